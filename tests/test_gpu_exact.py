@@ -83,6 +83,50 @@ def test_calibration_size_sandwich(oracle):
     assert (val[0] - raw) / val[0] < 0.01
 
 
+def _recursion(U, B, n):
+    """The recursion as defined, fp32, smallest b on ties: (budgets, optimum)."""
+    f = np.full(B + 1, -np.inf, np.float32)
+    f[0] = 0
+    choice = []
+    for row in U:
+        g, arg = np.full(B + 1, -np.inf, np.float32), np.zeros(B + 1, np.int64)
+        for b in range(min(n, B) + 1):
+            c = f[:B + 1 - b] + row[b]
+            better = c > g[b:]
+            g[b:][better], arg[b:][better] = c[better], b
+        f = g
+        choice.append(arg)
+    x, out = B, []
+    for arg in reversed(choice):
+        out.append(int(arg[x]))
+        x -= out[-1]
+    return out[::-1], f[B]
+
+
+@pytest.mark.parametrize("kind", ["rough", "steps", "decay", "falling"])
+@pytest.mark.parametrize("N,T,w,Bs", [(7, 130, 3, [1, 63, 64, 65, 128, 500, 7 * 127 - 1]),   # block and tile edges
+                                      (3, 4096, 1, [4095, 4096, 8191])])                      # the longest curves
+def test_budgets_of_the_full_recursion(kind, N, T, w, Bs):
+    """Blocks are skipped on a bound: the budgets and the optimum stay those of the full recursion, bit for bit, on
+    curves with and without a single maximum, with equal increments (ties) and falling ones."""
+    rng = np.random.default_rng(82)
+    inc = rng.exponential(size=(N, T)).astype(np.float32)
+    if kind == "rough":
+        inc -= 0.9
+    elif kind == "steps":
+        inc = np.floor(2 * inc)
+    elif kind == "decay":
+        inc *= (np.arange(1, T + 1) ** -rng.uniform(0.2, 1.6, size=(N, 1))).astype(np.float32)
+    else:
+        inc = -inc
+    U = np.zeros((N, T + 1), np.float32)
+    U[:, 1:] = np.cumsum(inc, axis=1)
+    b, _, val = gpu_exact(N, T, w, U, Bs)
+    for q, B in enumerate(Bs):
+        ref, best = _recursion(U, B, T - w)
+        assert list(b[q]) == ref and np.float32(val[q]) == best
+
+
 def test_unsupported_shapes():
     f = torch.empty(1, device="cuda")
     p = lukv.make_params(1, 1, 4, 1, 64, 64, 8, 1, "fp32", 33)      # 2 tokens per segment
