@@ -264,7 +264,7 @@ LUKV_API int lukv_compress_profile(const lukv_params_t* params, const void* q_wi
  * not call cudaMalloc at the point where budgets are needed -- a serving process whose
  * device memory is fully owned by its own pool allocator, or code running inside a region
  * where allocation is forbidden -- and so have no workspace to pass.  This entry point takes
- * none: the hull gains go to a fixed array of LUKV_STATIC_GAINS_MAX = 262144 floats (1 MiB)
+ * none: the hull goes to a fixed array for LUKV_STATIC_GAINS_MAX = 262144 curve segments (2.5 MiB)
  * that is part of the library image and is resident on every GPU that loads the library
  * until the process exits.  It calls no allocating routine.
  *
@@ -273,7 +273,7 @@ LUKV_API int lukv_compress_profile(const lukv_params_t* params, const void* q_wi
  *   - The first call on each device looks up the array's device address (a one-time runtime
  *     query, cached per device); make that first call before any stream capture begins.
  *   - All calls on a device share the one array.  It keeps the previous call's contents,
- *     which is harmless: every call rewrites the gains it uses before reading them.  Calls
+ *     which is harmless: every call rewrites what it uses before reading it.  Calls
  *     whose kernels can overlap on the GPU (different streams, or threads) race on it and
  *     must be serialised by the caller.
  *   - Arguments, results and error codes otherwise as lukv_allocate (no ws, ws_bytes).

@@ -1,13 +1,16 @@
 // Stage (b): global head-level budget allocation (paper Sec. 4.2, App. A.2).
-//   hull_kernel    PAVA projection of every head's curve increments onto a non-increasing,
-//                  non-negative sequence (Eq. "marginal_gain"); merge decisions equal to the
-//                  comparison of fp64 block means, gains fp64 with explicit round-to-nearest
-//                  operations, rounded once to fp32.
+//   hull_kernel    projection of every head's curve increments onto a non-increasing,
+//                  non-negative sequence (Eq. "marginal_gain": what pooling adjacent violators gives);
+//                  slopes compared as fp64 quotients, gains fp64 with explicit round-to-nearest
+//                  operations, rounded once to fp32.  The result is a short list per head: the
+//                  blocks of equal gain, steepest first.
 //   greedy_kernel  the marginal-utility greedy, computed as a weighted selection: the greedy
 //                  consumes curve segments in the order (gain desc, k asc, hid asc); the
-//                  kernel finds the segment at which the budget runs out by bisection over
-//                  the key bits (one binary search per head and bit) and gives every head
-//                  the capacity of its segments before that point.
+//                  kernel finds the gain at which the budget runs out by bisection over the
+//                  bits of the gain (one binary search per head and bit), then the segment
+//                  index and the head among the segments of exactly that gain.
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace lukv {
@@ -15,20 +18,237 @@ namespace {
 
 // ---- hull ----------------------------------------------------------------------------
 
+// Where the blocks of one curve go.
+struct HullOut {
+  float* gain;
+  unsigned short* start;
+};
+
+// A vertex walk: the blocks that pooling adjacent violators ends up with are the edges of the least concave majorant of
+// the points (k, U[k]); from a vertex i the next one is the point j > i with the steepest slope from i, the last of them
+// if several share it.  Slopes are compared in fp32; points whose slopes fp32 cannot tell apart are compared by their
+// correctly rounded fp64 quotients.  Once no slope is positive the rest is one block of gain 0.
+// Both forms below run it with one warp per curve and return the number of blocks.
+
+// The last point among the candidates of the warp (j < 0: none in this lane) with the largest fp64 quotient.
+__device__ __noinline__ int hull_resolve(float uj, int j, float ui, int i) {
+  double q = j >= 0 ? __ddiv_rn(__dsub_rn((double)uj, (double)ui), (double)(j - i)) : -INFINITY;
+#pragma unroll 1
+  for (int off = 16; off > 0; off >>= 1) {
+    const double qo = __shfl_xor_sync(0xffffffffu, q, off);
+    const int jo = __shfl_xor_sync(0xffffffffu, j, off);
+    if (qo > q || (qo == q && jo > j)) {
+      q = qo;
+      j = jo;
+    }
+  }
+  return j;
+}
+// The blocks found so far: lane l holds block 32 (count / 32) + l, its start and the curve there, until 32 are complete
+// or the walk ends.  A gain is an fp64 division, a chain of some 700 clocks: 32 of them at a time, off the walk's chain.
+struct HullBlocks {
+  int count = 0, start = 0;
+  float u = 0.f;
+  // the block that starts at point i (value ui) and ends at point `end` (value u_end); gain 0 when `flat`
+  __device__ __forceinline__ void add(int i, float ui, int end, float u_end, bool flat, bool last, int lane,
+                                      const HullOut& out) {
+    if (lane == (count & 31)) {
+      start = i;
+      u = ui;
+    }
+    ++count;
+    if (!last && (count & 31)) return;
+    const int base = (count - 1) & ~31, in = count - base;
+    int r = __shfl_down_sync(0xffffffffu, start, 1);
+    float ur = __shfl_down_sync(0xffffffffu, u, 1);
+    if (lane == in - 1) {
+      r = end;
+      ur = u_end;
+    }
+    if (lane < in) {
+      double mean = __ddiv_rn(__dsub_rn((double)ur, (double)u), (double)(r - start));
+      if (!(mean > 0.0) || (flat && lane == in - 1)) mean = 0.0;
+      out.gain[base + lane] = __double2float_rn(mean);
+      out.start[base + lane] = (unsigned short)start;
+    }
+  }
+};
+
+// P <= 32 NT: every point in a register, all slopes of a step at once, no branches: about 300 clocks a step.
+template <int NT>
+__device__ __forceinline__ int hull_walk_regs(const float* __restrict__ U, int P, int lane, HullOut out) {
+  float u[NT];
+#pragma unroll
+  for (int t = 0; t < NT; ++t) u[t] = lane + 32 * t < P ? __ldg(U + lane + 32 * t) : -INFINITY;
+  float ui = __shfl_sync(0xffffffffu, u[0], 0);
+  int i = 0;
+  HullBlocks blocks;
+#pragma unroll 1
+  while (i < P - 1) {
+    float sl[NT], best = -INFINITY;
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+      const int dist = lane + 32 * t - i;
+      sl[t] = dist > 0 ? __fdividef(u[t] - ui, (float)dist) : -INFINITY;
+      best = fmaxf(best, sl[t]);
+    }
+    best = warp_max(best);
+    const float near = best - 2e-6f * fabsf(best);
+    int mine = -1, found = 0;
+    float u_mine = 0.f;
+#pragma unroll
+    for (int t = 0; t < NT; ++t)
+      if (sl[t] >= near) {
+        mine = lane + 32 * t;
+        u_mine = u[t];
+        ++found;
+      }
+    int next = __reduce_max_sync(0xffffffffu, mine);
+    if (next < 0) next = P - 1;  // not a number: the rest is one block
+    if (__reduce_add_sync(0xffffffffu, found) > 1) {
+      // a lane with several candidates offers them one by one
+      int win = -1;
+      float u_win = 0.f;
+#pragma unroll 1
+      for (int t = 0; t < NT; ++t) {
+        float ut = u[0], st = sl[0];
+#pragma unroll
+        for (int x = 1; x < NT; ++x)
+          if (x == t) ut = u[x], st = sl[x];
+        const int at = hull_resolve(ut, st >= near ? lane + 32 * t : -1, ui, i);
+        if (at < 0) continue;
+        const float u_at = __shfl_sync(0xffffffffu, ut, at & 31);
+        // the winner of this turn against the winner so far
+        const int a2 = hull_resolve(lane == 0 ? u_at : u_win, lane == 0 ? at : lane == 1 ? win : -1, ui, i);
+        if (a2 == at) win = at, u_win = u_at;
+      }
+      next = win;
+      mine = win;
+      u_mine = u_win;
+    }
+    const bool flat = !(best > 0.f);
+    if (flat) next = P - 1;
+    const float u_next = __shfl_sync(0xffffffffu, u_mine, next & 31);
+    blocks.add(i, ui, next, u_next, flat, next == P - 1, lane, out);
+    ui = u_next;
+    i = next;
+  }
+  return blocks.count;
+}
+
+// Any P: the curve in shared memory `Us`, at most 32 chunks of 32 PPL points.  Chunk maxima of U bound the slope that any
+// point of a chunk can reach (one chunk per lane); the chunks whose bound comes up to the steepest slope found are
+// evaluated, PPL points per lane.  Returns -1 for a curve with many vertices, which hull_dense_kernel takes: a step costs
+// the same whether it skips one point or a thousand.  The walk stops after one vertex per 32 points, or before it starts
+// when more than three quarters of the increments are no larger than the one before (half of them on noisy curves).
+template <int PPL>
+__device__ __forceinline__ int hull_walk_chunks(const float* Us, int P, int lane, HullOut out) {
+  constexpr int C = 32 * PPL;
+  const int nchunk = (P + C - 1) / C;
+  float cmax = -INFINITY;  // maximum of chunk `lane`
+#pragma unroll 1
+  for (int c = 0; c < nchunk; ++c) {
+    float m = -INFINITY;
+#pragma unroll
+    for (int t = 0; t < PPL; ++t)
+      if (c * C + 32 * t + lane < P) m = fmaxf(m, Us[c * C + 32 * t + lane]);
+    m = warp_max(m);
+    if (lane == c) cmax = m;
+  }
+  int falls = 0;
+#pragma unroll 4
+  for (int j = lane + 1; j + 1 < P; j += 32) falls += Us[j + 1] - Us[j] <= Us[j] - Us[j - 1];
+  if (4 * __reduce_add_sync(0xffffffffu, falls) > 3 * P) return -1;
+  const int c_first = lane * C, c_last = min(c_first + C, P) - 1;
+  const float f_lane = (float)lane;
+  HullBlocks blocks;
+  int i = 0;
+  float ui = Us[0];
+#pragma unroll 1
+  while (i < P - 1) {
+    // slopes from i to the points j0 + lane + 32 t
+    auto slope = [&](int j0, int t) {
+      const float dist = f_lane + (float)(j0 + 32 * t - i);
+      const int j = j0 + 32 * t + lane;
+      return dist > 0.f && j < P ? __fdividef(Us[j] - ui, dist) : -INFINITY;
+    };
+    // upper bound of the slope from i to a point of this lane's chunk, above the rounding of the slopes
+    float bound = -INFINITY;
+    if (lane < nchunk && c_last > i) {
+      const float rise = cmax - ui;
+      bound = __fdividef(rise, (float)(rise > 0.f ? max(c_first, i + 1) - i : c_last - i));
+      bound += 1e-6f * fabsf(bound);
+    }
+    float best = -INFINITY, chunk_best = -INFINITY;
+    uint32_t todo = __ballot_sync(0xffffffffu, bound > -INFINITY);
+    int c = __ffs(__ballot_sync(0xffffffffu, bound == warp_max(bound)) & todo) - 1;
+    int next = P - 1;
+    if (c >= 0) {  // else not a number: the rest is one block
+#pragma unroll 1
+      for (;;) {
+        float m = -INFINITY;
+#pragma unroll
+        for (int t = 0; t < PPL; ++t) m = fmaxf(m, slope(c * C, t));
+        m = warp_max(m);
+        if (lane == c) chunk_best = m;
+        best = fmaxf(best, m);
+        todo &= ~(1u << c) & __ballot_sync(0xffffffffu, bound >= best);
+        if (!todo) break;
+        c = __ffs(todo) - 1;
+      }
+      // every point that may hold the steepest slope
+      const float near = best - 2e-6f * fabsf(best);
+      const uint32_t chunks = __ballot_sync(0xffffffffu, chunk_best >= near);
+      int mine = -1, found = 0;
+#pragma unroll 1
+      for (uint32_t left = chunks; left; left &= left - 1) {
+        const int j0 = (__ffs(left) - 1) * C;
+#pragma unroll
+        for (int t = 0; t < PPL; ++t)
+          if (slope(j0, t) >= near) {
+            mine = j0 + 32 * t + lane;
+            ++found;
+          }
+      }
+      next = __reduce_max_sync(0xffffffffu, mine);
+      if (__reduce_add_sync(0xffffffffu, found) > 1) {
+        next = -1;
+#pragma unroll 1
+        for (uint32_t left = chunks; left; left &= left - 1) {
+          const int j0 = (__ffs(left) - 1) * C;
+#pragma unroll 1
+          for (int t = 0; t < PPL; ++t) {
+            const int j = j0 + 32 * t + lane;
+            const int at = hull_resolve(j < P ? Us[j] : 0.f, slope(j0, t) >= near ? j : -1, ui, i);
+            if (at < 0) continue;
+            const int pick = lane == 0 ? at : lane == 1 ? next : -1;
+            next = hull_resolve(pick >= 0 ? Us[pick] : 0.f, pick, ui, i);
+          }
+        }
+      }
+    }
+    const bool flat = !(best > 0.f);
+    if (flat) next = P - 1;
+    if (blocks.count > P / 32) return -1;
+    const float u_next = Us[next];
+    blocks.add(i, ui, next, u_next, flat, next == P - 1, lane, out);
+    ui = u_next;
+    i = next;
+  }
+  return blocks.count;
+}
+
+// ---- curves with many vertices: pool adjacent violators on 32 runs, then join -------------------------------------
+
 // mean of block 1 <= mean of block 2, where a block's mean is (its curve rise) / (its length) and
 // the rises are differences of two fp32 curve values: decided exactly as the comparison of the two
-// correctly rounded fp64 quotients.  Three tiers, cheapest first (the fp64 pipe is slow, and the
-// walk below is one dependent chain):
+// correctly rounded fp64 quotients.  Three tiers, cheapest first:
 //   fp32 cross products, when they are further apart than fp32 rounding can explain;
 //   fp64 cross products, when they are clearly apart;
 //   the fp64 quotients themselves.
+// (the last two out of line: they are rare, and an fp64 operation costs the walk some 50 clocks)
 // Block 1 rises from u_l1 to u_r1 over len1 points, block 2 from u_l2 to u_r2 over len2.
-__device__ __forceinline__ bool mean_le(float u_l1, float u_r1, int len1, float u_l2, float u_r2, int len2) {
-  const float fa = u_r1 - u_l1, fb = (float)len1, fc = u_r2 - u_l2, fd = (float)len2;
-  const float q1 = fa * fd, q2 = fc * fb;
-  const float ftol = 4e-7f * fmaxf(fabsf(q1), fabsf(q2));  // each product carries two roundings of 2^-24
-  if (q1 < q2 - ftol) return true;
-  if (q1 > q2 + ftol) return false;
+__device__ __noinline__ bool mean_le_f64(float u_l1, float u_r1, int len1, float u_l2, float u_r2, int len2) {
   const double a = __dsub_rn((double)u_r1, (double)u_l1), b = (double)len1;
   const double c = __dsub_rn((double)u_r2, (double)u_l2), d = (double)len2;
   const double p1 = __dmul_rn(a, d), p2 = __dmul_rn(c, b);
@@ -38,280 +258,706 @@ __device__ __forceinline__ bool mean_le(float u_l1, float u_r1, int len1, float 
   if (diff > tol) return false;
   return __ddiv_rn(a, b) <= __ddiv_rn(c, d);
 }
+__device__ __forceinline__ bool mean_le(float u_l1, float u_r1, int len1, float u_l2, float u_r2, int len2) {
+  const float q1 = (u_r1 - u_l1) * (float)len2, q2 = (u_r2 - u_l2) * (float)len1;
+  const float diff = q1 - q2;
+  // each product carries two roundings of 2^-24, the difference one
+  if (fabsf(diff) > 5e-7f * fmaxf(fabsf(q1), fabsf(q2))) return diff < 0.f;
+  return mean_le_f64(u_l1, u_r1, len1, u_l2, u_r2, len2);
+}
 
-// Shared memory of one warp of the hull kernel: the stack of block starts, [P] 16-bit indices.
-__host__ __device__ inline size_t hull_bytes_per_warp(int P) { return ((size_t)P * 2 + 15) & ~(size_t)15; }
+// Increments per lane: an odd count, so that the lanes' runs start in different banks.
+__host__ __device__ inline int hull_run(int P) { return ((P - 1 + 31) / 32) | 1; }
+inline size_t hull_dense_smem_bytes(int P) { return (size_t)P * 4 + (size_t)hull_run(P) * 64 + 128; }
 
-// One warp per curve.  Lane 0 runs the pool-adjacent-violators stack (the sequence of merge
-// decisions is the algorithm; it is serial by nature).  The walk is one dependent chain, so what it
-// touches per step is kept short: the curve values at the starts of the top block and of the
-// current block live in registers, the next curve point is requested one step ahead (the curve is
-// read through L1: the walk streams it, a pop re-reads a point that was read not long before), and
-// the stack of block starts is the only thing in shared memory (2 bytes per point, so that many
-// warps fit an SM when thousands of long curves are projected at once).  The other lanes join for
-// the output: one block of the result per lane at a time.
-// Stack entries are block start points; a block's end is the next entry's start.
-__global__ void hull_kernel(const float* __restrict__ curves, float* __restrict__ gains, int N, int P) {
-  extern __shared__ __align__(16) unsigned char hull_smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int warps = blockDim.x >> 5;
-  const int hid = blockIdx.x * warps + warp;
-  if (hid >= N) return;  // whole warps leave together; only __syncwarp is used below
+// One warp per curve.  Every lane runs the pool-adjacent-violators stack over its run of the curve (a merge or a push per
+// turn, so that the lanes stay together), which leaves the hull of the run as a list of block starts.  Then neighbouring
+// hulls are joined pairwise, five times: the block across the joint absorbs blocks from the left while their mean does
+// not exceed its own and from the right while its own does not exceed theirs, which is where the serial algorithm ends
+// up as well (the projection is unique).
+__global__ void hull_dense_kernel(const float* __restrict__ curves, HullLists lists, int P) {
+  extern __shared__ float hull_smem[];
+  const int hid = blockIdx.x, lane = threadIdx.x;
+  pdl_launch_dependents();
+  pdl_wait();
+  if (lists.count[hid] >= 0) return;  // the vertex walk took this curve
   const float* U = curves + (size_t)hid * P;
-  unsigned short* Ls = reinterpret_cast<unsigned short*>(hull_smem + (size_t)warp * hull_bytes_per_warp(P));
+  const int run = hull_run(P);
+  float* Us = hull_smem;
+  unsigned short* Ls = reinterpret_cast<unsigned short*>(Us + P);  // [32][run]
+  volatile unsigned short* first = Ls + 32 * run;                  // [32] first entry of the lane's list
+  volatile unsigned short* end = first + 32;                       // [32] one past its last entry
+#pragma unroll 16
+  for (int i = lane; i < P; i += 32) Us[i] = __ldg(U + i);
+  __syncwarp();
+
+  // the lane's own run: increments k0 .. k1-1
+  const int k0 = min(lane * run, P - 1), k1 = min(k0 + run, P - 1);
+  unsigned short* own = Ls + lane * run;
   int sp = 0;
-  if (lane == 0) {
-    int top_l = 0;        // start of the block on top of the stack; it ends where the current block starts
-    float u_top = 0.f;    // U[top_l]
-    float u_k = __ldg(U), u_next = __ldg(U + 1);
-    for (int k = 0; k + 1 < P; ++k) {
-      const float u_ahead = k + 2 < P ? __ldg(U + k + 2) : 0.f;  // for the next step
-      int cur_l = k;
-      float u_cur = u_k;  // U[cur_l]
-      while (sp > 0 && mean_le(u_top, u_cur, cur_l - top_l, u_cur, u_next, k + 1 - cur_l)) {
+  if (k0 < k1) {
+    int k = k0, cur_l = k0, top_l = k0;
+    float u_cur = Us[k0], u_next = Us[k0 + 1], u_top = u_cur;
+    // the current block is [cur_l, k+1); below it on the stack lies [top_l, cur_l)
+    while (k < k1) {
+      if (sp > 0 && mean_le(u_top, u_cur, cur_l - top_l, u_cur, u_next, k + 1 - cur_l)) {
         cur_l = top_l;
         u_cur = u_top;
         --sp;
         if (sp > 0) {
-          top_l = Ls[sp - 1];
-          u_top = __ldg(U + top_l);
+          top_l = own[sp - 1];
+          u_top = Us[top_l];
         }
+      } else {
+        own[sp++] = (unsigned short)cur_l;
+        top_l = cur_l;
+        u_top = u_cur;
+        ++k;
+        cur_l = k;
+        u_cur = u_next;
+        if (k < k1) u_next = Us[k + 1];
       }
-      Ls[sp++] = (unsigned short)cur_l;
-      top_l = cur_l;
-      u_top = u_cur;
-      u_k = u_next;
-      u_next = u_ahead;
     }
   }
-  sp = __shfl_sync(0xffffffffu, sp, 0);
-  __syncwarp();
-  float* out = gains + (size_t)hid * (P - 1);
-  for (int i = lane; i < sp; i += 32) {
-    const int l = Ls[i];
-    const int r = (i + 1 < sp) ? (int)Ls[i + 1] : P - 1;
-    const double mean = __ddiv_rn(__dsub_rn((double)__ldg(U + r), (double)__ldg(U + l)), (double)(r - l));
-    const float g = __double2float_rn(mean > 0.0 ? mean : 0.0);
-    for (int k = l; k < r; ++k) out[k] = g;
+  first[lane] = 0;
+  end[lane] = (unsigned short)sp;
+
+  // join hulls of `width` runs pairwise; the leader of a pair walks
+#pragma unroll 1
+  for (int width = 1; width < 32; width <<= 1) {
+    __syncwarp();
+    if ((lane & (2 * width - 1)) == 0) {
+      const int last = lane + 2 * width - 1, stop = min((last + 1) * run, P - 1);  // the right hull ends at point `stop`
+      int la = lane + width - 1, lb = lane + width;
+      while (la > lane && first[la] == end[la]) --la;
+      while (lb <= last && first[lb] == end[lb]) ++lb;
+      if (lb <= last) {
+        // start of the block behind entry `at` of list `list`, or the end of the right hull
+        auto next_right = [&](int& list, int& at) {
+          ++at;
+          while (list <= last && at == end[list]) {
+            ++list;
+            if (list <= last) at = first[list];
+          }
+          return list <= last ? (int)Ls[list * run + at] : stop;
+        };
+        int ea = end[la];                                  // the left hull's last block is entry ea - 1 of list la
+        int l = Ls[la * run + ea - 1], m = Ls[lb * run + first[lb]];
+        int rl = lb, ra = first[lb];                       // where the right hull goes on
+        int r = next_right(rl, ra);
+        float ul = Us[l], um = Us[m], ur = Us[r];
+        if (mean_le(ul, um, m - l, um, ur, r - m)) {
+          bool more = true;
+          while (more) {  // the joint block is [l, r)
+            more = false;
+            int pl = la, pe = ea - 1;                      // the block before it
+            while (pl > lane && pe == first[pl]) {
+              --pl;
+              pe = end[pl];
+            }
+            if (pe > first[pl]) {
+              const int p = Ls[pl * run + pe - 1];
+              const float up = Us[p];
+              if (mean_le(up, ul, l - p, ul, ur, r - l)) {
+                end[la] = (unsigned short)(ea - 1);        // l is no block start any more
+                la = pl;                                   // the lists in between are empty
+                ea = pe;
+                l = p;
+                ul = up;
+                more = true;
+              }
+            }
+            if (r < stop) {
+              int nl = rl, na = ra;
+              const int r2 = next_right(nl, na);
+              const float u2 = Us[r2];
+              if (mean_le(ul, ur, r - l, ur, u2, r2 - r)) {
+                r = r2;
+                ur = u2;
+                rl = nl;
+                ra = na;
+                more = true;
+              }
+            }
+          }
+          // the right hull keeps its blocks from entry ra of list rl on
+          for (int i = lb; i < rl && i <= last; ++i) first[i] = end[i];
+          if (rl <= last) first[rl] = (unsigned short)ra;
+        }
+      }
+    }
   }
+  __syncwarp();
+
+  // the lists one behind the other: block starts and gains
+  const int f0 = first[lane], cnt = end[lane] - f0;
+  int incl = cnt;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int o = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += o;
+  }
+  const int total = __shfl_sync(0xffffffffu, incl, 31);
+  // end of this lane's last block: the first block start of the next non-empty list
+  const uint32_t filled = __ballot_sync(0xffffffffu, cnt > 0);
+  const uint32_t above = lane < 31 ? filled & ~((2u << lane) - 1u) : 0u;
+  const int my_first = cnt > 0 ? (int)own[f0] : 0;
+  const int next_first = __shfl_sync(0xffffffffu, my_first, above ? __ffs(above) - 1 : 0);
+  const int tail = above ? next_first : P - 1;
+  float* g_out = lists.gain + (size_t)hid * (P - 1) + (incl - cnt);
+  unsigned short* s_out = lists.start + (size_t)hid * (P - 1) + (incl - cnt);
+  for (int i = 0; i < cnt; ++i) {
+    const int l = own[f0 + i], r = i + 1 < cnt ? (int)own[f0 + i + 1] : tail;
+    const double mean = __ddiv_rn(__dsub_rn((double)Us[r], (double)Us[l]), (double)(r - l));
+    g_out[i] = __double2float_rn(mean > 0.0 ? mean : 0.0);
+    s_out[i] = (unsigned short)l;
+  }
+  if (lane == 0) lists.count[hid] = total;
+}
+
+constexpr int kHullRegsMaxP = 32 * 17;
+
+__device__ __forceinline__ int hull_walk_short(const float* U, int P, int lane, HullOut out) {
+  if (P <= 96) return hull_walk_regs<3>(U, P, lane, out);
+  if (P <= 160) return hull_walk_regs<5>(U, P, lane, out);
+  if (P <= 288) return hull_walk_regs<9>(U, P, lane, out);
+  return hull_walk_regs<17>(U, P, lane, out);
+}
+
+// One warp (a block of its own) per curve.
+// Bound by the latency of a step; a curve has few vertices: 6 of 257 points on the benchmark's curves, 53 of 4001 on the
+// calibration curves.  Measured against one serial stack walk per curve: 256 curves of 257 points 59 -> 5 us, 7680 of 4001
+// 3.07 -> 0.29 ms; pooling on 32 runs per curve (below) takes 0.5 ms there, but is the faster one on concave curves.
+template <int PPL>
+__global__ void hull_kernel(const float* __restrict__ curves, HullLists lists, int P) {
+  extern __shared__ float hull_smem[];
+  const int hid = blockIdx.x, lane = threadIdx.x;
+  const float* U = curves + (size_t)hid * P;
+  const HullOut out = {lists.gain + (size_t)hid * (P - 1), lists.start + (size_t)hid * (P - 1)};
+  pdl_launch_dependents();
+  int count;
+  if (PPL == 0) {
+    count = hull_walk_short(U, P, lane, out);
+  } else {
+#pragma unroll 16
+    for (int i = lane; i < P; i += 32) hull_smem[i] = __ldg(U + i);
+    __syncwarp();
+    count = hull_walk_chunks<PPL == 0 ? 1 : PPL>(hull_smem, P, lane, out);
+  }
+  if (lane == 0) lists.count[hid] = count;
 }
 
 // ---- greedy --------------------------------------------------------------------------
 
 constexpr int kGreedyMaxThreads = 1024;
-constexpr int kSeqPerLaunch = 32;
+constexpr int kGreedyMaxGroups = 8;
+constexpr int kSeqPerLaunch = 128;
 
 struct GreedyArgs {
   long long budget[kSeqPerLaunch];    // B_q
   long long row_base[kSeqPerLaunch];  // packed rows before sequence q
   int T[kSeqPerLaunch];               // context length of sequence q (the curve grid is T/(P-1) tokens per segment)
   int floor_tok[kSeqPerLaunch];       // tokens every head of sequence q keeps at least
-  int seq0;                           // first sequence of this launch
+  int seq0, count;                    // sequences seq0 .. seq0 + count - 1
 };
 
 struct SetStride {
-  size_t gains, budgets, offsets;  // elements between consecutive curve sets
+  size_t budgets, offsets;  // elements between consecutive curve sets
 };
-
-// Sort key of segment (hid,k): ascending key order == greedy consumption order.
-__device__ __forceinline__ unsigned long long seg_key(float gain, unsigned k, unsigned hid, unsigned N) {
-  return ((unsigned long long)(~__float_as_uint(gain)) << 32) | (unsigned long long)(k * N + hid);
-}
 
 // Tokens for sale in segments [0,c) of a head whose first `floor_tok` tokens were handed to it up
 // front (the minimum retention of App. E; 0 = none).
-__device__ __forceinline__ long long capsum(int c, int seg, int n, int floor_tok) {
-  long long t = (long long)c * seg;
-  t = (t < n ? t : (long long)n) - floor_tok;
-  return t > 0 ? t : 0;
+__device__ __forceinline__ int capsum(int c, int seg, int n, int floor_tok) {
+  return max(min(c * seg, n) - floor_tok, 0);  // c * seg <= T
 }
 
-// Block-wide sum; every thread gets the result.  `buf` holds one value per warp.  One barrier per
-// call is enough only if consecutive calls use different buffers: the caller alternates between two.
-__device__ __forceinline__ long long block_sum_ll(long long v, long long* buf) {
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  if ((threadIdx.x & 31) == 0) buf[threadIdx.x >> 5] = v;
-  __syncthreads();
-  long long total = 0;
-  const int warps = blockDim.x >> 5;
-  for (int x = 0; x < warps; ++x) total += buf[x];
-  return total;
-}
-
-// One CTA per (sequence, curve set), one thread per head (a CTA of fewer threads than heads loops).
-// The greedy buys segments in ascending key order until the budget is spent; the kernel finds the
-// key at which that happens by bisection over the 64 key bits.  Within a head the keys increase
-// with k (gains are non-increasing), so the segments of a head that share the key prefix fixed so
-// far form a range [lo,hi), segments before lo are bought, and inside the range the next key bit is
-// 0 up to some index and 1 from there on: one binary search per head and bit finds that index (no
-// search at all when the range's two ends agree), the capacities below it are summed over the
-// heads, and the budget decides which half holds the cut.  Keys are unique, so after the last bit
-// one segment remains: the partially bought one.
-//
-// blockIdx.y selects one of several independent curve sets (the calibration queries of the
-// offline profile, which share the budgets): set i reads gains + i*set.gains, writes
-// budgets + i*set.budgets and offsets + i*set.offsets.  The hot path launches one set.
-__global__ void __launch_bounds__(kGreedyMaxThreads) greedy_kernel(const float* __restrict__ gains, GreedyArgs args,
-                                                                   int32_t* __restrict__ budgets,
-                                                                   int32_t* __restrict__ offsets, SetStride set,
-                                                                   int N, int P, int w) {
-  // the sequence's own grid: n rankable positions, seg tokens per curve segment, nseg segments with capacity
-  const int n = args.T[blockIdx.x] - w, seg = args.T[blockIdx.x] / (P - 1), nseg = (n + seg - 1) / seg;
-  const int floor_tok = args.floor_tok[blockIdx.x];
-  gains += (size_t)blockIdx.y * set.gains;
-  budgets += (size_t)blockIdx.y * set.budgets;
-  offsets += (size_t)blockIdx.y * set.offsets;
-  extern __shared__ __align__(16) unsigned char greedy_smem[];
-  int* lo = reinterpret_cast<int*>(greedy_smem);  // [N]
-  int* hi = lo + N;                               // [N]
-  int* mid = hi + N;                              // [N]
-  __shared__ long long sum_buf[2][kGreedyMaxThreads / 32];
-  __shared__ long long warp_sums[kGreedyMaxThreads / 32];
-
-  const int q = args.seq0 + blockIdx.x;
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  const int G1 = P - 1;
-  long long R = args.budget[blockIdx.x] - (long long)N * floor_tok;  // the floor is spent before the greedy
-  const bool all_taken = (long long)N * (n - floor_tok) <= R;
-  for (int h = tid; h < N; h += nthr) {
-    lo[h] = all_taken ? nseg : 0;
-    hi[h] = nseg;
+// Threads that solve one problem together: whole warps, with a barrier of their own.
+struct Group {
+  int tid, nthr, bar;
+  __device__ __forceinline__ void sync() const {
+    if (nthr == 32) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(bar), "r"(nthr) : "memory");
   }
-  // (each thread only ever touches the heads it owns, so lo/hi/mid need no barrier of their own)
+};
+
+// Sums of two values over the group; every thread gets them.  `buf` holds one pair per warp.  One barrier per
+// call is enough only if consecutive calls use different buffers: the caller alternates between two.
+__device__ __forceinline__ uint2 group_sum2(unsigned a, unsigned b, uint2* buf, const Group& g) {
+  a = __reduce_add_sync(0xffffffffu, a);
+  b = __reduce_add_sync(0xffffffffu, b);
+  const int warps = g.nthr >> 5, lane = g.tid & 31;
+  if (warps == 1) return make_uint2(a, b);
+  if (lane == 0) buf[g.tid >> 5] = make_uint2(a, b);
+  g.sync();
+  const uint2 v = lane < warps ? buf[lane] : make_uint2(0u, 0u);
+  return make_uint2(__reduce_add_sync(0xffffffffu, v.x), __reduce_add_sync(0xffffffffu, v.y));
+}
+
+// Exclusive scan over the group in thread order.  `sums` holds one value per warp; barriers inside.
+__device__ __forceinline__ int group_scan(int v, int* sums, const Group& g) {
+  const int lane = g.tid & 31, wv = g.tid >> 5;
+  int incl = v;
+#pragma unroll
+  for (int off = 1; off < 32; off <<= 1) {
+    const int o = __shfl_up_sync(0xffffffffu, incl, off);
+    if (lane >= off) incl += o;
+  }
+  g.sync();  // the previous scan's sums are read
+  if (lane == 31) sums[wv] = incl;
+  g.sync();
+  const int before = __reduce_add_sync(0xffffffffu, lane < wv ? sums[lane] : 0);
+  return before + incl - v;
+}
+
+// The lists of a curve set as a CTA reads them: staged in shared memory (one behind the other, head h from at[h] on, each
+// with one more entry that holds the end of the curve) or in place.
+template <bool STAGED>
+struct ListView {
+  const float* gain_;
+  const unsigned short* start_;
+  const int* at_;     // staged: [N + 1] where a head's list starts
+  const int* count_;  // in place
+  int G1;
+  __device__ int blocks(int h) const { return STAGED ? at_[h + 1] - at_[h] - 1 : count_[h]; }
+  __device__ float gain(int h, int i) const { return STAGED ? gain_[at_[h] + i] : gain_[(size_t)h * G1 + i]; }
+  __device__ int start(int h, int i) const {  // first segment of block i; the end of the curve behind the last block
+    if (STAGED) return (int)start_[at_[h] + i];
+    return i < count_[h] ? (int)start_[(size_t)h * G1 + i] : G1;
+  }
+};
+
+struct GreedyShared {
+  uint2 sum[2][32];
+  int scan[32];
+  unsigned cut[2];
+};
+constexpr int kGreedyCountMax = 256;  // blocks in all up to which the cut is found by counting
+
+// One problem: sequence i of `args` on the lists of one curve set, by the threads of a group; thread t owns the heads
+// [t*per, (t+1)*per) (ONE: the head t).  The greedy buys segments in the order (gain desc, k asc, hid asc) until the
+// budget is spent.
+//   gain  With few blocks every thread adds up the capacities of the blocks that are steeper than its own: the block at
+//         which the sum passes the budget names the gain.  Otherwise by bisection over the bits of the gain: the lists
+//         are sorted by falling gain, so the blocks of a head whose gain agrees with the bits fixed so far form a range
+//         [lo,hi); inside it the next bit is 1 up to some index and 0 from there on: one binary search per head and bit
+//         (none when the range's ends agree).  The capacities of the 1s, summed over the heads, and the budget decide
+//         which half holds the cut.  The bits end early when a single block is left.
+//   k     Of the segments with exactly that gain (a range [a,e) per head) those with the smaller index are bought
+//         first: the index K at which the budget runs out, by bisection; not needed when one head has such segments.
+//   hid   Segment K of the heads that have it, in head order, each whole while the budget lasts.
+// lo, hi, mid: [N] words per head (unused when ONE).  weight: room for kGreedyCountMax words when STAGED.
+template <bool STAGED, bool ONE>
+__device__ __forceinline__ void greedy_problem(const ListView<STAGED> lists, const GreedyArgs& args, int i, int N, int w,
+                                               int* lo, int* hi, int* mid, int* weight, GreedyShared& sh,
+                                               const Group grp, int32_t* __restrict__ budgets, int32_t* __restrict__ offsets) {
+  const int tid = grp.tid, nthr = grp.nthr, G1 = lists.G1;
+  const int per = ONE ? 1 : (N + nthr - 1) / nthr;
+  const int h_begin = min(N, tid * per), h_end = min(N, h_begin + per);
+  int lo1 = 0, hi1 = 0, mid1 = 0;
+  auto LO = [&](int h) -> int& { return ONE ? lo1 : lo[h]; };
+  auto HI = [&](int h) -> int& { return ONE ? hi1 : hi[h]; };
+  auto MID = [&](int h) -> int& { return ONE ? mid1 : mid[h]; };
+  // the sequence's own grid: n rankable positions, seg tokens per curve segment, nseg segments with capacity
+  const int n = args.T[i] - w, seg = args.T[i] / G1, nseg = (n + seg - 1) / seg;
+  const int floor_tok = args.floor_tok[i], q = args.seq0 + i;
+  const long long left = args.budget[i] - (long long)N * floor_tok;  // the floor is spent before the greedy
+  const bool all_taken = (long long)N * (n - floor_tok) <= left;
+  unsigned R = (unsigned)left;  // budgets are below 2^31
+  unsigned round = 0;
   if (!all_taken) {
-    // the low key word is k*N + hid < N*(P-1): its bits from idx_bits up are zero in every key, a pass over
-    // them would change nothing
-    int idx_bits = 0;
-    while (idx_bits < 32 && ((unsigned long long)N * (unsigned)G1) >> idx_bits) ++idx_bits;
-    int round = 0;  // executed iterations: selects the sum buffer (the skipped bits must not count)
-    for (int bit = 63; bit >= 0; --bit) {
-      if (bit < 32 && bit >= idx_bits) continue;
-      long long local = 0;
-      for (int h = tid; h < N; h += nthr) {
-        const int l = lo[h], r = hi[h];
-        int m = l;
-        if (l < r) {
-          const float* g = gains + (size_t)h * G1;
-          auto bit_at = [&](int k) { return (int)((seg_key(__ldg(g + k), k, h, N) >> bit) & 1ull); };
-          if (bit_at(l)) {
-            m = l;
-          } else if (!bit_at(r - 1)) {
-            m = r;
-          } else {
-            int a = l, b = r - 1;  // bit(a) == 0, bit(b) == 1
-            while (b - a > 1) {
-              const int c = (a + b) >> 1;
-              if (bit_at(c)) b = c; else a = c;
-            }
-            m = b;
-          }
+    const int total = STAGED ? lists.at_[N] - N : kGreedyCountMax + 1;
+    if (STAGED && total <= kGreedyCountMax) {
+      // entries of all lists, the ends of the curves among them as blocks without capacity
+      const int entries = total + N;
+      for (int h = tid >> 5; h < N; h += nthr >> 5)
+        for (int e = lists.at_[h] + (tid & 31); e < lists.at_[h + 1]; e += 32) {
+          const bool end = e + 1 == lists.at_[h + 1];
+          weight[e] = end ? 0 : capsum(lists.start_[e + 1], seg, n, floor_tok) - capsum(lists.start_[e], seg, n, floor_tok);
         }
-        mid[h] = m;
-        local += capsum(m, seg, n, floor_tok) - capsum(l, seg, n, floor_tok);
+      grp.sync();
+      for (int e = tid; e < entries; e += nthr) {
+        const float g = lists.gain_[e];
+        unsigned steeper = 0, same = 0;
+#pragma unroll 4
+        for (int x = 0; x < entries; ++x) {
+          const float gx = lists.gain_[x];
+          const unsigned wx = (unsigned)weight[x];
+          steeper += gx > g ? wx : 0u;
+          same += gx == g ? wx : 0u;
+        }
+        if (steeper <= R && R < steeper + same) {  // one gain; every thread that holds it writes the same
+          sh.cut[0] = __float_as_uint(g);
+          sh.cut[1] = R - steeper;
+        }
       }
-      const long long tokens0 = block_sum_ll(local, sum_buf[round++ & 1]);
-      if (tokens0 > R) {
-        for (int h = tid; h < N; h += nthr) hi[h] = mid[h];
-      } else {
-        R -= tokens0;
-        for (int h = tid; h < N; h += nthr) lo[h] = mid[h];
+      grp.sync();
+      const float g = __uint_as_float(sh.cut[0]);
+      R = sh.cut[1];
+      for (int h = h_begin; h < h_end; ++h) {
+        const int c = lists.blocks(h);
+        int l = 0;
+        while (l < c && lists.gain(h, l) > g) ++l;
+        int r = l;
+        while (r < c && lists.gain(h, r) == g) ++r;
+        LO(h) = l;
+        HI(h) = r;
+      }
+    } else {
+      for (int h = h_begin; h < h_end; ++h) {
+        LO(h) = 0;
+        HI(h) = lists.blocks(h);
+      }
+#pragma unroll 1
+      for (int bit = 30; bit >= 0; --bit) {  // gains are not negative
+        unsigned local = 0, alive = 0;
+        for (int h = h_begin; h < h_end; ++h) {
+          const int l = LO(h), r = HI(h);
+          int m = l;
+          if (l < r) {
+            alive += r - l;
+            auto bit_at = [&](int k) { return (__float_as_uint(lists.gain(h, k)) >> bit) & 1u; };
+            const unsigned bl = bit_at(l), br = bit_at(r - 1);
+            if (bl) {
+              m = r;
+              if (!br) {
+                int x = l, y = r - 1;  // bit(x) == 1, bit(y) == 0
+#pragma unroll 1
+                while (y - x > 1) {
+                  const int c = (x + y) >> 1;
+                  if (bit_at(c)) x = c; else y = c;
+                }
+                m = y;
+              }
+              local += capsum(lists.start(h, m), seg, n, floor_tok) - capsum(lists.start(h, l), seg, n, floor_tok);
+            }
+          }
+          MID(h) = m;
+        }
+        const uint2 sum = group_sum2(local, alive, sh.sum[round++ & 1], grp);
+        if (sum.y <= 1) break;  // the gain of the one block left
+        if (sum.x > R) {
+          for (int h = h_begin; h < h_end; ++h) HI(h) = MID(h);
+        } else {
+          R -= sum.x;
+          for (int h = h_begin; h < h_end; ++h) LO(h) = MID(h);
+        }
       }
     }
   }
-
-  // budgets, then offsets = row_base + exclusive scan of (budget + w)
-  const int per = (N + nthr - 1) / nthr;
-  const int h_begin = min(N, tid * per), h_end = min(N, h_begin + per);
-  __syncthreads();  // the scan below re-partitions the heads over the threads
-  long long local = 0;
+  // segments [a,e) of every head have the gain at which the budget runs out, those before a are bought
+  unsigned with = 0;
   for (int h = h_begin; h < h_end; ++h) {
-    long long b = floor_tok + capsum(lo[h], seg, n, floor_tok);
-    if (hi[h] > lo[h]) b += R;  // the one partially bought segment
-    mid[h] = (int)b;
-    local += b + w;
+    int a = nseg, e = nseg;
+    if (!all_taken) {
+      a = min(lists.start(h, LO(h)), nseg);
+      e = HI(h) > LO(h) ? min(lists.start(h, HI(h)), nseg) : a;
+    }
+    LO(h) = a;
+    HI(h) = e;
+    with += e > a;
   }
-  long long incl = local;
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const long long o = __shfl_up_sync(0xffffffffu, incl, off);
-    if ((tid & 31) >= off) incl += o;
+  const bool tie = group_sum2(with, 0u, sh.sum[round++ & 1], grp).x > 1;
+  int K = 0, rank = 0;
+  unsigned cap_K = 0;
+  if (tie) {
+    // largest K with (tokens of the segments below K in the ranges) <= R
+    auto below = [&](int k) {
+      unsigned local = 0;
+      for (int h = h_begin; h < h_end; ++h) {
+        const int a = LO(h), e = HI(h);
+        local += capsum(min(max(k, a), e), seg, n, floor_tok) - capsum(a, seg, n, floor_tok);
+      }
+      return group_sum2(local, 0u, sh.sum[round++ & 1], grp).x;
+    };
+    int top = 1;
+    while (top <= nseg) top <<= 1;
+    unsigned spent = 0;
+#pragma unroll 1
+    for (int b = top >> 1; b > 0; b >>= 1) {
+      if (K + b > nseg) continue;
+      const unsigned s = below(K + b);
+      if (s <= R) {
+        K += b;
+        spent = s;
+      }
+    }
+    R -= spent;
+    cap_K = (unsigned)(capsum(K + 1, seg, n, floor_tok) - capsum(K, seg, n, floor_tok));
+    int mine = 0;
+    for (int h = h_begin; h < h_end; ++h) mine += LO(h) <= K && K < HI(h);
+    rank = group_scan(mine, sh.scan, grp);
   }
-  if ((tid & 31) == 31) warp_sums[tid >> 5] = incl;
-  __syncthreads();
-  long long before = 0;
-  for (int wv = 0; wv < (tid >> 5); ++wv) before += warp_sums[wv];
-  long long run = args.row_base[blockIdx.x] + before + incl - local;
+  // budgets, then offsets = row_base + exclusive scan of (budget + w)
+  int rows = 0;
+  for (int h = h_begin; h < h_end; ++h) {
+    const int a = LO(h), e = HI(h);
+    int b = floor_tok + capsum(a, seg, n, floor_tok);
+    if (tie) {
+      b = floor_tok + capsum(min(max(K, a), e), seg, n, floor_tok);
+      if (a <= K && K < e) {
+        const unsigned before = (unsigned)rank++ * cap_K;
+        b += before < R ? (int)min(cap_K, R - before) : 0;
+      }
+    } else if (e > a) {
+      b += (int)R;
+    }
+    MID(h) = b;
+    rows += b + w;
+  }
+  long long run = args.row_base[i] + group_scan(rows, sh.scan, grp);
   if (q == 0 && tid == 0) offsets[0] = 0;
   for (int h = h_begin; h < h_end; ++h) {
-    budgets[(size_t)q * N + h] = mid[h];
-    run += mid[h] + w;
+    budgets[(size_t)q * N + h] = MID(h);
+    run += MID(h) + w;
     offsets[(size_t)q * N + h + 1] = (int32_t)run;
   }
+  grp.sync();  // the shared words start over
+}
+
+// Shared memory of the greedy kernel: at [N+1], gain and start [cap + N] and the counted weights when lists are staged;
+// lo, hi, mid [N] when a thread owns several heads.
+inline size_t greedy_smem_bytes(int N, int cap, int groups, bool one) {
+  const size_t e = (size_t)cap + N, weights = (size_t)groups * (kGreedyCountMax + N);
+  return (cap > 0 ? ((size_t)N + 1) * 4 + e * 4 + ((e * 2 + 3) & ~(size_t)3) + weights * 4 : 0) +
+         (one ? 0 : (size_t)N * 12);
+}
+
+// One CTA per (share of the sequences, curve set), of one or more groups of `group` threads, each with a sequence of its
+// own at a time.  The lists of a set are short (6 blocks a head on the benchmark's curves, 53 of 4000 on the calibration
+// curves) and are staged in shared memory once for all sequences of the CTA when they fit, else read through L1.
+// Bound by latency, up to 31 rounds of a search and a group-wide sum, hence several groups per CTA where there are that
+// many problems.  65536 segments in 256 heads beside the scorer: 91 us with a search per head for each of the 64
+// bits of (gain, k, hid) over expanded segments, 34 us now; 2970 problems of 256 x 4000 segments 0.6 -> 0.16 ms.
+// blockIdx.y selects one of several independent curve sets (the calibration queries of the offline profile, which
+// share the budgets): set i reads the lists of curves i*N .., writes budgets + i*set.budgets and offsets +
+// i*set.offsets.  The hot path launches one set.
+template <bool ONE>
+__global__ void __launch_bounds__(kGreedyMaxThreads) greedy_kernel(HullLists lists, const __grid_constant__ GreedyArgs args,
+                                                                   int32_t* __restrict__ budgets,
+                                                                   int32_t* __restrict__ offsets, SetStride set,
+                                                                   int N, int P, int w, int cap, int group) {
+  extern __shared__ __align__(16) unsigned char greedy_smem[];
+  __shared__ GreedyShared shared[kGreedyMaxGroups];
+  const int groups = blockDim.x / group;
+  const int mine = threadIdx.x / group;
+  const Group grp = {(int)threadIdx.x - mine * group, group, mine + 1}, all = {(int)threadIdx.x, (int)blockDim.x, 0};
+  GreedyShared& sh = shared[mine];
+  int* lo = reinterpret_cast<int*>(greedy_smem);     // [N] each, unless ONE
+  int* hi = lo + (ONE ? 0 : N);
+  int* mid = hi + (ONE ? 0 : N);
+  int* at = mid + (ONE ? 0 : N);                     // [N + 1]
+  int* weights = at + N + 1;                         // [groups][kGreedyCountMax + N]
+  float* s_gain = reinterpret_cast<float*>(weights + groups * (kGreedyCountMax + N));
+  unsigned short* s_start = reinterpret_cast<unsigned short*>(s_gain + cap + N);
+
+  const int tid = threadIdx.x, nthr = blockDim.x, G1 = P - 1;
+  const size_t curve0 = (size_t)blockIdx.y * N;
+  budgets += (size_t)blockIdx.y * set.budgets;
+  offsets += (size_t)blockIdx.y * set.offsets;
+  pdl_launch_dependents();
+  pdl_wait();  // the lists come from the launch before
+  const int* count = lists.count + curve0;
+
+  bool staged = false;
+  if (cap > 0) {
+    const int per = (N + nthr - 1) / nthr;
+    const int h_begin = min(N, tid * per), h_end = min(N, h_begin + per);
+    int local = 0;
+    for (int h = h_begin; h < h_end; ++h) local += count[h] + 1;
+    int run = group_scan(local, shared[0].scan, all);
+    for (int h = h_begin; h < h_end; ++h) {
+      at[h] = run;
+      run += count[h] + 1;
+      if (h == N - 1) at[N] = run;
+    }
+    __syncthreads();
+    staged = at[N] - N <= cap;
+    if (staged) {
+      // eight lanes per list: four lists of a warp in flight at a time
+      const int sub = tid & 7;
+#pragma unroll 2
+      for (int h = tid >> 3; h < N; h += nthr >> 3) {
+        const int a0 = at[h], c = at[h + 1] - a0 - 1;
+        const float* g = lists.gain + (curve0 + h) * G1;
+        const unsigned short* s = lists.start + (curve0 + h) * G1;
+#pragma unroll 4
+        for (int x = sub; x <= c; x += 8) {
+          s_gain[a0 + x] = x < c ? g[x] : 0.f;
+          s_start[a0 + x] = x < c ? s[x] : (unsigned short)G1;
+        }
+      }
+    }
+    __syncthreads();
+  }
+  const ListView<true> in_smem = {s_gain, s_start, at, nullptr, G1};
+  const ListView<false> in_place = {lists.gain + curve0 * G1, lists.start + curve0 * G1, nullptr, count, G1};
+  int* weight = weights + mine * (kGreedyCountMax + N);
+  for (int i = blockIdx.x * groups + mine; i < args.count; i += gridDim.x * groups) {
+    if (staged) greedy_problem<true, ONE>(in_smem, args, i, N, w, lo, hi, mid, weight, sh, grp, budgets, offsets);
+    else greedy_problem<false, ONE>(in_place, args, i, N, w, lo, hi, mid, weight, sh, grp, budgets, offsets);
+  }
+}
+
+// Hull and greedy of up to 32 heads in one launch: one CTA per sequence, a warp per head walks the head's curve into
+// shared memory (the curves are shared by the sequences; a walk costs less than handing lists over between launches).
+// For calls of one or a few layers, where allocation is on the critical path: 8 heads x 129 points 29 + 34 us as two
+// kernels before, 7 us now.
+constexpr int kSmallMaxHeads = 32;
+
+inline size_t alloc_small_smem_bytes(int N, int P) {
+  return (size_t)N * P * 4 + (((size_t)N * P * 2 + 3) & ~(size_t)3);
+}
+
+__global__ void __launch_bounds__(32 * kSmallMaxHeads) alloc_small_kernel(const float* __restrict__ curves,
+                                                                          const __grid_constant__ GreedyArgs args,
+                                                                          int32_t* __restrict__ budgets,
+                                                                          int32_t* __restrict__ offsets, int N, int P,
+                                                                          int w) {
+  extern __shared__ __align__(16) unsigned char small_smem[];
+  __shared__ GreedyShared sh;
+  __shared__ int at[kSmallMaxHeads + 1];
+  __shared__ int weight[kGreedyCountMax + kSmallMaxHeads];
+  float* gain = reinterpret_cast<float*>(small_smem);                              // [N][P], then packed
+  unsigned short* start = reinterpret_cast<unsigned short*>(gain + (size_t)N * P);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int count = 0;
+  if (warp < N) {
+    count = hull_walk_short(curves + (size_t)warp * P, P, lane, HullOut{gain + (size_t)warp * P, start + (size_t)warp * P});
+    if (lane == 0) {  // the end of the curve
+      gain[(size_t)warp * P + count] = 0.f;
+      start[(size_t)warp * P + count] = (unsigned short)(P - 1);
+      at[warp + 1] = count + 1;
+    }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    int v = lane < N ? at[lane + 1] : 0;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int o = __shfl_up_sync(0xffffffffu, v, off);
+      if (lane >= off) v += o;
+    }
+    if (lane < N) at[lane + 1] = v;
+    if (lane == 0) at[0] = 0;
+  }
+  __syncthreads();
+  // pack the lists, head by head (a list only moves towards the front)
+  for (int h = 1; h < N; ++h) {
+    const int to = at[h], len = at[h + 1] - to;
+    for (int x0 = 0; x0 < len; x0 += blockDim.x) {
+      const int x = x0 + threadIdx.x;
+      const float g = x < len ? gain[(size_t)h * P + x] : 0.f;
+      const unsigned short s = x < len ? start[(size_t)h * P + x] : (unsigned short)0;
+      __syncthreads();
+      if (x < len) {
+        gain[to + x] = g;
+        start[to + x] = s;
+      }
+    }
+  }
+  __syncthreads();
+  const ListView<true> lists = {gain, start, at, nullptr, P - 1};
+  const Group grp = {(int)threadIdx.x, (int)blockDim.x, 0};
+  greedy_problem<true, true>(lists, args, blockIdx.x, N, w, nullptr, nullptr, nullptr, weight, sh, grp, budgets, offsets);
+}
+
+GreedyArgs greedy_args(const Dims& dm, const int64_t* budgets_host, int q0, int cnt, long long* row_base) {
+  GreedyArgs args = {};
+  for (int i = 0; i < cnt; ++i) {
+    args.budget[i] = budgets_host[q0 + i];
+    args.row_base[i] = *row_base;
+    args.T[i] = dm.seq_T ? dm.seq_T[q0 + i] : dm.T;
+    args.floor_tok[i] = dm.seq_T ? seq_floor_tokens(dm, q0 + i) : dm.floor_tok;
+    *row_base += budgets_host[q0 + i] + (long long)dm.N * dm.w;
+  }
+  args.seq0 = q0;
+  args.count = cnt;
+  return args;
 }
 
 }  // namespace
 
-cudaError_t launch_hull(const float* curves, float* gains, int64_t n_curves, int P, LaunchCtx& lc) {
-  // one warp per curve; few curves: small blocks, so that they spread over the SMs (each walk is a
-  // latency-bound chain); many curves: up to 8 warps per block
-  int dev = 0, sms = 148;
-  if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  int hw = (int)((n_curves + sms - 1) / sms);
-  hw = hw > 8 ? 8 : (hw < 1 ? 1 : hw);
-  const size_t hull_smem = hull_bytes_per_warp(P) * hw;
+HullLists hull_lists(void* base, int64_t n_curves, int P) {
+  HullLists h;
+  char* p = static_cast<char*>(base);
+  const size_t cells = (size_t)n_curves * (P - 1);
+  h.gain = reinterpret_cast<float*>(p);
+  h.start = reinterpret_cast<unsigned short*>(p + cells * 4);
+  h.count = reinterpret_cast<int*>(p + ((cells * 6 + 3) & ~(size_t)3));
+  return h;
+}
+size_t hull_lists_bytes(int64_t n_curves, int P) {
+  return (((size_t)n_curves * (P - 1) * 6 + 3) & ~(size_t)3) + (size_t)n_curves * 4;
+}
+
+cudaError_t launch_hull(const float* curves, const HullLists& out, int64_t n_curves, int P, LaunchCtx& lc) {
+  const unsigned grid = (unsigned)n_curves;
+  const size_t smem = P <= kHullRegsMaxP ? 0 : (size_t)P * sizeof(float);  // at most 16.4 KB
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(hull_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hull_smem)) != cudaSuccess)
-    return e;
-  hull_kernel<<<(unsigned)((n_curves + hw - 1) / hw), hw * 32, hull_smem, lc.st>>>(curves, gains, (int)n_curves, P);
+  if (P <= kHullRegsMaxP) hull_kernel<0><<<grid, 32, smem, lc.st>>>(curves, out, P);
+  else if (P <= 1024) hull_kernel<1><<<grid, 32, smem, lc.st>>>(curves, out, P);
+  else if (P <= 2048) hull_kernel<2><<<grid, 32, smem, lc.st>>>(curves, out, P);
+  else if (P <= 4096) hull_kernel<4><<<grid, 32, smem, lc.st>>>(curves, out, P);
+  else hull_kernel<5><<<grid, 32, smem, lc.st>>>(curves, out, P);
   lc.mark("hull");
+  if (P > kHullRegsMaxP) {
+    const size_t dense = hull_dense_smem_bytes(P);  // at most 25 KB
+    if ((e = launch_pdl(hull_dense_kernel, dim3(grid), dim3(32), dense, lc.st, true, curves, out, P)) != cudaSuccess) return e;
+    lc.mark("hull_dense");
+  }
   return cudaGetLastError();
 }
 
-cudaError_t launch_greedy(const Dims& dm, const float* gains, const int64_t* budgets_host, int32_t* budgets,
+cudaError_t launch_greedy(const Dims& dm, const HullLists& lists, const int64_t* budgets_host, int32_t* budgets,
                           int32_t* offsets, int n_sets, LaunchCtx& lc) {
   cudaError_t e;
-  const size_t greedy_smem = (size_t)dm.N * 3 * sizeof(int);
-  int threads = (dm.N + 31) & ~31;  // one thread per head, whole warps
-  if (threads > kGreedyMaxThreads) threads = kGreedyMaxThreads;
-  if ((e = cudaFuncSetAttribute(greedy_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)greedy_smem)) != cudaSuccess)
-    return e;
+  // lists of up to 16384 blocks in all are staged (two CTAs per SM then); with many heads the per-head words take the room
+  const long long cells = (long long)dm.N * (dm.P - 1);
+  const int cap = dm.N > 2048 ? 0 : (int)std::min(cells, 16384LL);
+  const bool one = dm.N <= kGreedyMaxThreads;
+  int group = (dm.N + 31) & ~31;  // one thread per head, whole warps
+  if (group > kGreedyMaxThreads) group = kGreedyMaxThreads;
+  // several problems per CTA where many sets share the budgets (never when a thread owns several heads)
+  const int groups = n_sets > 1 && one ? std::min(kGreedyMaxGroups, std::max(1, std::min(dm.S, kGreedyMaxThreads / group))) : 1;
+  const size_t smem = greedy_smem_bytes(dm.N, cap, groups, one);
+  auto kern = one ? greedy_kernel<true> : greedy_kernel<false>;
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
   SetStride set;
-  set.gains = (size_t)dm.N * (dm.P - 1);
   set.budgets = (size_t)dm.S * dm.N;
   set.offsets = (size_t)dm.S * dm.N + 1;
   long long base = 0;
   for (int q0 = 0; q0 < dm.S; q0 += kSeqPerLaunch) {
-    GreedyArgs args;
     const int cnt = dm.S - q0 < kSeqPerLaunch ? dm.S - q0 : kSeqPerLaunch;
-    for (int i = 0; i < kSeqPerLaunch; ++i) {
-      args.budget[i] = 0;
-      args.row_base[i] = 0;
-      args.T[i] = dm.T;
-      args.floor_tok[i] = dm.floor_tok;
-    }
-    for (int i = 0; i < cnt; ++i) {
-      args.budget[i] = budgets_host[q0 + i];
-      args.row_base[i] = base;
-      if (dm.seq_T) {
-        args.T[i] = dm.seq_T[q0 + i];
-        args.floor_tok[i] = seq_floor_tokens(dm, q0 + i);
-      }
-      base += budgets_host[q0 + i] + (long long)dm.N * dm.w;
-    }
-    args.seq0 = q0;
-    greedy_kernel<<<dim3(cnt, n_sets), threads, greedy_smem, lc.st>>>(gains, args, budgets, offsets, set, dm.N, dm.P,
-                                                                      dm.w);
+    const GreedyArgs args = greedy_args(dm, budgets_host, q0, cnt, &base);
+    // one CTA per sequence; where many sets share the budgets, a set's staged lists serve several of them
+    int ctas = (cnt + groups - 1) / groups;
+    if (n_sets > 1) ctas = std::max(1, std::min(ctas, 2 * 148 / n_sets));
+    e = launch_pdl(kern, dim3(ctas, n_sets), dim3(group * groups), smem, lc.st, q0 == 0, lists, args, budgets, offsets, set,
+                   dm.N, dm.P, dm.w, cap, group);
+    if (e != cudaSuccess) return e;
     lc.mark("greedy");
   }
   return cudaGetLastError();
 }
 
-cudaError_t launch_allocate(const Dims& dm, const float* curves, const int64_t* budgets_host, float* gains,
+cudaError_t launch_allocate(const Dims& dm, const float* curves, const int64_t* budgets_host, const HullLists& lists,
                             int32_t* budgets, int32_t* offsets, LaunchCtx& lc) {
-  cudaError_t e = launch_hull(curves, gains, dm.N, dm.P, lc);
+  if (dm.N <= kSmallMaxHeads && dm.P <= kHullRegsMaxP) {
+    const size_t smem = alloc_small_smem_bytes(dm.N, dm.P);
+    cudaError_t e = cudaFuncSetAttribute(alloc_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    long long base = 0;
+    for (int q0 = 0; q0 < dm.S; q0 += kSeqPerLaunch) {
+      const int cnt = dm.S - q0 < kSeqPerLaunch ? dm.S - q0 : kSeqPerLaunch;
+      const GreedyArgs args = greedy_args(dm, budgets_host, q0, cnt, &base);
+      alloc_small_kernel<<<cnt, 32 * dm.N, smem, lc.st>>>(curves, args, budgets, offsets, dm.N, dm.P, dm.w);
+      lc.mark("allocate");
+    }
+    return cudaGetLastError();
+  }
+  cudaError_t e = launch_hull(curves, lists, dm.N, dm.P, lc);
   if (e != cudaSuccess) return e;
-  return launch_greedy(dm, gains, budgets_host, budgets, offsets, 1, lc);
+  return launch_greedy(dm, lists, budgets_host, budgets, offsets, 1, lc);
 }
 
 }  // namespace lukv

@@ -32,7 +32,7 @@ Workspace carve_workspace(const Dims& dm, void* base) {
   if (keydiff_scratch_bytes(dm) > stats_bytes) stats_bytes = keydiff_scratch_bytes(dm);
   ws.stats = static_cast<float*>(take(stats_bytes));
   ws.lse = static_cast<float*>(take(heads * dm.M * sizeof(float)));
-  ws.gains = static_cast<float*>(take((size_t)dm.N * (dm.P - 1) * sizeof(float)));
+  ws.hull = hull_lists(take(hull_lists_bytes(dm.N, dm.P)), dm.N, dm.P);
   ws.head_flags = static_cast<int*>(take(score_tc_flag_bytes(dm)));
   ws.bytes = off;
   return ws;
@@ -182,7 +182,7 @@ static int run_compress(const Dims& dm, const void* q_win, const void* k, const 
     ls.st = side->stream;
     if (cudaEventRecord(side->fork, lc.st) != cudaSuccess || cudaStreamWaitEvent(ls.st, side->fork, 0) != cudaSuccess)
       return LUKV_ERR_CUDA;
-    if (launch_allocate(dm, curves, budgets_in, w.gains, budgets, offsets, ls) != cudaSuccess) rc = LUKV_ERR_CUDA;
+    if (launch_allocate(dm, curves, budgets_in, w.hull, budgets, offsets, ls) != cudaSuccess) rc = LUKV_ERR_CUDA;
     if (cudaEventRecord(side->join, ls.st) != cudaSuccess) rc = LUKV_ERR_CUDA;
     lc.launches += ls.launches;
     if (rc == LUKV_OK && dm.keydiff) {
@@ -198,7 +198,7 @@ static int run_compress(const Dims& dm, const void* q_win, const void* k, const 
     if (cudaStreamWaitEvent(lc.st, side->join, 0) != cudaSuccess) rc = LUKV_ERR_CUDA;
     if (rc != LUKV_OK) return rc;
   } else {
-    if (launch_allocate(dm, curves, budgets_in, w.gains, budgets, offsets, lc) != cudaSuccess) return LUKV_ERR_CUDA;
+    if (launch_allocate(dm, curves, budgets_in, w.hull, budgets, offsets, lc) != cudaSuccess) return LUKV_ERR_CUDA;
     if (run_score(dm, q_win, k, w, w.pooled, dev_status, lc) != cudaSuccess) return LUKV_ERR_CUDA;
   }
   if (launch_select(dm, w.pooled, budgets, offsets, kept_idx, rows_cap, all_heads(dm), lc) != cudaSuccess)
@@ -302,7 +302,7 @@ int lukv_allocate(const lukv_params_t* params, const float* curves, const int64_
   if ((rc = check_ws(dm, ws, ws_bytes, &w)) != LUKV_OK) return rc;
   LaunchCtx lc;
   lc.st = (cudaStream_t)stream;
-  if (launch_allocate(dm, curves, budgets_in, w.gains, budgets, offsets, lc) != cudaSuccess) return LUKV_ERR_CUDA;
+  if (launch_allocate(dm, curves, budgets_in, w.hull, budgets, offsets, lc) != cudaSuccess) return LUKV_ERR_CUDA;
   g_last_launches = lc.launches;
   return LUKV_OK;
 }
@@ -419,26 +419,26 @@ int lukv_compress_profile(const lukv_params_t* params, const void* q_win, const 
 }
 
 // ---- allocation without a caller-provided workspace ---------------------------------------
-// Scratch of lukv_allocate_static: the hull gains [N][P-1].  The array lives in every GPU
-// context that loads this library, from load until exit.
+// Scratch of lukv_allocate_static: the hull lists, at most 6 bytes per segment and 4 per curve.  The array lives in
+// every GPU context that loads this library, from load until exit.
 #define LUKV_STATIC_GAINS_MAX (256 * 1024)
-static __device__ __align__(256) float g_static_gains[LUKV_STATIC_GAINS_MAX];
+static __device__ __align__(256) unsigned char g_static_hull[LUKV_STATIC_GAINS_MAX * 10];
 
-// In host code `g_static_gains` is only a handle for the runtime, not a device address; the
+// In host code `g_static_hull` is only a handle for the runtime, not a device address; the
 // address on the current device is looked up once per device and cached here.
-static float* g_static_gains_ptr[64] = {nullptr};
-static std::mutex g_static_gains_mutex;
+static void* g_static_hull_ptr[64] = {nullptr};
+static std::mutex g_static_hull_mutex;
 
-static int static_gains_address(float** out) {
+static int static_hull_address(void** out) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return LUKV_ERR_CUDA;
-  std::lock_guard<std::mutex> lock(g_static_gains_mutex);
-  if (!g_static_gains_ptr[dev]) {
-    float* ptr = nullptr;
-    if (cudaGetSymbolAddress((void**)&ptr, g_static_gains) != cudaSuccess || !ptr) return LUKV_ERR_CUDA;
-    g_static_gains_ptr[dev] = ptr;
+  std::lock_guard<std::mutex> lock(g_static_hull_mutex);
+  if (!g_static_hull_ptr[dev]) {
+    void* ptr = nullptr;
+    if (cudaGetSymbolAddress(&ptr, g_static_hull) != cudaSuccess || !ptr) return LUKV_ERR_CUDA;
+    g_static_hull_ptr[dev] = ptr;
   }
-  *out = g_static_gains_ptr[dev];
+  *out = g_static_hull_ptr[dev];
   return LUKV_OK;
 }
 
@@ -452,13 +452,13 @@ int lukv_allocate_static(const lukv_params_t* params, const float* curves, const
   int64_t rows;
   if ((rc = check_budgets(dm, budgets_in, &rows)) != LUKV_OK) return rc;
   if (rows >= (int64_t)1 << 31) return LUKV_ERR_UNSUPPORTED;
-  float* gains = nullptr;
-  if ((rc = static_gains_address(&gains)) != LUKV_OK) return rc;
+  void* base = nullptr;
+  if ((rc = static_hull_address(&base)) != LUKV_OK) return rc;
   LaunchCtx lc;
   lc.st = (cudaStream_t)stream;
-  // the hull kernel overwrites gains[0 .. N*(P-1)) before the greedy kernel reads them, so
+  // the hull kernel overwrites every list before the greedy kernel reads it, so
   // nothing left by an earlier call is ever consumed
-  if (launch_allocate(dm, curves, budgets_in, gains, budgets, offsets, lc) != cudaSuccess) return LUKV_ERR_CUDA;
+  if (launch_allocate(dm, curves, budgets_in, hull_lists(base, dm.N, dm.P), budgets, offsets, lc) != cudaSuccess) return LUKV_ERR_CUDA;
   g_last_launches = lc.launches;
   return LUKV_OK;
 }
@@ -467,7 +467,7 @@ int lukv_allocate_static(const lukv_params_t* params, const float* curves, const
 
 namespace {
 struct ProfileWs {
-  float* gains;      // [Mq][N][P-1]
+  HullLists hull;    // of Mq * N curves
   int32_t* budgets;  // [Mq][R][N]
   int32_t* offsets;  // [Mq][R*N+1] (written by the greedy kernel, not used further)
   size_t bytes;
@@ -482,7 +482,7 @@ ProfileWs carve_profile_ws(const Dims& dm, int n_queries, void* base) {
     return r;
   };
   const size_t Mq = (size_t)n_queries, RN = (size_t)dm.S * dm.N;
-  ws.gains = static_cast<float*>(take(Mq * dm.N * (dm.P - 1) * sizeof(float)));
+  ws.hull = hull_lists(take(hull_lists_bytes((int64_t)Mq * dm.N, dm.P)), (int64_t)Mq * dm.N, dm.P);
   ws.budgets = static_cast<int32_t*>(take(Mq * RN * sizeof(int32_t)));
   ws.offsets = static_cast<int32_t*>(take(Mq * (RN + 1) * sizeof(int32_t)));
   ws.bytes = off;
@@ -531,8 +531,8 @@ int lukv_profile_build(const lukv_params_t* calib, const float* curves, int32_t 
   }
   LaunchCtx lc;
   lc.st = (cudaStream_t)stream;
-  cudaError_t e = launch_hull(curves, w.gains, (int64_t)n_queries * dm.N, dm.P, lc);
-  if (e == cudaSuccess) e = launch_greedy(dm, w.gains, B, w.budgets, w.offsets, n_queries, lc);
+  cudaError_t e = launch_hull(curves, w.hull, (int64_t)n_queries * dm.N, dm.P, lc);
+  if (e == cudaSuccess) e = launch_greedy(dm, w.hull, B, w.budgets, w.offsets, n_queries, lc);
   free(B);  // the budgets travel by value in the launch arguments
   if (e == cudaSuccess) e = launch_profile_mean(w.budgets, profile, n_queries, (int64_t)dm.S * dm.N, dm.n, lc);
   if (e != cudaSuccess) return LUKV_ERR_CUDA;

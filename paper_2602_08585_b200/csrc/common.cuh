@@ -31,6 +31,16 @@ struct Dims {
   size_t esize() const { return dtype == LUKV_DTYPE_BF16 ? 2 : 4; }
 };
 
+// The hull of every curve as a list of its blocks of equal gain, steepest first: row i of `gain` and `start` ([curves]
+// [P-1]) holds count[i] entries, `start` the first curve segment of the block.
+struct HullLists {
+  float* gain;
+  unsigned short* start;
+  int* count;
+};
+HullLists hull_lists(void* base, int64_t n_curves, int P);
+size_t hull_lists_bytes(int64_t n_curves, int P);
+
 // Workspace carve-up (all offsets 256-byte aligned).
 struct Workspace {
   float* raw;        // [S*N][n]   un-pooled scores
@@ -38,7 +48,7 @@ struct Workspace {
   float* stats;      // partial (reference, sum-exp) per row: [S*N][chunks][M][2] (FP32-pipe scorer) or
                      // [S*N][items][256][2] (tensor-core scorer)
   float* lse;        // [S*N][M]   row log-sum-exp in the exp2 domain
-  float* gains;      // [N][P-1]   hull gains
+  HullLists hull;    // blocks of equal gain of every head's curve
   int* head_flags;   // tensor-core scorer: [S*N] items delivered per head, then the (lse, tag) rows
   size_t bytes;
 };
@@ -92,6 +102,35 @@ struct LaunchCtx {
   }
 };
 
+// Programmatic dependent launch: a kernel launched with launch_pdl(..., overlap = true) may start while the kernel before
+// it on the stream still runs; it touches nothing that kernel (or any before it) reads or writes until pdl_wait, which
+// returns once they are complete.  Both are no-ops in an ordinary launch.
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Maximum over the warp.
+__device__ __forceinline__ float warp_max(float v) {
+  float d;
+  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(d) : "f"(v));
+  return d;
+}
+template <typename Kernel, typename... Args>
+inline cudaError_t launch_pdl(Kernel kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool overlap,
+                              const Args&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+#endif
+
 // Heads [h0, h0+nh) of the S*N heads of a call (the stages after allocation work head by head).
 struct HeadRange {
   int h0, nh;
@@ -111,13 +150,13 @@ cudaError_t launch_score_tc(const Dims& dm, const void* q, const void* k, const 
 cudaError_t launch_score_onepass(const Dims& dm, const void* q, const void* k, const Workspace& ws,
                                  int32_t* dev_status, HeadRange hr, bool clear_flags, int spare_sms, LaunchCtx& lc);
 cudaError_t launch_pool(const Dims& dm, const float* raw, float* pooled, HeadRange hr, LaunchCtx& lc);
-cudaError_t launch_allocate(const Dims& dm, const float* curves, const int64_t* budgets_host, float* gains,
+cudaError_t launch_allocate(const Dims& dm, const float* curves, const int64_t* budgets_host, const HullLists& lists,
                             int32_t* budgets, int32_t* offsets, LaunchCtx& lc);
 // The two halves of launch_allocate.  launch_hull treats its input as n_curves independent curves;
-// launch_greedy solves n_sets curve sets (gains [n_sets][N][P-1]) for the same dm.S budgets and
+// launch_greedy solves n_sets curve sets (lists of n_sets * N curves) for the same dm.S budgets and
 // writes budgets [n_sets][S][N] and offsets [n_sets][S*N+1].
-cudaError_t launch_hull(const float* curves, float* gains, int64_t n_curves, int P, LaunchCtx& lc);
-cudaError_t launch_greedy(const Dims& dm, const float* gains, const int64_t* budgets_host, int32_t* budgets,
+cudaError_t launch_hull(const float* curves, const HullLists& out, int64_t n_curves, int P, LaunchCtx& lc);
+cudaError_t launch_greedy(const Dims& dm, const HullLists& lists, const int64_t* budgets_host, int32_t* budgets,
                           int32_t* offsets, int n_sets, LaunchCtx& lc);
 // Offline profile (mean of the local ratios) and online lookup + budgeting.
 cudaError_t launch_profile_mean(const int32_t* budgets, float* profile, int n_queries, int64_t count, int n,

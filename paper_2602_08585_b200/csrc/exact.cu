@@ -47,12 +47,6 @@ __device__ __forceinline__ float max3(float a, float b, float c) {
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
-__device__ __forceinline__ float warp_max(float v) {
-  float d;
-  asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(d) : "f"(v));
-  return d;
-}
-
 // Maxima of every curve over runs of 16 values of b; -inf beyond n.  One CTA per head.
 __global__ void __launch_bounds__(kDpURuns) dp_runs_kernel(const float* __restrict__ curves, float* __restrict__ runs, int n,
                                                            int P) {
@@ -148,8 +142,8 @@ __global__ void __launch_bounds__(kDpThreads, 5) dp_step_kernel(const DpStep a) 
   const unsigned char* fw = F2 + (xg - bg + 3) * kDpGroup;
   const unsigned char* ub = U2 + bg * kDpGroup;
 
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_launch_dependents();
+  pdl_wait();
   if (x0 > a.hi) return;  // whole warps; nothing below waits for another warp
 
   // Upper bound of (f(y) - s (y - x0)) + (U(b) - s b) over the pairs of block `blk` from the run maxima of its 64 values of

@@ -1,0 +1,41 @@
+"""GPU parity of stage (b) at the sizes where its kernels change: points per lane of the hull walk, curves in registers or
+shared memory, one launch or two, heads per thread, lists staged or in place.  Bit-exact against the oracle."""
+import numpy as np
+import pytest
+
+from gpu_helpers import gpu_allocate
+from paper_2602_08585_b200 import lukv
+
+pytestmark = pytest.mark.gpu
+
+
+def _curves(rng, N, P, kind):
+    inc = rng.exponential(size=(N, P - 1)) * np.where(rng.random((N, P - 1)) < 0.2, 3.0, 1.0)
+    if kind == "concave":
+        inc = -np.sort(-inc, axis=1)                       # every point is a vertex
+    elif kind == "ties":
+        inc = -np.sort(-np.floor(inc * 2), axis=1)         # equal slopes inside and across heads
+    elif kind == "mixed":
+        inc = inc * np.arange(1, P) ** -0.7 - 0.02         # few vertices, falling tails
+    U = np.zeros((N, P), np.float32)
+    U[:, 1:] = np.cumsum(inc, axis=1)
+    return U
+
+
+@pytest.mark.parametrize("kind", ["rough", "concave", "ties", "mixed"])
+@pytest.mark.parametrize("N,P", [(1, 2), (4, 65), (7, 97), (32, 161), (3, 289), (32, 544), (5, 545), (33, 98), (40, 1025),
+                                 (3, 2049), (2, 4097), (300, 257), (1025, 5), (2100, 9)])
+def test_allocation_at_the_edges(oracle, N, P, kind):
+    rng = np.random.default_rng(1000 * N + P)
+    s, w = (3, 4) if P < 1000 else (1, 2)
+    T = s * (P - 1)
+    if T <= w:
+        T, w = 8 * (P - 1), 3
+    U = _curves(rng, N, P, kind)
+    most = N * (T - w)
+    Bs = [0, 1, most // 5, most // 2 + 1, most - 1, most]
+    p = lukv.make_params(len(Bs), 1, N, 1, 64, T, w, 1, "bf16", P)
+    b, o = gpu_allocate(p, U, Bs)
+    b_ref, o_ref = oracle.allocate(U, T, w, Bs)
+    np.testing.assert_array_equal(b, b_ref)
+    np.testing.assert_array_equal(o, o_ref)
