@@ -2,12 +2,14 @@
 //   I_j = max over decode steps k of  sum_g A_{g,k,j} * || v_j W_O^(g) ||_2 ,
 // A the attention weights (Eq. 1) of the G query heads of the KV head at decode step k, the softmax running over
 // the T cached keys and, if decode keys are given, the keys of steps 1..k; each layer then divided by its total.
-// An offline tool (it feeds the curve builder and the profile build), on the FP32 pipes in the tiling of the
-// general-shape scorer: 64 x 64 dot products per shared-memory tile pair, a 4 x 4 register tile per thread.
+// An offline tool (it feeds the curve builder and the profile build).  bf16 inputs run on the tensor cores
+// (value_norm_tc.cu, importance_tc.cu); the kernels here are for fp32 inputs and groups of more than eight query heads, on
+// the FP32 pipes in the tiling of the general-shape scorer: 64 x 64 dot products per shared-memory tile pair, a 4 x 4 register tile per thread.
 //   value_norm_kernel   || v_j W_O^(g) ||_2 for every (head, g, rankable position)
 //   imp_lse_kernel      row log-sum-exp of every (head, g, step), exp2 domain
 //   imp_kernel          probabilities x value norms, summed over g inside a thread, maximum over the steps
 //   imp_normalize_kernel  one CTA per (sequence, layer): fp64 total in a fixed order, then the division
+#include <algorithm>
 #include <cstdlib>
 
 #include "simt_tile.cuh"
@@ -272,11 +274,16 @@ cudaError_t launch_importance_t(const Dims& dm, ImpDims id, const void* q_dec, c
     kn<<<dim3(heads * id.G, pos_tiles), kSimtThreads, smem, lc.st>>>((const TIn*)v, (const TIn*)w_o, vnorm, id);
     lc.mark("value_norm");
   }
-  kl<<<dim3(heads, (unsigned)((id.Kmax + 15) / 16)), kSimtThreads, smem, lc.st>>>((const TIn*)q_dec, (const TIn*)k,
-                                                                                 (const TIn*)k_dec, lse, id);
-  lc.mark("imp_lse");
-  ki<<<dim3(heads, pos_tiles), kSimtThreads, smem, lc.st>>>((const TIn*)q_dec, (const TIn*)k, lse, vnorm, importance, id);
-  lc.mark("importance");
+  if (importance_tc_supported(dm, id.Kmax) && !value_norm_force_simt()) {
+    if ((e = launch_importance_tc(dm, id.Kmax, q_dec, k, k_dec, vnorm, lse, importance, lc)) != cudaSuccess) return e;
+  } else {
+    kl<<<dim3(heads, (unsigned)((id.Kmax + 15) / 16)), kSimtThreads, smem, lc.st>>>((const TIn*)q_dec, (const TIn*)k,
+                                                                                   (const TIn*)k_dec, lse, id);
+    lc.mark("imp_lse");
+    ki<<<dim3(heads, pos_tiles), kSimtThreads, smem, lc.st>>>((const TIn*)q_dec, (const TIn*)k, lse, vnorm, importance,
+                                                              id);
+    lc.mark("importance");
+  }
   if (normalize) {
     imp_normalize_kernel<<<(unsigned)(dm.S * dm.L), 1024, 0, lc.st>>>(importance, (long long)dm.H * dm.n);
     lc.mark("imp_normalize");
@@ -288,7 +295,8 @@ cudaError_t launch_importance_t(const Dims& dm, ImpDims id, const void* q_dec, c
 
 size_t importance_workspace_bytes(const Dims& dm, int k_max) {
   const size_t a = ((size_t)dm.heads() * dm.G * dm.n * sizeof(float) + 255) & ~(size_t)255;
-  const size_t b = ((size_t)dm.heads() * dm.G * k_max * sizeof(float) + 255) & ~(size_t)255;
+  const size_t rows = (size_t)dm.heads() * dm.G * k_max * sizeof(float);  // row log-sum-exps, or their partials
+  const size_t b = (std::max(rows, dm.G <= 8 ? importance_tc_part_bytes(dm, k_max) : 0) + 255) & ~(size_t)255;
   return a + b;
 }
 

@@ -307,12 +307,12 @@ EncodeTiledFn encode_fn() {
   return fn;
 }
 
-// 2-D bf16 tensor [rows][128] with boxes of 64 channels x 128 rows, 128-byte swizzle, zero fill.
-bool make_map(CUtensorMap* map, const void* base, uint64_t rows) {
+// 2-D bf16 tensor [rows][d] with boxes of 64 channels x 128 rows, 128-byte swizzle, zero fill.
+bool make_map(CUtensorMap* map, const void* base, uint64_t rows, int d = 128) {
   EncodeTiledFn fn = encode_fn();
   if (!fn) return false;
-  const cuuint64_t dims[2] = {128, rows};
-  const cuuint64_t strides[1] = {256};
+  const cuuint64_t dims[2] = {(cuuint64_t)d, rows};
+  const cuuint64_t strides[1] = {(cuuint64_t)d * 2};
   const cuuint32_t box[2] = {64, 128};
   const cuuint32_t estr[2] = {1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,

@@ -1,15 +1,15 @@
 // Value norms of the oracle importance (Sec. 4.1, Eq. "oracle_importance"; App. E: L2 norm of the projected value),
 //   vnorm[u][g][j] = || v[u][j] W_O^(g) ||_2 ,   u a KV head, g one of its G query heads, j a rankable position,
-// on the tensor cores for bf16 inputs with d = 128.  Per (u, g) this is a dense contraction (n x d) * (d x D_model)
+// on the tensor cores for bf16 inputs.  Per (u, g) this is a dense contraction (n x d) * (d x D_model)
 // followed by a sum of squares over the D_model output columns: 98 % of the flops of the importance computation.
 //
 // One persistent kernel, one CTA per SM, work items (u, g, chunk of 4096 positions).  For an item the CTA walks the
 // projection in panels of 256 output columns and, per panel, the chunk's tiles of 128 positions:
-//   warp 0      TMA producer: value tiles (128 positions x 128 channels, the layout of the key tiles of the scorer)
+//   warp 0      TMA producer: value tiles (128 positions x d channels, the layout of the key tiles of the scorer)
 //   warp 1      allocates tensor memory; one lane issues the MMAs, D[position][column] = V tile * panel^T, N = 256
 //   warps 2-5   epilogue: read the accumulator (a row per thread), add the squares to the row's running sum in
 //               shared memory; after the last panel write the square roots
-//   warps 6-9   panel writers: W_O^(g) is stored [d][D_model], the MMA wants each output column's 128 channels
+//   warps 6-9   panel writers: W_O^(g) is stored [d][D_model], the MMA wants each output column's d channels
 //               contiguous, so the panel is transposed on its way into shared memory (8 loads of 4 columns -> 4 rows
 //               of 8 channels, stored in the 128-byte-swizzled layout the MMA descriptor describes); a panel serves all
 //               tiles of the chunk, and the next one is written while the current one is in use
@@ -23,17 +23,15 @@ constexpr int kVnRowTile = 128;                      // positions per MMA (M)
 constexpr int kVnColTile = 256;                      // projection columns per MMA (N)
 constexpr int kVnChunkTiles = 32;                    // row tiles per work item
 constexpr int kVnChunkRows = kVnChunkTiles * kVnRowTile;
-constexpr int kVnABytes = kVnRowTile * 128 * 2;      // one value tile: two halves of 64 channels
-constexpr int kVnAHalf = kVnABytes / 2;
-constexpr int kVnBBytes = kVnColTile * 128 * 2;      // one panel: two halves of 64 channels, 256 rows each
-constexpr int kVnBHalf = kVnBBytes / 2;
+constexpr int kVnAHalf = kVnRowTile * 128;           // 64 channels of a value tile; d = 64 NH channels make NH of them
+constexpr int kVnBHalf = kVnColTile * 128;           // 64 channels of a panel: 256 rows
 constexpr int kVnThreads = 320;
-constexpr int kVnSmem = 2 * kVnABytes + 2 * kVnBBytes + kVnChunkRows * 4 + 1024;
+constexpr int vn_smem(int NH) { return 2 * NH * (kVnAHalf + kVnBHalf) + kVnChunkRows * 4 + 1024; }
 
 enum { kVnAFull = 0, kVnAEmpty = 2, kVnBFull = 4, kVnBEmpty = 6, kVnTFull = 8, kVnTEmpty = 10, kVnBars = 12 };
 
 struct VnArgs {
-  const __nv_bfloat16* w_o;  // [L][H*G][128][Dm]
+  const __nv_bfloat16* w_o;  // [L][H*G][d][Dm]
   float* vnorm;              // [heads][G][n]
   int L, H, G, T, n, Dm;
   int chunks;                // row chunks per (u, g)
@@ -41,14 +39,15 @@ struct VnArgs {
   uint32_t spin_limit;
 };
 
-// Writes the panel of output columns [m0, m0 + 256) of one projection slice w [128][Dm] into shared memory as 256
-// rows (columns of W) of 128 channels, in two halves of 64 channels, rows of 128 bytes, 16-byte chunk c of row m at
+// Writes the panel of output columns [m0, m0 + 256) of one projection slice w [64 NH][Dm] into shared memory as 256
+// rows (columns of W) of 64 NH channels, in halves of 64 channels, rows of 128 bytes, 16-byte chunk c of row m at
 // chunk position c ^ (m & 7).  Columns at or beyond Dm are zero.  128 threads.
+template <int NH>
 __device__ __forceinline__ void vn_write_panel(unsigned char* panel, const __nv_bfloat16* w, int Dm, int m0, int t,
                                                bool vec) {
   if (vec) {
-    // unit = (4 columns, 8 channels): 64 x 16 units, 8 per thread; lanes take consecutive column groups
-    for (int unit = t; unit < 64 * 16; unit += 128) {
+    // unit = (4 columns, 8 channels): 64 x 8 NH units; lanes take consecutive column groups
+    for (int unit = t; unit < 64 * 8 * NH; unit += 128) {
       const int mq = unit & 63, c8 = unit >> 6;
       const int m = m0 + 4 * mq;
       uint2 r[8];
@@ -73,7 +72,7 @@ __device__ __forceinline__ void vn_write_panel(unsigned char* panel, const __nv_
     }
   } else {
     // any Dm and alignment: one column and 8 channels per unit
-    for (int unit = t; unit < 256 * 16; unit += 128) {
+    for (int unit = t; unit < 256 * 8 * NH; unit += 128) {
       const int row = unit & 255, c8 = unit >> 8;
       const int m = m0 + row;
       uint4 o = make_uint4(0u, 0u, 0u, 0u);
@@ -97,6 +96,7 @@ struct VnItem {
   int u, g, row0, ntiles;
   const __nv_bfloat16* w;
 };
+template <int NH>
 __device__ __forceinline__ VnItem vn_item(const VnArgs& a, long long idx) {
   VnItem it;
   const int chunk = (int)(idx % a.chunks);
@@ -106,12 +106,14 @@ __device__ __forceinline__ VnItem vn_item(const VnArgs& a, long long idx) {
   it.row0 = chunk * kVnChunkRows;
   it.ntiles = (min(kVnChunkRows, a.n - it.row0) + kVnRowTile - 1) / kVnRowTile;
   const int layer = (it.u / a.H) % a.L, h = it.u % a.H;
-  it.w = a.w_o + ((size_t)layer * a.H * a.G + (size_t)h * a.G + it.g) * 128 * a.Dm;
+  it.w = a.w_o + ((size_t)layer * a.H * a.G + (size_t)h * a.G + it.g) * (64 * NH) * a.Dm;
   return it;
 }
 
+template <int NH>
 __global__ void __launch_bounds__(kVnThreads, 1)
     value_norm_tc_kernel(const __grid_constant__ CUtensorMap v_map, const VnArgs a) {
+  constexpr int kVnABytes = NH * kVnAHalf, kVnBBytes = NH * kVnBHalf;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   unsigned char* a_tiles = smem;                              // [2][kVnABytes]
@@ -150,7 +152,7 @@ __global__ void __launch_bounds__(kVnThreads, 1)
       uint32_t tt = 0;
       bool ok = true;
       for (long long idx = blockIdx.x; idx < a.items && ok; idx += gridDim.x) {
-        const VnItem it = vn_item(a, idx);
+        const VnItem it = vn_item<NH>(a, idx);
         for (int cp = 0; cp < npanels && ok; ++cp)
           for (int rt = 0; rt < it.ntiles; ++rt, ++tt) {
             const uint32_t s = tt & 1, ph = (tt >> 1) & 1;
@@ -158,8 +160,7 @@ __global__ void __launch_bounds__(kVnThreads, 1)
             mbar_expect_tx(bar(kVnAFull, s), kVnABytes);
             const uint32_t dst = smem_u32(a_tiles + s * kVnABytes);
             const int row = it.u * a.T + it.row0 + rt * kVnRowTile;  // rows past the head are never written back
-            tma_load_2d(dst, &v_map, bar(kVnAFull, s), 0, row);
-            tma_load_2d(dst + kVnAHalf, &v_map, bar(kVnAFull, s), 64, row);
+            for (int h = 0; h < NH; ++h) tma_load_2d(dst + h * kVnAHalf, &v_map, bar(kVnAFull, s), h * 64, row);
           }
       }
     }
@@ -170,7 +171,7 @@ __global__ void __launch_bounds__(kVnThreads, 1)
       uint32_t tt = 0, pc = 0;
       bool ok = true;
       for (long long idx = blockIdx.x; idx < a.items && ok; idx += gridDim.x) {
-        const VnItem it = vn_item(a, idx);
+        const VnItem it = vn_item<NH>(a, idx);
         for (int cp = 0; cp < npanels && ok; ++cp, ++pc) {
           const uint32_t pb = pc & 1;
           if (!(ok = mbar_wait(bar(kVnBFull, pb), (pc >> 1) & 1, abort_flag, nullptr, a.spin_limit))) break;
@@ -182,7 +183,7 @@ __global__ void __launch_bounds__(kVnThreads, 1)
             tc_fence_after();
             const uint32_t at = smem_u32(a_tiles + s * kVnABytes);
 #pragma unroll
-            for (int ks = 0; ks < 8; ++ks) {
+            for (int ks = 0; ks < 4 * NH; ++ks) {
               const int h = ks >> 2, sub = ks & 3;
               const uint64_t da = smem_desc_sw128(at + h * kVnAHalf) + (uint64_t)(sub * 2);
               const uint64_t db = smem_desc_sw128(bp + h * kVnBHalf) + (uint64_t)(sub * 2);
@@ -202,7 +203,7 @@ __global__ void __launch_bounds__(kVnThreads, 1)
     uint32_t tt = 0;
     bool ok = true;
     for (long long idx = blockIdx.x; idx < a.items && ok; idx += gridDim.x) {
-      const VnItem it = vn_item(a, idx);
+      const VnItem it = vn_item<NH>(a, idx);
       for (int cp = 0; cp < npanels && ok; ++cp)
         for (int rt = 0; rt < it.ntiles; ++rt, ++tt) {
           const uint32_t s = tt & 1, ph = (tt >> 1) & 1;
@@ -242,11 +243,11 @@ __global__ void __launch_bounds__(kVnThreads, 1)
     uint32_t pc = 0;
     bool ok = true;
     for (long long idx = blockIdx.x; idx < a.items && ok; idx += gridDim.x) {
-      const VnItem it = vn_item(a, idx);
+      const VnItem it = vn_item<NH>(a, idx);
       for (int cp = 0; cp < npanels; ++cp, ++pc) {
         const uint32_t pb = pc & 1;
         if (!(ok = mbar_wait(bar(kVnBEmpty, pb), ((pc >> 1) & 1) ^ 1, abort_flag, nullptr, a.spin_limit))) break;
-        vn_write_panel(panels + pb * kVnBBytes, it.w, a.Dm, cp * kVnColTile, t, vec);
+        vn_write_panel<NH>(panels + pb * kVnBBytes, it.w, a.Dm, cp * kVnColTile, t, vec);
         // the MMA reads shared memory through the asynchronous proxy: order these writes before it
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
@@ -271,13 +272,13 @@ __global__ void __launch_bounds__(kVnThreads, 1)
 }  // namespace
 
 bool value_norm_tc_supported(const Dims& dm) {
-  return dm.dtype == LUKV_DTYPE_BF16 && dm.d == 128 && dm.heads() * (int64_t)dm.T < ((int64_t)1 << 31);
+  return dm.dtype == LUKV_DTYPE_BF16 && dm.heads() * (int64_t)dm.T < ((int64_t)1 << 31);
 }
 
 cudaError_t launch_value_norm_tc(const Dims& dm, int d_model, const void* v, const void* w_o, float* vnorm,
                                  LaunchCtx& lc) {
   CUtensorMap vm;
-  if (!make_map(&vm, v, (uint64_t)dm.heads() * dm.T)) return cudaErrorNotSupported;
+  if (!make_map(&vm, v, (uint64_t)dm.heads() * dm.T, dm.d)) return cudaErrorNotSupported;
   VnArgs a;
   a.w_o = static_cast<const __nv_bfloat16*>(w_o);
   a.vnorm = vnorm;
@@ -290,10 +291,11 @@ cudaError_t launch_value_norm_tc(const Dims& dm, int d_model, const void* v, con
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(value_norm_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kVnSmem)) != cudaSuccess)
-    return e;
+  auto kern = dm.d == 128 ? value_norm_tc_kernel<2> : value_norm_tc_kernel<1>;
+  const int smem = vn_smem(dm.d / 64);
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
   const long long grid = a.items < sms ? a.items : sms;  // one CTA per SM: each owns the SM's tensor memory
-  value_norm_tc_kernel<<<(unsigned)grid, kVnThreads, kVnSmem, lc.st>>>(vm, a);
+  kern<<<(unsigned)grid, kVnThreads, smem, lc.st>>>(vm, a);
   lc.mark("value_norm_tc");
   return cudaGetLastError();
 }

@@ -76,6 +76,23 @@ def test_value_norms_tensor_core_against_fp32_pipes(monkeypatch):
     np.testing.assert_allclose(tc, simt, rtol=2e-5, atol=1e-30)
 
 
+@pytest.mark.parametrize("S,L,H,G,d,T,w,Kmax,Dm,with_kd", [
+    (1, 1, 2, 1, 64, 130, 1, 1, 64, True),        # one step, one query head; a key tile with two keys
+    (1, 1, 2, 2, 128, 129, 32, 65, 40, True),     # steps just past one query tile; odd panel width
+    (2, 1, 1, 3, 64, 700, 32, 33, 256, False),    # padded group, two sequences
+    (1, 2, 2, 4, 128, 300, 16, 130, 72, True),    # five query tiles: the maximum runs over three launches; two decode tiles
+    (1, 1, 1, 7, 64, 4000, 32, 17, 512, True),    # the keys of a row in several parts
+    (1, 1, 2, 8, 128, 256, 32, 16, 64, False),    # whole steps and key tiles only
+])
+def test_tensor_core_importance_against_fp32_pipes(monkeypatch, S, L, H, G, d, T, w, Kmax, Dm, with_kd):
+    q, k, v, kd, wo = _inputs(S, L, H, G, d, T, Kmax, Dm, torch.bfloat16, seed=T + G, scale=1.5)
+    p = lukv.make_params(S, L, H, G, d, T, w, 1, torch.bfloat16, 2)
+    tc = gpu_importance(p, Kmax, Dm, q, k, v, kd if with_kd else None, wo, False)
+    monkeypatch.setenv("LUKV_FORCE_SIMT", "1")
+    simt = gpu_importance(p, Kmax, Dm, q, k, v, kd if with_kd else None, wo, False)
+    np.testing.assert_allclose(tc, simt, rtol=1e-4, atol=1e-30)
+
+
 def test_importance_at_the_benchmark_size_sampled_heads(oracle):
     """The size bench.py times (one calibration query of 4000 tokens, 256 KV heads x 4 query heads, 64 decode steps,
     model width 4096; the value norms run on the tensor cores over 1024 work items): two sampled heads against the
