@@ -1,4 +1,4 @@
-// Stage (a) on the 5th-generation tensor cores (bf16, head_dim 128): one persistent kernel
+// Stage (a) on the 5th-generation tensor cores (bf16): one persistent kernel
 // computes the un-pooled observation-window scores of every head.
 //
 // The window logits S = Q K^T of Eq. 1 (Sec. 3.1) come from tcgen05.mma with fp32
@@ -34,7 +34,8 @@ namespace {
 
 // ---- shared-memory layout ---------------------------------------------------------------------
 
-template <int MT, int NQ>
+// NH: halves of 64 channels, d = 64 NH.
+template <int MT, int NQ, int NH>
 struct Plan {
   static_assert(MT == 1 || NQ == 2, "two query-row blocks are split over exactly two quads");
   // An mbarrier wait only knows the parity of the phase it waits for, so the successive phases of a
@@ -53,7 +54,8 @@ struct Plan {
   // odd count the two issuers would take turns on a stage, and the one that runs ahead could wait
   // for a phase two ahead of the barrier -- which a parity wait reports as complete while the
   // previous load of that stage is still in flight.
-  static constexpr int kStages = MT == 1 ? 4 : 2;
+  static constexpr int kStages = (MT == 1 ? 4 : 2) * (3 - NH);
+  static constexpr int kStageBytes = NH * kHalfBytes;
   static_assert(kStages % 2 == 0, "a key stage must always be consumed by the same MMA issuer");
   static constexpr int kQSlots = 2;                    // query tiles of the job in the tensor pipe and the next one
   static constexpr int kQBytes = MT * kStageBytes;     // [half][MT*128 rows][128 B]
@@ -159,12 +161,12 @@ __device__ __forceinline__ Job decode_job(int idx, int K, const FusedArgs& a) {
   return make_job<RAGGED>(K - lead + (r - pairs), true, a);
 }
 
-template <int MT, int NQ, bool RAGGED>
-__global__ void __launch_bounds__(Plan<MT, NQ>::kThreads, 1)
+template <int MT, int NQ, int NH, bool RAGGED>
+__global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
     score_fused_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                        const FusedArgs a) {
-  using P = Plan<MT, NQ>;
-  constexpr int kStages = P::kStages;
+  using P = Plan<MT, NQ, NH>;
+  constexpr int kStages = P::kStages, kStageBytes = P::kStageBytes;
   constexpr int kNumBufs = P::kNumBufs;
   constexpr int kEpiWarps = P::kEpiWarps;
   constexpr int kRowsPad = 128 * MT;
@@ -229,7 +231,7 @@ __global__ void __launch_bounds__(Plan<MT, NQ>::kThreads, 1)
         if (!mbar_wait(bar(P::kBarQEmpty, slot), ((jq / P::kQSlots) & 1) ^ 1, abort_flag, a.dev_status, a.spin_limit)) break;
         mbar_expect_tx(bar(P::kBarQFull, slot), P::kQBytes);
         const uint32_t qd = q_s + slot * P::kQBytes;
-        for (int h = 0; h < 2; ++h)
+        for (int h = 0; h < NH; ++h)
           for (int mt = 0; mt < MT; ++mt) {
             const uint32_t dst = qd + h * (MT * kHalfBytes) + mt * kHalfBytes;
             if (a.l2_hints) tma_load_2d_hint(dst, &q_map, bar(P::kBarQFull, slot), h * 64, j.u * a.M + mt * 128, keep);
@@ -245,11 +247,9 @@ __global__ void __launch_bounds__(Plan<MT, NQ>::kThreads, 1)
           const uint32_t dst = k_s + s * kStageBytes;
           if (a.l2_hints) {
             const uint64_t pol = j.p2 ? drop : keep;
-            tma_load_2d_hint(dst, &k_map, bar(P::kBarFull, s), 0, row, pol);
-            tma_load_2d_hint(dst + kHalfBytes, &k_map, bar(P::kBarFull, s), 64, row, pol);
+            for (int h = 0; h < NH; ++h) tma_load_2d_hint(dst + h * kHalfBytes, &k_map, bar(P::kBarFull, s), h * 64, row, pol);
           } else {
-            tma_load_2d(dst, &k_map, bar(P::kBarFull, s), 0, row);
-            tma_load_2d(dst + kHalfBytes, &k_map, bar(P::kBarFull, s), 64, row);
+            for (int h = 0; h < NH; ++h) tma_load_2d(dst + h * kHalfBytes, &k_map, bar(P::kBarFull, s), h * 64, row);
           }
         }
         if (!ok) break;
@@ -289,7 +289,7 @@ __global__ void __launch_bounds__(Plan<MT, NQ>::kThreads, 1)
 #pragma unroll
             for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-              for (int ks = 0; ks < 8; ++ks) {
+              for (int ks = 0; ks < 4 * NH; ++ks) {
                 const int h = ks >> 2, sub = ks & 3;
                 const uint64_t da = smem_desc_sw128(qd + h * (MT * kHalfBytes) + mt * kHalfBytes) + (uint64_t)(sub * 2);
                 const uint64_t db = smem_desc_sw128(kt + h * kHalfBytes) + (uint64_t)(sub * 2);
@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(Plan<MT, NQ>::kThreads, 1)
             // D[key][q row]: A = K tile, B = Q (npad rows)
             const uint32_t idesc = instr_desc_bf16(128, a.npad);
 #pragma unroll
-            for (int ks = 0; ks < 8; ++ks) {
+            for (int ks = 0; ks < 4 * NH; ++ks) {
               const int h = ks >> 2, sub = ks & 3;
               const uint64_t da = smem_desc_sw128(kt + h * kHalfBytes) + (uint64_t)(sub * 2);
               const uint64_t db = smem_desc_sw128(qd + h * (MT * kHalfBytes)) + (uint64_t)(sub * 2);
@@ -610,12 +610,12 @@ __global__ void __launch_bounds__(Plan<MT, NQ>::kThreads, 1)
 
 // ---- host side --------------------------------------------------------------------------------
 
-template <int MT, int NQ, bool RAGGED = false>
+template <int MT, int NQ, int NH, bool RAGGED = false>
 cudaError_t launch_fused(const CUtensorMap& qm, const CUtensorMap& km, FusedArgs args, int spare_sms, LaunchCtx& lc,
                          const int32_t* seq_T_host = nullptr) {
-  using P = Plan<MT, NQ>;
+  using P = Plan<MT, NQ, NH>;
   const int smem = P::kTotal;
-  auto kern = score_fused_kernel<MT, NQ, RAGGED>;
+  auto kern = score_fused_kernel<MT, NQ, NH, RAGGED>;
   cudaError_t e;
   if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
   int dev = 0, sms = 0, per_sm = 0;
@@ -705,7 +705,7 @@ size_t score_tc_flag_bytes(const Dims& dm) {
 }
 
 bool score_tc_supported(const Dims& dm) {
-  return dm.dtype == LUKV_DTYPE_BF16 && dm.d == 128 && encode_fn() != nullptr;
+  return dm.dtype == LUKV_DTYPE_BF16 && encode_fn() != nullptr;
 }
 
 cudaError_t launch_score_tc(const Dims& dm, const void* q, const void* k, const Workspace& ws, int32_t* dev_status,
@@ -719,7 +719,7 @@ cudaError_t launch_score_tc(const Dims& dm, const void* q, const void* k, const 
     if (e1 != cudaErrorNotSupported) return e1;
   }
   CUtensorMap qm, km;
-  if (!make_map(&qm, q, (uint64_t)dm.heads() * dm.M) || !make_map(&km, k, (uint64_t)dm.heads() * dm.T))
+  if (!make_map(&qm, q, (uint64_t)dm.heads() * dm.M, dm.d) || !make_map(&km, k, (uint64_t)dm.heads() * dm.T, dm.d))
     return cudaErrorInvalidValue;
   FusedArgs args;
   args.stats = ws.stats;
@@ -758,13 +758,18 @@ cudaError_t launch_score_tc(const Dims& dm, const void* q, const void* k, const 
   if (dm.seq_T) {
     // sequences of different lengths: the whole call in one launch (no head ranges), work items dealt per sequence
     if (hr.h0 != 0 || hr.nh != (int)dm.heads() || dm.S > kMaxRaggedSeqs) return cudaErrorInvalidValue;
-    return dm.M > 128 ? launch_fused<2, 2, true>(qm, km, args, spare_sms, lc, dm.seq_T)
-                      : launch_fused<1, 2, true>(qm, km, args, spare_sms, lc, dm.seq_T);
+    if (dm.d == 64)
+      return dm.M > 128 ? launch_fused<2, 2, 1, true>(qm, km, args, spare_sms, lc, dm.seq_T)
+                        : launch_fused<1, 2, 1, true>(qm, km, args, spare_sms, lc, dm.seq_T);
+    return dm.M > 128 ? launch_fused<2, 2, 2, true>(qm, km, args, spare_sms, lc, dm.seq_T)
+                      : launch_fused<1, 2, 2, true>(qm, km, args, spare_sms, lc, dm.seq_T);
   }
-  if (dm.M > 128) return launch_fused<2, 2>(qm, km, args, spare_sms, lc);
+  if (dm.d == 64)
+    return dm.M > 128 ? launch_fused<2, 2, 1>(qm, km, args, spare_sms, lc) : launch_fused<1, 2, 1>(qm, km, args, spare_sms, lc);
+  if (dm.M > 128) return launch_fused<2, 2, 2>(qm, km, args, spare_sms, lc);
   static const int quads = env_int("LUKV_QUADS", 2, 3, 2);
-  if (quads == 3) return launch_fused<1, 3>(qm, km, args, spare_sms, lc);
-  return launch_fused<1, 2>(qm, km, args, spare_sms, lc);
+  if (quads == 3) return launch_fused<1, 3, 2>(qm, km, args, spare_sms, lc);
+  return launch_fused<1, 2, 2>(qm, km, args, spare_sms, lc);
 }
 
 }  // namespace lukv
