@@ -50,6 +50,25 @@ def test_calibration_size(oracle):
     assert (np.diff(got.astype(np.float64), axis=-1) >= 0).all()
 
 
+@pytest.mark.parametrize("n,w,n_sink", [(511, 1, 0), (512, 8, 512), (513, 7, 4), (4096, 4, 3), (4097, 3, 0), (8193, 7, 5),
+                                        (16384, 16, 4)])
+@pytest.mark.parametrize("values", ["lognormal", "signed", "runs", "two"])
+def test_bucket_kernel_edges(oracle, n, w, n_sink, values):
+    """Sizes around the thread counts and value distributions that fill the buckets differently: scores over orders of
+    magnitude, of both signs, in runs of equals, and so few values that the kernel sorts instead."""
+    rng = np.random.default_rng(n + n_sink)
+    s = rng.standard_normal(n)
+    s = {"lognormal": np.exp(2 * s), "signed": s / 4, "runs": np.repeat(np.exp(s), 7)[:n],
+         "two": (s > 0).astype(float)}[values]
+    scores = np.ascontiguousarray(s, np.float32).reshape(1, 1, n)
+    imp = rng.exponential(size=(1, 1, n)).astype(np.float32)
+    T = n + w
+    P = 5 if T % 4 == 0 else 2
+    p = lukv.make_params(1, 1, 1, 1, 64, T, w, 1, "fp32", P, n_sink=n_sink)
+    ref = oracle.build_curves(scores.reshape(1, n), imp.reshape(1, n), T, w, P, n_sink=n_sink)
+    np.testing.assert_allclose(gpu_curves(p, scores, imp).reshape(1, P), ref, rtol=RTOL, atol=0)
+
+
 def test_beyond_the_sorting_kernel(oracle):
     # more than 16384 positions: ranks by counting instead of the shared-memory sort
     _case(oracle, 1, 1, 2, 20000, 32, 126, n_sink=4, seed=6, ties=True)
