@@ -732,11 +732,9 @@ inline size_t greedy_smem_bytes(int N, int cap, int groups, bool one) {
 // share the budgets): set i reads the lists of curves i*N .., writes budgets + i*set.budgets and offsets +
 // i*set.offsets.  The hot path launches one set.
 template <bool ONE>
-__global__ void __launch_bounds__(kGreedyMaxThreads) greedy_kernel(HullLists lists, const __grid_constant__ GreedyArgs args,
-                                                                   int32_t* __restrict__ budgets,
-                                                                   int32_t* __restrict__ offsets, SetStride set,
-                                                                   int N, int P, int w, int cap, int group) {
-  extern __shared__ __align__(16) unsigned char greedy_smem[];
+__device__ __forceinline__ void greedy_cta(unsigned char* greedy_smem, const HullLists& lists, const GreedyArgs& args,
+                                           int32_t* __restrict__ budgets, int32_t* __restrict__ offsets,
+                                           const SetStride& set, int N, int P, int w, int cap, int group) {
   __shared__ GreedyShared shared[kGreedyMaxGroups];
   const int groups = blockDim.x / group;
   const int mine = threadIdx.x / group;
@@ -754,8 +752,6 @@ __global__ void __launch_bounds__(kGreedyMaxThreads) greedy_kernel(HullLists lis
   const size_t curve0 = (size_t)blockIdx.y * N;
   budgets += (size_t)blockIdx.y * set.budgets;
   offsets += (size_t)blockIdx.y * set.offsets;
-  pdl_launch_dependents();
-  pdl_wait();  // the lists come from the launch before
   const int* count = lists.count + curve0;
 
   bool staged = false;
@@ -798,6 +794,39 @@ __global__ void __launch_bounds__(kGreedyMaxThreads) greedy_kernel(HullLists lis
   }
 }
 
+template <bool ONE>
+__global__ void __launch_bounds__(kGreedyMaxThreads) greedy_kernel(HullLists lists, const __grid_constant__ GreedyArgs args,
+                                                                   int32_t* __restrict__ budgets,
+                                                                   int32_t* __restrict__ offsets, SetStride set,
+                                                                   int N, int P, int w, int cap, int group) {
+  extern __shared__ __align__(16) unsigned char greedy_smem[];
+  pdl_launch_dependents();
+  pdl_wait();  // the lists come from the launch before
+  greedy_cta<ONE>(greedy_smem, lists, args, budgets, offsets, set, N, P, w, cap, group);
+}
+
+// Hull and greedy of up to 1024 heads by one CTA: a warp walks every 32nd curve, then the groups take the sequences.  It
+// fits the SM that a persistent scorer leaves free and is done long before the scorer where heads are many, so that the whole
+// path needs no second stream: the scorer, this kernel as its programmatic
+// dependent, which does not wait for the scorer before its own end, then the selection, which waits for this one.
+__global__ void __launch_bounds__(kGreedyMaxThreads) alloc_kernel(const float* __restrict__ curves, HullLists lists,
+                                                                  const __grid_constant__ GreedyArgs args,
+                                                                  int32_t* __restrict__ budgets,
+                                                                  int32_t* __restrict__ offsets, int N, int P, int w, int cap,
+                                                                  int group) {
+  extern __shared__ __align__(16) unsigned char greedy_smem[];
+  pdl_launch_dependents();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int h = warp; h < N; h += blockDim.x >> 5) {
+    const int count = hull_walk_short(curves + (size_t)h * P, P, lane,
+                                      HullOut{lists.gain + (size_t)h * (P - 1), lists.start + (size_t)h * (P - 1)});
+    if (lane == 0) lists.count[h] = count;
+  }
+  __syncthreads();
+  greedy_cta<true>(greedy_smem, lists, args, budgets, offsets, SetStride{0, 0}, N, P, w, cap, group);
+  pdl_wait();
+}
+
 // Hull and greedy of up to 32 heads in one launch: one CTA per sequence, a warp per head walks the head's curve into
 // shared memory (the curves are shared by the sequences; a walk costs less than handing lists over between launches).
 // For calls of one or a few layers, where allocation is on the critical path: 8 heads x 129 points 29 + 34 us as two
@@ -819,6 +848,7 @@ __global__ void __launch_bounds__(32 * kSmallMaxHeads) alloc_small_kernel(const 
   __shared__ int weight[kGreedyCountMax + kSmallMaxHeads];
   float* gain = reinterpret_cast<float*>(small_smem);                              // [N][P], then packed
   unsigned short* start = reinterpret_cast<unsigned short*>(gain + (size_t)N * P);
+  pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int count = 0;
   if (warp < N) {
@@ -859,6 +889,7 @@ __global__ void __launch_bounds__(32 * kSmallMaxHeads) alloc_small_kernel(const 
   const ListView<true> lists = {gain, start, at, nullptr, P - 1};
   const Group grp = {(int)threadIdx.x, (int)blockDim.x, 0};
   greedy_problem<true, true>(lists, args, blockIdx.x, N, w, nullptr, nullptr, nullptr, weight, sh, grp, budgets, offsets);
+  pdl_wait();
 }
 
 GreedyArgs greedy_args(const Dims& dm, const int64_t* budgets_host, int q0, int cnt, long long* row_base) {
@@ -921,7 +952,7 @@ cudaError_t launch_greedy(const Dims& dm, const HullLists& lists, const int64_t*
   const int groups = n_sets > 1 && one ? std::min(kGreedyMaxGroups, std::max(1, std::min(dm.S, kGreedyMaxThreads / group))) : 1;
   const size_t smem = greedy_smem_bytes(dm.N, cap, groups, one);
   auto kern = one ? greedy_kernel<true> : greedy_kernel<false>;
-  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+  if ((e = allow_smem((const void*)kern, smem)) != cudaSuccess) return e;
   SetStride set;
   set.budgets = (size_t)dm.S * dm.N;
   set.offsets = (size_t)dm.S * dm.N + 1;
@@ -940,21 +971,38 @@ cudaError_t launch_greedy(const Dims& dm, const HullLists& lists, const int64_t*
   return cudaGetLastError();
 }
 
+bool allocate_one_launch(const Dims& dm) {
+  return dm.N <= kGreedyMaxThreads && dm.P <= kHullRegsMaxP && dm.S <= kSeqPerLaunch;
+}
+
+cudaError_t launch_allocate_one(const Dims& dm, const float* curves, const int64_t* budgets_host, const HullLists& lists,
+                                int32_t* budgets, int32_t* offsets, bool beside, LaunchCtx& lc) {
+  long long base = 0;
+  const GreedyArgs args = greedy_args(dm, budgets_host, 0, dm.S, &base);
+  cudaError_t e;
+  if (dm.N <= kSmallMaxHeads) {
+    const size_t smem = alloc_small_smem_bytes(dm.N, dm.P);
+    if ((e = allow_smem((const void*)alloc_small_kernel, smem)) != cudaSuccess) return e;
+    e = launch_pdl(alloc_small_kernel, dim3(dm.S), dim3(32 * dm.N), smem, lc.st, beside, curves, args, budgets, offsets, dm.N,
+                   dm.P, dm.w);
+  } else {
+    const int group = (dm.N + 31) & ~31, groups = std::min(kGreedyMaxGroups, kGreedyMaxThreads / group);
+    const int cap = (int)std::min((long long)dm.N * (dm.P - 1), 16384LL);
+    const size_t smem = greedy_smem_bytes(dm.N, cap, groups, true);
+    if ((e = allow_smem((const void*)alloc_kernel, smem)) != cudaSuccess) return e;
+    e = launch_pdl(alloc_kernel, dim3(1), dim3(group * groups), smem, lc.st, beside, curves, lists, args, budgets, offsets,
+                   dm.N, dm.P, dm.w, cap, group);
+  }
+  if (e != cudaSuccess) return e;
+  lc.mark("allocate");
+  return cudaGetLastError();
+}
+
 cudaError_t launch_allocate(const Dims& dm, const float* curves, const int64_t* budgets_host, const HullLists& lists,
                             int32_t* budgets, int32_t* offsets, LaunchCtx& lc) {
-  if (dm.N <= kSmallMaxHeads && dm.P <= kHullRegsMaxP) {
-    const size_t smem = alloc_small_smem_bytes(dm.N, dm.P);
-    cudaError_t e = cudaFuncSetAttribute(alloc_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    long long base = 0;
-    for (int q0 = 0; q0 < dm.S; q0 += kSeqPerLaunch) {
-      const int cnt = dm.S - q0 < kSeqPerLaunch ? dm.S - q0 : kSeqPerLaunch;
-      const GreedyArgs args = greedy_args(dm, budgets_host, q0, cnt, &base);
-      alloc_small_kernel<<<cnt, 32 * dm.N, smem, lc.st>>>(curves, args, budgets, offsets, dm.N, dm.P, dm.w);
-      lc.mark("allocate");
-    }
-    return cudaGetLastError();
-  }
+  // alone: up to 32 heads in one launch; more heads walk their curves on as many SMs as there are
+  if (allocate_one_launch(dm) && dm.N <= kSmallMaxHeads)
+    return launch_allocate_one(dm, curves, budgets_host, lists, budgets, offsets, false, lc);
   cudaError_t e = launch_hull(curves, lists, dm.N, dm.P, lc);
   if (e != cudaSuccess) return e;
   return launch_greedy(dm, lists, budgets_host, budgets, offsets, 1, lc);

@@ -3,7 +3,9 @@
 #include <math.h>
 #include <stdlib.h>
 
+#include <atomic>
 #include <mutex>
+#include <unordered_map>
 
 #include "common.cuh"
 
@@ -23,15 +25,14 @@ Workspace carve_workspace(const Dims& dm, void* base) {
     return r;
   };
   const size_t heads = (size_t)dm.heads();
-  ws.raw = static_cast<float*>(take(heads * dm.n * sizeof(float)));
-  ws.pooled = static_cast<float*>(take(heads * dm.n * sizeof(float)));
+  ws.raw = static_cast<float*>(take(heads * dm.raw_stride() * sizeof(float)));
+  ws.pooled = static_cast<float*>(take(heads * dm.raw_stride() * sizeof(float)));
   const size_t stats_simt = heads * score_chunks(dm) * dm.M * 2 * sizeof(float);
   size_t stats_bytes = score_tc_stats_bytes(dm);
   if (stats_simt > stats_bytes) stats_bytes = stats_simt;
   if (score_onepass_stats_bytes(dm) > stats_bytes) stats_bytes = score_onepass_stats_bytes(dm);
   if (keydiff_scratch_bytes(dm) > stats_bytes) stats_bytes = keydiff_scratch_bytes(dm);
   ws.stats = static_cast<float*>(take(stats_bytes));
-  ws.lse = static_cast<float*>(take(heads * dm.M * sizeof(float)));
   ws.hull = hull_lists(take(hull_lists_bytes(dm.N, dm.P)), dm.N, dm.P);
   ws.head_flags = static_cast<int*>(take(score_tc_flag_bytes(dm)));
   ws.bytes = off;
@@ -123,20 +124,63 @@ static bool force_simt() {
   return v;
 }
 
-static HeadRange all_heads(const Dims& dm) { return HeadRange{0, (int)dm.heads()}; }
-
-static cudaError_t run_score(const Dims& dm, const void* q, const void* k, const Workspace& ws, float* pooled_out,
-                             int32_t* dev_status, LaunchCtx& lc) {
-  if (dm.keydiff) return launch_keydiff(dm, k, pooled_out, ws.stats, dev_status, 0, lc);  // nothing to pool
-  cudaError_t e = (score_tc_supported(dm) && !force_simt())
-                      ? launch_score_tc(dm, q, k, ws, dev_status, all_heads(dm), true, 0, lc)
-                      : launch_score_simt(dm, q, k, ws, lc);
-  if (e != cudaSuccess) return e;
-  return launch_pool(dm, ws.raw, pooled_out, all_heads(dm), lc);
+// Scores of all heads into the workspace: un-pooled ones, or the KeyDiff scores (nothing to pool).  `beside`: an allocation
+// kernel was launched just before (general-shape scorer) or follows (persistent scorers, which leave it `spare` SMs).
+static cudaError_t run_score(const Dims& dm, const void* q, const void* k, const Workspace& ws, int spare, bool beside,
+                             LaunchCtx& lc) {
+  if (dm.keydiff) return launch_keydiff(dm, k, ws.raw, dm.raw_stride(), ws.stats, nullptr, spare, lc);
+  if (score_tc_supported(dm) && !force_simt()) return launch_score_tc(dm, q, k, ws, spare, lc);
+  return launch_score_simt(dm, q, k, ws, beside, lc);
 }
 
-// An auxiliary stream and the two events that tie it to the caller's stream, created on first
-// use on a device and kept until the process exits (handles only, no device memory).
+// The scorer's status word, or null where it has no bounded wait.
+static const int* score_status(const Dims& dm, const Workspace& ws) {
+  if (dm.keydiff) return keydiff_status(dm, ws.stats);
+  return score_tc_supported(dm) && !force_simt() ? score_tc_status(dm, ws) : nullptr;
+}
+
+int device_index() {
+  int dev = -1;
+  return cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64 ? dev : -1;
+}
+
+cudaError_t device_sms(int* sms) {
+  static std::atomic<int> table[64];
+  const int dev = device_index();
+  if (dev < 0) return cudaErrorInvalidDevice;
+  int v = table[dev].load(std::memory_order_relaxed);
+  if (v == 0) {
+    const cudaError_t e = cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    table[dev].store(v, std::memory_order_relaxed);
+  }
+  *sms = v;
+  return cudaSuccess;
+}
+
+cudaError_t allow_smem(const void* kernel, size_t bytes) {
+  if (bytes <= 48 * 1024) return cudaSuccess;
+  static std::mutex mu;
+  static std::unordered_map<const void*, uint64_t> done;  // bit d: set on device d
+  const int dev = device_index();
+  if (dev < 0) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lock(mu);
+  uint64_t& bits = done[kernel];
+  if ((bits >> dev) & 1) return cudaSuccess;
+  cudaFuncAttributes fa;
+  cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
+  if (e != cudaSuccess) return e;
+  int most = 0;
+  if ((e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes)) !=
+      cudaSuccess)
+    return e;
+  bits |= 1ull << dev;
+  return cudaSuccess;
+}
+
+// An auxiliary stream and the two events that tie it to the caller's stream (allocations too large for one launch), created
+// on first use on a device and kept until the process exits (handles only, no device memory).
 struct SideStream {
   cudaStream_t stream = nullptr;
   cudaEvent_t fork = nullptr, join = nullptr;
@@ -162,48 +206,63 @@ static SideStream* side_stream() {
   return &s;
 }
 
-// The whole path.  Allocation depends only on the curves, scoring only on Q/K; selection needs
-// both, the gather follows.  With `overlap` the two allocation kernels run on an auxiliary stream
-// beside the scorer, which then leaves one SM to them (its CTAs fill theirs completely); the
-// caller's stream waits for the budgets before selection, so stream order is preserved.
+// The whole path.  Allocation depends only on the curves, scoring only on Q/K; selection needs both, the gather follows.
+// With `overlap` allocation runs beside the scorer, normally as one CTA: behind a persistent scorer (tensor-core, KeyDiff),
+// which leaves it an SM, or ahead of the general-shape scorer's first sweep.  Neighbours in the stream are programmatic
+// dependents; whichever of scorer and allocation comes second ends after the first, so that the selection, which waits for
+// the second, sees both.  Allocations too large for one launch run on an auxiliary stream.
 static int run_compress(const Dims& dm, const void* q_win, const void* k, const void* v, const float* curves,
                         const int64_t* budgets_in, void* k_out, void* v_out, int32_t* kept_idx, int32_t* budgets,
                         int32_t* offsets, int64_t rows_cap, int32_t* dev_status, const Workspace& w, LaunchCtx& lc,
                         bool overlap) {
-  if (dev_status && cudaMemsetAsync(dev_status, 0, sizeof(int32_t), lc.st) != cudaSuccess) return LUKV_ERR_CUDA;
-  const bool tc = score_tc_supported(dm) && !force_simt();
-  // the persistent scorers (tensor-core, KeyDiff) leave one SM to the allocation kernels of the auxiliary stream;
-  // the FP32-pipe scorer's ordinary grids simply share the SMs with them
-  SideStream* side = overlap ? side_stream() : nullptr;
-  int rc = LUKV_OK;
-  if (side) {
+  const bool persistent = dm.keydiff || (score_tc_supported(dm) && !force_simt());
+  bool chained = overlap;  // the selection is the dependent of the launch before it
+  if (overlap && allocate_one_launch(dm)) {
+    auto allocate = [&](bool beside) {
+      return launch_allocate_one(dm, curves, budgets_in, w.hull, budgets, offsets, beside, lc);
+    };
+    if (!persistent && allocate(false) != cudaSuccess) return LUKV_ERR_CUDA;
+    if (run_score(dm, q_win, k, w, 1, true, lc) != cudaSuccess) return LUKV_ERR_CUDA;
+    if (persistent && allocate(true) != cudaSuccess) return LUKV_ERR_CUDA;
+  } else if (SideStream* side = overlap ? side_stream() : nullptr) {
     std::lock_guard<std::mutex> in_use(side->use);
     LaunchCtx ls;
     ls.st = side->stream;
+    int rc = LUKV_OK;
     if (cudaEventRecord(side->fork, lc.st) != cudaSuccess || cudaStreamWaitEvent(ls.st, side->fork, 0) != cudaSuccess)
       return LUKV_ERR_CUDA;
     if (launch_allocate(dm, curves, budgets_in, w.hull, budgets, offsets, ls) != cudaSuccess) rc = LUKV_ERR_CUDA;
     if (cudaEventRecord(side->join, ls.st) != cudaSuccess) rc = LUKV_ERR_CUDA;
     lc.launches += ls.launches;
-    if (rc == LUKV_OK && dm.keydiff) {
-      if (launch_keydiff(dm, k, w.pooled, w.stats, dev_status, 1, lc) != cudaSuccess) rc = LUKV_ERR_CUDA;
-    } else if (rc == LUKV_OK && tc) {
-      if (launch_score_tc(dm, q_win, k, w, dev_status, all_heads(dm), true, 1, lc) != cudaSuccess ||
-          launch_pool(dm, w.raw, w.pooled, all_heads(dm), lc) != cudaSuccess)
-        rc = LUKV_ERR_CUDA;
-    } else if (rc == LUKV_OK) {
-      if (run_score(dm, q_win, k, w, w.pooled, dev_status, lc) != cudaSuccess) rc = LUKV_ERR_CUDA;
-    }
+    if (rc == LUKV_OK && run_score(dm, q_win, k, w, 1, false, lc) != cudaSuccess) rc = LUKV_ERR_CUDA;
     // join even after a failure: the caller's stream must not run ahead of work already enqueued
     if (cudaStreamWaitEvent(lc.st, side->join, 0) != cudaSuccess) rc = LUKV_ERR_CUDA;
     if (rc != LUKV_OK) return rc;
+    chained = false;
   } else {
     if (launch_allocate(dm, curves, budgets_in, w.hull, budgets, offsets, lc) != cudaSuccess) return LUKV_ERR_CUDA;
-    if (run_score(dm, q_win, k, w, w.pooled, dev_status, lc) != cudaSuccess) return LUKV_ERR_CUDA;
+    if (run_score(dm, q_win, k, w, 0, false, lc) != cudaSuccess) return LUKV_ERR_CUDA;
+    chained = false;
   }
-  if (launch_select(dm, w.pooled, budgets, offsets, kept_idx, rows_cap, all_heads(dm), lc) != cudaSuccess)
+  const float* scores = w.raw;
+  const bool pool = !dm.keydiff && select_pools(dm);
+  if (!dm.keydiff && !pool) {
+    if (launch_pool(dm, w.raw, w.pooled, dm.raw_stride(), lc) != cudaSuccess) return LUKV_ERR_CUDA;
+    scores = w.pooled;
+    chained = false;
+  }
+  if (launch_select(dm, scores, dm.raw_stride(), pool, budgets, offsets, kept_idx, rows_cap, score_status(dm, w), dev_status,
+                    chained, lc) != cudaSuccess)
     return LUKV_ERR_CUDA;
-  if (launch_gather(dm, offsets, kept_idx, k, v, k_out, v_out, rows_cap, all_heads(dm), lc) != cudaSuccess)
+  if (launch_gather(dm, offsets, kept_idx, k, v, k_out, v_out, rows_cap, overlap, lc) != cudaSuccess) return LUKV_ERR_CUDA;
+  return LUKV_OK;
+}
+
+// Scores for the caller: [heads][n].
+static int score_to(const Dims& dm, const void* q, const void* k, float* scores, const Workspace& w, LaunchCtx& lc) {
+  if (dm.keydiff)
+    return launch_keydiff(dm, k, scores, dm.n, w.stats, nullptr, 0, lc) == cudaSuccess ? LUKV_OK : LUKV_ERR_CUDA;
+  if (run_score(dm, q, k, w, 0, false, lc) != cudaSuccess || launch_pool(dm, w.raw, scores, dm.n, lc) != cudaSuccess)
     return LUKV_ERR_CUDA;
   return LUKV_OK;
 }
@@ -252,7 +311,7 @@ int lukv_score(const lukv_params_t* params, const void* q_win, const void* k, fl
   if ((rc = check_ws(dm, ws, ws_bytes, &w)) != LUKV_OK) return rc;
   LaunchCtx lc;
   lc.st = (cudaStream_t)stream;
-  if (run_score(dm, q_win, k, w, scores, nullptr, lc) != cudaSuccess) return LUKV_ERR_CUDA;
+  if ((rc = score_to(dm, q_win, k, scores, w, lc)) != LUKV_OK) return rc;
   g_last_launches = lc.launches;
   return LUKV_OK;
 }
@@ -268,7 +327,7 @@ int lukv_score_keydiff(const lukv_params_t* params, const void* k, float* scores
   LaunchCtx lc;
   lc.st = (cudaStream_t)stream;
   if (dev_status && cudaMemsetAsync(dev_status, 0, sizeof(int32_t), lc.st) != cudaSuccess) return LUKV_ERR_CUDA;
-  if (launch_keydiff(dm, k, scores, w.stats, dev_status, 0, lc) != cudaSuccess) return LUKV_ERR_CUDA;
+  if (launch_keydiff(dm, k, scores, dm.n, w.stats, dev_status, 0, lc) != cudaSuccess) return LUKV_ERR_CUDA;
   g_last_launches = lc.launches;
   return LUKV_OK;
 }
@@ -284,7 +343,7 @@ int lukv_score_ragged(const lukv_params_t* params, const int32_t* ctx_lens, cons
   if ((rc = check_ws(dm, ws, ws_bytes, &w)) != LUKV_OK) return rc;
   LaunchCtx lc;
   lc.st = (cudaStream_t)stream;
-  if (run_score(dm, q_win, k, w, scores, nullptr, lc) != cudaSuccess) return LUKV_ERR_CUDA;
+  if ((rc = score_to(dm, q_win, k, scores, w, lc)) != LUKV_OK) return rc;
   g_last_launches = lc.launches;
   return LUKV_OK;
 }
@@ -322,10 +381,9 @@ static int select_gather_impl(const lukv_params_t* params, const int32_t* ctx_le
   if ((rc = check_ws(dm, ws, ws_bytes, &w)) != LUKV_OK) return rc;
   LaunchCtx lc;
   lc.st = (cudaStream_t)stream;
-  if (launch_select(dm, scores, budgets, offsets, kept_idx, rows_cap, all_heads(dm), lc) != cudaSuccess)
+  if (launch_select(dm, scores, dm.n, false, budgets, offsets, kept_idx, rows_cap, nullptr, nullptr, false, lc) != cudaSuccess)
     return LUKV_ERR_CUDA;
-  if (launch_gather(dm, offsets, kept_idx, k, v, k_out, v_out, rows_cap, all_heads(dm), lc) != cudaSuccess)
-    return LUKV_ERR_CUDA;
+  if (launch_gather(dm, offsets, kept_idx, k, v, k_out, v_out, rows_cap, true, lc) != cudaSuccess) return LUKV_ERR_CUDA;
   g_last_launches = lc.launches;
   return LUKV_OK;
 }

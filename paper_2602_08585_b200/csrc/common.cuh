@@ -28,6 +28,7 @@ struct Dims {
   float min_keep = 0.f;  // as given (the per-sequence floors of a ragged call are derived from it)
   bool keydiff = false;  // stage (a) is the KeyDiff metric (keys only, no pooling)
   int64_t heads() const { return (int64_t)S * N; }
+  int raw_stride() const { return (n + 3) & ~3; }  // floats between the rows of the un-pooled scores: 16-byte rows
   size_t esize() const { return dtype == LUKV_DTYPE_BF16 ? 2 : 4; }
 };
 
@@ -43,19 +44,19 @@ size_t hull_lists_bytes(int64_t n_curves, int P);
 
 // Workspace carve-up (all offsets 256-byte aligned).
 struct Workspace {
-  float* raw;        // [S*N][n]   un-pooled scores
-  float* pooled;     // [S*N][n]   pooled scores (fused path)
+  float* raw;        // [S*N][raw_stride]  un-pooled scores
+  float* pooled;     // [S*N][raw_stride]  pooled scores (whole path, where the selection does not pool)
   float* stats;      // partial (reference, sum-exp) per row: [S*N][chunks][M][2] (FP32-pipe scorer) or
                      // [S*N][items][256][2] (tensor-core scorer)
-  float* lse;        // [S*N][M]   row log-sum-exp in the exp2 domain
   HullLists hull;    // blocks of equal gain of every head's curve
-  int* head_flags;   // tensor-core scorer: [S*N] items delivered per head, then the (lse, tag) rows
+  int* head_flags;   // tensor-core scorer: [S*N] items delivered per head and the status word, then the (lse, tag) rows
   size_t bytes;
 };
 
 int score_chunks(const Dims& dm);                       // key chunks per head of the SIMT scorer
 size_t score_tc_stats_bytes(const Dims& dm);            // pass-1 partials of the two-sweep tensor-core scorer
-size_t score_tc_flag_bytes(const Dims& dm);             // zero-initialised block: [heads] counters, then the (lse, tag) rows
+size_t score_tc_flag_bytes(const Dims& dm);             // zero-initialised block: [heads] counters, status, then the (lse, tag) rows
+inline int* score_tc_status(const Dims& dm, const Workspace& ws) { return ws.head_flags + dm.heads(); }
 size_t score_tc_lse_offset(const Dims& dm);             // offset of the (lse, tag) rows inside that block
 void score_test_hooks(uint32_t* spin_limit, int* drop_item);  // environment hooks for the timeout tests
 // Single-sweep tensor-core scorer: takes a shape if a head's work items fit kOnePassMaxItems CTAs.
@@ -131,28 +132,33 @@ inline cudaError_t launch_pdl(Kernel kernel, dim3 grid, dim3 block, size_t smem,
 }
 #endif
 
-// Heads [h0, h0+nh) of the S*N heads of a call (the stages after allocation work head by head).
-struct HeadRange {
-  int h0, nh;
-};
+// Multiprocessors of the current device (looked up once per device).
+cudaError_t device_sms(int* sms);
+// Lets a kernel use `bytes` of dynamic shared memory (the attribute is set once per kernel and device, to the most it can
+// have).
+cudaError_t allow_smem(const void* kernel, size_t bytes);
 
 // Launchers.  Each returns cudaGetLastError() after its launches.
-cudaError_t launch_score_simt(const Dims& dm, const void* q, const void* k, const Workspace& ws, LaunchCtx& lc);
-// Folds per-chunk (max, sum-exp) partials [heads][chunks][M][2] into lse[heads][M] (exp2 domain).
-cudaError_t launch_lse(const Dims& dm, const float* stats, float* lse, int chunks, LaunchCtx& lc);
-// Tensor-core scorer (bf16, head_dim 128).  dev_status may be null.
+// The first sweep may run beside a kernel launched just before it (overlap); it ends after that kernel.
+cudaError_t launch_score_simt(const Dims& dm, const void* q, const void* k, const Workspace& ws, bool overlap, LaunchCtx& lc);
+// Tensor-core scorer (bf16).  A bounded wait that runs out stores LUKV_ERR_TIMEOUT to score_tc_status().
+// spare_sms: SMs the persistent grid leaves to kernels that run beside it
 bool score_tc_supported(const Dims& dm);
-// clear_flags: zero the scorer's counters and (lse, tag) rows first (once per call, before the first range)
-// spare_sms: SMs the persistent grid leaves to kernels of other streams
-cudaError_t launch_score_tc(const Dims& dm, const void* q, const void* k, const Workspace& ws, int32_t* dev_status,
-                            HeadRange hr, bool clear_flags, int spare_sms, LaunchCtx& lc);
+cudaError_t launch_score_tc(const Dims& dm, const void* q, const void* k, const Workspace& ws, int spare_sms, LaunchCtx& lc);
 // The single-sweep kernel alone; cudaErrorNotSupported (nothing launched) if the device has too few SMs for the shape.
-cudaError_t launch_score_onepass(const Dims& dm, const void* q, const void* k, const Workspace& ws,
-                                 int32_t* dev_status, HeadRange hr, bool clear_flags, int spare_sms, LaunchCtx& lc);
-cudaError_t launch_pool(const Dims& dm, const float* raw, float* pooled, HeadRange hr, LaunchCtx& lc);
+cudaError_t launch_score_onepass(const Dims& dm, const void* q, const void* k, const Workspace& ws, int spare_sms,
+                                 LaunchCtx& lc);
+// raw [heads][raw_stride] -> pooled [heads][stride]
+cudaError_t launch_pool(const Dims& dm, const float* raw, float* pooled, int stride, LaunchCtx& lc);
+// Allocation in one launch of one CTA: up to 1024 heads, 544 curve points and 128 sequences.  With `beside` it may run
+// beside the kernel launched just before it, whose results it does not touch; it ends after that kernel.
+bool allocate_one_launch(const Dims& dm);
+cudaError_t launch_allocate_one(const Dims& dm, const float* curves, const int64_t* budgets_host, const HullLists& lists,
+                                int32_t* budgets, int32_t* offsets, bool beside, LaunchCtx& lc);
+// Any size: the above where it applies, else hull and greedy.
 cudaError_t launch_allocate(const Dims& dm, const float* curves, const int64_t* budgets_host, const HullLists& lists,
                             int32_t* budgets, int32_t* offsets, LaunchCtx& lc);
-// The two halves of launch_allocate.  launch_hull treats its input as n_curves independent curves;
+// The two halves.  launch_hull treats its input as n_curves independent curves;
 // launch_greedy solves n_sets curve sets (lists of n_sets * N curves) for the same dm.S budgets and
 // writes budgets [n_sets][S][N] and offsets [n_sets][S*N+1].
 cudaError_t launch_hull(const float* curves, const HullLists& out, int64_t n_curves, int P, LaunchCtx& lc);
@@ -168,9 +174,11 @@ cudaError_t launch_profile_budgets(const float* profile, const int* row_lo, cons
 size_t curves_smem_bytes(int n, int P);
 cudaError_t launch_build_curves(const Dims& dm, const float* scores, const float* importance, float* curves,
                                 LaunchCtx& lc);
-// KeyDiff proxy scores (key-only metric): scores [heads][n]; scratch of keydiff_scratch_bytes().
+// KeyDiff proxy scores (key-only metric): scores [heads][stride]; scratch of keydiff_scratch_bytes().  A bounded wait that
+// runs out stores LUKV_ERR_TIMEOUT to dev_status, or to keydiff_status() when that is null.
 size_t keydiff_scratch_bytes(const Dims& dm);
-cudaError_t launch_keydiff(const Dims& dm, const void* k, float* scores, float* scratch, int32_t* dev_status,
+int* keydiff_status(const Dims& dm, float* scratch);
+cudaError_t launch_keydiff(const Dims& dm, const void* k, float* scores, int stride, float* scratch, int32_t* dev_status,
                            int spare_sms, LaunchCtx& lc);
 // Value norms || v_j W_O^(g) ||_2 of the oracle importance on the tensor cores (bf16): vnorm [heads][G][n].
 bool value_norm_tc_supported(const Dims& dm);
@@ -191,9 +199,14 @@ cudaError_t launch_importance(const Dims& dm, int k_max, int d_model, const void
 size_t exact_workspace_bytes(const Dims& dm, int64_t max_budget);
 cudaError_t launch_exact_allocate(const Dims& dm, const float* curves, const int64_t* budgets_host, int32_t* budgets,
                                   int32_t* offsets, double* values, void* ws, LaunchCtx& lc);
-cudaError_t launch_select(const Dims& dm, const float* scores, const int32_t* budgets, const int32_t* offsets,
-                          int32_t* kept_idx, int64_t rows_cap, HeadRange hr, LaunchCtx& lc);
+// Selection from scores [heads][stride]; with `pool` the scores are max-pooled on the way in (select_pools() sizes).
+// status: the scorer's status word, copied to dev_status (both may be null).  overlap: launched as the programmatic
+// dependent of the kernel before it.
+bool select_pools(const Dims& dm);
+cudaError_t launch_select(const Dims& dm, const float* scores, int stride, bool pool, const int32_t* budgets,
+                          const int32_t* offsets, int32_t* kept_idx, int64_t rows_cap, const int* status,
+                          int32_t* dev_status, bool overlap, LaunchCtx& lc);
 cudaError_t launch_gather(const Dims& dm, const int32_t* offsets, const int32_t* kept_idx, const void* k,
-                          const void* v, void* k_out, void* v_out, int64_t rows_cap, HeadRange hr, LaunchCtx& lc);
+                          const void* v, void* k_out, void* v_out, int64_t rows_cap, bool overlap, LaunchCtx& lc);
 
 }  // namespace lukv

@@ -341,14 +341,13 @@ cudaError_t launch_build_curves(const Dims& dm, const float* scores, const float
   if (curve_pow2(dm.n) <= kSortMaxN) {
     const int np = bucket_pow2(dm.n);
     auto kern = np <= 4096 ? build_curves_bucket_kernel<8> : build_curves_bucket_kernel<16>;
-    if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    if ((e = allow_smem((const void*)kern, smem)) != cudaSuccess) return e;
     kern<<<(unsigned)dm.heads(), np <= 4096 ? np / 8 : np / 16, smem, lc.st>>>(
         scores, importance, curves, dm.n, np, dm.P, dm.seg, dm.n_sink);
     lc.mark("build_curves_bucket");
     return cudaGetLastError();
   }
-  if ((e = cudaFuncSetAttribute(build_curves_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-    return e;
+  if ((e = allow_smem((const void*)build_curves_kernel, smem)) != cudaSuccess) return e;
   build_curves_kernel<<<(unsigned)dm.heads(), kCurveThreads, smem, lc.st>>>(scores, importance, curves, dm.n, dm.P,
                                                                             dm.seg, dm.n_sink);
   lc.mark("build_curves");

@@ -9,7 +9,6 @@
 //   imp_lse_kernel      row log-sum-exp of every (head, g, step), exp2 domain
 //   imp_kernel          probabilities x value norms, summed over g inside a thread, maximum over the steps
 //   imp_normalize_kernel  one CTA per (sequence, layer): fp64 total in a fixed order, then the division
-#include <algorithm>
 #include <cstdlib>
 
 #include "simt_tile.cuh"
@@ -263,9 +262,9 @@ cudaError_t launch_importance_t(const Dims& dm, ImpDims id, const void* q_dec, c
   auto kn = value_norm_kernel<TIn, D>;
   auto kl = imp_lse_kernel<TIn, D>;
   auto ki = imp_kernel<TIn, D>;
-  if ((e = cudaFuncSetAttribute(kn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(kl, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(ki, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+  if ((e = allow_smem((const void*)kn, smem)) != cudaSuccess) return e;
+  if ((e = allow_smem((const void*)kl, smem)) != cudaSuccess) return e;
+  if ((e = allow_smem((const void*)ki, smem)) != cudaSuccess) return e;
   const unsigned heads = (unsigned)dm.heads();
   const unsigned pos_tiles = (unsigned)((dm.n + kTile - 1) / kTile);
   if (value_norm_tc_supported(dm) && !value_norm_force_simt()) {
@@ -295,8 +294,8 @@ cudaError_t launch_importance_t(const Dims& dm, ImpDims id, const void* q_dec, c
 
 size_t importance_workspace_bytes(const Dims& dm, int k_max) {
   const size_t a = ((size_t)dm.heads() * dm.G * dm.n * sizeof(float) + 255) & ~(size_t)255;
-  const size_t rows = (size_t)dm.heads() * dm.G * k_max * sizeof(float);  // row log-sum-exps, or their partials
-  const size_t b = (std::max(rows, dm.G <= 8 ? importance_tc_part_bytes(dm, k_max) : 0) + 255) & ~(size_t)255;
+  const size_t rows = (size_t)dm.heads() * dm.G * k_max * sizeof(float);  // row log-sum-exps; room for their partials
+  const size_t b = (rows + (dm.G <= 8 ? importance_tc_part_bytes(dm, k_max) : 0) + 255) & ~(size_t)255;
   return a + b;
 }
 

@@ -381,15 +381,14 @@ cudaError_t launch_importance_tc_t(const Dims& dm, int k_max, const void* q_dec,
   a.scale_log2 = dm.scale_log2;
   int drop = 0;
   score_test_hooks(&a.spin_limit, &drop);
-  int dev = 0, sms = 0;
+  int sms = 0;
   cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = device_sms(&sms)) != cudaSuccess) return e;
   auto lse = imp_tc_kernel<NH, true>;
   auto imp = imp_tc_kernel<NH, false>;
   constexpr int lse_smem = ItPlan<NH, true>::kTotal, imp_smem = ItPlan<NH, false>::kTotal;
-  if ((e = cudaFuncSetAttribute(lse, cudaFuncAttributeMaxDynamicSharedMemorySize, lse_smem)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(imp, cudaFuncAttributeMaxDynamicSharedMemorySize, imp_smem)) != cudaSuccess) return e;
+  if ((e = allow_smem((const void*)lse, lse_smem)) != cudaSuccess) return e;
+  if ((e = allow_smem((const void*)imp, imp_smem)) != cudaSuccess) return e;
   a.tiles_T = (dm.T + 127) / 128;
   a.tiles_D = k_dec ? (k_max + 127) / 128 : 0;
   a.tiles_per_split = (a.tiles_T + a.tiles_D + a.splits - 1) / a.splits;

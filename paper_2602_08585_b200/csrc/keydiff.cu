@@ -49,13 +49,13 @@ struct Vec16<float> {
 
 struct KdArgs {
   const unsigned char* k;  // [heads][T][d]
-  float* scores;           // [heads][n]
+  float* scores;           // [heads][stride]
   float* pieces;           // [2][kKdMaxGrid + group][d]: partial sums of unit keys, by parity of the group
   float* anchors;          // [heads][d]   mean unit key
   float* inv_norm;         // [heads]      1 / max(||anchor||, eps)
   int* head_count;         // [heads]      pieces delivered; one more once the anchor is published.  Starts at 0.
   int32_t* dev_status;     // may be null
-  int T, n, heads, group;
+  int T, n, stride, heads, group;
   uint32_t spin_limit;
   int drop_head;           // test hook: this head's anchor is never published (-1: none)
 };
@@ -123,6 +123,7 @@ __global__ void __launch_bounds__(kKdThreads, 2) keydiff_kernel(const KdArgs a) 
   __shared__ int last_s;
   __shared__ int abort_s;
   volatile int* abort_flag = &abort_s;
+  pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = (a.heads + a.group - 1) / a.group;
   const bool odd_cta = blockIdx.x & 1;
@@ -305,7 +306,7 @@ __global__ void __launch_bounds__(kKdThreads, 2) keydiff_kernel(const KdArgs a) 
               av[i][e] = __ldcg(a.anchors + (size_t)u * D + (4 * ((i + odd_row) % V) + l) * E + e);
           const float inv_an = __ldcg(a.inv_norm + u);
           const int j_end = min(j_end_all, a.n);
-          float* out = a.scores + (size_t)u * a.n;
+          float* out = a.scores + (size_t)u * a.stride;
           for (int j = j_begin; j < j_end; j += kKdStageRows, ++cnt) {
             const uint32_t s = cnt % kStages, use = cnt / kStages;
             mbar_wait(smem_u32(&bars[s]), use & 1, abort_flag, a.dev_status, a.spin_limit);
@@ -360,18 +361,24 @@ size_t kd_pieces_bytes(const Dims& dm) {
   return kd_align((size_t)2 * (kKdMaxGrid + group) * dm.d * sizeof(float));
 }
 size_t kd_anchor_bytes(const Dims& dm) { return kd_align((size_t)dm.heads() * dm.d * sizeof(float)); }
-size_t kd_head_bytes(const Dims& dm) { return kd_align((size_t)dm.heads() * sizeof(float)); }
+size_t kd_head_bytes(const Dims& dm) { return kd_align(((size_t)dm.heads() + 1) * sizeof(float)); }
+size_t kd_count_offset(const Dims& dm) { return kd_pieces_bytes(dm) + kd_anchor_bytes(dm) + kd_head_bytes(dm); }
+
+}  // namespace
+
+int* keydiff_status(const Dims& dm, float* scratch) {
+  return reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(scratch) + kd_count_offset(dm)) + dm.heads();
+}
+
+namespace {
 
 template <typename TIn, int D>
-cudaError_t launch_keydiff_t(const Dims& dm, const void* k, float* scores, float* scratch, int32_t* dev_status,
+cudaError_t launch_keydiff_t(const Dims& dm, const void* k, float* scores, int stride, float* scratch, int32_t* dev_status,
                              int spare_sms, LaunchCtx& lc) {
   auto kern = keydiff_kernel<TIn, D>;
-  int dev = 0, sms = 0, per_sm = 0;
+  int sms = 0, per_sm = 0;
   cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kKdRingBytes)) != cudaSuccess)
-    return e;
+  if ((e = device_sms(&sms)) != cudaSuccess || (e = allow_smem((const void*)kern, kKdRingBytes)) != cudaSuccess) return e;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kKdThreads, kKdRingBytes)) != cudaSuccess)
     return e;
   if (per_sm < 1) return cudaErrorLaunchOutOfResources;
@@ -383,11 +390,11 @@ cudaError_t launch_keydiff_t(const Dims& dm, const void* k, float* scores, float
   a.pieces = reinterpret_cast<float*>(sc);
   a.anchors = reinterpret_cast<float*>(sc + kd_pieces_bytes(dm));
   a.inv_norm = reinterpret_cast<float*>(sc + kd_pieces_bytes(dm) + kd_anchor_bytes(dm));
-  a.head_count = reinterpret_cast<int*>(sc + kd_pieces_bytes(dm) + kd_anchor_bytes(dm) + kd_head_bytes(dm));
-  a.dev_status = dev_status;
-  a.T = dm.T, a.n = dm.n, a.heads = (int)dm.heads(), a.group = keydiff_group(dm);
+  a.head_count = reinterpret_cast<int*>(sc + kd_count_offset(dm));
+  a.dev_status = dev_status ? dev_status : keydiff_status(dm, scratch);
+  a.T = dm.T, a.n = dm.n, a.stride = stride, a.heads = (int)dm.heads(), a.group = keydiff_group(dm);
   score_test_hooks(&a.spin_limit, &a.drop_head);
-  if ((e = cudaMemsetAsync(a.head_count, 0, (size_t)a.heads * sizeof(int), lc.st)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(a.head_count, 0, ((size_t)a.heads + 1) * sizeof(int), lc.st)) != cudaSuccess) return e;
   // a slice is at least one stage: small problems get a smaller grid
   const long long slices = ((long long)a.group * dm.T + kKdStageRows - 1) / kKdStageRows;
   long long grid = (long long)sms * (per_sm > 2 ? 2 : per_sm);
@@ -402,18 +409,18 @@ cudaError_t launch_keydiff_t(const Dims& dm, const void* k, float* scores, float
 
 }  // namespace
 
-// scratch of the KeyDiff scorer: pieces, anchors, their norms, the per-head counters
+// scratch of the KeyDiff scorer: pieces, anchors, their norms, the per-head counters and the status word
 size_t keydiff_scratch_bytes(const Dims& dm) {
   return kd_pieces_bytes(dm) + kd_anchor_bytes(dm) + 2 * kd_head_bytes(dm);
 }
 
-cudaError_t launch_keydiff(const Dims& dm, const void* k, float* scores, float* scratch, int32_t* dev_status,
+cudaError_t launch_keydiff(const Dims& dm, const void* k, float* scores, int stride, float* scratch, int32_t* dev_status,
                            int spare_sms, LaunchCtx& lc) {
   if (dm.dtype == LUKV_DTYPE_BF16)
-    return dm.d == 128 ? launch_keydiff_t<__nv_bfloat16, 128>(dm, k, scores, scratch, dev_status, spare_sms, lc)
-                       : launch_keydiff_t<__nv_bfloat16, 64>(dm, k, scores, scratch, dev_status, spare_sms, lc);
-  return dm.d == 128 ? launch_keydiff_t<float, 128>(dm, k, scores, scratch, dev_status, spare_sms, lc)
-                     : launch_keydiff_t<float, 64>(dm, k, scores, scratch, dev_status, spare_sms, lc);
+    return dm.d == 128 ? launch_keydiff_t<__nv_bfloat16, 128>(dm, k, scores, stride, scratch, dev_status, spare_sms, lc)
+                       : launch_keydiff_t<__nv_bfloat16, 64>(dm, k, scores, stride, scratch, dev_status, spare_sms, lc);
+  return dm.d == 128 ? launch_keydiff_t<float, 128>(dm, k, scores, stride, scratch, dev_status, spare_sms, lc)
+                     : launch_keydiff_t<float, 64>(dm, k, scores, stride, scratch, dev_status, spare_sms, lc);
 }
 
 }  // namespace lukv

@@ -85,12 +85,12 @@ struct Plan {
 struct FusedArgs {
   float* stats;        // pass 1 partials: [heads][items_per_head][128*MT] log-sum-exp of the item's keys, exp2 domain
   float* lse;          // [heads][lse_rows] (row log-sum-exp in the exp2 domain, tag); zero at launch
-  float* raw;          // pass 2 out: [heads][n]
+  float* raw;          // pass 2 out: [heads][n_stride]
   int* head_cnt;       // [heads] items whose partials were delivered (zero at launch)
   int32_t* dev_status;
   int M, T, w, n;
   int lse_rows;        // M rounded up to a multiple of 4
-  int head0, nheads;   // heads [head0, head0+nheads) are scored by this launch
+  int nheads;
   int item_tiles, items_per_head, tiles_T, tiles_n;
   int adapt_items;     // host only: let the launcher pick a multiple of item_tiles
   int npad;            // pass 2: query rows rounded up to a multiple of 32 (MMA N and columns read)
@@ -128,7 +128,7 @@ __device__ __forceinline__ Job make_job(int k, bool p2, const FusedArgs& a) {
     j.iph = a.items_per_head;
     const int hu = item / a.items_per_head;
     j.c = item - hu * a.items_per_head;
-    j.u = a.head0 + hu;
+    j.u = hu;
   } else {
     int lo = 0, hi = a.n_seq;  // the sequence whose items contain `item`
     while (hi - lo > 1) {
@@ -182,6 +182,7 @@ __global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
   float2* pub_s = reinterpret_cast<float2*>(smem + P::kPubOff);   // [NQ][128]
   float* nlse_s = reinterpret_cast<float*>(smem + P::kLseOff);    // [kMaxLag][256]
 
+  pdl_launch_dependents();  // kernels that do not read the scores may start on SMs this grid leaves free
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int total_items = a.total_items;
   const int K = (total_items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;  // items of this CTA (>= 1)
@@ -617,12 +618,8 @@ cudaError_t launch_fused(const CUtensorMap& qm, const CUtensorMap& km, FusedArgs
   const int smem = P::kTotal;
   auto kern = score_fused_kernel<MT, NQ, NH, RAGGED>;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
-  int dev = 0, sms = 0, per_sm = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, P::kThreads, smem)) != cudaSuccess) return e;
-  if (per_sm < 1 || sms < 1) return cudaErrorLaunchOutOfResources;
+  int sms = 0;
+  if ((e = allow_smem((const void*)kern, smem)) != cudaSuccess || (e = device_sms(&sms)) != cudaSuccess) return e;
   if (spare_sms > 0 && sms > 8 * spare_sms) sms -= spare_sms;
   // A CTA runs pass 1 of later items before pass 2 of the current one, so a head's items must
   // not outnumber the CTAs (else a CTA would wait for partials that it is due to produce itself).
@@ -663,7 +660,8 @@ cudaError_t launch_fused(const CUtensorMap& qm, const CUtensorMap& km, FusedArgs
   args.total_items = total_items;
   const int grid = total_items < sms ? total_items : sms;  // one CTA per SM: each owns the SM's tensor memory
   void* params[] = {(void*)&qm, (void*)&km, (void*)&args};
-  // cooperative launch: the CTAs of a head wait for one another, so all must be resident
+  // cooperative launch: the CTAs of a head wait for one another, so all must be resident (one per SM: the launch fails if
+  // they cannot be)
   e = cudaLaunchCooperativeKernel((const void*)kern, dim3((unsigned)grid), dim3(P::kThreads), params, (size_t)smem,
                                   lc.st);
   lc.mark("score_fused");
@@ -672,8 +670,8 @@ cudaError_t launch_fused(const CUtensorMap& qm, const CUtensorMap& km, FusedArgs
 
 }  // namespace
 
-// Offset of the (lse, tag) rows inside the zero-initialised block that starts with the [heads] counters.
-size_t score_tc_lse_offset(const Dims& dm) { return ((size_t)dm.heads() * sizeof(int) + 255) & ~(size_t)255; }
+// Offset of the (lse, tag) rows inside the zero-initialised block that starts with the [heads] counters and the status.
+size_t score_tc_lse_offset(const Dims& dm) { return (((size_t)dm.heads() + 1) * sizeof(int) + 255) & ~(size_t)255; }
 
 // Test hooks of the tensor-core scorers, read from the environment at every call: LUKV_TEST_SPIN_LIMIT shortens
 // the limit of every device-side wait, LUKV_TEST_DROP_ITEM names one work item whose partial results never
@@ -698,7 +696,7 @@ size_t score_tc_stats_bytes(const Dims& dm) {
   const size_t items = (tiles + score_item_tiles() - 1) / score_item_tiles();
   return (size_t)dm.heads() * items * 256 * 2 * sizeof(float);
 }
-// Bytes of the block that must be zero at launch: [heads] counters, then [heads][lse_rows][2] floats.
+// Bytes of the block that must be zero at launch: [heads] counters, the status word, then [heads][lse_rows][2] floats.
 size_t score_tc_flag_bytes(const Dims& dm) {
   // the single-sweep kernel strides the rows of a head by 128 or 256, the two-sweep kernel by M rounded up to 4
   return score_tc_lse_offset(dm) + (size_t)dm.heads() * ((dm.M + 127) & ~127) * 2 * sizeof(float);
@@ -708,14 +706,13 @@ bool score_tc_supported(const Dims& dm) {
   return dm.dtype == LUKV_DTYPE_BF16 && encode_fn() != nullptr;
 }
 
-cudaError_t launch_score_tc(const Dims& dm, const void* q, const void* k, const Workspace& ws, int32_t* dev_status,
-                            HeadRange hr, bool clear_flags, int spare_sms, LaunchCtx& lc) {
+cudaError_t launch_score_tc(const Dims& dm, const void* q, const void* k, const Workspace& ws, int spare_sms, LaunchCtx& lc) {
   // The two-sweep kernel below is the default.  LUKV_SCORER=onesweep selects the single-sweep kernel where the
   // shape allows it (it parks a head's exponentials in tensor memory and is bound by the latency of the
   // log-sum-exp exchange between CTAs; at long contexts the two sweeps are faster).
   const char* which = getenv("LUKV_SCORER");
   if (which && which[0] == 'o' && !dm.seq_T && score_onepass_eligible(dm)) {
-    const cudaError_t e1 = launch_score_onepass(dm, q, k, ws, dev_status, hr, clear_flags, spare_sms, lc);
+    const cudaError_t e1 = launch_score_onepass(dm, q, k, ws, spare_sms, lc);
     if (e1 != cudaErrorNotSupported) return e1;
   }
   CUtensorMap qm, km;
@@ -726,18 +723,17 @@ cudaError_t launch_score_tc(const Dims& dm, const void* q, const void* k, const 
   args.lse = reinterpret_cast<float*>(reinterpret_cast<char*>(ws.head_flags) + score_tc_lse_offset(dm));
   args.raw = ws.raw;
   args.head_cnt = ws.head_flags;
-  args.dev_status = dev_status;
+  args.dev_status = score_tc_status(dm, ws);
   args.M = dm.M;
   args.T = dm.T;
   args.w = dm.w;
   args.n = dm.n;
   args.T_stride = dm.T;
-  args.n_stride = dm.n;
+  args.n_stride = dm.raw_stride();
   args.n_seq = dm.S;
   args.heads_per_seq = dm.N;
   args.lse_rows = (dm.M + 3) & ~3;
-  args.head0 = hr.h0;
-  args.nheads = hr.nh;
+  args.nheads = (int)dm.heads();
   args.tiles_T = (dm.T + kTileKeys - 1) / kTileKeys;
   args.item_tiles = score_item_tiles();
   args.adapt_items = getenv("LUKV_ITEM_TILES") ? 0 : 1;
@@ -751,13 +747,11 @@ cudaError_t launch_score_tc(const Dims& dm, const void* q, const void* k, const 
   args.scale_log2 = dm.scale_log2;
   score_test_hooks(&args.spin_limit, &args.drop_item);
   // the per-head counters and the (value, tag) rows must start at zero; they are adjacent in the workspace
-  if (clear_flags) {
-    const cudaError_t e = cudaMemsetAsync(ws.head_flags, 0, score_tc_flag_bytes(dm), lc.st);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = cudaMemsetAsync(ws.head_flags, 0, score_tc_flag_bytes(dm), lc.st);
+  if (e != cudaSuccess) return e;
   if (dm.seq_T) {
-    // sequences of different lengths: the whole call in one launch (no head ranges), work items dealt per sequence
-    if (hr.h0 != 0 || hr.nh != (int)dm.heads() || dm.S > kMaxRaggedSeqs) return cudaErrorInvalidValue;
+    // sequences of different lengths: work items dealt per sequence
+    if (dm.S > kMaxRaggedSeqs) return cudaErrorInvalidValue;
     if (dm.d == 64)
       return dm.M > 128 ? launch_fused<2, 2, 1, true>(qm, km, args, spare_sms, lc, dm.seq_T)
                         : launch_fused<1, 2, 1, true>(qm, km, args, spare_sms, lc, dm.seq_T);

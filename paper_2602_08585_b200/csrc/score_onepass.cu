@@ -57,10 +57,11 @@ struct OnePlan {
 struct OneArgs {
   float* stats;        // [heads][M][tiles_pad] log-sum-exp of (row, key tile), exp2 domain; all-ones bits at launch
   float* lse;          // [heads][128*MT] (row log-sum-exp, tag); zero at launch
-  float* raw;          // out: [heads][n] un-pooled scores
+  float* raw;          // out: [heads][n_stride] un-pooled scores
+  int n_stride;
   int32_t* dev_status;
   int M, T, w, n;
-  int head0, nheads;   // heads [head0, head0+nheads) are scored by this launch
+  int nheads;   // heads [head0, head0+nheads) are scored by this launch
   int items_per_head, tiles_T, tiles_pad;
   float scale_log2;
   uint32_t spin_limit; // iterations a wait may take
@@ -81,7 +82,7 @@ __device__ __forceinline__ Item make_item(int k, const OneArgs& a) {
   it.index = (int)blockIdx.x + k * (int)gridDim.x;
   const int hu = it.index / a.items_per_head;
   it.c = it.index - hu * a.items_per_head;
-  it.u = a.head0 + hu;
+  it.u = hu;
   it.tile0 = it.c * OnePlan<MT>::kItemTiles;
   it.ntiles = min(OnePlan<MT>::kItemTiles, a.tiles_T - it.tile0);
   return it;
@@ -553,11 +554,11 @@ __global__ void __launch_bounds__(OnePlan<MT>::kThreads, 1)
           if (MT == 1) {
             const float* pq = part_k + quad * 512 + qtid;
             const float s = (pq[0] + pq[128]) + (pq[256] + pq[384]);
-            if (key < a.n) a.raw[(size_t)it.u * a.n + key] = s;
+            if (key < a.n) a.raw[(size_t)it.u * a.n_stride + key] = s;
           } else if (quad == 0) {
             const float* pq = part_k + qtid;
             const float s = ((pq[0] + pq[128]) + (pq[256] + pq[384])) + ((pq[512] + pq[640]) + (pq[768] + pq[896]));
-            if (key < a.n) a.raw[(size_t)it.u * a.n + key] = s;
+            if (key < a.n) a.raw[(size_t)it.u * a.n_stride + key] = s;
           }
         } else {
           // the item has no tile for this quad: only keep the accumulator's barriers in step
@@ -623,8 +624,8 @@ size_t score_onepass_stats_bytes(const Dims& dm) {
 }
 
 // Returns cudaErrorNotSupported (and launches nothing) when the device has fewer SMs than a head has items.
-cudaError_t launch_score_onepass(const Dims& dm, const void* q, const void* k, const Workspace& ws, int32_t* dev_status,
-                                 HeadRange hr, bool clear_flags, int spare_sms, LaunchCtx& lc) {
+cudaError_t launch_score_onepass(const Dims& dm, const void* q, const void* k, const Workspace& ws, int spare_sms,
+                                 LaunchCtx& lc) {
   int dev = 0, sms = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -641,23 +642,21 @@ cudaError_t launch_score_onepass(const Dims& dm, const void* q, const void* k, c
   args.stats = ws.stats;
   args.lse = reinterpret_cast<float*>(reinterpret_cast<char*>(ws.head_flags) + score_tc_lse_offset(dm));
   args.raw = ws.raw;
-  args.dev_status = dev_status;
+  args.dev_status = score_tc_status(dm, ws);
+  args.n_stride = dm.raw_stride();
   args.M = dm.M;
   args.T = dm.T;
   args.w = dm.w;
   args.n = dm.n;
-  args.head0 = hr.h0;
-  args.nheads = hr.nh;
+  args.nheads = (int)dm.heads();
   args.tiles_T = onepass_tiles(dm);
   args.tiles_pad = onepass_tiles_pad(dm);
   args.scale_log2 = dm.scale_log2;
   score_test_hooks(&args.spin_limit, &args.drop_item);
-  if (clear_flags) {
-    // the (lse, tag) rows start at zero, the partials as all-ones bit patterns
-    if ((e = cudaMemsetAsync(ws.head_flags, 0, score_tc_flag_bytes(dm), lc.st)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(ws.stats, 0xFF, score_onepass_stats_bytes(dm), lc.st)) != cudaSuccess) return e;
-  }
-  const long long total_items = (long long)hr.nh * args.items_per_head;
+  // the (lse, tag) rows start at zero, the partials as all-ones bit patterns
+  if ((e = cudaMemsetAsync(ws.head_flags, 0, score_tc_flag_bytes(dm), lc.st)) != cudaSuccess) return e;
+  if ((e = cudaMemsetAsync(ws.stats, 0xFF, score_onepass_stats_bytes(dm), lc.st)) != cudaSuccess) return e;
+  const long long total_items = (long long)dm.heads() * args.items_per_head;
   const int grid = (int)(total_items < sms ? total_items : sms);
   if (grid < args.items_per_head) return cudaErrorNotSupported;
   return dm.M > 128 ? launch_onepass<2>(qm, km, args, grid, lc) : launch_onepass<1>(qm, km, args, grid, lc);

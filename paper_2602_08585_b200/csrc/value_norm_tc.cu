@@ -287,13 +287,12 @@ cudaError_t launch_value_norm_tc(const Dims& dm, int d_model, const void* v, con
   a.items = (long long)dm.heads() * dm.G * a.chunks;
   int drop = 0;
   score_test_hooks(&a.spin_limit, &drop);
-  int dev = 0, sms = 0;
+  int sms = 0;
   cudaError_t e;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  if ((e = device_sms(&sms)) != cudaSuccess) return e;
   auto kern = dm.d == 128 ? value_norm_tc_kernel<2> : value_norm_tc_kernel<1>;
   const int smem = vn_smem(dm.d / 64);
-  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
+  if ((e = allow_smem((const void*)kern, smem)) != cudaSuccess) return e;
   const long long grid = a.items < sms ? a.items : sms;  // one CTA per SM: each owns the SM's tensor memory
   kern<<<(unsigned)grid, kVnThreads, smem, lc.st>>>(vm, a);
   lc.mark("value_norm_tc");
