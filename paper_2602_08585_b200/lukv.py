@@ -117,15 +117,36 @@ def _ptr(t) -> Optional[int]:
     return None if t is None else t.data_ptr()
 
 
+_have_device: Optional[bool] = None
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # the current stream's handle, without an object for it
+
+
 def _stream(stream) -> int:
     if stream is None:
         # without a device only argument validation can be exercised; it never launches
-        return torch.cuda.current_stream().cuda_stream if torch.cuda.is_available() else 0
+        global _have_device
+        if _have_device is None:
+            _have_device = torch.cuda.is_available()
+        if not _have_device:
+            return 0
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
+        return torch.cuda.current_stream().cuda_stream
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
-def _host_budgets(budgets_in: Sequence[int]) -> np.ndarray:
-    return np.ascontiguousarray(np.asarray(budgets_in, dtype=np.int64))
+def _host_array(values, ctype, dtype):
+    """(what keeps it alive, address) of host values as a C array: a list or tuple of plain ints directly, anything else
+    through numpy."""
+    if type(values) in (list, tuple) and all(type(v) is int for v in values):
+        a = (ctype * len(values))(*values)
+        return a, a
+    b = np.ascontiguousarray(np.asarray(values, dtype=dtype))
+    return b, b.ctypes.data
+
+
+def _host_budgets(budgets_in: Sequence[int]):
+    return _host_array(budgets_in, ctypes.c_int64, np.int64)
 
 
 def lukv_workspace_bytes(params: Params) -> int:
@@ -154,8 +175,8 @@ def lukv_score(params: Params, q_win, k, scores, ws, stream=None, check: bool = 
 
 
 def lukv_allocate(params: Params, curves, budgets_in, budgets, offsets, ws, stream=None, check: bool = True) -> int:
-    b = _host_budgets(budgets_in)
-    rc = lib().lukv_allocate(ctypes.byref(params), _ptr(curves), b.ctypes.data, _ptr(budgets), _ptr(offsets),
+    _keep, b = _host_budgets(budgets_in)
+    rc = lib().lukv_allocate(ctypes.byref(params), _ptr(curves), b, _ptr(budgets), _ptr(offsets),
                              _ptr(ws), 0 if ws is None else ws.numel() * ws.element_size(), _stream(stream))
     return _check(rc, "lukv_allocate", check)
 
@@ -164,14 +185,19 @@ def lukv_allocate_static(params: Params, curves, budgets_in, budgets, offsets, s
     """lukv_allocate without a workspace argument: the scratch is a fixed array inside the library
     (at most 262144 gains), for callers that cannot allocate device memory.  Calls sharing a device
     must not overlap on the GPU."""
-    b = _host_budgets(budgets_in)
-    rc = lib().lukv_allocate_static(ctypes.byref(params), _ptr(curves), b.ctypes.data, _ptr(budgets), _ptr(offsets),
+    _keep, b = _host_budgets(budgets_in)
+    rc = lib().lukv_allocate_static(ctypes.byref(params), _ptr(curves), b, _ptr(budgets), _ptr(offsets),
                                     _stream(stream))
     return _check(rc, "lukv_allocate_static", check)
 
 
-def _host_f32(x) -> np.ndarray:
-    return np.ascontiguousarray(np.asarray(x, dtype=np.float32).reshape(-1))
+def _host_f32(x):
+    """(what keeps it alive, address, count) of host values as a flat float array."""
+    if type(x) in (list, tuple) and all(type(v) is float for v in x):
+        a = (ctypes.c_float * len(x))(*x)
+        return a, a, len(x)
+    b = np.ascontiguousarray(np.asarray(x, dtype=np.float32).reshape(-1))
+    return b, b.ctypes.data, int(b.shape[0])
 
 
 def lukv_profile_workspace_bytes(calib: Params, n_queries: int, n_ratios: int) -> int:
@@ -185,8 +211,8 @@ def lukv_profile_workspace_bytes(calib: Params, n_queries: int, n_ratios: int) -
 def lukv_profile_build(calib: Params, curves, n_queries: int, ratios, profile, ws, stream=None,
                        check: bool = True) -> int:
     """Offline profile: curves [n_queries][N][P] (device), ratios (host) -> profile [len(ratios)][N] (device)."""
-    r = _host_f32(ratios)
-    rc = lib().lukv_profile_build(ctypes.byref(calib), _ptr(curves), int(n_queries), r.ctypes.data, int(r.shape[0]),
+    _keep, r, n_ratios = _host_f32(ratios)
+    rc = lib().lukv_profile_build(ctypes.byref(calib), _ptr(curves), int(n_queries), r, n_ratios,
                                   _ptr(profile), _ptr(ws), 0 if ws is None else ws.numel() * ws.element_size(),
                                   _stream(stream))
     return _check(rc, "lukv_profile_build", check)
@@ -195,23 +221,23 @@ def lukv_profile_build(calib: Params, curves, n_queries: int, ratios, profile, w
 def lukv_profile_budgets(params: Params, profile, ratios, sigma, budgets, offsets, stream=None,
                          check: bool = True) -> int:
     """Online lookup + budgeting: profile (device), ratios and per-sequence sigma (host) -> budgets, offsets."""
-    r, sg = _host_f32(ratios), _host_f32(sigma)
-    if sg.shape[0] != params.batch:
+    (_keep, r, n_ratios), (_keep_sigma, sg, n_sigma) = _host_f32(ratios), _host_f32(sigma)
+    if n_sigma != params.batch:
         raise ValueError("one target ratio per sequence")
-    rc = lib().lukv_profile_budgets(ctypes.byref(params), _ptr(profile), r.ctypes.data, int(r.shape[0]),
-                                    sg.ctypes.data, _ptr(budgets), _ptr(offsets), _stream(stream))
+    rc = lib().lukv_profile_budgets(ctypes.byref(params), _ptr(profile), r, n_ratios, sg, _ptr(budgets), _ptr(offsets),
+                                    _stream(stream))
     return _check(rc, "lukv_profile_budgets", check)
 
 
 def lukv_profile_budgets_ragged(params: Params, ctx_lens, profile, ratios, sigma, budgets, offsets, stream=None,
                                 check: bool = True) -> int:
     """lukv_profile_budgets for sequences of different lengths: ctx_lens [S] host ints."""
-    r, sg, lens = _host_f32(ratios), _host_f32(sigma), _host_lens(ctx_lens)
-    if sg.shape[0] != params.batch:
+    (_keep, r, n_ratios), (_keep_sigma, sg, n_sigma) = _host_f32(ratios), _host_f32(sigma)
+    _keep_lens, lens = _host_lens(ctx_lens)
+    if n_sigma != params.batch:
         raise ValueError("one target ratio per sequence")
-    rc = lib().lukv_profile_budgets_ragged(ctypes.byref(params), lens.ctypes.data, _ptr(profile), r.ctypes.data,
-                                           int(r.shape[0]), sg.ctypes.data, _ptr(budgets), _ptr(offsets),
-                                           _stream(stream))
+    rc = lib().lukv_profile_budgets_ragged(ctypes.byref(params), lens, _ptr(profile), r, n_ratios, sg, _ptr(budgets),
+                                           _ptr(offsets), _stream(stream))
     return _check(rc, "lukv_profile_budgets_ragged", check)
 
 
@@ -250,8 +276,8 @@ def lukv_exact_workspace_bytes(params: Params, max_budget: int) -> int:
 def lukv_exact_allocate(params: Params, curves, budgets_in, budgets, offsets, values, ws, stream=None,
                         check: bool = True) -> int:
     """Exact allocation on token-resolution curves; values is a float64 device tensor [S]."""
-    b = _host_budgets(budgets_in)
-    rc = lib().lukv_exact_allocate(ctypes.byref(params), _ptr(curves), b.ctypes.data, _ptr(budgets), _ptr(offsets),
+    _keep, b = _host_budgets(budgets_in)
+    rc = lib().lukv_exact_allocate(ctypes.byref(params), _ptr(curves), b, _ptr(budgets), _ptr(offsets),
                                    _ptr(values), _ptr(ws), 0 if ws is None else ws.numel() * ws.element_size(),
                                    _stream(stream))
     return _check(rc, "lukv_exact_allocate", check)
@@ -268,8 +294,8 @@ def lukv_select_gather(params: Params, scores, budgets, offsets, k, v, k_out, v_
 def lukv_select_gather_ragged(params: Params, ctx_lens, scores, budgets, offsets, k, v, k_out, v_out, kept_idx,
                               rows_cap: int, ws, stream=None, check: bool = True) -> int:
     """lukv_select_gather for sequences of different lengths: ctx_lens [S] host ints."""
-    lens = _host_lens(ctx_lens)
-    rc = lib().lukv_select_gather_ragged(ctypes.byref(params), lens.ctypes.data, _ptr(scores), _ptr(budgets),
+    _keep_lens, lens = _host_lens(ctx_lens)
+    rc = lib().lukv_select_gather_ragged(ctypes.byref(params), lens, _ptr(scores), _ptr(budgets),
                                          _ptr(offsets), _ptr(k), _ptr(v), _ptr(k_out), _ptr(v_out), _ptr(kept_idx),
                                          int(rows_cap), _ptr(ws), 0 if ws is None else ws.numel() * ws.element_size(),
                                          _stream(stream))
@@ -278,8 +304,8 @@ def lukv_select_gather_ragged(params: Params, ctx_lens, scores, budgets, offsets
 
 def lukv_compress(params: Params, q_win, k, v, curves, budgets_in, k_out, v_out, kept_idx, budgets, offsets,
                   rows_cap: int, dev_status, ws, stream=None, check: bool = True) -> int:
-    b = _host_budgets(budgets_in)
-    rc = lib().lukv_compress(ctypes.byref(params), _ptr(q_win), _ptr(k), _ptr(v), _ptr(curves), b.ctypes.data,
+    _keep, b = _host_budgets(budgets_in)
+    rc = lib().lukv_compress(ctypes.byref(params), _ptr(q_win), _ptr(k), _ptr(v), _ptr(curves), b,
                              _ptr(k_out), _ptr(v_out), _ptr(kept_idx), _ptr(budgets), _ptr(offsets), int(rows_cap),
                              _ptr(dev_status), _ptr(ws), 0 if ws is None else ws.numel() * ws.element_size(),
                              _stream(stream))
@@ -293,24 +319,24 @@ def lukv_score_keydiff(params: Params, k, scores, ws, dev_status=None, stream=No
     return _check(rc, "lukv_score_keydiff", check)
 
 
-def _host_lens(ctx_lens) -> np.ndarray:
-    return np.ascontiguousarray(np.asarray(ctx_lens, dtype=np.int32))
+def _host_lens(ctx_lens):
+    return _host_array(ctx_lens, ctypes.c_int32, np.int32)
 
 
 def lukv_score_ragged(params: Params, ctx_lens, q_win, k, scores, ws, stream=None, check: bool = True) -> int:
     """lukv_score for sequences of different lengths: params.ctx_len is the row stride, ctx_lens [S] host ints."""
-    lens = _host_lens(ctx_lens)
-    rc = lib().lukv_score_ragged(ctypes.byref(params), lens.ctypes.data, _ptr(q_win), _ptr(k), _ptr(scores), _ptr(ws),
+    _keep_lens, lens = _host_lens(ctx_lens)
+    rc = lib().lukv_score_ragged(ctypes.byref(params), lens, _ptr(q_win), _ptr(k), _ptr(scores), _ptr(ws),
                                  0 if ws is None else ws.numel() * ws.element_size(), _stream(stream))
     return _check(rc, "lukv_score_ragged", check)
 
 
 def lukv_compress_ragged(params: Params, ctx_lens, q_win, k, v, curves, budgets_in, k_out, v_out, kept_idx, budgets,
                          offsets, rows_cap: int, dev_status, ws, stream=None, check: bool = True) -> int:
-    b = _host_budgets(budgets_in)
-    lens = _host_lens(ctx_lens)
-    rc = lib().lukv_compress_ragged(ctypes.byref(params), lens.ctypes.data, _ptr(q_win), _ptr(k), _ptr(v), _ptr(curves),
-                                    b.ctypes.data, _ptr(k_out), _ptr(v_out), _ptr(kept_idx), _ptr(budgets),
+    _keep, b = _host_budgets(budgets_in)
+    _keep_lens, lens = _host_lens(ctx_lens)
+    rc = lib().lukv_compress_ragged(ctypes.byref(params), lens, _ptr(q_win), _ptr(k), _ptr(v), _ptr(curves),
+                                    b, _ptr(k_out), _ptr(v_out), _ptr(kept_idx), _ptr(budgets),
                                     _ptr(offsets), int(rows_cap), _ptr(dev_status), _ptr(ws),
                                     0 if ws is None else ws.numel() * ws.element_size(), _stream(stream))
     return _check(rc, "lukv_compress_ragged", check)
@@ -319,10 +345,10 @@ def lukv_compress_ragged(params: Params, ctx_lens, q_win, k, v, curves, budgets_
 def lukv_compress_profile(params: Params, q_win, k, v, curves, budgets_in, k_out, v_out, kept_idx, budgets, offsets,
                           rows_cap: int, dev_status, ws, stream=None, max_times: int = 64):
     """lukv_compress with a CUDA event after every kernel; synchronises.  Returns [(kernel name, ms)]."""
-    b = _host_budgets(budgets_in)
+    _keep, b = _host_budgets(budgets_in)
     times = (KernelTime * max_times)()
     cnt = ctypes.c_int(0)
-    rc = lib().lukv_compress_profile(ctypes.byref(params), _ptr(q_win), _ptr(k), _ptr(v), _ptr(curves), b.ctypes.data,
+    rc = lib().lukv_compress_profile(ctypes.byref(params), _ptr(q_win), _ptr(k), _ptr(v), _ptr(curves), b,
                                      _ptr(k_out), _ptr(v_out), _ptr(kept_idx), _ptr(budgets), _ptr(offsets),
                                      int(rows_cap), _ptr(dev_status), _ptr(ws),
                                      0 if ws is None else ws.numel() * ws.element_size(), _stream(stream), times,
