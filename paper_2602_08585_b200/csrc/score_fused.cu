@@ -527,6 +527,12 @@ __global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
             const int j0 = (j.tile0 + t) * kTileKeys;
             const bool masked = j0 + kTileKeys > j.n;             // tile reaches into the window / past T
             const uint32_t tcol = tmem_base + lane_addr + buf * P::kBufCols + (MT == 2 ? 128 * quad : 0);
+            // the accumulator is free as soon as its last columns are in registers
+            auto release = [&](uint32_t n) {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(bar(P::kBarTEmpty, buf), n);
+            };
             float va[32], vb[32];
             tmem_ld32(tcol, va);
 #pragma unroll
@@ -539,14 +545,12 @@ __global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
               }
               tmem_ld_wait(vb);
               if (c + 2 < 4) tmem_ld32(tcol + 32 * (c + 2), va);
+              else release(1);
               if (lim >= 0) {
                 if (masked) p1_chunk<true>(vb, j0 + 32 * (c + 1), lim, a.scale_log2, m, l);
                 else p1_chunk<false>(vb, j0 + 32 * (c + 1), lim, a.scale_log2, m, l);
               }
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(P::kBarTEmpty, buf), 1);
           }
         }
         // hand the partial to the publisher warp
@@ -569,6 +573,11 @@ __global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
             const int key = (j.tile0 + t) * kTileKeys + qtid;
             const uint32_t tcol = tmem_base + lane_addr + buf * P::kBufCols;
             uint64_t acc0 = 0ull, acc1 = 0ull;
+            auto release = [&](uint32_t n) {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(bar(P::kBarTEmpty, buf), n);
+            };
             float va[32], vb[32];
             tmem_ld32(tcol, va);
 #pragma unroll 1
@@ -576,16 +585,15 @@ __global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
               tmem_ld_wait(va);
               const bool two = c0 + 32 < a.npad;
               if (two) tmem_ld32(tcol + c0 + 32, vb);
+              else release(MT == 2 ? 2 : 1);
               p2_chunk(va, nlse + c0, sc2, acc0, acc1);
               if (two) {
                 tmem_ld_wait(vb);
                 if (c0 + 64 < a.npad) tmem_ld32(tcol + c0 + 64, va);
+                else release(MT == 2 ? 2 : 1);
                 p2_chunk(vb, nlse + c0 + 32, sc2, acc0, acc1);
               }
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(P::kBarTEmpty, buf), MT == 2 ? 2 : 1);
             if (key < j.n) a.raw[(size_t)j.u * a.n_stride + key] = sum4(acc0, acc1);
           }
         }
