@@ -195,14 +195,13 @@ LUKV_API int lukv_select_gather(const lukv_params_t* params, const float* scores
  *   dev_status [1] int32, may be NULL: set to 0 by the call; a kernel that gives up on a
  *   bounded wait stores LUKV_ERR_TIMEOUT there (the tensor-core scorer's CTAs wait for one
  *   another; it is launched cooperatively, so this only happens if the device is taken away).
- * The allocation kernels run on an auxiliary stream beside the scorer; that stream and two
- * events are created on the first call on a device and kept until the process exits.  The
- * caller's stream waits for them inside the call, so everything the call enqueues is ordered
- * after earlier work on `stream` and before later work on it.  Host threads may call
- * concurrently on one device (each with its own workspace and outputs): the call holds a
- * per-device lock while it enqueues on the auxiliary stream, so such calls enqueue one after
- * the other.  The call only enqueues (kernels, memsets, the event pair), so it may be captured into a CUDA
- * graph once the auxiliary stream exists (after one plain call on the device).
+ * The allocation runs beside the scorer: for up to 32 heads per sequence on the caller's stream, for more on an auxiliary
+ * stream that, with two events, is created on the first such call on a device and kept until the process exits.  The
+ * caller's stream waits for it inside the call, so everything the call enqueues is ordered after earlier work on `stream`
+ * and before later work on it.  Host threads may call concurrently on one device (each with its own workspace and
+ * outputs): the call holds a per-device lock while it enqueues on the auxiliary stream, so such calls enqueue one after
+ * the other.  The call only enqueues (kernels, a memset, the event pair), so it may be captured into a CUDA graph once the
+ * auxiliary stream exists (after one plain call on the device).
  */
 LUKV_API int lukv_compress(const lukv_params_t* params, const void* q_win, const void* k, const void* v,
                   const float* curves, const int64_t* budgets_in, void* k_out, void* v_out, int32_t* kept_idx,

@@ -732,9 +732,13 @@ inline size_t greedy_smem_bytes(int N, int cap, int groups, bool one) {
 // share the budgets): set i reads the lists of curves i*N .., writes budgets + i*set.budgets and offsets +
 // i*set.offsets.  The hot path launches one set.
 template <bool ONE>
-__device__ __forceinline__ void greedy_cta(unsigned char* greedy_smem, const HullLists& lists, const GreedyArgs& args,
-                                           int32_t* __restrict__ budgets, int32_t* __restrict__ offsets,
-                                           const SetStride& set, int N, int P, int w, int cap, int group) {
+__global__ void __launch_bounds__(kGreedyMaxThreads) greedy_kernel(HullLists lists, const __grid_constant__ GreedyArgs args,
+                                                                   int32_t* __restrict__ budgets,
+                                                                   int32_t* __restrict__ offsets, SetStride set,
+                                                                   int N, int P, int w, int cap, int group) {
+  extern __shared__ __align__(16) unsigned char greedy_smem[];
+  pdl_launch_dependents();
+  pdl_wait();  // the lists come from the launch before
   __shared__ GreedyShared shared[kGreedyMaxGroups];
   const int groups = blockDim.x / group;
   const int mine = threadIdx.x / group;
@@ -792,39 +796,6 @@ __device__ __forceinline__ void greedy_cta(unsigned char* greedy_smem, const Hul
     if (staged) greedy_problem<true, ONE>(in_smem, args, i, N, w, lo, hi, mid, weight, sh, grp, budgets, offsets);
     else greedy_problem<false, ONE>(in_place, args, i, N, w, lo, hi, mid, weight, sh, grp, budgets, offsets);
   }
-}
-
-template <bool ONE>
-__global__ void __launch_bounds__(kGreedyMaxThreads) greedy_kernel(HullLists lists, const __grid_constant__ GreedyArgs args,
-                                                                   int32_t* __restrict__ budgets,
-                                                                   int32_t* __restrict__ offsets, SetStride set,
-                                                                   int N, int P, int w, int cap, int group) {
-  extern __shared__ __align__(16) unsigned char greedy_smem[];
-  pdl_launch_dependents();
-  pdl_wait();  // the lists come from the launch before
-  greedy_cta<ONE>(greedy_smem, lists, args, budgets, offsets, set, N, P, w, cap, group);
-}
-
-// Hull and greedy of up to 1024 heads by one CTA: a warp walks every 32nd curve, then the groups take the sequences.  It
-// fits the SM that a persistent scorer leaves free and is done long before the scorer where heads are many, so that the whole
-// path needs no second stream: the scorer, this kernel as its programmatic
-// dependent, which does not wait for the scorer before its own end, then the selection, which waits for this one.
-__global__ void __launch_bounds__(kGreedyMaxThreads) alloc_kernel(const float* __restrict__ curves, HullLists lists,
-                                                                  const __grid_constant__ GreedyArgs args,
-                                                                  int32_t* __restrict__ budgets,
-                                                                  int32_t* __restrict__ offsets, int N, int P, int w, int cap,
-                                                                  int group) {
-  extern __shared__ __align__(16) unsigned char greedy_smem[];
-  pdl_launch_dependents();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int h = warp; h < N; h += blockDim.x >> 5) {
-    const int count = hull_walk_short(curves + (size_t)h * P, P, lane,
-                                      HullOut{lists.gain + (size_t)h * (P - 1), lists.start + (size_t)h * (P - 1)});
-    if (lane == 0) lists.count[h] = count;
-  }
-  __syncthreads();
-  greedy_cta<true>(greedy_smem, lists, args, budgets, offsets, SetStride{0, 0}, N, P, w, cap, group);
-  pdl_wait();
 }
 
 // Hull and greedy of up to 32 heads in one launch: one CTA per sequence, a warp per head walks the head's curve into
@@ -940,7 +911,7 @@ cudaError_t launch_hull(const float* curves, const HullLists& out, int64_t n_cur
 }
 
 cudaError_t launch_greedy(const Dims& dm, const HullLists& lists, const int64_t* budgets_host, int32_t* budgets,
-                          int32_t* offsets, int n_sets, LaunchCtx& lc) {
+                          int32_t* offsets, int n_sets, bool one_cta, LaunchCtx& lc) {
   cudaError_t e;
   // lists of up to 16384 blocks in all are staged (two CTAs per SM then); with many heads the per-head words take the room
   const long long cells = (long long)dm.N * (dm.P - 1);
@@ -948,8 +919,10 @@ cudaError_t launch_greedy(const Dims& dm, const HullLists& lists, const int64_t*
   const bool one = dm.N <= kGreedyMaxThreads;
   int group = (dm.N + 31) & ~31;  // one thread per head, whole warps
   if (group > kGreedyMaxThreads) group = kGreedyMaxThreads;
-  // several problems per CTA where many sets share the budgets (never when a thread owns several heads)
-  const int groups = n_sets > 1 && one ? std::min(kGreedyMaxGroups, std::max(1, std::min(dm.S, kGreedyMaxThreads / group))) : 1;
+  // several problems per CTA where many sets share the budgets, or where one CTA takes all (never when a thread owns several
+  // heads)
+  const bool pack = (n_sets > 1 || one_cta) && one;
+  const int groups = pack ? std::min(kGreedyMaxGroups, std::max(1, std::min(dm.S, kGreedyMaxThreads / group))) : 1;
   const size_t smem = greedy_smem_bytes(dm.N, cap, groups, one);
   auto kern = one ? greedy_kernel<true> : greedy_kernel<false>;
   if ((e = allow_smem((const void*)kern, smem)) != cudaSuccess) return e;
@@ -960,10 +933,11 @@ cudaError_t launch_greedy(const Dims& dm, const HullLists& lists, const int64_t*
   for (int q0 = 0; q0 < dm.S; q0 += kSeqPerLaunch) {
     const int cnt = dm.S - q0 < kSeqPerLaunch ? dm.S - q0 : kSeqPerLaunch;
     const GreedyArgs args = greedy_args(dm, budgets_host, q0, cnt, &base);
-    // one CTA per sequence; where many sets share the budgets, a set's staged lists serve several of them
-    int ctas = (cnt + groups - 1) / groups;
+    // one CTA per sequence; where many sets share the budgets, a set's staged lists serve several of them; beside a
+    // persistent scorer a single CTA, which fits the SM that the scorer leaves free
+    int ctas = one_cta ? 1 : (cnt + groups - 1) / groups;
     if (n_sets > 1) ctas = std::max(1, std::min(ctas, 2 * 148 / n_sets));
-    e = launch_pdl(kern, dim3(ctas, n_sets), dim3(group * groups), smem, lc.st, q0 == 0, lists, args, budgets, offsets, set,
+    e = launch_pdl(kern, dim3(ctas, n_sets), dim3(group * groups), smem, lc.st, true, lists, args, budgets, offsets, set,
                    dm.N, dm.P, dm.w, cap, group);
     if (e != cudaSuccess) return e;
     lc.mark("greedy");
@@ -971,28 +945,17 @@ cudaError_t launch_greedy(const Dims& dm, const HullLists& lists, const int64_t*
   return cudaGetLastError();
 }
 
-bool allocate_one_launch(const Dims& dm) {
-  return dm.N <= kGreedyMaxThreads && dm.P <= kHullRegsMaxP && dm.S <= kSeqPerLaunch;
-}
+bool allocate_small(const Dims& dm) { return dm.N <= kSmallMaxHeads && dm.P <= kHullRegsMaxP && dm.S <= kSeqPerLaunch; }
 
-cudaError_t launch_allocate_one(const Dims& dm, const float* curves, const int64_t* budgets_host, const HullLists& lists,
-                                int32_t* budgets, int32_t* offsets, bool beside, LaunchCtx& lc) {
+cudaError_t launch_allocate_small(const Dims& dm, const float* curves, const int64_t* budgets_host, int32_t* budgets,
+                                  int32_t* offsets, bool beside, LaunchCtx& lc) {
   long long base = 0;
   const GreedyArgs args = greedy_args(dm, budgets_host, 0, dm.S, &base);
+  const size_t smem = alloc_small_smem_bytes(dm.N, dm.P);
   cudaError_t e;
-  if (dm.N <= kSmallMaxHeads) {
-    const size_t smem = alloc_small_smem_bytes(dm.N, dm.P);
-    if ((e = allow_smem((const void*)alloc_small_kernel, smem)) != cudaSuccess) return e;
-    e = launch_pdl(alloc_small_kernel, dim3(dm.S), dim3(32 * dm.N), smem, lc.st, beside, curves, args, budgets, offsets, dm.N,
-                   dm.P, dm.w);
-  } else {
-    const int group = (dm.N + 31) & ~31, groups = std::min(kGreedyMaxGroups, kGreedyMaxThreads / group);
-    const int cap = (int)std::min((long long)dm.N * (dm.P - 1), 16384LL);
-    const size_t smem = greedy_smem_bytes(dm.N, cap, groups, true);
-    if ((e = allow_smem((const void*)alloc_kernel, smem)) != cudaSuccess) return e;
-    e = launch_pdl(alloc_kernel, dim3(1), dim3(group * groups), smem, lc.st, beside, curves, lists, args, budgets, offsets,
-                   dm.N, dm.P, dm.w, cap, group);
-  }
+  if ((e = allow_smem((const void*)alloc_small_kernel, smem)) != cudaSuccess) return e;
+  e = launch_pdl(alloc_small_kernel, dim3(dm.S), dim3(32 * dm.N), smem, lc.st, beside, curves, args, budgets, offsets, dm.N,
+                 dm.P, dm.w);
   if (e != cudaSuccess) return e;
   lc.mark("allocate");
   return cudaGetLastError();
@@ -1000,12 +963,10 @@ cudaError_t launch_allocate_one(const Dims& dm, const float* curves, const int64
 
 cudaError_t launch_allocate(const Dims& dm, const float* curves, const int64_t* budgets_host, const HullLists& lists,
                             int32_t* budgets, int32_t* offsets, LaunchCtx& lc) {
-  // alone: up to 32 heads in one launch; more heads walk their curves on as many SMs as there are
-  if (allocate_one_launch(dm) && dm.N <= kSmallMaxHeads)
-    return launch_allocate_one(dm, curves, budgets_host, lists, budgets, offsets, false, lc);
+  if (allocate_small(dm)) return launch_allocate_small(dm, curves, budgets_host, budgets, offsets, false, lc);
   cudaError_t e = launch_hull(curves, lists, dm.N, dm.P, lc);
   if (e != cudaSuccess) return e;
-  return launch_greedy(dm, lists, budgets_host, budgets, offsets, 1, lc);
+  return launch_greedy(dm, lists, budgets_host, budgets, offsets, 1, false, lc);
 }
 
 }  // namespace lukv

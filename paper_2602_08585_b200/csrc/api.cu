@@ -179,7 +179,7 @@ cudaError_t allow_smem(const void* kernel, size_t bytes) {
   return cudaSuccess;
 }
 
-// An auxiliary stream and the two events that tie it to the caller's stream (allocations too large for one launch), created
+// An auxiliary stream and the two events that tie it to the caller's stream (allocations of more than 32 heads), created
 // on first use on a device and kept until the process exits (handles only, no device memory).
 struct SideStream {
   cudaStream_t stream = nullptr;
@@ -207,23 +207,26 @@ static SideStream* side_stream() {
 }
 
 // The whole path.  Allocation depends only on the curves, scoring only on Q/K; selection needs both, the gather follows.
-// With `overlap` allocation runs beside the scorer, normally as one CTA: behind a persistent scorer (tensor-core, KeyDiff),
-// which leaves it an SM, or ahead of the general-shape scorer's first sweep.  Neighbours in the stream are programmatic
-// dependents; whichever of scorer and allocation comes second ends after the first, so that the selection, which waits for
-// the second, sees both.  Allocations too large for one launch run on an auxiliary stream.
+// With `overlap` allocation runs beside the scorer.  Up to 32 heads: one CTA per sequence, on the caller's stream, behind a
+// persistent scorer (tensor-core, KeyDiff), which leaves it an SM, or ahead of the general-shape scorer's first sweep;
+// neighbours in the stream are programmatic dependents, and whichever of scorer and allocation comes second ends after the
+// first, so that the selection, which waits for the second, sees both.  More heads: hulls and greedy on an auxiliary
+// stream, whose hulls take the SMs before the scorer does (256 heads x 513 points with 1536 keys: 87 us a call; hulls by
+// one CTA behind the scorer 134 us, hulls ahead of the scorer on its own stream 97 us).
 static int run_compress(const Dims& dm, const void* q_win, const void* k, const void* v, const float* curves,
                         const int64_t* budgets_in, void* k_out, void* v_out, int32_t* kept_idx, int32_t* budgets,
                         int32_t* offsets, int64_t rows_cap, int32_t* dev_status, const Workspace& w, LaunchCtx& lc,
                         bool overlap) {
   const bool persistent = dm.keydiff || (score_tc_supported(dm) && !force_simt());
-  bool chained = overlap;  // the selection is the dependent of the launch before it
-  if (overlap && allocate_one_launch(dm)) {
+  bool chained = false;  // the selection is the dependent of the launch before it
+  if (overlap && allocate_small(dm)) {
     auto allocate = [&](bool beside) {
-      return launch_allocate_one(dm, curves, budgets_in, w.hull, budgets, offsets, beside, lc);
+      return launch_allocate_small(dm, curves, budgets_in, budgets, offsets, beside, lc);
     };
     if (!persistent && allocate(false) != cudaSuccess) return LUKV_ERR_CUDA;
     if (run_score(dm, q_win, k, w, 1, true, lc) != cudaSuccess) return LUKV_ERR_CUDA;
     if (persistent && allocate(true) != cudaSuccess) return LUKV_ERR_CUDA;
+    chained = true;
   } else if (SideStream* side = overlap ? side_stream() : nullptr) {
     std::lock_guard<std::mutex> in_use(side->use);
     LaunchCtx ls;
@@ -231,18 +234,18 @@ static int run_compress(const Dims& dm, const void* q_win, const void* k, const 
     int rc = LUKV_OK;
     if (cudaEventRecord(side->fork, lc.st) != cudaSuccess || cudaStreamWaitEvent(ls.st, side->fork, 0) != cudaSuccess)
       return LUKV_ERR_CUDA;
-    if (launch_allocate(dm, curves, budgets_in, w.hull, budgets, offsets, ls) != cudaSuccess) rc = LUKV_ERR_CUDA;
+    if (launch_hull(curves, w.hull, dm.N, dm.P, ls) != cudaSuccess ||
+        launch_greedy(dm, w.hull, budgets_in, budgets, offsets, 1, persistent, ls) != cudaSuccess)
+      rc = LUKV_ERR_CUDA;
     if (cudaEventRecord(side->join, ls.st) != cudaSuccess) rc = LUKV_ERR_CUDA;
     lc.launches += ls.launches;
     if (rc == LUKV_OK && run_score(dm, q_win, k, w, 1, false, lc) != cudaSuccess) rc = LUKV_ERR_CUDA;
     // join even after a failure: the caller's stream must not run ahead of work already enqueued
     if (cudaStreamWaitEvent(lc.st, side->join, 0) != cudaSuccess) rc = LUKV_ERR_CUDA;
     if (rc != LUKV_OK) return rc;
-    chained = false;
   } else {
     if (launch_allocate(dm, curves, budgets_in, w.hull, budgets, offsets, lc) != cudaSuccess) return LUKV_ERR_CUDA;
     if (run_score(dm, q_win, k, w, 0, false, lc) != cudaSuccess) return LUKV_ERR_CUDA;
-    chained = false;
   }
   const float* scores = w.raw;
   const bool pool = !dm.keydiff && select_pools(dm);
@@ -590,7 +593,7 @@ int lukv_profile_build(const lukv_params_t* calib, const float* curves, int32_t 
   LaunchCtx lc;
   lc.st = (cudaStream_t)stream;
   cudaError_t e = launch_hull(curves, w.hull, (int64_t)n_queries * dm.N, dm.P, lc);
-  if (e == cudaSuccess) e = launch_greedy(dm, w.hull, B, w.budgets, w.offsets, n_queries, lc);
+  if (e == cudaSuccess) e = launch_greedy(dm, w.hull, B, w.budgets, w.offsets, n_queries, false, lc);
   free(B);  // the budgets travel by value in the launch arguments
   if (e == cudaSuccess) e = launch_profile_mean(w.budgets, profile, n_queries, (int64_t)dm.S * dm.N, dm.n, lc);
   if (e != cudaSuccess) return LUKV_ERR_CUDA;

@@ -150,20 +150,20 @@ cudaError_t launch_score_onepass(const Dims& dm, const void* q, const void* k, c
                                  LaunchCtx& lc);
 // raw [heads][raw_stride] -> pooled [heads][stride]
 cudaError_t launch_pool(const Dims& dm, const float* raw, float* pooled, int stride, LaunchCtx& lc);
-// Allocation in one launch of one CTA: up to 1024 heads, 544 curve points and 128 sequences.  With `beside` it may run
-// beside the kernel launched just before it, whose results it does not touch; it ends after that kernel.
-bool allocate_one_launch(const Dims& dm);
-cudaError_t launch_allocate_one(const Dims& dm, const float* curves, const int64_t* budgets_host, const HullLists& lists,
-                                int32_t* budgets, int32_t* offsets, bool beside, LaunchCtx& lc);
+// Allocation of up to 32 heads (544 curve points, 128 sequences) in one launch.  With `beside` it may run beside the kernel
+// launched just before it, whose results it does not touch; it ends after that kernel.
+bool allocate_small(const Dims& dm);
+cudaError_t launch_allocate_small(const Dims& dm, const float* curves, const int64_t* budgets_host, int32_t* budgets,
+                                  int32_t* offsets, bool beside, LaunchCtx& lc);
 // Any size: the above where it applies, else hull and greedy.
 cudaError_t launch_allocate(const Dims& dm, const float* curves, const int64_t* budgets_host, const HullLists& lists,
                             int32_t* budgets, int32_t* offsets, LaunchCtx& lc);
 // The two halves.  launch_hull treats its input as n_curves independent curves;
 // launch_greedy solves n_sets curve sets (lists of n_sets * N curves) for the same dm.S budgets and
-// writes budgets [n_sets][S][N] and offsets [n_sets][S*N+1].
+// writes budgets [n_sets][S][N] and offsets [n_sets][S*N+1].  one_cta: by a single CTA (n_sets == 1).
 cudaError_t launch_hull(const float* curves, const HullLists& out, int64_t n_curves, int P, LaunchCtx& lc);
 cudaError_t launch_greedy(const Dims& dm, const HullLists& lists, const int64_t* budgets_host, int32_t* budgets,
-                          int32_t* offsets, int n_sets, LaunchCtx& lc);
+                          int32_t* offsets, int n_sets, bool one_cta, LaunchCtx& lc);
 // Offline profile (mean of the local ratios) and online lookup + budgeting.
 cudaError_t launch_profile_mean(const int32_t* budgets, float* profile, int n_queries, int64_t count, int n,
                                 LaunchCtx& lc);
