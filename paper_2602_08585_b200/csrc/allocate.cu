@@ -28,7 +28,7 @@ struct HullOut {
 // the points (k, U[k]); from a vertex i the next one is the point j > i with the steepest slope from i, the last of them
 // if several share it.  Slopes are compared in fp32; points whose slopes fp32 cannot tell apart are compared by their
 // correctly rounded fp64 quotients.  Once no slope is positive the rest is one block of gain 0.
-// Both forms below run it with one warp per curve and return the number of blocks.
+// One warp per curve; returns the number of blocks.
 
 // The last point among the candidates of the warp (j < 0: none in this lane) with the largest fp64 quotient.
 __device__ __noinline__ int hull_resolve(float uj, int j, float ui, int i) {
@@ -136,117 +136,17 @@ __device__ __forceinline__ int hull_walk_regs(const float* __restrict__ U, int P
   return blocks.count;
 }
 
-// Any P: the curve in shared memory `Us`, at most 32 chunks of 32 PPL points.  Chunk maxima of U bound the slope that any
-// point of a chunk can reach (one chunk per lane); the chunks whose bound comes up to the steepest slope found are
-// evaluated, PPL points per lane.  Returns -1 for a curve with many vertices, which hull_dense_kernel takes: a step costs
-// the same whether it skips one point or a thousand.  The walk stops after one vertex per 32 points, or before it starts
-// when more than three quarters of the increments are no larger than the one before (half of them on noisy curves).
-template <int PPL>
-__device__ __forceinline__ int hull_walk_chunks(const float* Us, int P, int lane, HullOut out) {
-  constexpr int C = 32 * PPL;
-  const int nchunk = (P + C - 1) / C;
-  float cmax = -INFINITY;  // maximum of chunk `lane`
-#pragma unroll 1
-  for (int c = 0; c < nchunk; ++c) {
-    float m = -INFINITY;
-#pragma unroll
-    for (int t = 0; t < PPL; ++t)
-      if (c * C + 32 * t + lane < P) m = fmaxf(m, Us[c * C + 32 * t + lane]);
-    m = warp_max(m);
-    if (lane == c) cmax = m;
-  }
-  int falls = 0;
-#pragma unroll 4
-  for (int j = lane + 1; j + 1 < P; j += 32) falls += Us[j + 1] - Us[j] <= Us[j] - Us[j - 1];
-  if (4 * __reduce_add_sync(0xffffffffu, falls) > 3 * P) return -1;
-  const int c_first = lane * C, c_last = min(c_first + C, P) - 1;
-  const float f_lane = (float)lane;
-  HullBlocks blocks;
-  int i = 0;
-  float ui = Us[0];
-#pragma unroll 1
-  while (i < P - 1) {
-    // slopes from i to the points j0 + lane + 32 t
-    auto slope = [&](int j0, int t) {
-      const float dist = f_lane + (float)(j0 + 32 * t - i);
-      const int j = j0 + 32 * t + lane;
-      return dist > 0.f && j < P ? __fdividef(Us[j] - ui, dist) : -INFINITY;
-    };
-    // upper bound of the slope from i to a point of this lane's chunk, above the rounding of the slopes
-    float bound = -INFINITY;
-    if (lane < nchunk && c_last > i) {
-      const float rise = cmax - ui;
-      bound = __fdividef(rise, (float)(rise > 0.f ? max(c_first, i + 1) - i : c_last - i));
-      bound += 1e-6f * fabsf(bound);
-    }
-    float best = -INFINITY, chunk_best = -INFINITY;
-    uint32_t todo = __ballot_sync(0xffffffffu, bound > -INFINITY);
-    int c = __ffs(__ballot_sync(0xffffffffu, bound == warp_max(bound)) & todo) - 1;
-    int next = P - 1;
-    if (c >= 0) {  // else not a number: the rest is one block
-#pragma unroll 1
-      for (;;) {
-        float m = -INFINITY;
-#pragma unroll
-        for (int t = 0; t < PPL; ++t) m = fmaxf(m, slope(c * C, t));
-        m = warp_max(m);
-        if (lane == c) chunk_best = m;
-        best = fmaxf(best, m);
-        todo &= ~(1u << c) & __ballot_sync(0xffffffffu, bound >= best);
-        if (!todo) break;
-        c = __ffs(todo) - 1;
-      }
-      // every point that may hold the steepest slope
-      const float near = best - 2e-6f * fabsf(best);
-      const uint32_t chunks = __ballot_sync(0xffffffffu, chunk_best >= near);
-      int mine = -1, found = 0;
-#pragma unroll 1
-      for (uint32_t left = chunks; left; left &= left - 1) {
-        const int j0 = (__ffs(left) - 1) * C;
-#pragma unroll
-        for (int t = 0; t < PPL; ++t)
-          if (slope(j0, t) >= near) {
-            mine = j0 + 32 * t + lane;
-            ++found;
-          }
-      }
-      next = __reduce_max_sync(0xffffffffu, mine);
-      if (__reduce_add_sync(0xffffffffu, found) > 1) {
-        next = -1;
-#pragma unroll 1
-        for (uint32_t left = chunks; left; left &= left - 1) {
-          const int j0 = (__ffs(left) - 1) * C;
-#pragma unroll 1
-          for (int t = 0; t < PPL; ++t) {
-            const int j = j0 + 32 * t + lane;
-            const int at = hull_resolve(j < P ? Us[j] : 0.f, slope(j0, t) >= near ? j : -1, ui, i);
-            if (at < 0) continue;
-            const int pick = lane == 0 ? at : lane == 1 ? next : -1;
-            next = hull_resolve(pick >= 0 ? Us[pick] : 0.f, pick, ui, i);
-          }
-        }
-      }
-    }
-    const bool flat = !(best > 0.f);
-    if (flat) next = P - 1;
-    if (blocks.count > P / 32) return -1;
-    const float u_next = Us[next];
-    blocks.add(i, ui, next, u_next, flat, next == P - 1, lane, out);
-    ui = u_next;
-    i = next;
-  }
-  return blocks.count;
-}
-
-// ---- curves with many vertices: pool adjacent violators on 32 runs, then join -------------------------------------
+// ---- long curves: drop the points that lie on or below the chord of their neighbours, until none does ----------------
 
 // mean of block 1 <= mean of block 2, where a block's mean is (its curve rise) / (its length) and
 // the rises are differences of two fp32 curve values: decided exactly as the comparison of the two
-// correctly rounded fp64 quotients.  Three tiers, cheapest first:
+// correctly rounded fp64 quotients.  Cheapest first:
 //   fp32 cross products, when they are further apart than fp32 rounding can explain;
+//   their exact values in two words, when both rises are exact in fp32 (neighbouring points of a long curve differ by a few
+//   units in the last place, and ties are common): 24 + 13 bits, which fp64 quotients tell apart if they differ;
 //   fp64 cross products, when they are clearly apart;
 //   the fp64 quotients themselves.
-// (the last two out of line: they are rare, and an fp64 operation costs the walk some 50 clocks)
+// (the last two out of line: they are rare, and an fp64 operation costs a warp some 50 clocks)
 // Block 1 rises from u_l1 to u_r1 over len1 points, block 2 from u_l2 to u_r2 over len2.
 __device__ __noinline__ bool mean_le_f64(float u_l1, float u_r1, int len1, float u_l2, float u_r2, int len2) {
   const double a = __dsub_rn((double)u_r1, (double)u_l1), b = (double)len1;
@@ -258,13 +158,148 @@ __device__ __noinline__ bool mean_le_f64(float u_l1, float u_r1, int len1, float
   if (diff > tol) return false;
   return __ddiv_rn(a, b) <= __ddiv_rn(c, d);
 }
+// Whether d = fl(a - b) is a - b exactly: a sufficient condition (Sterbenz: the one at most twice the other).
+__device__ __forceinline__ bool exact_diff(float a, float b, float d) { return fabsf(d) <= fminf(fabsf(a), fabsf(b)); }
+// d1 / n1 <= d2 / n2 for exact rises d and lengths n below 2^13: exact cross products in two words.
+__device__ __forceinline__ bool exact_le(float d1, float n1, float d2, float n2) {
+  const float q1 = d1 * n2, q2 = d2 * n1;
+  return (q1 < q2) | ((q1 == q2) & (fmaf(d1, n2, -q1) <= fmaf(d2, n1, -q2)));  // no branches
+}
 __device__ __forceinline__ bool mean_le(float u_l1, float u_r1, int len1, float u_l2, float u_r2, int len2) {
-  const float q1 = (u_r1 - u_l1) * (float)len2, q2 = (u_r2 - u_l2) * (float)len1;
+  const float d1 = u_r1 - u_l1, d2 = u_r2 - u_l2, n1 = (float)len1, n2 = (float)len2;
+  const float q1 = d1 * n2, q2 = d2 * n1;
   const float diff = q1 - q2;
   // each product carries two roundings of 2^-24, the difference one
   if (fabsf(diff) > 5e-7f * fmaxf(fabsf(q1), fabsf(q2))) return diff < 0.f;
+  if (exact_diff(u_r1, u_l1, d1) && exact_diff(u_r2, u_l2, d2)) return exact_le(d1, n1, d2, n2);
   return mean_le_f64(u_l1, u_r1, len1, u_l2, u_r2, len2);
 }
+
+// Survivors of the first pass that the shared memory of a curve holds; a fifth of the points of a noisy curve survive.
+inline int hull_prune_cap(int P) { return (P * 2 / 5 + 63) & ~63; }
+constexpr int kHullPasses = 48;
+
+// One warp per curve.  A point on or below the chord of two other points is no vertex of the majorant, whichever points
+// they are, so a pass may test all points against their current neighbours at once; a polygon without such a point is the
+// majorant.  The first pass reads the curve once, into registers, and drops what lies clearly below the chord of the points
+// 1, 2, 4, 8 or 16 places to either side (4001 points: about 800 stay); the survivors (value and index) are compacted in
+// shared memory and tested against their neighbours, exactly, until none is dropped (9 passes over 1900 points in all, 53
+// stay).  A curve of which more than two fifths survive the first pass, or that needs more than kHullPasses, is left to
+// hull_dense_kernel (count -1).  Blocks beyond the last positive slope are one block of gain 0.
+// Bound by instruction issue.  7680 curves of 4001 points: 3.07 ms as one serial stack walk per curve, 0.31 ms as a walk from
+// vertex to vertex over chunk maxima, 0.22 ms with neighbours alone in the first pass, 0.15 ms now.
+__global__ void __launch_bounds__(32) hull_prune_kernel(const float* __restrict__ curves, HullLists lists, int P, int cap) {
+  extern __shared__ float hull_smem[];
+  const int hid = blockIdx.x, lane = threadIdx.x;
+  const float* U = curves + (size_t)hid * P;
+  float* us = hull_smem;                                                    // [cap]
+  unsigned short* is = reinterpret_cast<unsigned short*>(hull_smem + cap);  // [cap]
+  const uint32_t lt_mask = (1u << lane) - 1u;
+  pdl_launch_dependents();
+  constexpr int kAhead = 8;  // vectors of 32 points at a time; the next ones are on their way
+  int cnt = 0;
+  float cur[kAhead], nxt[kAhead], prev = 0.f;
+#pragma unroll
+  for (int t = 0; t < kAhead; ++t) nxt[t] = __ldg(U + min(32 * t + lane, P - 1));
+#pragma unroll 1
+  for (int base = 0; base < P; base += 32 * kAhead) {
+#pragma unroll
+    for (int t = 0; t < kAhead; ++t) cur[t] = nxt[t];
+#pragma unroll
+    for (int t = 0; t < kAhead; ++t) nxt[t] = __ldg(U + min(base + 32 * (kAhead + t) + lane, P - 1));
+#pragma unroll
+    for (int t = 0; t < kAhead; ++t) {
+      const int j = base + 32 * t + lane;
+      const float u = cur[t], up = t > 0 ? cur[t > 0 ? t - 1 : 0] : prev, un = t + 1 < kAhead ? cur[t + 1 < kAhead ? t + 1 : 0] : nxt[0];
+      // below the chord by more than the roundings of the two sides (2.4e-7 |u| where they are close)
+      const float lim = fmaf(5e-7f, fabsf(u), 2.f * u), small = 0.25f * fabsf(u);
+      bool below = false;
+      const bool edge = base + 32 * t < 32 || base + 32 * t + 48 > P;
+#pragma unroll
+      for (int k = 1; k <= 16; k <<= 1) {
+        // lanes whose value wraps around stand for the vector before, or behind
+        const float l = __shfl_sync(0xffffffffu, lane >= 32 - k ? up : u, (lane + 32 - k) & 31);
+        const float r = __shfl_sync(0xffffffffu, lane < k ? un : u, (lane + k) & 31);
+        bool b;
+        if (k <= 2) {
+          // rises of at most a quarter of u are exact in fp32 (late on a curve they are a few units in the last place)
+          const float d1 = u - l, d2 = r - u;
+          b = (d1 <= d2) & (fmaxf(fabsf(d1), fabsf(d2)) <= small);
+        } else {
+          b = l + r > lim;
+        }
+        if (edge) b = b & (j >= k) & (j + k < P);
+        below |= b;
+      }
+      const bool keep = (j < P) & !below;
+      const uint32_t kept = __ballot_sync(0xffffffffu, keep);
+      const int at = cnt + __popc(kept & lt_mask);
+      if (keep && at < cap) {
+        us[at] = u;
+        is[at] = (unsigned short)j;
+      }
+      cnt += __popc(kept);
+    }
+    prev = cur[kAhead - 1];
+  }
+  bool done = false;
+  if (cnt <= cap) {
+#pragma unroll 1
+    for (int pass = 0; pass < kHullPasses && !done; ++pass) {
+      __syncwarp();
+      int out = 0;
+#pragma unroll 1
+      for (int base = 0; base < cnt; base += 32) {
+        // in place: the writes of a turn end before the points that the next one reads, but for the last, unless nothing
+        // was dropped yet, when they write what is there
+        const int i = base + lane, ii = min(i, cnt - 1), il = max(ii - 1, 0), ir = min(ii + 1, cnt - 1);
+        const float um = us[ii], ul = us[il], ur = us[ir];
+        const int km = is[ii], kl = is[il], kr = is[ir];
+        // 2^23 + k as a float: differences of two are the lengths
+        auto place = [](int k) { return __int_as_float(0x4B000000 | k); };
+        const float d1 = um - ul, d2 = ur - um;
+        bool keep;
+        if (__all_sync(0xffffffffu, exact_diff(um, ul, d1) & exact_diff(ur, um, d2)))
+          keep = !exact_le(d1, place(km) - place(kl), d2, place(kr) - place(km));
+        else
+          keep = !mean_le(ul, um, km - kl, um, ur, kr - km);
+        keep = (i < cnt) & ((i == 0) | (i == cnt - 1) | keep);
+        const uint32_t kept = __ballot_sync(0xffffffffu, keep);
+        if (keep) {
+          const int at = out + __popc(kept & lt_mask);
+          us[at] = um;
+          is[at] = (unsigned short)km;
+        }
+        out += __popc(kept);
+        __syncwarp();
+      }
+      done = out == cnt;
+      cnt = out;
+    }
+  }
+  int total = -1;
+  if (done) {
+    total = 0;
+    float* g_out = lists.gain + (size_t)hid * (P - 1);
+    unsigned short* s_out = lists.start + (size_t)hid * (P - 1);
+    for (int base = 0; base < cnt - 1; base += 32) {
+      const int i = base + lane;
+      const bool block = i < cnt - 1, rises = block && us[i + 1] > us[i];
+      const int rising = __popc(__ballot_sync(0xffffffffu, rises));
+      if (block && lane <= rising) {
+        double mean = 0.0;
+        if (rises) mean = __ddiv_rn(__dsub_rn((double)us[i + 1], (double)us[i]), (double)(is[i + 1] - is[i]));
+        g_out[i] = __double2float_rn(mean);
+        s_out[i] = is[i];
+      }
+      total = min(base + rising + 1, cnt - 1);
+      if (rising < 32) break;  // the rest has no positive slope
+    }
+  }
+  if (lane == 0) lists.count[hid] = total;
+}
+
+// ---- long curves with many vertices: pool adjacent violators on 32 runs, then join --------------------------------
 
 // Increments per lane: an odd count, so that the lanes' runs start in different banks.
 __host__ __device__ inline int hull_run(int P) { return ((P - 1 + 31) / 32) | 1; }
@@ -280,7 +315,7 @@ __global__ void hull_dense_kernel(const float* __restrict__ curves, HullLists li
   const int hid = blockIdx.x, lane = threadIdx.x;
   pdl_launch_dependents();
   pdl_wait();
-  if (lists.count[hid] >= 0) return;  // the vertex walk took this curve
+  if (lists.count[hid] >= 0) return;  // the kernel before took this curve
   const float* U = curves + (size_t)hid * P;
   const int run = hull_run(P);
   float* Us = hull_smem;
@@ -424,26 +459,14 @@ __device__ __forceinline__ int hull_walk_short(const float* U, int P, int lane, 
   return hull_walk_regs<17>(U, P, lane, out);
 }
 
-// One warp (a block of its own) per curve.
-// Bound by the latency of a step; a curve has few vertices: 6 of 257 points on the benchmark's curves, 53 of 4001 on the
-// calibration curves.  Measured against one serial stack walk per curve: 256 curves of 257 points 59 -> 5 us, 7680 of 4001
-// 3.07 -> 0.29 ms; pooling on 32 runs per curve (below) takes 0.5 ms there, but is the faster one on concave curves.
-template <int PPL>
+// One warp (a block of its own) per curve of up to kHullRegsMaxP points.
+// Bound by the latency of a step; a curve has few vertices (6 of 257 points on the benchmark's curves).  256 curves of 257
+// points: 59 us beside the scorer as one serial stack walk per curve, 5 us now.
 __global__ void hull_kernel(const float* __restrict__ curves, HullLists lists, int P) {
-  extern __shared__ float hull_smem[];
   const int hid = blockIdx.x, lane = threadIdx.x;
-  const float* U = curves + (size_t)hid * P;
   const HullOut out = {lists.gain + (size_t)hid * (P - 1), lists.start + (size_t)hid * (P - 1)};
   pdl_launch_dependents();
-  int count;
-  if (PPL == 0) {
-    count = hull_walk_short(U, P, lane, out);
-  } else {
-#pragma unroll 16
-    for (int i = lane; i < P; i += 32) hull_smem[i] = __ldg(U + i);
-    __syncwarp();
-    count = hull_walk_chunks<PPL == 0 ? 1 : PPL>(hull_smem, P, lane, out);
-  }
+  const int count = hull_walk_short(curves + (size_t)hid * P, P, lane, out);
   if (lane == 0) lists.count[hid] = count;
 }
 
@@ -894,19 +917,18 @@ size_t hull_lists_bytes(int64_t n_curves, int P) {
 
 cudaError_t launch_hull(const float* curves, const HullLists& out, int64_t n_curves, int P, LaunchCtx& lc) {
   const unsigned grid = (unsigned)n_curves;
-  const size_t smem = P <= kHullRegsMaxP ? 0 : (size_t)P * sizeof(float);  // at most 16.4 KB
-  cudaError_t e;
-  if (P <= kHullRegsMaxP) hull_kernel<0><<<grid, 32, smem, lc.st>>>(curves, out, P);
-  else if (P <= 1024) hull_kernel<1><<<grid, 32, smem, lc.st>>>(curves, out, P);
-  else if (P <= 2048) hull_kernel<2><<<grid, 32, smem, lc.st>>>(curves, out, P);
-  else if (P <= 4096) hull_kernel<4><<<grid, 32, smem, lc.st>>>(curves, out, P);
-  else hull_kernel<5><<<grid, 32, smem, lc.st>>>(curves, out, P);
-  lc.mark("hull");
-  if (P > kHullRegsMaxP) {
-    const size_t dense = hull_dense_smem_bytes(P);  // at most 25 KB
-    if ((e = launch_pdl(hull_dense_kernel, dim3(grid), dim3(32), dense, lc.st, true, curves, out, P)) != cudaSuccess) return e;
-    lc.mark("hull_dense");
+  if (P <= kHullRegsMaxP) {
+    hull_kernel<<<grid, 32, 0, lc.st>>>(curves, out, P);
+    lc.mark("hull");
+    return cudaGetLastError();
   }
+  const int cap = hull_prune_cap(P);
+  hull_prune_kernel<<<grid, 32, (size_t)cap * 6, lc.st>>>(curves, out, P, cap);
+  lc.mark("hull_prune");
+  const cudaError_t e = launch_pdl(hull_dense_kernel, dim3(grid), dim3(32), hull_dense_smem_bytes(P), lc.st, true, curves,
+                                   out, P);  // at most 25 KB
+  if (e != cudaSuccess) return e;
+  lc.mark("hull_dense");
   return cudaGetLastError();
 }
 
