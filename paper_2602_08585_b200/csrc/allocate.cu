@@ -482,6 +482,7 @@ struct GreedyArgs {
   int T[kSeqPerLaunch];               // context length of sequence q (the curve grid is T/(P-1) tokens per segment)
   int floor_tok[kSeqPerLaunch];       // tokens every head of sequence q keeps at least
   int seq0, count;                    // sequences seq0 .. seq0 + count - 1
+  int uniform;                        // all of one length
 };
 
 struct SetStride {
@@ -552,27 +553,101 @@ struct ListView {
 struct GreedyShared {
   uint2 sum[2][32];
   int scan[32];
-  unsigned cut[2];
+  unsigned cut[2];    // gain at which the budget runs out, tokens left for it
+  unsigned range[2];  // smallest and largest gain
+  unsigned sel[2];    // bin, tokens above it
+  unsigned listed;
 };
-constexpr int kGreedyCountMax = 256;  // blocks in all up to which the cut is found by counting
+constexpr int kGreedyBins = 512;
+constexpr int kGreedyList = kGreedyBins / 2;  // blocks that are ranked directly
+constexpr int kGreedyWords = kGreedyBins + 2; // scratch of a group: bins, or a list of pairs
+
+// body(gain bits, tokens) for the staged blocks with from <= gain <= to; the ends of the curves count as blocks without
+// capacity.
+template <typename Body>
+__device__ __forceinline__ void each_block(const ListView<true>& lists, int N, int seg, int n, int floor_tok, unsigned from,
+                                           unsigned to, const Group& grp, Body&& body) {
+  const int entries = lists.at_[N] - 1;
+#pragma unroll 4
+  for (int e = grp.tid; e < entries; e += grp.nthr) {
+    const unsigned g = __float_as_uint(lists.gain_[e]);
+    if (g - from <= to - from)
+      body(g, (unsigned)max(0, capsum(lists.start_[e + 1], seg, n, floor_tok) - capsum(lists.start_[e], seg, n, floor_tok)));
+  }
+}
+// Smallest and largest positive gain of the staged lists (bit patterns; from > to: none).
+__device__ __forceinline__ void gain_range(const ListView<true>& lists, int N, const Group& grp, GreedyShared& sh,
+                                           unsigned& from, unsigned& to) {
+  if (grp.tid == 0) {
+    sh.range[0] = 0xFFFFFFFFu;
+    sh.range[1] = 0u;
+  }
+  grp.sync();
+  from = 0xFFFFFFFFu;
+  to = 0u;
+  for (int h = grp.tid; h < N; h += grp.nthr) {
+    int x = lists.blocks(h) - 1;
+    while (x > 0 && lists.gain(h, x) == 0.f) --x;
+    const unsigned g = __float_as_uint(lists.gain(h, x));
+    if (g != 0u) from = min(from, g);
+    to = max(to, __float_as_uint(lists.gain(h, 0)));
+  }
+  from = __reduce_min_sync(0xffffffffu, from);
+  to = __reduce_max_sync(0xffffffffu, to);
+  if ((grp.tid & 31) == 0) {
+    atomicMin(&sh.range[0], from);
+    atomicMax(&sh.range[1], to);
+  }
+  grp.sync();
+  from = sh.range[0];
+  to = sh.range[1];
+}
+__device__ __forceinline__ int bin_bits(unsigned from, unsigned to) { return max(0, 23 - __clz(to - from)); }
+// Tokens in the bins at or above each of the kGreedyBins bins (entry kGreedyBins: 0) over the range [from, to].
+__device__ __forceinline__ void bins_at_least(const ListView<true>& lists, int N, int seg, int n, int floor_tok, unsigned from,
+                                              unsigned to, const Group& grp, GreedyShared& sh, unsigned* bins) {
+  for (int x = grp.tid; x <= kGreedyBins; x += grp.nthr) bins[x] = 0u;
+  grp.sync();
+  const int bits = bin_bits(from, to);
+  each_block(lists, N, seg, n, floor_tok, from, to, grp,
+             [&](unsigned g, unsigned tokens) { atomicAdd(&bins[(g - from) >> bits], tokens); });
+  grp.sync();
+  // a thread owns consecutive bins from the top
+  const int own = (kGreedyBins + grp.nthr - 1) / grp.nthr, top = kGreedyBins - 1 - grp.tid * own;
+  unsigned mine = 0;
+  for (int x = top; x > top - own && x >= 0; --x) mine += bins[x];
+  unsigned run = (unsigned)group_scan((int)mine, sh.scan, grp);
+  for (int x = top; x > top - own && x >= 0; --x) {
+    run += bins[x];
+    bins[x] = run;
+  }
+  grp.sync();
+}
+
+// The first split of the gains, shared by the problems of a CTA where all have the same grid; bins null: none.
+struct FirstSplit {
+  const unsigned* bins;
+  unsigned from, to;
+};
 
 // One problem: sequence i of `args` on the lists of one curve set, by the threads of a group; thread t owns the heads
 // [t*per, (t+1)*per) (ONE: the head t).  The greedy buys segments in the order (gain desc, k asc, hid asc) until the
 // budget is spent.
-//   gain  With few blocks every thread adds up the capacities of the blocks that are steeper than its own: the block at
-//         which the sum passes the budget names the gain.  Otherwise by bisection over the bits of the gain: the lists
-//         are sorted by falling gain, so the blocks of a head whose gain agrees with the bits fixed so far form a range
-//         [lo,hi); inside it the next bit is 1 up to some index and 0 from there on: one binary search per head and bit
-//         (none when the range's ends agree).  The capacities of the 1s, summed over the heads, and the budget decide
-//         which half holds the cut.  The bits end early when a single block is left.
+//   gain  Staged lists: the capacities of all blocks go into bins along the range of the gains (their bit patterns: a
+//         logarithmic scale); the bin in which the budget runs out is split again until it holds at most kGreedyList blocks,
+//         of which every thread adds up those that are steeper than its own.  Lists in place: bisection over the bits of the
+//         gain; they are sorted by falling gain, so the blocks of a head whose gain agrees with the bits fixed so far form
+//         a range [lo,hi); inside it the next bit is 1 up to some index and 0 from there on: one binary search per head
+//         and bit (none when the range's ends agree), and the capacities of the 1s, summed over the heads, and the budget
+//         decide which half holds the cut.
 //   k     Of the segments with exactly that gain (a range [a,e) per head) those with the smaller index are bought
 //         first: the index K at which the budget runs out, by bisection; not needed when one head has such segments.
 //   hid   Segment K of the heads that have it, in head order, each whole while the budget lasts.
-// lo, hi, mid: [N] words per head (unused when ONE).  weight: room for kGreedyCountMax words when STAGED.
+// lo, hi, mid: [N] words per head (unused when ONE).  bins: kGreedyWords words when STAGED.
 template <bool STAGED, bool ONE>
 __device__ __forceinline__ void greedy_problem(const ListView<STAGED> lists, const GreedyArgs& args, int i, int N, int w,
-                                               int* lo, int* hi, int* mid, int* weight, GreedyShared& sh,
-                                               const Group grp, int32_t* __restrict__ budgets, int32_t* __restrict__ offsets) {
+                                               int* lo, int* hi, int* mid, unsigned* bins, GreedyShared& sh,
+                                               const FirstSplit first, const Group grp, int32_t* __restrict__ budgets, int32_t* __restrict__ offsets) {
   const int tid = grp.tid, nthr = grp.nthr, G1 = lists.G1;
   const int per = ONE ? 1 : (N + nthr - 1) / nthr;
   const int h_begin = min(N, tid * per), h_end = min(N, h_begin + per);
@@ -588,39 +663,86 @@ __device__ __forceinline__ void greedy_problem(const ListView<STAGED> lists, con
   unsigned R = (unsigned)left;  // budgets are below 2^31
   unsigned round = 0;
   if (!all_taken) {
-    const int total = STAGED ? lists.at_[N] - N : kGreedyCountMax + 1;
-    if (STAGED && total <= kGreedyCountMax) {
-      // entries of all lists, the ends of the curves among them as blocks without capacity
-      const int entries = total + N;
-      for (int h = tid >> 5; h < N; h += nthr >> 5)
-        for (int e = lists.at_[h] + (tid & 31); e < lists.at_[h + 1]; e += 32) {
-          const bool end = e + 1 == lists.at_[h + 1];
-          weight[e] = end ? 0 : capsum(lists.start_[e + 1], seg, n, floor_tok) - capsum(lists.start_[e], seg, n, floor_tok);
-        }
-      grp.sync();
-      for (int e = tid; e < entries; e += nthr) {
-        const float g = lists.gain_[e];
-        unsigned steeper = 0, same = 0;
+    if constexpr (STAGED) {
+      unsigned from = first.from, to = first.to, gain = 0u;
+      if (!first.bins) gain_range(lists, N, grp, sh, from, to);
+      const unsigned* at_least = first.bins;                     // of the present range, if known
+      bool rank = !at_least && lists.at_[N] - N <= kGreedyList;  // few blocks: no bins
+#pragma unroll 1
+      while (from <= to) {
+        if (rank) {
+          if (tid == 0) {
+            sh.listed = 0u;
+            sh.cut[0] = 0u;
+          }
+          grp.sync();
+          uint2* list = reinterpret_cast<uint2*>(bins);
+          each_block(lists, N, seg, n, floor_tok, from, to, grp, [&](unsigned g, unsigned tokens) {
+            const unsigned x = atomicAdd(&sh.listed, 1u);
+            if (x < kGreedyList) list[x] = make_uint2(g, tokens);
+          });
+          grp.sync();
+          const int m = (int)sh.listed;
+          if (m <= kGreedyList) {
+            unsigned all = 0;
+            for (int e = tid; e < m; e += nthr) {
+              const unsigned g = list[e].x;
+              unsigned steeper = 0, same = 0;
 #pragma unroll 4
-        for (int x = 0; x < entries; ++x) {
-          const float gx = lists.gain_[x];
-          const unsigned wx = (unsigned)weight[x];
-          steeper += gx > g ? wx : 0u;
-          same += gx == g ? wx : 0u;
+              for (int x = 0; x < m; ++x) {
+                const uint2 o = list[x];
+                steeper += o.x > g ? o.y : 0u;
+                same += o.x == g ? o.y : 0u;
+              }
+              if (steeper <= R && R < steeper + same) {  // one gain; every thread that holds it writes the same
+                sh.cut[0] = g;
+                sh.cut[1] = R - steeper;
+              }
+              all += list[e].y;
+            }
+            all = group_sum2(all, 0u, sh.sum[round++ & 1], grp).x;
+            grp.sync();
+            gain = sh.cut[0];
+            R = gain != 0u ? sh.cut[1] : R - all;  // else the budget reaches the segments without gain
+            break;
+          }
+          grp.sync();
         }
-        if (steeper <= R && R < steeper + same) {  // one gain; every thread that holds it writes the same
-          sh.cut[0] = __float_as_uint(g);
-          sh.cut[1] = R - steeper;
+        if (!at_least) {
+          bins_at_least(lists, N, seg, n, floor_tok, from, to, grp, sh, bins);
+          at_least = bins;
         }
+        if (R >= at_least[0]) {  // the budget reaches the segments without gain
+          R -= at_least[0];
+          break;
+        }
+        for (int x = tid; x < kGreedyBins; x += nthr)
+          if (at_least[x + 1] <= R && R < at_least[x]) {
+            sh.sel[0] = (unsigned)x;
+            sh.sel[1] = at_least[x + 1];
+          }
+        grp.sync();
+        const int bits = bin_bits(from, to);
+        R -= sh.sel[1];
+        from += sh.sel[0] << bits;
+        to = min(to, from + ((1u << bits) - 1u));
+        if (bits == 0) {
+          gain = from;
+          break;
+        }
+        rank = true;
+        at_least = nullptr;
+        grp.sync();
       }
-      grp.sync();
-      const float g = __uint_as_float(sh.cut[0]);
-      R = sh.cut[1];
+      const float g = __uint_as_float(gain);
       for (int h = h_begin; h < h_end; ++h) {
         const int c = lists.blocks(h);
-        int l = 0;
-        while (l < c && lists.gain(h, l) > g) ++l;
-        int r = l;
+        int l = 0, r = c;  // first block that is not steeper than g
+        while (l < r) {
+          const int m = (l + r) >> 1;
+          if (lists.gain(h, m) > g) l = m + 1; else r = m;
+        }
+        r = l;
         while (r < c && lists.gain(h, r) == g) ++r;
         LO(h) = l;
         HI(h) = r;
@@ -737,20 +859,21 @@ __device__ __forceinline__ void greedy_problem(const ListView<STAGED> lists, con
   grp.sync();  // the shared words start over
 }
 
-// Shared memory of the greedy kernel: at [N+1], gain and start [cap + N] and the counted weights when lists are staged;
+// Shared memory of the greedy kernel: at [N+1], the groups' bins, gain and start [cap + N] when lists are staged;
 // lo, hi, mid [N] when a thread owns several heads.
 inline size_t greedy_smem_bytes(int N, int cap, int groups, bool one) {
-  const size_t e = (size_t)cap + N, weights = (size_t)groups * (kGreedyCountMax + N);
-  return (cap > 0 ? ((size_t)N + 1) * 4 + e * 4 + ((e * 2 + 3) & ~(size_t)3) + weights * 4 : 0) +
-         (one ? 0 : (size_t)N * 12);
+  const size_t e = (size_t)cap + N, bins = (size_t)groups * kGreedyWords;
+  return (cap > 0 ? ((size_t)N + 1) * 4 + e * 4 + ((e * 2 + 3) & ~(size_t)3) + bins * 4 + 4 : 0) +
+         (one ? 0 : (size_t)N * 12 + 4);
 }
 
 // One CTA per (share of the sequences, curve set), of one or more groups of `group` threads, each with a sequence of its
 // own at a time.  The lists of a set are short (6 blocks a head on the benchmark's curves, 53 of 4000 on the calibration
 // curves) and are staged in shared memory once for all sequences of the CTA when they fit, else read through L1.
-// Bound by latency, up to 31 rounds of a search and a group-wide sum, hence several groups per CTA where there are that
-// many problems.  65536 segments in 256 heads beside the scorer: 91 us with a search per head for each of the 64
-// bits of (gain, k, hid) over expanded segments, 34 us now; 2970 problems of 256 x 4000 segments 0.6 -> 0.16 ms.
+// Bound by latency (a pass over the blocks, a scan, a ranking), hence several groups per CTA where there are that many
+// problems.  65536 segments in 256 heads: 91 us beside the scorer with a search per head for each of the 64 bits of (gain,
+// k, hid) over expanded segments, 34 us with the bits of the gain over block lists, and about that now; 2970 problems of
+// 256 x 4000 segments 0.6 ms, 0.12 ms, 0.07 ms now that the first split is shared.
 // blockIdx.y selects one of several independent curve sets (the calibration queries of the offline profile, which
 // share the budgets): set i reads the lists of curves i*N .., writes budgets + i*set.budgets and offsets +
 // i*set.offsets.  The hot path launches one set.
@@ -770,9 +893,9 @@ __global__ void __launch_bounds__(kGreedyMaxThreads) greedy_kernel(HullLists lis
   int* lo = reinterpret_cast<int*>(greedy_smem);     // [N] each, unless ONE
   int* hi = lo + (ONE ? 0 : N);
   int* mid = hi + (ONE ? 0 : N);
-  int* at = mid + (ONE ? 0 : N);                     // [N + 1]
-  int* weights = at + N + 1;                         // [groups][kGreedyCountMax + N]
-  float* s_gain = reinterpret_cast<float*>(weights + groups * (kGreedyCountMax + N));
+  int* at = lo + (ONE ? 0 : (3 * N + 1) & ~1);       // [N + 1]
+  unsigned* bins = reinterpret_cast<unsigned*>(at + ((N + 2) & ~1));  // [groups][kGreedyWords], 8-byte aligned
+  float* s_gain = reinterpret_cast<float*>(bins + groups * kGreedyWords);
   unsigned short* s_start = reinterpret_cast<unsigned short*>(s_gain + cap + N);
 
   const int tid = threadIdx.x, nthr = blockDim.x, G1 = P - 1;
@@ -814,10 +937,20 @@ __global__ void __launch_bounds__(kGreedyMaxThreads) greedy_kernel(HullLists lis
   }
   const ListView<true> in_smem = {s_gain, s_start, at, nullptr, G1};
   const ListView<false> in_place = {lists.gain + curve0 * G1, lists.start + curve0 * G1, nullptr, count, G1};
-  int* weight = weights + mine * (kGreedyCountMax + N);
+  unsigned* my_bins = bins + mine * kGreedyWords;
+  FirstSplit first = {nullptr, 0u, 0u};
+  if (staged && args.uniform && args.count > (int)(gridDim.x * groups)) {  // a group takes several problems of one grid
+    __shared__ unsigned first_bins[kGreedyBins + 1];
+    gain_range(in_smem, N, all, shared[0], first.from, first.to);
+    const int T = args.T[0], n = T - w;
+    if (first.from <= first.to)
+      bins_at_least(in_smem, N, T / G1, n, args.floor_tok[0], first.from, first.to, all, shared[0], first_bins);
+    first.bins = first_bins;
+    __syncthreads();  // the groups go their own ways
+  }
   for (int i = blockIdx.x * groups + mine; i < args.count; i += gridDim.x * groups) {
-    if (staged) greedy_problem<true, ONE>(in_smem, args, i, N, w, lo, hi, mid, weight, sh, grp, budgets, offsets);
-    else greedy_problem<false, ONE>(in_place, args, i, N, w, lo, hi, mid, weight, sh, grp, budgets, offsets);
+    if (staged) greedy_problem<true, ONE>(in_smem, args, i, N, w, lo, hi, mid, my_bins, sh, first, grp, budgets, offsets);
+    else greedy_problem<false, ONE>(in_place, args, i, N, w, lo, hi, mid, my_bins, sh, first, grp, budgets, offsets);
   }
 }
 
@@ -839,7 +972,7 @@ __global__ void __launch_bounds__(32 * kSmallMaxHeads) alloc_small_kernel(const 
   extern __shared__ __align__(16) unsigned char small_smem[];
   __shared__ GreedyShared sh;
   __shared__ int at[kSmallMaxHeads + 1];
-  __shared__ int weight[kGreedyCountMax + kSmallMaxHeads];
+  __shared__ __align__(8) unsigned bins[kGreedyWords];
   float* gain = reinterpret_cast<float*>(small_smem);                              // [N][P], then packed
   unsigned short* start = reinterpret_cast<unsigned short*>(gain + (size_t)N * P);
   pdl_launch_dependents();
@@ -882,7 +1015,7 @@ __global__ void __launch_bounds__(32 * kSmallMaxHeads) alloc_small_kernel(const 
   __syncthreads();
   const ListView<true> lists = {gain, start, at, nullptr, P - 1};
   const Group grp = {(int)threadIdx.x, (int)blockDim.x, 0};
-  greedy_problem<true, true>(lists, args, blockIdx.x, N, w, nullptr, nullptr, nullptr, weight, sh, grp, budgets, offsets);
+  greedy_problem<true, true>(lists, args, blockIdx.x, N, w, nullptr, nullptr, nullptr, bins, sh, FirstSplit{nullptr, 0u, 0u}, grp, budgets, offsets);
   pdl_wait();
 }
 
@@ -897,6 +1030,7 @@ GreedyArgs greedy_args(const Dims& dm, const int64_t* budgets_host, int q0, int 
   }
   args.seq0 = q0;
   args.count = cnt;
+  args.uniform = dm.seq_T == nullptr;
   return args;
 }
 
