@@ -62,6 +62,24 @@ def test_keydiff_many_groups(oracle, monkeypatch, group_mb):
     np.testing.assert_allclose(got, oracle.keydiff(bits(k), w), rtol=0, atol=ATOL)
 
 
+@pytest.mark.parametrize("heads, T, d, dtype", [
+    (66, 16001, 128, torch.bfloat16),   # 11 heads per group, six whole groups: the fewest that are split off
+    (150, 8192, 64, torch.float32),     # short heads, fewer pieces than one warp takes at once; a smaller last group
+    (20, 50001, 128, torch.bfloat16),   # three heads per group, 99 pieces per head: anchors made in quarters
+    (13, 40001, 128, torch.float32),    # two heads per group, the last group is one head
+])
+def test_keydiff_groups_that_stay_in_l2(heads, T, d, dtype):
+    """Enough keys for the library's own choice of groups, against the same formula in fp32."""
+    g = torch.Generator(device="cuda").manual_seed(heads)
+    k = (torch.randn((1, 1, heads, T, d), generator=g, device="cuda") + 0.3).to(dtype)
+    p = lukv.make_params(1, 1, heads, 1, d, T, 1, 1, dtype, 2)
+    got = gpu_keydiff(p, k)[0]
+    unit = torch.nn.functional.normalize(k[0, 0].float(), dim=-1, eps=1e-8)
+    anchor = torch.nn.functional.normalize(unit.mean(dim=1, dtype=torch.float64).float(), dim=-1, eps=1e-8)
+    ref = -(unit * anchor[:, None]).sum(dim=-1)[:, :T - 1]
+    np.testing.assert_allclose(got.cpu().numpy(), ref.cpu().numpy(), rtol=0, atol=ATOL)
+
+
 def test_keydiff_wait_runs_out(monkeypatch):
     """A head whose anchor is never published (a host-side switch of the library drops the publication): the CTAs
     that score it give up after the bounded wait, the call reports LUKV_ERR_TIMEOUT in dev_status, the device stays
