@@ -6,9 +6,9 @@
 //                  blocks of equal gain, steepest first.
 //   greedy_kernel  the marginal-utility greedy, computed as a weighted selection: the greedy
 //                  consumes curve segments in the order (gain desc, k asc, hid asc); the
-//                  kernel finds the gain at which the budget runs out by bisection over the
-//                  bits of the gain (one binary search per head and bit), then the segment
-//                  index and the head among the segments of exactly that gain.
+//                  kernel finds the gain at which the budget runs out (capacities in bins of the
+//                  gain, then a ranking; or bisection over its bits), then the segment index
+//                  and the head among the segments of exactly that gain.
 #include <algorithm>
 
 #include "common.cuh"
