@@ -92,7 +92,7 @@ struct FusedArgs {
   int lse_rows;        // M rounded up to a multiple of 4
   int nheads;
   int item_tiles, items_per_head, tiles_T, tiles_n;
-  int adapt_items, least_tiles;  // host only: let the launcher pick the tiles per item, least_tiles or more
+  int adapt_items;     // host only: let the launcher pick a multiple of item_tiles
   int npad;            // pass 2: query rows rounded up to a multiple of 32 (MMA N and columns read)
   int lag;             // 2..kMaxLag: pass 1 of item k+lag-1 precedes pass 2 of item k
   int l2_hints;        // 1: pass-1 key loads ask L2 to keep the lines, pass-2 loads to drop them first
@@ -637,9 +637,9 @@ cudaError_t launch_fused(const CUtensorMap& qm, const CUtensorMap& km, FusedArgs
     // per-item overhead); measured on 256 heads x 256 tiles and 148 CTAs: 0.89 ms with 8 tiles per item,
     // 0.84 with 16, 0.82 with 32, 0.81 with 64.  The price of large items is that pass 2 no longer finds all its key
     // tiles in L2; the kernel is bound by the exp2 unit, not by HBM, so re-reading part of K costs nothing.
-    int best = args.least_tiles;
+    int best = args.item_tiles;
     double best_cost = 1e30;
-    for (int it = args.least_tiles; it <= 8 * args.item_tiles; it *= 2) {
+    for (int it = args.item_tiles; it <= 8 * args.item_tiles; it *= 2) {
       const long long per_head = (args.tiles_T + it - 1) / it;
       const long long items = (long long)args.nheads * per_head;
       const long long ctas = items < sms ? items : sms;
@@ -691,21 +691,17 @@ void score_test_hooks(uint32_t* spin_limit, int* drop_item) {
   *drop_item = (drop && d >= 0 && d <= (1L << 30)) ? (int)d : -1;
 }
 
-// Key tiles per work item (the smallest the scorer uses; it grows for very long contexts).
+// Key tiles per work item (the smallest the scorer uses; it grows for very long contexts).  Items of two tiles where eight
+// leave SMs without one are faster (8 heads x 8192 keys: 17.3 us instead of 23.4), but a row's sum is then added up in
+// another order, which changes the last bits of the scores and so, where two scores nearly tie, the kept positions.
 // LUKV_ITEM_TILES (1..64) overrides the default for tuning runs.
 int score_item_tiles() {
   static const int v = env_int("LUKV_ITEM_TILES", 1, 64, 8);
   return v;
 }
-// The smallest work item the launcher may choose: two tiles where eight would leave SMs without an item.
-int score_min_item_tiles(const Dims& dm) {
-  const long long tiles = dm.heads() * (long long)((dm.T + kTileKeys - 1) / kTileKeys);
-  const int it = score_item_tiles();
-  return tiles <= 148LL * it && it > 2 ? 2 : it;
-}
 // Bytes of pass-1 partials the tensor-core scorer may write for these sizes.
 size_t score_tc_stats_bytes(const Dims& dm) {
-  const size_t tiles = ((size_t)dm.T + kTileKeys - 1) / kTileKeys, least = score_min_item_tiles(dm);
+  const size_t tiles = ((size_t)dm.T + kTileKeys - 1) / kTileKeys, least = score_item_tiles();
   return (size_t)dm.heads() * ((tiles + least - 1) / least) * 256 * sizeof(float);
 }
 // Bytes of the block that must be zero at launch: [heads] counters, the status word, then [heads][lse_rows][2] floats.
@@ -749,7 +745,6 @@ cudaError_t launch_score_tc(const Dims& dm, const void* q, const void* k, const 
   args.tiles_T = (dm.T + kTileKeys - 1) / kTileKeys;
   args.item_tiles = score_item_tiles();
   args.adapt_items = getenv("LUKV_ITEM_TILES") ? 0 : 1;
-  args.least_tiles = score_min_item_tiles(dm);
   args.tiles_n = (dm.n + kTileKeys - 1) / kTileKeys;
   args.items_per_head = 0;  // set by the launcher
   args.npad = (dm.M + 31) & ~31;
