@@ -277,6 +277,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) select_kernel(const __grid_con
         k_eq = (int)found[1];
         break;
       }
+      __syncthreads();  // every thread has read sel: the next split writes it
     }
   }
 

@@ -1,0 +1,53 @@
+"""Selection at the branches of its threshold search, bit-exact against the oracle: scores given directly, so that the
+keys around the cut are chosen."""
+import numpy as np
+import pytest
+import torch
+
+from gpu_helpers import gpu_select_gather
+from paper_2602_08585_b200 import lukv
+
+pytestmark = pytest.mark.gpu
+
+
+def _case(S, N, T, w, budgets, n_sink=0):
+    """Parameters, budgets and offsets on the device, K and V (K's first channel tells the position) and the rows."""
+    p = lukv.make_params(S, 1, N, 1, 64, T, w, 1, "bf16", 2, n_sink=n_sink)
+    b = np.asarray(budgets, np.int32).reshape(-1)
+    off = np.concatenate([[0], np.cumsum(b + w)]).astype(np.int32)
+    k = torch.zeros((S, 1, N, T, 64), dtype=torch.bfloat16, device="cuda")
+    k[..., 0] = (torch.arange(T, device="cuda") % 251).to(torch.bfloat16)
+    k[..., 1] = (torch.arange(T, device="cuda") // 251).to(torch.bfloat16)
+    return p, torch.from_numpy(b).cuda(), torch.from_numpy(off).cuda(), off, k, int(off[-1])
+
+
+def _resplit_scores(rng, n, kind):
+    """Signed scores over the whole key range whose cut lies in a bin of more keys than are ranked directly."""
+    x = rng.uniform(-1.0, 1.0, n).astype(np.float32)
+    base = np.float32(0.5).view(np.uint32)
+    dense = rng.permutation(n)[: n * 3 // 4]
+    m = dense.size
+    if kind == "one":       # distinct keys, 16 apart: a second split leaves a few per bin
+        bits = base + 16 * np.arange(m, dtype=np.uint32)
+    elif kind == "two":     # runs of 700 equal keys in neighbouring key values: down to bins of one key value
+        bits = base + (np.arange(m, dtype=np.uint32) // 700)
+    else:                   # one value
+        bits = np.full(m, base, np.uint32)
+    x[dense] = bits.astype(np.uint32).view(np.float32)
+    return x
+
+
+@pytest.mark.parametrize("kind", ["one", "two", "tied"])
+@pytest.mark.parametrize("n", [3001, 7000, 16000, 32700, 60001, 120000, 250000])
+def test_cut_in_a_bin_that_is_split_again(oracle, n, kind):
+    rng = np.random.default_rng(n)
+    w, heads = 4, 6
+    scores = np.stack([_resplit_scores(rng, n, kind) for _ in range(heads)])
+    budgets = [n // 8, n // 4, n // 2, n * 3 // 4, 1, n - 1]
+    p, b, o, off, k, rows = _case(1, heads, n + w, w, budgets, n_sink=3)
+    _, _, kept = gpu_select_gather(p, torch.from_numpy(scores).cuda(), b, o, k, k, rows)
+    kept = kept.cpu().numpy()
+    for h in range(heads):
+        got = kept[off[h]:off[h + 1]]
+        np.testing.assert_array_equal(got[:budgets[h]], oracle.select(scores[h], budgets[h], 3))
+        np.testing.assert_array_equal(got[budgets[h]:], np.arange(n, n + w))
