@@ -574,15 +574,14 @@ __global__ void __launch_bounds__(kGatherThreads, 4) gather_kernel(const int32_t
 template <int LPR>
 cudaError_t launch_gather_t(const Dims& dm, const int32_t* offsets, const int32_t* kept_idx, const void* k, const void* v,
                             void* k_out, void* v_out, long long rows_cap, bool overlap, cudaStream_t st) {
-  // the row count is only known on the device; size the grid for the capacity
-  // (a capacity beyond what the call can ever produce sizes nothing: clamp it first)
-  const long long rows_max = (long long)dm.heads() * dm.T;
-  if (rows_cap > rows_max) rows_cap = rows_max;
+  // the row count is only known on the device; size the grid for the capacity, or for what these heads can hold where that
+  // is less (the kernel gets the capacity itself: a slice of a larger call's offsets starts beyond these heads' own rows)
+  const long long rows_max = (long long)dm.heads() * dm.T, rows_grid = rows_cap < rows_max ? rows_cap : rows_max;
   // one round of copies per warp (4 to 16 rows) unless that makes more warps than the chip holds
   constexpr int kOneRound = (32 / LPR) * (LPR < 4 ? LPR : 4);
-  const bool full = rows_cap > 148LL * 64 * kOneRound;
+  const bool full = rows_grid > 148LL * 64 * kOneRound;
   const int span = full ? 32 : kOneRound;
-  const long long spans = (rows_cap + span - 1) / span + 1;
+  const long long spans = (rows_grid + span - 1) / span + 1;
   long long blocks = (spans + kGatherThreads / 32 - 1) / (kGatherThreads / 32);
   const long long max_blocks = 148LL * 8 * 4;  // a few waves of resident CTAs; the loop covers the rest
   if (blocks > max_blocks) blocks = max_blocks;

@@ -51,3 +51,30 @@ def test_cut_in_a_bin_that_is_split_again(oracle, n, kind):
         got = kept[off[h]:off[h + 1]]
         np.testing.assert_array_equal(got[:budgets[h]], oracle.select(scores[h], budgets[h], 3))
         np.testing.assert_array_equal(got[budgets[h]:], np.arange(n, n + w))
+
+
+@pytest.mark.parametrize("d,dtype,T", [(64, "bf16", 600), (128, "bf16", 2064), (128, "fp32", 600), (64, "bf16", 100016)])
+def test_slices_of_a_larger_calls_offsets(d, dtype, T):
+    """Layer by layer on slices of one allocation's budgets and offsets, into outputs of the whole: from the third layer on
+    the slice's rows lie beyond the rows that its own heads could fill."""
+    L, H, w = 8, 2, 16
+    n = T - w
+    g = torch.Generator(device="cuda").manual_seed(T)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    k, v = (torch.randn((1, L, H, T, d), generator=g, device="cuda").to(dt) for _ in range(2))
+    scores = torch.randn((1, L * H, n), generator=g, device="cuda")
+    budgets = torch.from_numpy((n // 2 + 5 * np.arange(L * H)).astype(np.int32)).cuda()
+    offsets = torch.cat([torch.zeros(1, dtype=torch.int32, device="cuda"), torch.cumsum(budgets + w, 0).to(torch.int32)])
+    rows = int(offsets[-1])
+    whole = gpu_select_gather(lukv.make_params(1, L, H, 1, d, T, w, 1, dtype, 2), scores, budgets, offsets, k, v, rows)
+    assert rows > 3 * H * T
+    p = lukv.make_params(1, 1, H, 1, d, T, w, 1, dtype, 2)
+    ws = lukv.alloc_workspace(p)
+    k_out, v_out = (torch.zeros((rows, d), dtype=dt, device="cuda") for _ in range(2))
+    kept = torch.full((rows,), -1, dtype=torch.int32, device="cuda")
+    for layer in range(L):
+        lukv.lukv_select_gather(p, scores[0, layer * H:], budgets[layer * H:], offsets[layer * H:], k[0, layer], v[0, layer],
+                                k_out, v_out, kept, rows, ws)
+    torch.cuda.synchronize()
+    for got, want in zip((k_out, v_out, kept), whole):
+        assert torch.equal(got, want)
