@@ -143,7 +143,8 @@ __global__ void __launch_bounds__(kSelThreads, 1) select_kernel(const __grid_con
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int j = 4 * (quad0 + 32 * e) + i;
-        key[4 * e + i] = j >= n ? 0u : j < a.n_sink ? 0xFFFFFFFFu : score_key(y[i]);
+        // scored positions keep off the two marks, whatever the score (a NaN may be either): a head emits b rows
+        key[4 * e + i] = j >= n ? 0u : j < a.n_sink ? 0xFFFFFFFFu : min(max(score_key(y[i]), 1u), 0xFFFFFFFEu);
       }
     }
   }
@@ -223,7 +224,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) select_kernel(const __grid_con
       }
       sync();  // the histograms may be cleared again
       lo += (uint32_t)sel[0] << sh;
-      hi = min(hi, lo + ((1u << sh) - 1u));
+      hi = lo + min(hi - lo, (1u << sh) - 1u);
       want = sel[1];
       const int cnt = sel[2];
       if (sh == 0) {
@@ -316,6 +317,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) select_kernel(const __grid_con
   }
 
   // ---- emit in ascending position: all keys > thr, and the first k_eq keys == thr
+  const int room_b = (int)min(room, (long long)b);
   int run = run_gt + min(run_eq, k_eq);
   // counts per vector of a lane, four vectors to a word (a warp's vector holds at most 128 positions: no carries)
   auto counts = [&](uint32_t bits, int half) {
@@ -364,7 +366,7 @@ __global__ void __launch_bounds__(kSelThreads, 1) select_kernel(const __grid_con
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const bool keep = (kept >> (16 * h + 4 * e + i)) & 1u;
-        if (keep && pos < room) out[pos] = j + i;
+        if (keep && pos < room_b) out[pos] = j + i;
         pos += keep;
       }
       run += (int)((total >> (8 * e)) & 0xFFu);

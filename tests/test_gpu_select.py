@@ -4,8 +4,8 @@ import numpy as np
 import pytest
 import torch
 
-from gpu_helpers import gpu_select_gather
-from paper_2602_08585_b200 import lukv
+from gpu_helpers import gpu_compress, gpu_select_gather, params_of
+from paper_2602_08585_b200 import lukv, synth
 
 pytestmark = pytest.mark.gpu
 
@@ -78,3 +78,54 @@ def test_slices_of_a_larger_calls_offsets(d, dtype, T):
     torch.cuda.synchronize()
     for got, want in zip((k_out, v_out, kept), whole):
         assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("n,n_sink", [(1500, 4), (32700, 0), (60001, 4)])
+@pytest.mark.parametrize("bits,share", [(0x7FFFFFFF, 1.0), (0xFFFFFFFF, 1.0), (0x7FFFFFFF, 0.6), (0xFFFFFFFF, 0.6)])
+def test_scores_that_are_no_numbers_stay_in_their_head(oracle, n, n_sink, bits, share):
+    """A head with NaN scores still fills exactly its own rows (where they rank is left open, but equal ones tie: the lower
+    position first); the heads around it are not touched."""
+    rng = np.random.default_rng(n)
+    w, heads = 8, 5
+    scores = rng.standard_normal((heads, n)).astype(np.float32)
+    budgets = [n // 3, n // 2, n // 3, n - 2, 7]
+    nan_at = rng.random(n) < share
+    for h in (1, 3):
+        scores.view(np.uint32)[h, nan_at] = bits
+    p, b, o, off, k, rows = _case(1, heads, n + w, w, budgets, n_sink=n_sink)
+    _, _, kept = gpu_select_gather(p, torch.from_numpy(scores).cuda(), b, o, k, k, rows)
+    kept = kept.cpu().numpy()
+    for h in range(heads):
+        got, tail = np.split(kept[off[h]:off[h + 1]], [budgets[h]])
+        np.testing.assert_array_equal(tail, np.arange(n, n + w))
+        if h not in (1, 3):
+            np.testing.assert_array_equal(got, oracle.select(scores[h], budgets[h], n_sink))
+            continue
+        assert np.all(np.diff(got) > 0) and got[0] >= 0 and got[-1] < n
+        np.testing.assert_array_equal(got[:n_sink], np.arange(n_sink))
+        for part in (nan_at, ~nan_at):   # of either kind those that rank first
+            at = np.flatnonzero(part[n_sink:]) + n_sink
+            mine = np.intersect1d(got, at)
+            x = scores[h][at] if part is not nan_at else np.zeros(at.size, np.float32)
+            np.testing.assert_array_equal(np.searchsorted(at, mine), oracle.select(x, mine.size))
+
+
+def test_a_query_that_is_no_number_stays_in_its_head():
+    """One NaN in a query spoils all scores of its head: it still fills its own rows with positions in ascending order, and
+    every other head's rows are those of the call without the NaN."""
+    wl = synth.scaled(synth.CONFIGS["llama8b_1layer_8k"], H=4, T=4096, P=65)
+    q, k, v = synth.gen_tensors(wl, "cuda")
+    p, curves, Bs = params_of(wl), synth.gen_curves(wl), wl.budgets()
+    ref = gpu_compress(p, q, k, v, curves, Bs)
+    q[0, 0, 1 * wl.G, 3, 5] = float("nan")
+    out = gpu_compress(p, q, k, v, curves, Bs)
+    off, b = ref.offsets.cpu().numpy(), ref.budgets.cpu().numpy().reshape(-1)
+    assert torch.equal(out.offsets, ref.offsets) and 0 < b[1] < wl.n
+    for h in range(wl.N):
+        rows = slice(int(off[h]), int(off[h + 1]))
+        if h != 1:
+            assert torch.equal(out.kept_idx[rows], ref.kept_idx[rows])
+            assert torch.equal(out.k_out[rows], ref.k_out[rows]) and torch.equal(out.v_out[rows], ref.v_out[rows])
+    got = out.kept_idx[int(off[1]):int(off[2])].cpu().numpy()
+    assert np.all(np.diff(got) > 0) and got[0] >= 0 and got[b[1] - 1] < wl.n
+    np.testing.assert_array_equal(got[b[1]:], np.arange(wl.n, wl.T))
