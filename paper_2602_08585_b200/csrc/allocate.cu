@@ -861,6 +861,8 @@ __device__ __forceinline__ void greedy_problem(const ListView<STAGED> lists, con
 
 // Shared memory of the greedy kernel: at [N+1], the groups' bins, gain and start [cap + N] when lists are staged;
 // lo, hi, mid [N] when a thread owns several heads.
+// The largest head count must leave room for the static arrays of the form with several heads per thread.
+static_assert(sizeof(GreedyShared) + (kGreedyBins + 1) * 4 + 64 + kGreedyMaxHeads * 12 + 4 <= 227 * 1024, "kGreedyMaxHeads");
 inline size_t greedy_smem_bytes(int N, int cap, int groups, bool one) {
   const size_t e = (size_t)cap + N, bins = (size_t)groups * kGreedyWords;
   return (cap > 0 ? ((size_t)N + 1) * 4 + e * 4 + ((e * 2 + 3) & ~(size_t)3) + bins * 4 + 4 : 0) +
@@ -885,7 +887,7 @@ __global__ void __launch_bounds__(kGreedyMaxThreads) greedy_kernel(HullLists lis
   extern __shared__ __align__(16) unsigned char greedy_smem[];
   pdl_launch_dependents();
   pdl_wait();  // the lists come from the launch before
-  __shared__ GreedyShared shared[kGreedyMaxGroups];
+  __shared__ GreedyShared shared[ONE ? kGreedyMaxGroups : 1];  // several heads per thread: one group (launch_greedy)
   const int groups = blockDim.x / group;
   const int mine = threadIdx.x / group;
   const Group grp = {(int)threadIdx.x - mine * group, group, mine + 1}, all = {(int)threadIdx.x, (int)blockDim.x, 0};

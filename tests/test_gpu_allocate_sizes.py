@@ -2,8 +2,9 @@
 shared memory, one launch or two, heads per thread, lists staged or in place.  Bit-exact against the oracle."""
 import numpy as np
 import pytest
+import torch
 
-from gpu_helpers import gpu_allocate
+from gpu_helpers import gpu_allocate, gpu_compress
 from paper_2602_08585_b200 import lukv
 
 pytestmark = pytest.mark.gpu
@@ -39,3 +40,32 @@ def test_allocation_at_the_edges(oracle, N, P, kind):
     b_ref, o_ref = oracle.allocate(U, T, w, Bs)
     np.testing.assert_array_equal(b, b_ref)
     np.testing.assert_array_equal(o, o_ref)
+
+
+@pytest.mark.parametrize("N,P", [(18944, 5), (18751, 9)])
+def test_largest_head_counts(oracle, N, P):
+    """As many heads as the greedy's shared memory holds: the allocation, the whole path and the profile build."""
+    rng = np.random.default_rng(N)
+    T, w = 8 * (P - 1), 4
+    U = _curves(rng, N, P, "mixed")
+    most = N * (T - w)
+    Bs = [0, most // 3, most - 1]
+    p = lukv.make_params(len(Bs), N, 1, 1, 64, T, w, 1, "bf16", P)
+    b, o = gpu_allocate(p, U, Bs)
+    b_ref, o_ref = oracle.allocate(U, T, w, Bs)
+    np.testing.assert_array_equal(b, b_ref)
+    np.testing.assert_array_equal(o, o_ref)
+
+    p1 = lukv.make_params(1, N, 1, 1, 64, T, w, 1, "bf16", P)
+    g = torch.Generator(device="cuda").manual_seed(N)
+    q = torch.randn((1, N, 1, w, 64), generator=g, device="cuda").to(torch.bfloat16)
+    k = torch.randn((1, N, 1, T, 64), generator=g, device="cuda").to(torch.bfloat16)
+    out = gpu_compress(p1, q, k, k, U, Bs[1:2])
+    np.testing.assert_array_equal(out.budgets.cpu().numpy(), b_ref[1:2])
+
+    ratios = [0.25, 0.5]
+    curves = np.stack([U, _curves(rng, N, P, "concave")])
+    profile = torch.empty((2, N), device="cuda")
+    ws = torch.empty(lukv.lukv_profile_workspace_bytes(p1, 2, 2), dtype=torch.uint8, device="cuda")
+    lukv.lukv_profile_build(p1, torch.from_numpy(curves).cuda(), 2, ratios, profile, ws)
+    np.testing.assert_array_equal(profile.cpu().numpy(), oracle.profile_build(curves, T, w, ratios))
