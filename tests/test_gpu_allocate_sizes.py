@@ -69,3 +69,20 @@ def test_largest_head_counts(oracle, N, P):
     ws = torch.empty(lukv.lukv_profile_workspace_bytes(p1, 2, 2), dtype=torch.uint8, device="cuda")
     lukv.lukv_profile_build(p1, torch.from_numpy(curves).cuda(), 2, ratios, profile, ws)
     np.testing.assert_array_equal(profile.cpu().numpy(), oracle.profile_build(curves, T, w, ratios))
+
+
+@pytest.mark.parametrize("N,points", [(16, range(417, 513, 8)), (32, range(209, 257, 4)), (33, range(177, 241, 8)),
+                                      (56, (113, 121, 129, 137)), (200, (29, 33, 37, 41))])
+def test_shared_memory_around_48_kilobytes(oracle, N, points):
+    """Curves whose staging, with the kernels' static arrays, comes to just under and just over what a kernel gets without
+    asking."""
+    rng = np.random.default_rng(N)
+    for P in points:
+        T, w = 2 * (P - 1), 2
+        U = _curves(rng, N, P, "mixed")
+        Bs = [N * (T - w) // 3, N * (T - w) - 5]
+        p = lukv.make_params(len(Bs), 1, N, 1, 64, T, w, 1, "bf16", P)
+        b, o = gpu_allocate(p, U, Bs)
+        b_ref, o_ref = oracle.allocate(U, T, w, Bs)
+        np.testing.assert_array_equal(b, b_ref)
+        np.testing.assert_array_equal(o, o_ref)
