@@ -310,6 +310,10 @@ __global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
           umma_commit(bar(P::kBarEmpty, s));     // the stage may be refilled once these MMAs have read it
           umma_commit(bar(P::kBarTFull, buf + kNumBufs * (use & 1)));   // the accumulator is complete
         }
+        // An issuer without a tile in this job (a job of one tile) waits all the same: else it could hand the slot back twice
+        // while the other issuer still works on the job before in it, which would free that job's query tiles, and its
+        // next wait on this barrier would be two phases ahead, which a parity wait reports as complete.
+        if (ok && !have_q) ok = mbar_wait(bar(P::kBarQFull, slot), (jq / P::kQSlots) & 1, abort_flag, a.dev_status, a.spin_limit);
         if (!ok) break;
         umma_commit(bar(P::kBarQEmpty, slot));   // this issuer's share of the job no longer needs the query tiles
         ++jq;
