@@ -136,11 +136,13 @@ def _stream(stream) -> int:
 
 
 def _host_array(values, ctype, dtype):
-    """(what keeps it alive, address) of host values as a C array: a list or tuple of plain ints directly, anything else
-    through numpy."""
-    if type(values) in (list, tuple) and all(type(v) is int for v in values):
-        a = (ctype * len(values))(*values)
-        return a, a
+    """(what keeps it alive, address) of host values as a C array: a list or tuple of plain ints in range directly (ctypes
+    would cut off what does not fit), anything else through numpy, which raises OverflowError."""
+    if type(values) in (list, tuple):
+        most = 1 << (8 * ctypes.sizeof(ctype) - 1)
+        if all(type(v) is int and -most <= v < most for v in values):
+            a = (ctype * len(values))(*values)
+            return a, a
     b = np.ascontiguousarray(np.asarray(values, dtype=dtype))
     return b, b.ctypes.data
 

@@ -154,3 +154,26 @@ def test_deployment_settings_are_validated():
     assert lukv.lukv_score(_p(n_sink=-1), f, f, f, f, check=False) == lukv.ERR_INVALID_ARG
     assert lukv.lukv_score(_p(n_sink=249), f, f, f, f, check=False) == lukv.ERR_INVALID_ARG
     assert lukv.lukv_workspace_bytes(_p(n_sink=4, min_keep=0.01)) == lukv.lukv_workspace_bytes(_p())
+
+
+@pytest.mark.parametrize("as_type", [list, tuple, np.array])
+def test_host_integers_beyond_their_type_raise(as_type):
+    """A budget or context length that its C type cannot hold is an error, not its low bits."""
+    p = _p(S=2)
+    f = _Fake()
+    big = as_type([2 ** 64 + 5, 5]) if as_type is not np.array else np.array([2 ** 64 + 5, 5], dtype=object)
+    lens = as_type([2 ** 32 + 64, 64]) if as_type is not np.array else np.array([2 ** 32 + 64, 64], dtype=object)
+    for call in (lambda: lukv.lukv_allocate(p, f, big, f, f, f, check=False),
+                 lambda: lukv.lukv_allocate_static(p, f, big, f, f, check=False),
+                 lambda: lukv.lukv_compress(p, f, f, f, f, big, f, f, f, f, f, 1 << 30, None, f, check=False),
+                 lambda: lukv.lukv_exact_allocate(p, f, big, f, f, f, f, check=False),
+                 lambda: lukv.lukv_score_ragged(p, lens, f, f, f, f, check=False),
+                 lambda: lukv.lukv_select_gather_ragged(p, lens, f, f, f, f, f, f, f, f, 10, f, check=False),
+                 lambda: lukv.lukv_compress_ragged(p, lens, f, f, f, f, [5, 5], f, f, f, f, f, 1 << 30, None, f, check=False),
+                 lambda: lukv.lukv_profile_budgets_ragged(p, lens, f, [0.0, 1.0], [0.5, 0.5], f, f, check=False)):
+        with pytest.raises(OverflowError):
+            call()
+    # the ends of the ranges still arrive as they are
+    assert lukv.lukv_allocate(p, f, as_type([2 ** 63 - 1, 5]), f, f, f, check=False) == lukv.ERR_BUDGET
+    assert lukv.lukv_allocate(p, f, as_type([-2 ** 63, 5]), f, f, f, check=False) == lukv.ERR_BUDGET
+    assert lukv.lukv_score_ragged(p, as_type([2 ** 31 - 1, 64]), f, f, f, f, check=False) == lukv.ERR_INVALID_ARG
