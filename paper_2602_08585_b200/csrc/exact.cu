@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(kDpThreads, 5) dp_step_kernel(const DpStep a) 
       best[r] = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
     }
     s = (__shfl_sync(0xffffffffu, best[7], 7) - __shfl_sync(0xffffffffu, best[0], 0)) * (1.f / 63.f);
-    if (!(s > 0.f && s < 3e38f)) s = 0.f;
+    if (!(s > 0.f && s < 1e30f)) s = 0.f;  // s times a distance of up to 8192 stays a number
     float neg = -INFINITY;
 #pragma unroll
     for (int r = 0; r < 8; ++r) {

@@ -133,3 +133,18 @@ def test_unsupported_shapes():
     assert lukv.lukv_exact_allocate(p, f, [10], f, f, f, f, check=False) == lukv.ERR_UNSUPPORTED
     p = lukv.make_params(1, 1, 4, 1, 64, 64, 8, 1, "fp32", 65, min_keep=0.1)
     assert lukv.lukv_exact_allocate(p, f, [40], f, f, f, f, check=False) == lukv.ERR_UNSUPPORTED
+
+
+def test_curves_with_jumps_near_the_end_of_fp32():
+    """Jumps of 1e37 to 3e37: a slope over 64 budgets, times the distance to a block, is beyond fp32, and the bound that
+    skips blocks must not take that for "cannot matter"."""
+    T, w = 2400, 16
+    U = np.zeros((3, T + 1), np.float32)
+    U[0, 2230:] = 1.5e37
+    U[1, 2200:] = 1e37
+    U[2, 90:] = 3e37
+    Bs = [2210, 2295, 2300, 4600]
+    b, _, val = gpu_exact(3, T, w, U, Bs)
+    for q, B in enumerate(Bs):
+        ref, best = _recursion(U, B, T - w)
+        assert list(b[q]) == ref and np.float32(val[q]) == best
