@@ -24,6 +24,111 @@ struct HullOut {
   unsigned short* start;
 };
 
+// mean of block 1 <= mean of block 2, where a block's mean is (its curve rise) / (its length) and
+// the rises are differences of two fp32 curve values: decided exactly as the comparison of the two
+// correctly rounded fp64 quotients.  Cheapest first:
+//   fp32 cross products, when they are further apart than fp32 rounding can explain;
+//   their exact values in two words, when both rises are exact in fp32 (neighbouring points of a long curve differ by a few
+//   units in the last place, and ties are common): 24 + 13 bits, which fp64 quotients tell apart if they differ;
+//   fp64 cross products, when they are clearly apart;
+//   the fp64 quotients themselves.
+// (the last two out of line: they are rare, and an fp64 operation costs a warp some 50 clocks)
+// Block 1 rises from u_l1 to u_r1 over len1 points, block 2 from u_l2 to u_r2 over len2.
+__device__ __noinline__ bool mean_le_f64(float u_l1, float u_r1, int len1, float u_l2, float u_r2, int len2) {
+  const double a = __dsub_rn((double)u_r1, (double)u_l1), b = (double)len1;
+  const double c = __dsub_rn((double)u_r2, (double)u_l2), d = (double)len2;
+  const double p1 = __dmul_rn(a, d), p2 = __dmul_rn(c, b);
+  const double diff = __dsub_rn(p1, p2);
+  const double tol = fmax(fabs(p1), fabs(p2)) * 9.094947017729282e-13;  // 2^-40
+  if (diff < -tol) return true;
+  if (diff > tol) return false;
+  return __ddiv_rn(a, b) <= __ddiv_rn(c, d);
+}
+// Whether d = fl(a - b) is a - b exactly: a sufficient condition (Sterbenz: the one at most twice the other).
+__device__ __forceinline__ bool exact_diff(float a, float b, float d) { return fabsf(d) <= fminf(fabsf(a), fabsf(b)); }
+// d1 / n1 <= d2 / n2 for exact rises d and lengths n below 2^13: exact cross products in two words.
+__device__ __forceinline__ bool exact_le(float d1, float n1, float d2, float n2) {
+  const float q1 = d1 * n2, q2 = d2 * n1;
+  return (q1 < q2) | ((q1 == q2) & (fmaf(d1, n2, -q1) <= fmaf(d2, n1, -q2)));  // no branches
+}
+__device__ __forceinline__ bool mean_le(float u_l1, float u_r1, int len1, float u_l2, float u_r2, int len2) {
+  const float d1 = u_r1 - u_l1, d2 = u_r2 - u_l2, n1 = (float)len1, n2 = (float)len2;
+  const float q1 = d1 * n2, q2 = d2 * n1;
+  const float diff = q1 - q2;
+  // each product carries two roundings of 2^-24, the difference one
+  if (fabsf(diff) > 5e-7f * fmaxf(fabsf(q1), fabsf(q2))) return diff < 0.f;
+  if (exact_diff(u_r1, u_l1, d1) && exact_diff(u_r2, u_l2, d2)) return exact_le(d1, n1, d2, n2);
+  return mean_le_f64(u_l1, u_r1, len1, u_l2, u_r2, len2);
+}
+
+// The vertices among cnt points (values us, places is, ascending; the first and the last are ends) in the warp's shared
+// memory: a point on or below the chord of its neighbours is dropped, all of them tested at once, until a pass drops none.
+// In place; returns how many are left, or -1 if that took more than max_passes.
+__device__ __forceinline__ int hull_passes(float* us, unsigned short* is, int cnt, int max_passes, int lane) {
+  const uint32_t lt_mask = (1u << lane) - 1u;
+#pragma unroll 1
+  for (int pass = 0; pass < max_passes; ++pass) {
+    __syncwarp();
+    int out = 0;
+#pragma unroll 1
+    for (int base = 0; base < cnt; base += 32) {
+      // in place: the writes of a turn end before the points that the next one reads, but for the last, unless nothing
+      // was dropped yet, when they write what is there
+      const int i = base + lane, ii = min(i, cnt - 1), il = max(ii - 1, 0), ir = min(ii + 1, cnt - 1);
+      const float um = us[ii], ul = us[il], ur = us[ir];
+      const int km = is[ii], kl = is[il], kr = is[ir];
+      // 2^23 + k as a float: differences of two are the lengths
+      auto place = [](int k) { return __int_as_float(0x4B000000 | k); };
+      const float d1 = um - ul, d2 = ur - um;
+      bool keep;
+      if (__all_sync(0xffffffffu, exact_diff(um, ul, d1) & exact_diff(ur, um, d2)))
+        keep = !exact_le(d1, place(km) - place(kl), d2, place(kr) - place(km));
+      else
+        keep = !mean_le(ul, um, km - kl, um, ur, kr - km);
+      keep = (i < cnt) & ((i == 0) | (i == cnt - 1) | keep);
+      const uint32_t kept = __ballot_sync(0xffffffffu, keep);
+      if (keep) {
+        const int at = out + __popc(kept & lt_mask);
+        us[at] = um;
+        is[at] = (unsigned short)km;
+      }
+      out += __popc(kept);
+      __syncwarp();
+    }
+    if (out == cnt) return cnt;
+    cnt = out;
+  }
+  return -1;
+}
+
+// The blocks between cnt vertices; the part without a positive slope is one block of gain 0.  The output may be the place
+// of the vertices.  Returns the number of blocks.
+__device__ __forceinline__ int hull_emit(const float* us, const unsigned short* is, int cnt, float* gain, unsigned short* start,
+                                         int lane) {
+  for (int base = 0; base < cnt - 1; base += 32) {
+    const int i = base + lane;
+    const bool block = i < cnt - 1;
+    const float u = block ? us[i] : 0.f, u_next = block ? us[i + 1] : 0.f;
+    const int k = block ? is[i] : 0, k_next = block ? is[i + 1] : 0;
+    const bool rises = block && u_next > u;
+    const int rising = __popc(__ballot_sync(0xffffffffu, rises));  // every lane has read
+    if (block && lane <= rising) {
+      double mean = 0.0;
+      if (rises) mean = __ddiv_rn(__dsub_rn((double)u_next, (double)u), (double)(k_next - k));
+      gain[i] = __double2float_rn(mean);
+      start[i] = (unsigned short)k;
+    }
+    if (rising < 32) return min(base + rising + 1, cnt - 1);  // the rest has no positive slope
+  }
+  return cnt - 1;
+}
+
+// The blocks of cnt points, however many passes it takes (all but the last drop a point).
+__device__ __noinline__ int hull_rest(float* us, unsigned short* is, int cnt, float* gain, unsigned short* start, int lane) {
+  cnt = hull_passes(us, is, cnt, cnt, lane);
+  return hull_emit(us, is, cnt, gain, start, lane);
+}
+
 // A vertex walk: the blocks that pooling adjacent violators ends up with are the edges of the least concave majorant of
 // the points (k, U[k]); from a vertex i the next one is the point j > i with the steepest slope from i, the last of them
 // if several share it.  Slopes are compared in fp32; points whose slopes fp32 cannot tell apart are compared by their
@@ -44,39 +149,46 @@ __device__ __noinline__ int hull_resolve(float uj, int j, float ui, int i) {
   }
   return j;
 }
-// The blocks found so far: lane l holds block 32 (count / 32) + l, its start and the curve there, until 32 are complete
-// or the walk ends.  A gain is an fp64 division, a chain of some 700 clocks: 32 of them at a time, off the walk's chain.
+// Steps of the walk after which the rest of a curve goes to hull_passes.
+constexpr int kHullWalk = 16;
+// The blocks found so far: lane l holds block l, its start and the curve there, until kHullWalk are complete or the walk
+// ends.  A gain is an fp64 division, a chain of some 700 clocks: all of them at a time, off the walk's chain.
 struct HullBlocks {
   int count = 0, start = 0;
   float u = 0.f;
   // the block that starts at point i (value ui) and ends at point `end` (value u_end); gain 0 when `flat`
   __device__ __forceinline__ void add(int i, float ui, int end, float u_end, bool flat, bool last, int lane,
                                       const HullOut& out) {
-    if (lane == (count & 31)) {
+    if (lane == count) {
       start = i;
       u = ui;
     }
-    ++count;
-    if (!last && (count & 31)) return;
-    const int base = (count - 1) & ~31, in = count - base;
+    if (++count < kHullWalk && !last) return;
     int r = __shfl_down_sync(0xffffffffu, start, 1);
     float ur = __shfl_down_sync(0xffffffffu, u, 1);
-    if (lane == in - 1) {
+    if (lane == count - 1) {
       r = end;
       ur = u_end;
     }
-    if (lane < in) {
+    if (lane < count) {
       double mean = __ddiv_rn(__dsub_rn((double)ur, (double)u), (double)(r - start));
-      if (!(mean > 0.0) || (flat && lane == in - 1)) mean = 0.0;
-      out.gain[base + lane] = __double2float_rn(mean);
-      out.start[base + lane] = (unsigned short)start;
+      if (!(mean > 0.0) || (flat && lane == count - 1)) mean = 0.0;
+      out.gain[lane] = __double2float_rn(mean);
+      out.start[lane] = (unsigned short)start;
     }
   }
 };
 
-// P <= 32 NT: every point in a register, all slopes of a step at once, no branches: about 300 clocks a step.
+// P <= 32 NT: every point in a register, all slopes of a step at once, no branches: 300 to 1000 clocks a step, growing with
+// NT.  A curve of many vertices takes that many steps, while passes over its points in shared memory drop few of them and
+// end early (one pass if it is concave, some 8 if it is noisy; a step costs as much as two to ten vectors of a pass).  So
+// the first kHullWalk vertices are walked to, which is all there are on most rough curves (6 of 257 points on the
+// benchmark's), and what is left goes to hull_rest.  us, is: P - kHullWalk entries of the warp's shared memory, may be
+// out.gain + kHullWalk and out.start + kHullWalk.  Whole allocation of 8 concave curves of 513 points: 263 us as a walk
+// alone, 29 us now (rough ones 23); 256 of 513 points 386 and 73 us, 256 of 257 points 105 and 61 us.
 template <int NT>
-__device__ __forceinline__ int hull_walk_regs(const float* __restrict__ U, int P, int lane, HullOut out) {
+__device__ __forceinline__ int hull_walk_regs(const float* __restrict__ U, int P, int lane, HullOut out, float* us,
+                                              unsigned short* is) {
   float u[NT];
 #pragma unroll
   for (int t = 0; t < NT; ++t) u[t] = lane + 32 * t < P ? __ldg(U + lane + 32 * t) : -INFINITY;
@@ -84,7 +196,7 @@ __device__ __forceinline__ int hull_walk_regs(const float* __restrict__ U, int P
   int i = 0;
   HullBlocks blocks;
 #pragma unroll 1
-  while (i < P - 1) {
+  while (i < P - 1 && blocks.count < kHullWalk) {
     float sl[NT], best = -INFINITY;
 #pragma unroll
     for (int t = 0; t < NT; ++t) {
@@ -133,47 +245,17 @@ __device__ __forceinline__ int hull_walk_regs(const float* __restrict__ U, int P
     ui = u_next;
     i = next;
   }
-  return blocks.count;
+  if (i == P - 1) return blocks.count;
+#pragma unroll
+  for (int t = 0; t < NT; ++t)
+    if (lane + 32 * t >= i && lane + 32 * t < P) {
+      us[lane + 32 * t - i] = u[t];
+      is[lane + 32 * t - i] = (unsigned short)(lane + 32 * t);
+    }
+  return kHullWalk + hull_rest(us, is, P - i, out.gain + kHullWalk, out.start + kHullWalk, lane);
 }
 
 // ---- long curves: drop the points that lie on or below the chord of their neighbours, until none does ----------------
-
-// mean of block 1 <= mean of block 2, where a block's mean is (its curve rise) / (its length) and
-// the rises are differences of two fp32 curve values: decided exactly as the comparison of the two
-// correctly rounded fp64 quotients.  Cheapest first:
-//   fp32 cross products, when they are further apart than fp32 rounding can explain;
-//   their exact values in two words, when both rises are exact in fp32 (neighbouring points of a long curve differ by a few
-//   units in the last place, and ties are common): 24 + 13 bits, which fp64 quotients tell apart if they differ;
-//   fp64 cross products, when they are clearly apart;
-//   the fp64 quotients themselves.
-// (the last two out of line: they are rare, and an fp64 operation costs a warp some 50 clocks)
-// Block 1 rises from u_l1 to u_r1 over len1 points, block 2 from u_l2 to u_r2 over len2.
-__device__ __noinline__ bool mean_le_f64(float u_l1, float u_r1, int len1, float u_l2, float u_r2, int len2) {
-  const double a = __dsub_rn((double)u_r1, (double)u_l1), b = (double)len1;
-  const double c = __dsub_rn((double)u_r2, (double)u_l2), d = (double)len2;
-  const double p1 = __dmul_rn(a, d), p2 = __dmul_rn(c, b);
-  const double diff = __dsub_rn(p1, p2);
-  const double tol = fmax(fabs(p1), fabs(p2)) * 9.094947017729282e-13;  // 2^-40
-  if (diff < -tol) return true;
-  if (diff > tol) return false;
-  return __ddiv_rn(a, b) <= __ddiv_rn(c, d);
-}
-// Whether d = fl(a - b) is a - b exactly: a sufficient condition (Sterbenz: the one at most twice the other).
-__device__ __forceinline__ bool exact_diff(float a, float b, float d) { return fabsf(d) <= fminf(fabsf(a), fabsf(b)); }
-// d1 / n1 <= d2 / n2 for exact rises d and lengths n below 2^13: exact cross products in two words.
-__device__ __forceinline__ bool exact_le(float d1, float n1, float d2, float n2) {
-  const float q1 = d1 * n2, q2 = d2 * n1;
-  return (q1 < q2) | ((q1 == q2) & (fmaf(d1, n2, -q1) <= fmaf(d2, n1, -q2)));  // no branches
-}
-__device__ __forceinline__ bool mean_le(float u_l1, float u_r1, int len1, float u_l2, float u_r2, int len2) {
-  const float d1 = u_r1 - u_l1, d2 = u_r2 - u_l2, n1 = (float)len1, n2 = (float)len2;
-  const float q1 = d1 * n2, q2 = d2 * n1;
-  const float diff = q1 - q2;
-  // each product carries two roundings of 2^-24, the difference one
-  if (fabsf(diff) > 5e-7f * fmaxf(fabsf(q1), fabsf(q2))) return diff < 0.f;
-  if (exact_diff(u_r1, u_l1, d1) && exact_diff(u_r2, u_l2, d2)) return exact_le(d1, n1, d2, n2);
-  return mean_le_f64(u_l1, u_r1, len1, u_l2, u_r2, len2);
-}
 
 // Survivors of the first pass that the shared memory of a curve holds; a fifth of the points of a noisy curve survive.
 inline int hull_prune_cap(int P) { return (P * 2 / 5 + 63) & ~63; }
@@ -242,60 +324,9 @@ __global__ void __launch_bounds__(32) hull_prune_kernel(const float* __restrict_
     }
     prev = cur[kAhead - 1];
   }
-  bool done = false;
-  if (cnt <= cap) {
-#pragma unroll 1
-    for (int pass = 0; pass < kHullPasses && !done; ++pass) {
-      __syncwarp();
-      int out = 0;
-#pragma unroll 1
-      for (int base = 0; base < cnt; base += 32) {
-        // in place: the writes of a turn end before the points that the next one reads, but for the last, unless nothing
-        // was dropped yet, when they write what is there
-        const int i = base + lane, ii = min(i, cnt - 1), il = max(ii - 1, 0), ir = min(ii + 1, cnt - 1);
-        const float um = us[ii], ul = us[il], ur = us[ir];
-        const int km = is[ii], kl = is[il], kr = is[ir];
-        // 2^23 + k as a float: differences of two are the lengths
-        auto place = [](int k) { return __int_as_float(0x4B000000 | k); };
-        const float d1 = um - ul, d2 = ur - um;
-        bool keep;
-        if (__all_sync(0xffffffffu, exact_diff(um, ul, d1) & exact_diff(ur, um, d2)))
-          keep = !exact_le(d1, place(km) - place(kl), d2, place(kr) - place(km));
-        else
-          keep = !mean_le(ul, um, km - kl, um, ur, kr - km);
-        keep = (i < cnt) & ((i == 0) | (i == cnt - 1) | keep);
-        const uint32_t kept = __ballot_sync(0xffffffffu, keep);
-        if (keep) {
-          const int at = out + __popc(kept & lt_mask);
-          us[at] = um;
-          is[at] = (unsigned short)km;
-        }
-        out += __popc(kept);
-        __syncwarp();
-      }
-      done = out == cnt;
-      cnt = out;
-    }
-  }
   int total = -1;
-  if (done) {
-    total = 0;
-    float* g_out = lists.gain + (size_t)hid * (P - 1);
-    unsigned short* s_out = lists.start + (size_t)hid * (P - 1);
-    for (int base = 0; base < cnt - 1; base += 32) {
-      const int i = base + lane;
-      const bool block = i < cnt - 1, rises = block && us[i + 1] > us[i];
-      const int rising = __popc(__ballot_sync(0xffffffffu, rises));
-      if (block && lane <= rising) {
-        double mean = 0.0;
-        if (rises) mean = __ddiv_rn(__dsub_rn((double)us[i + 1], (double)us[i]), (double)(is[i + 1] - is[i]));
-        g_out[i] = __double2float_rn(mean);
-        s_out[i] = is[i];
-      }
-      total = min(base + rising + 1, cnt - 1);
-      if (rising < 32) break;  // the rest has no positive slope
-    }
-  }
+  if (cnt <= cap && (cnt = hull_passes(us, is, cnt, kHullPasses, lane)) > 0)
+    total = hull_emit(us, is, cnt, lists.gain + (size_t)hid * (P - 1), lists.start + (size_t)hid * (P - 1), lane);
   if (lane == 0) lists.count[hid] = total;
 }
 
@@ -452,21 +483,23 @@ __global__ void hull_dense_kernel(const float* __restrict__ curves, HullLists li
 
 constexpr int kHullRegsMaxP = 32 * 17;
 
-__device__ __forceinline__ int hull_walk_short(const float* U, int P, int lane, HullOut out) {
-  if (P <= 96) return hull_walk_regs<3>(U, P, lane, out);
-  if (P <= 160) return hull_walk_regs<5>(U, P, lane, out);
-  if (P <= 288) return hull_walk_regs<9>(U, P, lane, out);
-  return hull_walk_regs<17>(U, P, lane, out);
+__device__ __forceinline__ int hull_walk_short(const float* U, int P, int lane, HullOut out, float* us, unsigned short* is) {
+  if (P <= 96) return hull_walk_regs<3>(U, P, lane, out, us, is);
+  if (P <= 160) return hull_walk_regs<5>(U, P, lane, out, us, is);
+  if (P <= 288) return hull_walk_regs<9>(U, P, lane, out, us, is);
+  return hull_walk_regs<17>(U, P, lane, out, us, is);
 }
 
 // One warp (a block of its own) per curve of up to kHullRegsMaxP points.
 // Bound by the latency of a step; a curve has few vertices (6 of 257 points on the benchmark's curves).  256 curves of 257
 // points: 59 us beside the scorer as one serial stack walk per curve, 5 us now.
 __global__ void hull_kernel(const float* __restrict__ curves, HullLists lists, int P) {
+  __shared__ float us[kHullRegsMaxP];
+  __shared__ unsigned short is[kHullRegsMaxP];
   const int hid = blockIdx.x, lane = threadIdx.x;
   const HullOut out = {lists.gain + (size_t)hid * (P - 1), lists.start + (size_t)hid * (P - 1)};
   pdl_launch_dependents();
-  const int count = hull_walk_short(curves + (size_t)hid * P, P, lane, out);
+  const int count = hull_walk_short(curves + (size_t)hid * P, P, lane, out, us, is);
   if (lane == 0) lists.count[hid] = count;
 }
 
@@ -981,7 +1014,8 @@ __global__ void __launch_bounds__(32 * kSmallMaxHeads) alloc_small_kernel(const 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int count = 0;
   if (warp < N) {
-    count = hull_walk_short(curves + (size_t)warp * P, P, lane, HullOut{gain + (size_t)warp * P, start + (size_t)warp * P});
+    const HullOut out = {gain + (size_t)warp * P, start + (size_t)warp * P};
+    count = hull_walk_short(curves + (size_t)warp * P, P, lane, out, out.gain + kHullWalk, out.start + kHullWalk);
     if (lane == 0) {  // the end of the curve
       gain[(size_t)warp * P + count] = 0.f;
       start[(size_t)warp * P + count] = (unsigned short)(P - 1);

@@ -86,3 +86,30 @@ def test_shared_memory_around_48_kilobytes(oracle, N, points):
         b_ref, o_ref = oracle.allocate(U, T, w, Bs)
         np.testing.assert_array_equal(b, b_ref)
         np.testing.assert_array_equal(o, o_ref)
+
+
+@pytest.mark.parametrize("kind", ["concave", "noisy", "hump", "scallops"])
+@pytest.mark.parametrize("N,P", [(8, 18), (8, 65), (32, 129), (4, 257), (8, 513), (5, 544), (40, 257), (33, 513)])
+def test_curves_of_many_vertices(oracle, N, P, kind):
+    """Curves with more vertices than are walked to: the rest goes through passes over its points, in the lists of one
+    launch and of two; `hump` loses its points a few at a time, in dozens of passes."""
+    rng = np.random.default_rng(N + P)
+    t = np.arange(1, P)[None, :]
+    inc = np.exp(-t / (P * rng.uniform(0.2, 1.0, (N, 1))))
+    if kind == "noisy":
+        inc = inc * (1 + 0.1 * rng.standard_normal((N, P - 1)))
+    elif kind == "hump":      # a concave start, then a smooth convex stretch that turns concave
+        inc = np.maximum(3 - 0.1 * t, 0) + np.exp(-((t - 0.6 * P) / (P / 5)) ** 2)
+        inc = inc * rng.uniform(0.5, 2.0, (N, 1))
+    elif kind == "scallops":
+        inc = inc * (1 + 0.5 * np.sin(t / rng.uniform(0.5, 6.0, (N, 1))))
+    U = np.zeros((N, P), np.float32)
+    U[:, 1:] = np.cumsum(inc, axis=1)
+    T, w = 3 * (P - 1), 4
+    most = N * (T - w)
+    Bs = [most // 7, most // 3 + 1, most * 4 // 5]
+    p = lukv.make_params(len(Bs), 1, N, 1, 64, T, w, 1, "bf16", P)
+    b, o = gpu_allocate(p, U, Bs)
+    b_ref, o_ref = oracle.allocate(U, T, w, Bs)
+    np.testing.assert_array_equal(b, b_ref)
+    np.testing.assert_array_equal(o, o_ref)
