@@ -51,13 +51,16 @@ __device__ __forceinline__ bool exact_le(float d1, float n1, float d2, float n2)
   const float q1 = d1 * n2, q2 = d2 * n1;
   return (q1 < q2) | ((q1 == q2) & (fmaf(d1, n2, -q1) <= fmaf(d2, n1, -q2)));  // no branches
 }
+// Rises to or from a curve value of this magnitude, times a length, stay in fp32's range.
+__device__ __forceinline__ bool exact_range(float u) { return fabsf(u) <= 1e34f; }
 __device__ __forceinline__ bool mean_le(float u_l1, float u_r1, int len1, float u_l2, float u_r2, int len2) {
   const float d1 = u_r1 - u_l1, d2 = u_r2 - u_l2, n1 = (float)len1, n2 = (float)len2;
   const float q1 = d1 * n2, q2 = d2 * n1;
   const float diff = q1 - q2;
-  // each product carries two roundings of 2^-24, the difference one
+  // each product carries two roundings of 2^-24, the difference one; false if a product overflowed
   if (fabsf(diff) > 5e-7f * fmaxf(fabsf(q1), fabsf(q2))) return diff < 0.f;
-  if (exact_diff(u_r1, u_l1, d1) && exact_diff(u_r2, u_l2, d2)) return exact_le(d1, n1, d2, n2);
+  if (exact_range(u_l1) && exact_range(u_l2) && exact_diff(u_r1, u_l1, d1) && exact_diff(u_r2, u_l2, d2))
+    return exact_le(d1, n1, d2, n2);
   return mean_le_f64(u_l1, u_r1, len1, u_l2, u_r2, len2);
 }
 
@@ -81,7 +84,7 @@ __device__ __forceinline__ int hull_passes(float* us, unsigned short* is, int cn
       auto place = [](int k) { return __int_as_float(0x4B000000 | k); };
       const float d1 = um - ul, d2 = ur - um;
       bool keep;
-      if (__all_sync(0xffffffffu, exact_diff(um, ul, d1) & exact_diff(ur, um, d2)))
+      if (__all_sync(0xffffffffu, exact_range(um) & exact_diff(um, ul, d1) & exact_diff(ur, um, d2)))
         keep = !exact_le(d1, place(km) - place(kl), d2, place(kr) - place(km));
       else
         keep = !mean_le(ul, um, km - kl, um, ur, kr - km);
@@ -205,7 +208,7 @@ __device__ __forceinline__ int hull_walk_regs(const float* __restrict__ U, int P
       best = fmaxf(best, sl[t]);
     }
     best = warp_max(best);
-    const float near = best - 2e-6f * fabsf(best);
+    const float near = best * 0.999998f;  // infinite rises tie; if no slope is positive, nothing below matters
     int mine = -1, found = 0;
     float u_mine = 0.f;
 #pragma unroll

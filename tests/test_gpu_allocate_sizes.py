@@ -113,3 +113,23 @@ def test_curves_of_many_vertices(oracle, N, P, kind):
     b_ref, o_ref = oracle.allocate(U, T, w, Bs)
     np.testing.assert_array_equal(b, b_ref)
     np.testing.assert_array_equal(o, o_ref)
+
+
+@pytest.mark.parametrize("exponent", [-105, -90, 90, 112, 117])
+@pytest.mark.parametrize("kind", ["rough", "concave", "mixed"])
+@pytest.mark.parametrize("N,P", [(6, 513), (40, 257), (6, 1025), (3, 4001)])
+def test_curves_far_from_one(oracle, N, P, kind, exponent):
+    """Curves scaled by a power of two that leaves every value and gain a normal number have the budgets of the unscaled
+    curves: fp32 products that overflow or flush to zero decide nothing."""
+    rng = np.random.default_rng(P)
+    U = _curves(rng, N, P, kind)
+    assert U.max() < 2.0 ** 13
+    if exponent > 114:
+        U *= np.float32(2.0 ** -4)    # up to the last factor of four below the largest number
+    T, w = 2 * (P - 1), 2
+    Bs = [N * (T - w) // 9, N * (T - w) // 3, N * (T - w) * 3 // 4]
+    p = lukv.make_params(len(Bs), 1, N, 1, 64, T, w, 1, "bf16", P)
+    b, o = gpu_allocate(p, U * np.float32(2.0 ** exponent), Bs)
+    b_ref, o_ref = oracle.allocate(U, T, w, Bs)
+    np.testing.assert_array_equal(b, b_ref)
+    np.testing.assert_array_equal(o, o_ref)
