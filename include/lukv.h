@@ -382,6 +382,8 @@ LUKV_API int lukv_build_curves(const lukv_params_t* params, const float* scores,
  *   importance  [S][N][n] fp32          out
  *   ws          lukv_importance_workspace_bytes() bytes, 256-byte aligned (value norms and row log-sum-exps)
  * fp32 arithmetic on the inputs as given; params->pool_kernel and curve_points must be valid but are unused.
+ * The tensor-core kernels (bf16) wait with a limit; should a wait run out (it needs the device to be taken away in
+ * mid-kernel), the values that depend on it, or with normalize their whole layers, are NaN.
  */
 LUKV_API int lukv_importance_workspace_bytes(const lukv_params_t* params, int32_t k_max, size_t* bytes /* HOST, out */);
 LUKV_API int lukv_oracle_importance(const lukv_params_t* params, int32_t k_max, int32_t d_model, const void* q_dec,

@@ -180,16 +180,17 @@ size_t keydiff_scratch_bytes(const Dims& dm);
 int* keydiff_status(const Dims& dm, float* scratch);
 cudaError_t launch_keydiff(const Dims& dm, const void* k, float* scores, int stride, float* scratch, int32_t* dev_status,
                            int spare_sms, LaunchCtx& lc);
-// Value norms || v_j W_O^(g) ||_2 of the oracle importance on the tensor cores (bf16): vnorm [heads][G][n].
+// Value norms || v_j W_O^(g) ||_2 of the oracle importance on the tensor cores (bf16): vnorm [heads][G][n].  Here and in
+// the attention part a bounded wait that runs out stores LUKV_ERR_TIMEOUT to status.
 bool value_norm_tc_supported(const Dims& dm);
-cudaError_t launch_value_norm_tc(const Dims& dm, int d_model, const void* v, const void* w_o, float* vnorm,
+cudaError_t launch_value_norm_tc(const Dims& dm, int d_model, const void* v, const void* w_o, float* vnorm, int32_t* status,
                                  LaunchCtx& lc);
 // Attention part of the oracle importance on the tensor cores (bf16, up to 8 query heads per KV head): needs the value
 // norms, leaves the un-normalised importance; part: importance_tc_part_bytes() of scratch.
 bool importance_tc_supported(const Dims& dm, int k_max);
 size_t importance_tc_part_bytes(const Dims& dm, int k_max);
 cudaError_t launch_importance_tc(const Dims& dm, int k_max, const void* q_dec, const void* k, const void* k_dec,
-                                 const float* vnorm, float* part, float* importance, LaunchCtx& lc);
+                                 const float* vnorm, float* part, float* importance, int32_t* status, LaunchCtx& lc);
 // Oracle importance of Sec. 4.1 from decode queries, the cache and the output projection.
 size_t importance_workspace_bytes(const Dims& dm, int k_max);
 cudaError_t launch_importance(const Dims& dm, int k_max, int d_model, const void* q_dec, const void* k, const void* v,

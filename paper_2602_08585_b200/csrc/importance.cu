@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(kSimtThreads) imp_lse_kernel(const TIn* __rest
 template <typename TIn, int D>
 __global__ void __launch_bounds__(kSimtThreads) imp_kernel(const TIn* __restrict__ q_dec, const TIn* __restrict__ k,
                                                            const float* __restrict__ lse, const float* __restrict__ vnorm,
-                                                           float* __restrict__ importance, ImpDims dm) {
+                                                           float* __restrict__ importance, ImpDims dm, const int32_t* status) {
   constexpr int kPitch = D + 4;
   extern __shared__ __align__(16) float smem[];
   float* Qs = smem;
@@ -221,6 +221,8 @@ __global__ void __launch_bounds__(kSimtThreads) imp_kernel(const TIn* __restrict
     float m = colmax[0][tid];
 #pragma unroll
     for (int r = 1; r < 16; ++r) m = fmaxf(m, colmax[r][tid]);
+    // a wait of the value norms' kernel ran out: they are not to be used
+    if (status && *status != 0) m = __int_as_float(0x7FC00000);
     importance[(size_t)u * dm.n + j0 + tid] = m;
   }
 }
@@ -243,7 +245,7 @@ __global__ void __launch_bounds__(1024) imp_normalize_kernel(float* __restrict__
   }
   __syncthreads();
   const double total = total_s;
-  if (!(total > 0.0)) return;
+  if (total <= 0.0) return;  // (not a number: the whole layer is none)
   for (long long i = threadIdx.x; i < count; i += blockDim.x) base[i] = (float)((double)base[i] / total);
 }
 
@@ -256,7 +258,7 @@ bool value_norm_force_simt() {
 template <typename TIn, int D>
 cudaError_t launch_importance_t(const Dims& dm, ImpDims id, const void* q_dec, const void* k, const void* v,
                                 const void* k_dec, const void* w_o, bool normalize, float* importance, float* vnorm,
-                                float* lse, LaunchCtx& lc) {
+                                float* lse, int32_t* status, LaunchCtx& lc) {
   const size_t smem = (size_t)2 * kTile * (D + 4) * sizeof(float);
   cudaError_t e;
   auto kn = value_norm_kernel<TIn, D>;
@@ -267,20 +269,21 @@ cudaError_t launch_importance_t(const Dims& dm, ImpDims id, const void* q_dec, c
   if ((e = allow_smem((const void*)ki, smem)) != cudaSuccess) return e;
   const unsigned heads = (unsigned)dm.heads();
   const unsigned pos_tiles = (unsigned)((dm.n + kTile - 1) / kTile);
-  if (value_norm_tc_supported(dm) && !value_norm_force_simt()) {
-    if ((e = launch_value_norm_tc(dm, id.Dm, v, w_o, vnorm, lc)) != cudaSuccess) return e;
+  const bool norms_tc = value_norm_tc_supported(dm) && !value_norm_force_simt();
+  if (norms_tc) {
+    if ((e = launch_value_norm_tc(dm, id.Dm, v, w_o, vnorm, status, lc)) != cudaSuccess) return e;
   } else {
     kn<<<dim3(heads * id.G, pos_tiles), kSimtThreads, smem, lc.st>>>((const TIn*)v, (const TIn*)w_o, vnorm, id);
     lc.mark("value_norm");
   }
-  if (importance_tc_supported(dm, id.Kmax) && !value_norm_force_simt()) {
-    if ((e = launch_importance_tc(dm, id.Kmax, q_dec, k, k_dec, vnorm, lse, importance, lc)) != cudaSuccess) return e;
+  if (norms_tc && importance_tc_supported(dm, id.Kmax)) {
+    if ((e = launch_importance_tc(dm, id.Kmax, q_dec, k, k_dec, vnorm, lse, importance, status, lc)) != cudaSuccess) return e;
   } else {
     kl<<<dim3(heads, (unsigned)((id.Kmax + 15) / 16)), kSimtThreads, smem, lc.st>>>((const TIn*)q_dec, (const TIn*)k,
                                                                                    (const TIn*)k_dec, lse, id);
     lc.mark("imp_lse");
-    ki<<<dim3(heads, pos_tiles), kSimtThreads, smem, lc.st>>>((const TIn*)q_dec, (const TIn*)k, lse, vnorm, importance,
-                                                              id);
+    ki<<<dim3(heads, pos_tiles), kSimtThreads, smem, lc.st>>>((const TIn*)q_dec, (const TIn*)k, lse, vnorm, importance, id,
+                                                              norms_tc ? status : nullptr);
     lc.mark("importance");
   }
   if (normalize) {
@@ -292,12 +295,14 @@ cudaError_t launch_importance_t(const Dims& dm, ImpDims id, const void* q_dec, c
 
 }  // namespace
 
-size_t importance_workspace_bytes(const Dims& dm, int k_max) {
+// value norms, row log-sum-exps (or their partials), the status word
+static size_t importance_status_offset(const Dims& dm, int k_max) {
   const size_t a = ((size_t)dm.heads() * dm.G * dm.n * sizeof(float) + 255) & ~(size_t)255;
   const size_t rows = (size_t)dm.heads() * dm.G * k_max * sizeof(float);  // row log-sum-exps; room for their partials
   const size_t b = (rows + (dm.G <= 8 ? importance_tc_part_bytes(dm, k_max) : 0) + 255) & ~(size_t)255;
   return a + b;
 }
+size_t importance_workspace_bytes(const Dims& dm, int k_max) { return importance_status_offset(dm, k_max) + 256; }
 
 cudaError_t launch_importance(const Dims& dm, int k_max, int d_model, const void* q_dec, const void* k, const void* v,
                               const void* k_dec, const void* w_o, bool normalize, float* importance, void* ws,
@@ -308,14 +313,15 @@ cudaError_t launch_importance(const Dims& dm, int k_max, int d_model, const void
   float* vnorm = static_cast<float*>(ws);
   float* lse = reinterpret_cast<float*>(static_cast<char*>(ws) +
                                         (((size_t)dm.heads() * dm.G * dm.n * sizeof(float) + 255) & ~(size_t)255));
+  int32_t* status = reinterpret_cast<int32_t*>(static_cast<char*>(ws) + importance_status_offset(dm, k_max));
   if (dm.dtype == LUKV_DTYPE_BF16) {
     if (dm.d == 128)
-      return launch_importance_t<__nv_bfloat16, 128>(dm, id, q_dec, k, v, k_dec, w_o, normalize, importance, vnorm, lse, lc);
-    return launch_importance_t<__nv_bfloat16, 64>(dm, id, q_dec, k, v, k_dec, w_o, normalize, importance, vnorm, lse, lc);
+      return launch_importance_t<__nv_bfloat16, 128>(dm, id, q_dec, k, v, k_dec, w_o, normalize, importance, vnorm, lse, status, lc);
+    return launch_importance_t<__nv_bfloat16, 64>(dm, id, q_dec, k, v, k_dec, w_o, normalize, importance, vnorm, lse, status, lc);
   }
   if (dm.d == 128)
-    return launch_importance_t<float, 128>(dm, id, q_dec, k, v, k_dec, w_o, normalize, importance, vnorm, lse, lc);
-  return launch_importance_t<float, 64>(dm, id, q_dec, k, v, k_dec, w_o, normalize, importance, vnorm, lse, lc);
+    return launch_importance_t<float, 128>(dm, id, q_dec, k, v, k_dec, w_o, normalize, importance, vnorm, lse, status, lc);
+  return launch_importance_t<float, 64>(dm, id, q_dec, k, v, k_dec, w_o, normalize, importance, vnorm, lse, status, lc);
 }
 
 }  // namespace lukv

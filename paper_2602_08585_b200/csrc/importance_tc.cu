@@ -9,7 +9,7 @@
 //   imp_tc_kernel       D[key][row] (operands swapped): a thread owns a key and runs over the rows
 // Both are persistent with static items and warp roles: warps 0-7 two epilogue quads that take alternate key tiles out of
 // four accumulator buffers, warp 8 TMA producer, warp 9 tensor memory and MMA issue.  Every wait is bounded and between the
-// warps of one CTA only.
+// warps of one CTA only; should one run out, here or in the value norms, what depends on it becomes NaN.
 // Bound by the exp2 of the epilogue (2 x 2.6e8 for 256 heads x 256 rows x 4000 keys).  Measured there: 1.90 + 1.82 ms
 // on the FP32 pipes, 0.11 + 0.14 ms here.
 #define LUKV_POLY_SEL1(i) false  // every exp2 on the special-function unit: the values keep their precision
@@ -48,6 +48,8 @@ struct ItArgs {
   int items;
   float scale_log2;
   uint32_t spin_limit;
+  int drop_item;      // test hook: the query tiles of this item are never loaded (-1: none)
+  int32_t* status;    // where a wait that ran out is reported
 };
 
 // Both kernels (LSE: the row log-sum-exps): one item is a head, its query tiles (one, or up to two) and a run of key tiles.
@@ -68,7 +70,7 @@ __global__ void __launch_bounds__(kItThreads, 1)
   volatile int* abort_flag = &abort_s;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   auto bar = [&](int kind, int i) { return smem_u32(&bars[kind + i]); };
-  auto wait = [&](uint32_t b, uint32_t parity) { return mbar_wait(b, parity, abort_flag, nullptr, a.spin_limit); };
+  auto wait = [&](uint32_t b, uint32_t parity) { return mbar_wait(b, parity, abort_flag, a.status, a.spin_limit); };
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < kItStages; ++i) {
@@ -91,6 +93,8 @@ __global__ void __launch_bounds__(kItThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_slot;
+  // a wait of the kernels before, or of this one, ran out: their values are not to be used
+  const bool spoiled = !LSE && *reinterpret_cast<volatile int32_t*>(a.status) != 0;
 
   // an item: head u, query tiles [c0, c0 + nq), key tiles [t0, t0 + nt)
   struct Item {
@@ -128,7 +132,7 @@ __global__ void __launch_bounds__(kItThreads, 1)
         const uint32_t slot = jq & 1;
         if (!(ok = wait(bar(kItQEmpty, slot), ((jq >> 1) & 1) ^ 1))) break;
         mbar_expect_tx(bar(kItQFull, slot), it.nq * P::kTile);
-        for (int c = 0; c < it.nq; ++c)
+        for (int c = 0; c < it.nq && idx != a.drop_item; ++c)
           for (int h = 0; h < NH; ++h) {
             const uint32_t dst = smem_u32(smem) + (P::kQPer * slot + c) * P::kTile + h * kHalfBytes;
             asm volatile(
@@ -313,7 +317,7 @@ __global__ void __launch_bounds__(kItThreads, 1)
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(kItTEmpty, buf), 1);
           }
-          if (j < a.n) a.importance[(size_t)it.u * a.n + j] = best;
+          if (j < a.n) a.importance[(size_t)it.u * a.n + j] = ok && !spoiled ? best : __int_as_float(0x7FC00000);
         }
       }
     }
@@ -364,7 +368,7 @@ bool make_query_map(CUtensorMap* map, const void* base, int d, int G, int k_max,
 
 template <int NH>
 cudaError_t launch_importance_tc_t(const Dims& dm, int k_max, const void* q_dec, const void* k, const void* k_dec,
-                                   const float* vnorm, float* part, float* importance, LaunchCtx& lc) {
+                                   const float* vnorm, float* part, float* importance, int32_t* status, LaunchCtx& lc) {
   const int gp_log2 = log2_ceil(dm.G), gp = 1 << gp_log2;
   CUtensorMap qm, km, kdm;
   if (!make_query_map(&qm, q_dec, dm.d, dm.G, k_max, (uint64_t)dm.heads(), gp) ||
@@ -379,8 +383,8 @@ cudaError_t launch_importance_tc_t(const Dims& dm, int k_max, const void* q_dec,
   a.chunks = imp_chunks(dm, k_max);
   a.splits = imp_splits(dm, k_max);
   a.scale_log2 = dm.scale_log2;
-  int drop = 0;
-  score_test_hooks(&a.spin_limit, &drop);
+  a.status = status;
+  score_test_hooks(&a.spin_limit, &a.drop_item);
   int sms = 0;
   cudaError_t e;
   if ((e = device_sms(&sms)) != cudaSuccess) return e;
@@ -422,9 +426,9 @@ size_t importance_tc_part_bytes(const Dims& dm, int k_max) {
 }
 
 cudaError_t launch_importance_tc(const Dims& dm, int k_max, const void* q_dec, const void* k, const void* k_dec,
-                                 const float* vnorm, float* part, float* importance, LaunchCtx& lc) {
-  return dm.d == 128 ? launch_importance_tc_t<2>(dm, k_max, q_dec, k, k_dec, vnorm, part, importance, lc)
-                     : launch_importance_tc_t<1>(dm, k_max, q_dec, k, k_dec, vnorm, part, importance, lc);
+                                 const float* vnorm, float* part, float* importance, int32_t* status, LaunchCtx& lc) {
+  return dm.d == 128 ? launch_importance_tc_t<2>(dm, k_max, q_dec, k, k_dec, vnorm, part, importance, status, lc)
+                     : launch_importance_tc_t<1>(dm, k_max, q_dec, k, k_dec, vnorm, part, importance, status, lc);
 }
 
 }  // namespace lukv

@@ -37,6 +37,7 @@ struct VnArgs {
   int chunks;                // row chunks per (u, g)
   long long items;           // heads * G * chunks
   uint32_t spin_limit;
+  int32_t* status;           // where a wait that ran out is reported
 };
 
 // Writes the panel of output columns [m0, m0 + 256) of one projection slice w [64 NH][Dm] into shared memory as 256
@@ -136,6 +137,8 @@ __global__ void __launch_bounds__(kVnThreads, 1)
       mbar_init(bar(kVnTEmpty, i), 4);
     }
     abort_s = 0;
+    // the first kernel of the call clears the word; a wait runs out milliseconds after this, at the earliest
+    if (blockIdx.x == 0) atomicExch(a.status, 0);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   for (int i = threadIdx.x; i < kVnChunkRows; i += kVnThreads) ssq[i] = 0.f;
@@ -156,7 +159,7 @@ __global__ void __launch_bounds__(kVnThreads, 1)
         for (int cp = 0; cp < npanels && ok; ++cp)
           for (int rt = 0; rt < it.ntiles; ++rt, ++tt) {
             const uint32_t s = tt & 1, ph = (tt >> 1) & 1;
-            if (!(ok = mbar_wait(bar(kVnAEmpty, s), ph ^ 1, abort_flag, nullptr, a.spin_limit))) break;
+            if (!(ok = mbar_wait(bar(kVnAEmpty, s), ph ^ 1, abort_flag, a.status, a.spin_limit))) break;
             mbar_expect_tx(bar(kVnAFull, s), kVnABytes);
             const uint32_t dst = smem_u32(a_tiles + s * kVnABytes);
             const int row = it.u * a.T + it.row0 + rt * kVnRowTile;  // rows past the head are never written back
@@ -174,12 +177,12 @@ __global__ void __launch_bounds__(kVnThreads, 1)
         const VnItem it = vn_item<NH>(a, idx);
         for (int cp = 0; cp < npanels && ok; ++cp, ++pc) {
           const uint32_t pb = pc & 1;
-          if (!(ok = mbar_wait(bar(kVnBFull, pb), (pc >> 1) & 1, abort_flag, nullptr, a.spin_limit))) break;
+          if (!(ok = mbar_wait(bar(kVnBFull, pb), (pc >> 1) & 1, abort_flag, a.status, a.spin_limit))) break;
           const uint32_t bp = smem_u32(panels + pb * kVnBBytes);
           for (int rt = 0; rt < it.ntiles; ++rt, ++tt) {
             const uint32_t s = tt & 1, ph = (tt >> 1) & 1;
-            if (!(ok = mbar_wait(bar(kVnTEmpty, s), ph ^ 1, abort_flag, nullptr, a.spin_limit))) break;
-            if (!(ok = mbar_wait(bar(kVnAFull, s), ph, abort_flag, nullptr, a.spin_limit))) break;
+            if (!(ok = mbar_wait(bar(kVnTEmpty, s), ph ^ 1, abort_flag, a.status, a.spin_limit))) break;
+            if (!(ok = mbar_wait(bar(kVnAFull, s), ph, abort_flag, a.status, a.spin_limit))) break;
             tc_fence_after();
             const uint32_t at = smem_u32(a_tiles + s * kVnABytes);
 #pragma unroll
@@ -207,7 +210,7 @@ __global__ void __launch_bounds__(kVnThreads, 1)
       for (int cp = 0; cp < npanels && ok; ++cp)
         for (int rt = 0; rt < it.ntiles; ++rt, ++tt) {
           const uint32_t s = tt & 1, ph = (tt >> 1) & 1;
-          if (!(ok = mbar_wait(bar(kVnTFull, s), ph, abort_flag, nullptr, a.spin_limit))) break;
+          if (!(ok = mbar_wait(bar(kVnTFull, s), ph, abort_flag, a.status, a.spin_limit))) break;
           tc_fence_after();
           float ss0 = 0.f, ss1 = 0.f, ss2 = 0.f, ss3 = 0.f;
 #pragma unroll 1
@@ -246,7 +249,7 @@ __global__ void __launch_bounds__(kVnThreads, 1)
       const VnItem it = vn_item<NH>(a, idx);
       for (int cp = 0; cp < npanels; ++cp, ++pc) {
         const uint32_t pb = pc & 1;
-        if (!(ok = mbar_wait(bar(kVnBEmpty, pb), ((pc >> 1) & 1) ^ 1, abort_flag, nullptr, a.spin_limit))) break;
+        if (!(ok = mbar_wait(bar(kVnBEmpty, pb), ((pc >> 1) & 1) ^ 1, abort_flag, a.status, a.spin_limit))) break;
         vn_write_panel<NH>(panels + pb * kVnBBytes, it.w, a.Dm, cp * kVnColTile, t, vec);
         // the MMA reads shared memory through the asynchronous proxy: order these writes before it
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -275,7 +278,7 @@ bool value_norm_tc_supported(const Dims& dm) {
   return dm.dtype == LUKV_DTYPE_BF16 && dm.heads() * (int64_t)dm.T < ((int64_t)1 << 31);
 }
 
-cudaError_t launch_value_norm_tc(const Dims& dm, int d_model, const void* v, const void* w_o, float* vnorm,
+cudaError_t launch_value_norm_tc(const Dims& dm, int d_model, const void* v, const void* w_o, float* vnorm, int32_t* status,
                                  LaunchCtx& lc) {
   CUtensorMap vm;
   if (!make_map(&vm, v, (uint64_t)dm.heads() * dm.T, dm.d)) return cudaErrorNotSupported;
@@ -285,6 +288,7 @@ cudaError_t launch_value_norm_tc(const Dims& dm, int d_model, const void* v, con
   a.L = dm.L, a.H = dm.H, a.G = dm.G, a.T = dm.T, a.n = dm.n, a.Dm = d_model;
   a.chunks = (dm.n + kVnChunkRows - 1) / kVnChunkRows;
   a.items = (long long)dm.heads() * dm.G * a.chunks;
+  a.status = status;
   int drop = 0;
   score_test_hooks(&a.spin_limit, &drop);
   int sms = 0;

@@ -93,6 +93,28 @@ def test_tensor_core_importance_against_fp32_pipes(monkeypatch, S, L, H, G, d, T
     np.testing.assert_allclose(tc, simt, rtol=1e-4, atol=1e-30)
 
 
+@pytest.mark.parametrize("normalize", [False, True])
+def test_a_wait_that_runs_out_leaves_nan(monkeypatch, normalize):
+    """With the test hooks one work item's query tiles are never loaded and the wait limit is short: in the log-sum-exp
+    kernel (item 0) every value depends on it, in the last kernel (item 40, which only that one has) the 128 positions of
+    head 5 do, or with the normalisation their layer.  The next ordinary call gives the bits of a fresh one."""
+    S, L, H, G, d, T, w, Kmax, Dm = 1, 2, 4, 1, 64, 1024, 32, 8, 64
+    q, k, v, kd, wo = _inputs(S, L, H, G, d, T, Kmax, Dm, torch.bfloat16, seed=5)
+    p = lukv.make_params(S, L, H, G, d, T, w, 1, torch.bfloat16, 2)
+    ref = gpu_importance(p, Kmax, Dm, q, k, v, kd, wo, normalize)
+    monkeypatch.setenv("LUKV_TEST_SPIN_LIMIT", "20000")
+    monkeypatch.setenv("LUKV_TEST_DROP_ITEM", "0")
+    assert np.isnan(gpu_importance(p, Kmax, Dm, q, k, v, kd, wo, normalize)).all()
+    monkeypatch.setenv("LUKV_TEST_DROP_ITEM", "40")
+    got = gpu_importance(p, Kmax, Dm, q, k, v, kd, wo, normalize)
+    assert np.isnan(got[0, 5, :128]).all() and (not normalize or np.isnan(got[0, 4:]).all())
+    np.testing.assert_array_equal(got[~np.isnan(got)], ref[~np.isnan(got)])
+    assert not np.isnan(got[0, :4]).any() and (normalize or np.isnan(got).sum() == 128)
+    monkeypatch.delenv("LUKV_TEST_SPIN_LIMIT")
+    monkeypatch.delenv("LUKV_TEST_DROP_ITEM")
+    np.testing.assert_array_equal(gpu_importance(p, Kmax, Dm, q, k, v, kd, wo, normalize), ref)
+
+
 def test_importance_at_the_benchmark_size_sampled_heads(oracle):
     """The size bench.py times (one calibration query of 4000 tokens, 256 KV heads x 4 query heads, 64 decode steps,
     model width 4096; the value norms run on the tensor cores over 1024 work items): two sampled heads against the
