@@ -5,7 +5,6 @@
 
 #include <atomic>
 #include <mutex>
-#include <unordered_map>
 
 #include "common.cuh"
 
@@ -161,13 +160,18 @@ cudaError_t device_sms(int* sms) {
 cudaError_t allow_smem(const void* kernel, size_t bytes) {
   // a kernel may have 48 KB without the attribute, its static arrays (up to 10 KB here) included
   if (bytes <= 32 * 1024) return cudaSuccess;
+  // a fixed table: nothing behind the C entry points allocates host memory that could be refused by an exception
+  constexpr int kKernels = 256;
   static std::mutex mu;
-  static std::unordered_map<const void*, uint64_t> done;  // bit d: set on device d
+  static const void* known[kKernels];
+  static uint64_t done[kKernels];  // bit d: set on device d
+  static int count = 0;
   const int dev = device_index();
   if (dev < 0) return cudaErrorInvalidDevice;
   std::lock_guard<std::mutex> lock(mu);
-  uint64_t& bits = done[kernel];
-  if ((bits >> dev) & 1) return cudaSuccess;
+  int at = 0;
+  while (at < count && known[at] != kernel) ++at;
+  if (at < count && ((done[at] >> dev) & 1)) return cudaSuccess;
   cudaFuncAttributes fa;
   cudaError_t e = cudaFuncGetAttributes(&fa, kernel);
   if (e != cudaSuccess) return e;
@@ -176,7 +180,8 @@ cudaError_t allow_smem(const void* kernel, size_t bytes) {
   if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most - (int)fa.sharedSizeBytes)) !=
       cudaSuccess)
     return e;
-  bits |= 1ull << dev;
+  if (at == count && count < kKernels) known[count++] = kernel;  // beyond the table it is set at every call
+  if (at < count) done[at] |= 1ull << dev;
   return cudaSuccess;
 }
 
