@@ -137,11 +137,12 @@ def test_profile_path_with_floor(oracle):
     assert b_ref.min() >= oracle.floor_tokens(0.02, Tn - 32)
 
 
-def test_layer_by_layer_equals_one_call(oracle):
+@pytest.mark.parametrize("L,keep", [(3, 0.2), (8, 0.4)])   # the deeper one's offsets run past a layer's own heads * T
+def test_layer_by_layer_equals_one_call(oracle, L, keep):
     """A server can compress layer l as soon as its prefill is done: allocation once for the whole model
     (it only needs the curves), then scoring, selection and gather with one-layer parameters on that layer's
     tensors and its slice of the budgets and offsets.  The packed cache is the same as from one call."""
-    wl = synth.scaled(synth.CONFIGS["llama8b_1layer_8k"], L=3, H=2, T=4096, P=65)
+    wl = synth.scaled(synth.CONFIGS["llama8b_1layer_8k"], L=L, H=2, T=4096, P=65, keep=(keep,))
     q, k, v = synth.gen_tensors(wl, "cuda")
     curves = synth.gen_curves(wl)
     Bs = wl.budgets()

@@ -129,3 +129,31 @@ def test_a_query_that_is_no_number_stays_in_its_head():
     got = out.kept_idx[int(off[1]):int(off[2])].cpu().numpy()
     assert np.all(np.diff(got) > 0) and got[0] >= 0 and got[b[1] - 1] < wl.n
     np.testing.assert_array_equal(got[b[1]:], np.arange(wl.n, wl.T))
+
+
+@pytest.mark.parametrize("T,w", [(13, 5), (1024, 16), (1031, 7), (2050, 3), (4090, 9), (8195, 2), (16391, 6), (32774, 6),
+                                 (40003, 4), (100001, 3), (200002, 8), (262145, 2)])
+def test_pooling_inside_the_selection(oracle, T, w):
+    """The whole path pools on the way into the selection (up to nine positions; a separate pass beyond): its kept positions
+    are those of lukv_score, whose pooled scores are exactly the maxima of the un-pooled ones, and the oracle's selection.
+    Every register layout, thread count and cluster size, rows of every remainder modulo 4."""
+    H, G, d, n = 3, 1, 64, T - w
+    g = torch.Generator(device="cuda").manual_seed(T)
+    q = torch.randn((1, 1, H * G, w, d), generator=g, device="cuda")
+    k = torch.randn((1, 1, H, T, d), generator=g, device="cuda")
+    curves = np.array([[0.0, 3.0], [0.0, 2.0], [0.0, 1.0]], np.float32)
+    raw = None
+    for kp in (1, 3, 5, 7, 9, 11):
+        p = lukv.make_params(1, 1, H, G, d, T, w, kp, "fp32", 2, n_sink=min(4, n) if kp in (5, 11) else 0)
+        ws = lukv.alloc_workspace(p)
+        scores = torch.empty((1, H, n), device="cuda")
+        lukv.lukv_score(p, q, k, scores, ws)
+        raw = scores.clone() if raw is None else raw
+        assert torch.equal(scores, torch.nn.functional.max_pool1d(raw, kp, 1, kp // 2))
+        Bs = [n + n // 3]    # one head whole, a third of the next, nothing of the last
+        out = gpu_compress(p, q, k, k, curves, Bs)
+        off, b, kept = out.offsets.cpu().numpy(), out.budgets.cpu().numpy()[0], out.kept_idx.cpu().numpy()
+        for h in range(H):
+            got, tail = np.split(kept[off[h]:off[h + 1]], [b[h]])
+            np.testing.assert_array_equal(got, oracle.select(scores[0, h].cpu().numpy(), int(b[h]), p.n_sink))
+            np.testing.assert_array_equal(tail, np.arange(n, T))
