@@ -418,7 +418,9 @@ def run_ours(args):
 
             e2e_step = e2e_step_layers if layered else e2e_step_one_call
 
-            kept_one_call = out.kept_idx.clone()
+            one_call = [t.clone() for t in (out.k_out, out.v_out, out.kept_idx)]
+            for t in (out.k_out, out.v_out, out.kept_idx):
+                t.zero_()
             e2e_step()
             barrier()
             e0.record()
@@ -427,8 +429,10 @@ def run_ours(args):
             e1.record()
             torch.cuda.synchronize()
             e2e_ms = e0.elapsed_time(e1) / args.e2e_steps
-            assert torch.equal(out.kept_idx, kept_one_call) and torch.equal(host_out[2], kept_one_call.cpu()), \
-                "the end-to-end run did not reproduce the kept positions of the device-resident run"
+            for dev_, host_, ref_ in zip((out.k_out, out.v_out, out.kept_idx), host_out, one_call):
+                assert torch.equal(dev_, ref_) and torch.equal(host_, ref_.cpu()), \
+                    "the end-to-end run did not reproduce the packed rows and positions of the device-resident run"
+            del one_call
             e2e_ms = max_over_ranks(e2e_ms, dist, "cuda")
             e2e = {"value": tokens / (e2e_ms * 1e-3), "unit": UNIT, "ms_per_step": e2e_ms, "steps": args.e2e_steps,
                    "mode": ("per layer: host-to-device copy | lukv_score + lukv_select_gather | device-to-host copy "

@@ -343,7 +343,7 @@ LUKV_API int lukv_profile_budgets_ragged(const lukv_params_t* params, const int3
  * importance mass of its k highest-ranked positions; the curve handed to stage (b) and to the
  * profile build is U sampled every s = T/(P-1) tokens: curves[u][k] = U(min(k*s, n)).
  * The ranking is the selection's (sinks first, score descending, lower position first among
- * equals).  Sums are fp64 in ranking order, each point rounded once to fp32.  With S calibration
+ * equals).  Sums are fp64 prefix sums over the ranking, each point rounded once to fp32.  With S calibration
  * queries as the batch, the output is the [n_queries][N][P] input of lukv_profile_build.
  * The oracle importance (Eq. "oracle_importance") is an input here; lukv_oracle_importance computes it from
  * decode queries, the cache and the output projection.
@@ -351,9 +351,9 @@ LUKV_API int lukv_profile_budgets_ragged(const lukv_params_t* params, const int3
  *   scores      [S][N][n] fp32   proxy scores of the rankable positions (lukv_score)
  *   importance  [S][N][n] fp32   oracle importance of the same positions
  *   curves      [S][N][P] fp32   out; curves[..][0] = 0, non-decreasing for importance >= 0
- * Every position is ranked by counting the positions ahead of it (quadratic in n, no scratch
- * memory), which suits calibration contexts of a few thousand tokens; n beyond about 24,000
- * (8*n + 8*P bytes of shared memory above 200 KiB) returns LUKV_ERR_UNSUPPORTED.
+ * No scratch memory.  Up to 16384 positions are ranked in buckets of similar scores, longer heads by counting the
+ * positions ahead of each (quadratic in n); n beyond about 24,000 (8*n + 8*P bytes of shared memory above 200 KiB)
+ * returns LUKV_ERR_UNSUPPORTED.
  */
 LUKV_API int lukv_build_curves(const lukv_params_t* params, const float* scores, const float* importance,
                                float* curves, void* stream);
@@ -394,8 +394,9 @@ LUKV_API int lukv_oracle_importance(const lukv_params_t* params, int32_t k_max, 
  * Exact allocation (Sec. 4.2, Eq. "combinatorial_optimization": maximise the summed utility over
  * integer budgets with sum b = B on the curves as given, no relaxation; the paper names the exact
  * solver as the comparison point of its relaxation).  A tool for cross-checks, not part of the
- * hot path: the multiple-choice-knapsack recursion over the heads, N*B*n/2 additions in fp32, one
- * launch per head.  Token-resolution curves only (P = T+1, so s = 1), n <= 65535, min_keep = 0;
+ * hot path: the multiple-choice-knapsack recursion over the heads in fp32, one launch per head, up to N*B*n/2
+ * additions (blocks that an upper bound rules out are skipped; the results are those of the full recursion).
+ * Token-resolution curves only (P = T+1, so s = 1), n <= 65535, min_keep = 0;
  * anything else is LUKV_ERR_UNSUPPORTED.
  *
  *   curves      [N][P] fp32          as in lukv_allocate (need not be monotone or concave)
@@ -405,7 +406,7 @@ LUKV_API int lukv_oracle_importance(const lukv_params_t* params, int32_t k_max, 
  *   offsets     [S*N+1] int32        out, as in lukv_allocate
  *   values      [S] fp64             out: the optimum (accumulated in fp32)
  *   ws          lukv_exact_workspace_bytes(params, max_q B_q) bytes, 256-byte aligned:
- *               two fp32 rows of B+1 values and the 16-bit argmax of every (head, budget)
+ *               one fp32 row of B+1 values per head (256 heads, B = 304742: 312 MB) and run maxima
  */
 LUKV_API int lukv_exact_workspace_bytes(const lukv_params_t* params, int64_t max_budget, size_t* bytes /* HOST, out */);
 LUKV_API int lukv_exact_allocate(const lukv_params_t* params, const float* curves, const int64_t* budgets_in,

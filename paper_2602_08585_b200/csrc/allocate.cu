@@ -271,7 +271,8 @@ constexpr int kHullPasses = 48;
 // shared memory and tested against their neighbours, exactly, until none is dropped (9 passes over 1900 points in all, 53
 // stay).  A curve of which more than two fifths survive the first pass, or that needs more than kHullPasses, is left to
 // hull_dense_kernel (count -1).  Blocks beyond the last positive slope are one block of gain 0.
-// Bound by instruction issue.  7680 curves of 4001 points: 3.07 ms as one serial stack walk per curve, 0.31 ms as a walk from
+// Bound by the latency of a warp's own instructions at 21 warps per SM (9600 bytes of shared memory each): 57 % of the issue
+// slots are used.  7680 curves of 4001 points: 3.07 ms as one serial stack walk per curve, 0.31 ms as a walk from
 // vertex to vertex over chunk maxima, 0.22 ms with neighbours alone in the first pass, 0.15 ms now.
 __global__ void __launch_bounds__(32) hull_prune_kernel(const float* __restrict__ curves, HullLists lists, int P, int cap) {
   extern __shared__ float hull_smem[];
@@ -495,7 +496,7 @@ __device__ __forceinline__ int hull_walk_short(const float* U, int P, int lane, 
 
 // One warp (a block of its own) per curve of up to kHullRegsMaxP points.
 // Bound by the latency of a step; a curve has few vertices (6 of 257 points on the benchmark's curves).  256 curves of 257
-// points: 59 us beside the scorer as one serial stack walk per curve, 5 us now.
+// points: 59 us beside the scorer as one serial stack walk per curve, 6 us now (curves of six vertices).
 __global__ void hull_kernel(const float* __restrict__ curves, HullLists lists, int P) {
   __shared__ float us[kHullRegsMaxP];
   __shared__ unsigned short is[kHullRegsMaxP];
@@ -910,7 +911,7 @@ inline size_t greedy_smem_bytes(int N, int cap, int groups, bool one) {
 // curves) and are staged in shared memory once for all sequences of the CTA when they fit, else read through L1.
 // Bound by latency (a pass over the blocks, a scan, a ranking), hence several groups per CTA where there are that many
 // problems.  65536 segments in 256 heads: 91 us beside the scorer with a search per head for each of the 64 bits of (gain,
-// k, hid) over expanded segments, 34 us with the bits of the gain over block lists, and about that now; 2970 problems of
+// k, hid) over expanded segments, 34 us with the bits of the gain over block lists, 16 us now; 2970 problems of
 // 256 x 4000 segments 0.6 ms, 0.12 ms, 0.07 ms now that the first split is shared.
 // blockIdx.y selects one of several independent curve sets (the calibration queries of the offline profile, which
 // share the budgets): set i reads the lists of curves i*N .., writes budgets + i*set.budgets and offsets +

@@ -46,8 +46,8 @@ size_t hull_lists_bytes(int64_t n_curves, int P);
 struct Workspace {
   float* raw;        // [S*N][raw_stride]  un-pooled scores
   float* pooled;     // [S*N][raw_stride]  pooled scores (whole path, where the selection does not pool)
-  float* stats;      // partial (reference, sum-exp) per row: [S*N][chunks][M][2] (FP32-pipe scorer) or
-                     // [S*N][items][256][2] (tensor-core scorer)
+  float* stats;      // partials per row: (reference, sum-exp) [S*N][chunks][M][2] (FP32-pipe scorer) or the
+                     // log-sum-exp [S*N][items][128 or 256] (tensor-core scorer); pieces and anchors (KeyDiff)
   HullLists hull;    // blocks of equal gain of every head's curve
   int* head_flags;   // tensor-core scorer: [S*N] items delivered per head and the status word, then the (lse, tag) rows
   size_t bytes;

@@ -6,7 +6,7 @@
 //                           interpolation between the two neighbouring grid rows), b = floor((1-r)*n).
 //   offsets_scan_kernel     packed-row offsets of the resulting budgets.
 //   profile_lookup_kernel   the two in one launch of one CTA, for calls of up to 8192 heads (launches and their
-//                           gaps are the cost there: 6 us from the first start to the last end as two, 2.5 us as one).
+//                           gaps are the cost there: 6 us from the first start to the last end as two, 4 us as one).
 // All ratio arithmetic is fp64 with explicit round-to-nearest operations (no contraction), because a
 // floor follows it: the integer must not depend on how the compiler fuses the expression.
 #include "common.cuh"

@@ -61,7 +61,7 @@ struct OneArgs {
   int n_stride;
   int32_t* dev_status;
   int M, T, w, n;
-  int nheads;   // heads [head0, head0+nheads) are scored by this launch
+  int nheads;
   int items_per_head, tiles_T, tiles_pad;
   float scale_log2;
   uint32_t spin_limit; // iterations a wait may take
