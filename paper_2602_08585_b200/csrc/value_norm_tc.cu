@@ -1,7 +1,9 @@
 // Value norms of the oracle importance (Sec. 4.1, Eq. "oracle_importance"; App. E: L2 norm of the projected value),
 //   vnorm[u][g][j] = || v[u][j] W_O^(g) ||_2 ,   u a KV head, g one of its G query heads, j a rankable position,
 // on the tensor cores for bf16 inputs.  Per (u, g) this is a dense contraction (n x d) * (d x D_model)
-// followed by a sum of squares over the D_model output columns: 98 % of the flops of the importance computation.
+// followed by a sum of squares over the D_model output columns.  The Gram matrix of the projection (value_norm_gram.cu) needs
+// far fewer operations; this kernel serves narrow projections, few positions, unaligned ones, and the chunks of positions that
+// the other one flags.
 //
 // One persistent kernel, one CTA per SM, work items (u, g, chunk of 4096 positions).  For an item the CTA walks the
 // projection in panels of 256 output columns and, per panel, the chunk's tiles of 128 positions:
@@ -38,6 +40,7 @@ struct VnArgs {
   long long items;           // heads * G * chunks
   uint32_t spin_limit;
   int32_t* status;           // where a wait that ran out is reported
+  const unsigned char* flags;  // [items][128] or null (every item): items without a flag are left as they are
 };
 
 // Writes the panel of output columns [m0, m0 + 256) of one projection slice w [64 NH][Dm] into shared memory as 256
@@ -108,6 +111,15 @@ __device__ __forceinline__ VnItem vn_item(const VnArgs& a, long long idx) {
   it.ntiles = (min(kVnChunkRows, a.n - it.row0) + kVnRowTile - 1) / kVnRowTile;
   const int layer = (it.u / a.H) % a.L, h = it.u % a.H;
   it.w = a.w_o + ((size_t)layer * a.H * a.G + (size_t)h * a.G + it.g) * (64 * NH) * a.Dm;
+  if (a.flags) {
+    const uint4* f = reinterpret_cast<const uint4*>(a.flags + idx * 128);
+    uint32_t any = 0;
+    for (int i = 0; i < (it.ntiles + 3) / 4; ++i) {
+      const uint4 x = f[i];
+      any |= x.x | (4 * i + 1 < it.ntiles ? x.y : 0u) | (4 * i + 2 < it.ntiles ? x.z : 0u) | (4 * i + 3 < it.ntiles ? x.w : 0u);
+    }
+    if (!any) it.ntiles = 0;
+  }
   return it;
 }
 
@@ -127,6 +139,15 @@ __global__ void __launch_bounds__(kVnThreads, 1)
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   auto bar = [&](int kind, int i) { return smem_u32(&bars[kind + i]); };
 
+  pdl_wait();
+  if (a.flags) {  // most often nothing is left to do
+    int any = 0;
+    for (long long k = threadIdx.x; blockIdx.x + (k >> 3) * gridDim.x < a.items; k += kVnThreads) {
+      const uint4 f = reinterpret_cast<const uint4*>(a.flags)[(blockIdx.x + (k >> 3) * gridDim.x) * 8 + (k & 7)];
+      any |= (f.x | f.y | f.z | f.w) != 0;  // entries past a head's last tile hold anything: the items look again
+    }
+    if (!__syncthreads_or(any)) return;
+  }
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) {
       mbar_init(bar(kVnAFull, i), 1);
@@ -138,7 +159,7 @@ __global__ void __launch_bounds__(kVnThreads, 1)
     }
     abort_s = 0;
     // the first kernel of the call clears the word; a wait runs out milliseconds after this, at the earliest
-    if (blockIdx.x == 0) atomicExch(a.status, 0);
+    if (blockIdx.x == 0 && !a.flags) atomicExch(a.status, 0);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   for (int i = threadIdx.x; i < kVnChunkRows; i += kVnThreads) ssq[i] = 0.f;
@@ -156,6 +177,7 @@ __global__ void __launch_bounds__(kVnThreads, 1)
       bool ok = true;
       for (long long idx = blockIdx.x; idx < a.items && ok; idx += gridDim.x) {
         const VnItem it = vn_item<NH>(a, idx);
+        if (it.ntiles == 0) continue;
         for (int cp = 0; cp < npanels && ok; ++cp)
           for (int rt = 0; rt < it.ntiles; ++rt, ++tt) {
             const uint32_t s = tt & 1, ph = (tt >> 1) & 1;
@@ -175,6 +197,7 @@ __global__ void __launch_bounds__(kVnThreads, 1)
       bool ok = true;
       for (long long idx = blockIdx.x; idx < a.items && ok; idx += gridDim.x) {
         const VnItem it = vn_item<NH>(a, idx);
+        if (it.ntiles == 0) continue;
         for (int cp = 0; cp < npanels && ok; ++cp, ++pc) {
           const uint32_t pb = pc & 1;
           if (!(ok = mbar_wait(bar(kVnBFull, pb), (pc >> 1) & 1, abort_flag, a.status, a.spin_limit))) break;
@@ -207,6 +230,7 @@ __global__ void __launch_bounds__(kVnThreads, 1)
     bool ok = true;
     for (long long idx = blockIdx.x; idx < a.items && ok; idx += gridDim.x) {
       const VnItem it = vn_item<NH>(a, idx);
+      if (it.ntiles == 0) continue;
       for (int cp = 0; cp < npanels && ok; ++cp)
         for (int rt = 0; rt < it.ntiles; ++rt, ++tt) {
           const uint32_t s = tt & 1, ph = (tt >> 1) & 1;
@@ -247,6 +271,7 @@ __global__ void __launch_bounds__(kVnThreads, 1)
     bool ok = true;
     for (long long idx = blockIdx.x; idx < a.items && ok; idx += gridDim.x) {
       const VnItem it = vn_item<NH>(a, idx);
+      if (it.ntiles == 0) continue;
       for (int cp = 0; cp < npanels; ++cp, ++pc) {
         const uint32_t pb = pc & 1;
         if (!(ok = mbar_wait(bar(kVnBEmpty, pb), ((pc >> 1) & 1) ^ 1, abort_flag, a.status, a.spin_limit))) break;
@@ -278,8 +303,8 @@ bool value_norm_tc_supported(const Dims& dm) {
   return dm.dtype == LUKV_DTYPE_BF16 && dm.heads() * (int64_t)dm.T < ((int64_t)1 << 31);
 }
 
-cudaError_t launch_value_norm_tc(const Dims& dm, int d_model, const void* v, const void* w_o, float* vnorm, int32_t* status,
-                                 LaunchCtx& lc) {
+cudaError_t launch_value_norm_tc(const Dims& dm, int d_model, const void* v, const void* w_o, float* vnorm,
+                                 const unsigned char* flags, int32_t* status, LaunchCtx& lc) {
   CUtensorMap vm;
   if (!make_map(&vm, v, (uint64_t)dm.heads() * dm.T, dm.d)) return cudaErrorNotSupported;
   VnArgs a;
@@ -289,6 +314,7 @@ cudaError_t launch_value_norm_tc(const Dims& dm, int d_model, const void* v, con
   a.chunks = (dm.n + kVnChunkRows - 1) / kVnChunkRows;
   a.items = (long long)dm.heads() * dm.G * a.chunks;
   a.status = status;
+  a.flags = flags;
   int drop = 0;
   score_test_hooks(&a.spin_limit, &drop);
   int sms = 0;
@@ -298,9 +324,9 @@ cudaError_t launch_value_norm_tc(const Dims& dm, int d_model, const void* v, con
   const int smem = vn_smem(dm.d / 64);
   if ((e = allow_smem((const void*)kern, smem)) != cudaSuccess) return e;
   const long long grid = a.items < sms ? a.items : sms;  // one CTA per SM: each owns the SM's tensor memory
-  kern<<<(unsigned)grid, kVnThreads, smem, lc.st>>>(vm, a);
+  e = launch_pdl(kern, dim3((unsigned)grid), dim3(kVnThreads), smem, lc.st, flags != nullptr, vm, a);
   lc.mark("value_norm_tc");
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace lukv

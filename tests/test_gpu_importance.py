@@ -76,6 +76,34 @@ def test_value_norms_tensor_core_against_fp32_pipes(monkeypatch):
     np.testing.assert_allclose(tc, simt, rtol=2e-5, atol=1e-30)
 
 
+@pytest.mark.parametrize("S,L,H,G,d,T,w,Dm", [
+    (1, 1, 1, 1, 128, 130, 2, 2048),      # one tile, filled to the last position
+    (1, 3, 8, 7, 128, 161, 32, 1032),     # a tile with one position; 168 slices on 148 SMs; a last panel of 8 columns
+    (3, 1, 2, 2, 128, 900, 5, 1096),      # tiles of three sequences shared out over items
+    (2, 1, 3, 5, 64, 4096 + 700, 16, 2056),  # head size 64, two chunks of positions
+])
+@pytest.mark.parametrize("kind", ["normal", "null", "zero", "large"])
+def test_value_norms_through_the_gram_matrix(monkeypatch, kind, S, L, H, G, d, T, w, Dm):
+    """Sizes that take the Gram matrix of the projection against the FP32 pipes, which multiply it out.  Both round sums of
+    exact products to 24 bits.  "null": some values lie where the projection is 1e-4 of its size, their chunks are left to the
+    direct kernel; "zero": zero values and a zero projection; "large": squares beyond fp32's range are left to it as well."""
+    q, k, v, kd, wo = _inputs(S, L, H, G, d, T, 2, Dm, torch.bfloat16, seed=T + Dm)
+    if kind == "null":
+        wo[:, 0, -1] *= 1e-4
+        v[:, :, :, 5::131, :-1] = 0
+    elif kind == "zero":
+        v[:, :, :, ::3] = 0
+        wo[:, -1] = 0
+    elif kind == "large":
+        wo[:, 0] *= 2.0 ** 70
+        v[:, :, 0, ::64] *= 2.0 ** -60
+    p = lukv.make_params(S, L, H, G, d, T, w, 1, torch.bfloat16, 2)
+    gram = gpu_importance(p, 2, Dm, q, k, v, kd, wo, False)
+    monkeypatch.setenv("LUKV_FORCE_SIMT", "1")
+    simt = gpu_importance(p, 2, Dm, q, k, v, kd, wo, False)
+    np.testing.assert_allclose(gram, simt, rtol=2e-5, atol=1e-30)
+
+
 @pytest.mark.parametrize("S,L,H,G,d,T,w,Kmax,Dm,with_kd", [
     (1, 1, 2, 1, 64, 130, 1, 1, 64, True),        # one step, one query head; a key tile with two keys
     (1, 1, 2, 2, 128, 129, 32, 65, 40, True),     # steps just past one query tile; odd panel width
