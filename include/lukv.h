@@ -394,8 +394,9 @@ LUKV_API int lukv_oracle_importance(const lukv_params_t* params, int32_t k_max, 
  * Exact allocation (Sec. 4.2, Eq. "combinatorial_optimization": maximise the summed utility over
  * integer budgets with sum b = B on the curves as given, no relaxation; the paper names the exact
  * solver as the comparison point of its relaxation).  A tool for cross-checks, not part of the
- * hot path: the multiple-choice-knapsack recursion over the heads in fp32, one launch per head, up to N*B*n/2
- * additions (blocks that an upper bound rules out are skipped; the results are those of the full recursion).
+ * hot path: the multiple-choice-knapsack recursion over the heads in fp32, up to N*B*n/2 additions (tokens and
+ * budgets that cannot matter are left out; the results are those of the full recursion).  Should a device-side wait
+ * run out, values[q] is NaN and the budgets of the sequence are zero.
  * Token-resolution curves only (P = T+1, so s = 1), n <= 65535, min_keep = 0;
  * anything else is LUKV_ERR_UNSUPPORTED.
  *
@@ -406,7 +407,8 @@ LUKV_API int lukv_oracle_importance(const lukv_params_t* params, int32_t k_max, 
  *   offsets     [S*N+1] int32        out, as in lukv_allocate
  *   values      [S] fp64             out: the optimum (accumulated in fp32)
  *   ws          lukv_exact_workspace_bytes(params, max_q B_q) bytes, 256-byte aligned:
- *               one fp32 row of B+1 values per head (256 heads, B = 304742: 312 MB) and run maxima
+ *               one fp32 row of B+1 values per head (256 heads, B = 304742: 312 MB), the curves' hulls
+ *               (6 MB) and run maxima
  */
 LUKV_API int lukv_exact_workspace_bytes(const lukv_params_t* params, int64_t max_budget, size_t* bytes /* HOST, out */);
 LUKV_API int lukv_exact_allocate(const lukv_params_t* params, const float* curves, const int64_t* budgets_in,

@@ -2,28 +2,31 @@
 // "combinatorial_optimization"; the paper names the exact solver as the point of comparison for its
 // relaxation): the multiple-choice-knapsack recursion over the heads,
 //     f_h(x) = max over b in [0, min(x, n)] of  f_{h-1}(x - b) + U_h(b),      f_{-1}(0) = 0,
-// at token resolution (curve point b = utility of keeping b tokens).  One launch per head.  Only the states
-// that can still reach sum b = B are evaluated: after head h, x lies in [B - (N-1-h)*n, (h+1)*n].  Every row
-// f_h is kept, and the walk back from x = B looks the choices up again: the smallest b with
-// f_{h-1}(x - b) + U_h(b) == f_h(x), which is the smallest b that attains the maximum.
+// at token resolution (curve point b = utility of keeping b tokens).  Every row f_h is kept, and the walk back from x = B
+// looks the choices up again: the smallest b with f_{h-1}(x - b) + U_h(b) == f_h(x), which is the smallest b that attains the
+// maximum.
 //
-// What bounds it: additions and comparisons (2.2e11 pairs for 256 heads x 3968 tokens at B = 0.3 N n) if every pair is
-// evaluated, then the latency of a step.  Three measures:
-//   - a warp owns 64 budgets and skips every block of 64 values of b that an upper bound rules out: with s the slope of
-//     f_h over its budgets, a pair (y, b) can only matter if (f(y) - s y) + (U(b) - s b) reaches the smallest
-//     f_h(x) - s x found so far, and maxima of f and U over runs of 16 bound the left side (every step leaves the maxima
-//     of its row for the next one).  On utility curves the blocks far from the optimum drop out (6 % are evaluated); on
-//     curves where they do not, everything is evaluated.  The values are those of the full recursion, bit for bit: a
-//     skipped block holds no pair that could raise a maximum;
+// 2.2e11 pairs (x, b) for 256 heads x 3968 tokens at B = 0.3 N n if every one is evaluated.  What is done instead:
+//   - tokens that no optimal solution can contain, and budgets that such tokens cannot add up to, are left out before (see
+//     "which tokens can matter" below): 5 % of the budgets and 6 % of the tokens are left there;
+//   - of those, a warp owns 64 budgets and skips every block of 64 values of b that an upper bound rules out: for any slope s
+//     a pair (y, b) can only matter if (f(y) - s y) + (U(b) - s b) reaches the smallest f_h(x) - s x found so far, and maxima
+//     of f and U over runs of 16 bound the left side; half a block at a time is then bounded by its own values.  Where six
+//     blocks or fewer are left all are evaluated: the bounds would take longer (256 heads, B = 0.05 N n: 891 us with, 784
+//     without);
 //   - in a block, a pair of additions is one packed instruction and two comparisons are one three-input maximum, on a
 //     register tile of 8 budgets x 8 pairs of b per lane; the argmax is not carried along;
-//   - warps share nothing (a block's 128 values of f and 64 of U go through a warp's own shared memory), and a step
-//     starts while the one before it drains.
-// Measured (256 heads x 3968 tokens, B = 304742): 57.2 ms with every pair evaluated one by one and the argmax kept
-// (220 us a head); 3.9 ms now, 13 us a head, of which a warp's 2 to 4 dependent reads of L2 are the larger part, and
-// 0.47 ms for the walk back.  Tried: f and U staged once per CTA (5.4 ms: staging costs more than the few blocks that are
-// left), 32 instead of 20 warps per SM at 64 registers (4.5 ms, spills), three blocks fetched ahead (4.1 ms).
+//   - all rows in one launch: a CTA keeps its part of the row before and the curve in shared memory and polls the values that
+//     others compute themselves, so that a row costs one trip through L2.
+// The values are those of the full recursion wherever its solutions pass, bit for bit.
+// What bounds it now: the latency of a row (2.9 us: store, poll, two barriers and a tile's 2000 to 4000 dependent clocks) and
+// of the walk back (0.6 us a head).  256 heads x 3968 tokens, B = 304742: 57.2 ms with every pair evaluated one by one and the
+// argmax kept; 3.95 ms with bounds and a launch per row; 2.7 + 0.4 ms in one launch over all budgets, its parts signalled by
+// flags; 1.0 ms now, of which the greedy solution takes 0.09, the rows 0.74 and the walk 0.17.  CTAs of at least ten tiles
+// instead of two 1171 us, five 1070; the curve's tokens read from L2 in the walk 1.7 us a head.
 #include <math.h>
+
+#include <algorithm>
 
 #include "common.cuh"
 #include "tc_ptx.cuh"
@@ -31,370 +34,739 @@
 namespace lukv {
 namespace {
 
-constexpr int kDpWarps = 4;
+constexpr int kDpWarps = 20;
 constexpr int kDpThreads = 32 * kDpWarps;
-constexpr int kDpX = 64;                      // budgets per warp; values of b per block
-constexpr int kDpTile = kDpX * kDpWarps;      // budgets per CTA
+constexpr int kDpX = 64;                      // budgets per tile (one warp); values of b per block
 constexpr int kDpMaxBlocks = 64;              // n <= 4095: the curve grid has at most 4097 points
 constexpr int kDpRun = 16;                    // entries per stored maximum
 constexpr int kDpURuns = kDpMaxBlocks * kDpX / kDpRun;  // run maxima per curve
-constexpr int kDpGroup = 80;                  // bytes of 8 packed entries, padded: eight lanes at this stride hit all banks
+constexpr int kDpSub = 96;                    // most tiles whose part of the previous row is staged together
+constexpr int kDpGroup = 80;                  // bytes of 8 packed pairs of f, padded: eight lanes at this stride hit all banks
+constexpr int kDpWindow = 112;                // packed pairs of f that a warp makes of 128 values
+constexpr int kDpUBlock = 2 * 128;            // bytes of a block's 32 packed pairs of U
+constexpr int kDpWindowsPer = ((kDpMaxBlocks + kDpSub) * kDpX / kDpWindow + kDpWarps) / kDpWarps;  // per warp
+constexpr int kDpMinTiles = 2;                // least tiles of a CTA in a row
+constexpr int kDpWords = 2;                   // status, heads that have their tokens
+constexpr int kDpTable = 1024;                // rows whose parts are worked out ahead
+constexpr int kDpFewBlocks = 6;               // blocks of b that are evaluated without bounds
+constexpr uint32_t kDpUnset = 0xFFFFFFFFu;    // a value that is still to come (a NaN that no addition or maximum makes)
 constexpr int kDpBackThreads = 384;
-constexpr int kDpFBytes = 12 * kDpGroup, kDpUBytes = 4 * kDpGroup;
 
 __device__ __forceinline__ float max3(float a, float b, float c) {
   float d;
   asm("max.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
   return d;
 }
-// Maxima of every curve over runs of 16 values of b; -inf beyond n.  One CTA per head.
-__global__ void __launch_bounds__(kDpURuns) dp_runs_kernel(const float* __restrict__ curves, float* __restrict__ runs, int n,
-                                                           int P) {
+// Maxima of every curve over runs of 16 values of b; -inf beyond n.  One CTA per head; the first also clears the words of
+// the next kernel.
+__global__ void __launch_bounds__(kDpURuns) dp_runs_kernel(const float* __restrict__ curves, float* __restrict__ runs,
+                                                           int* __restrict__ words, int n_words, int n, int P) {
   const float* U = curves + (size_t)blockIdx.x * P;
   const int b0 = threadIdx.x * kDpRun;
   float m = -INFINITY;
   for (int b = b0; b < b0 + kDpRun && b <= n; ++b) m = fmaxf(m, __ldg(U + b));
   runs[(size_t)blockIdx.x * kDpURuns + threadIdx.x] = m;
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i < n_words; i += kDpURuns) words[i] = 0;
 }
 
-struct DpStep {
-  const float* U;          // curve of this head
-  const float* u_runs;     // its run maxima
-  const float* prev;       // f_{h-1}, or null for the first head (f = 0 at y = 0)
-  const float* prev_runs;  // maxima of f_{h-1} over runs of 16, for the runs of the tiles that hold [plo, phi]
-  float* next;             // f_h
-  float* next_runs;
-  int lo, hi;              // budgets to evaluate
-  int plo, phi;            // where prev is defined; anything outside counts as -inf
-  int n;
+struct DpArgs {
+  const float* curves;  // [N][P]
+  const float* u_runs;  // [N][kDpURuns]
+  float* f;             // [N][stride]
+  const int4* rows;     // [N] lowest and highest budget of the row, fewest and most tokens of the head
+  int* words;           // [0] the status word
+  long long stride;
+  int P, N, n;
+  uint32_t spin_limit;
+  int drop;             // test hook: this CTA stores nothing (-1: none)
 };
-
-// What a lane fetches of one block: f at y0 + 4 lane .. + 3, U at b0 + lane and b0 + 32 + lane.
-struct DpFetch {
-  float4 f;
-  float u0, u1;
+// Shared memory: the staged part of the previous row as packed pairs and its run maxima; the curve of this head and the
+// next one as packed pairs and their run maxima; the rows' parts.
+struct DpPlan {
+  int blocks, entries, runs_off, u_off, u_bytes, u_runs_off, table_off, total;
 };
-__device__ __forceinline__ DpFetch dp_fetch(const DpStep& a, int x0, int blk, int lane) {
-  DpFetch r;
-  r.f = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-  const int y = x0 - kDpX * (blk + 1) + 4 * lane;  // a multiple of 4, as the rows' start
-  if (y + 3 >= a.plo && y <= a.phi) {
-    const float4 v = a.prev ? *reinterpret_cast<const float4*>(a.prev + y) : make_float4(0.f, 0.f, 0.f, 0.f);
-    if (y >= a.plo) r.f.x = v.x;  // y <= phi here
-    if (y + 1 >= a.plo && y + 1 <= a.phi) r.f.y = v.y;
-    if (y + 2 >= a.plo && y + 2 <= a.phi) r.f.z = v.z;
-    if (y + 3 <= a.phi) r.f.w = v.w;
-  }
-  const int b = kDpX * blk + lane;
-  r.u0 = b <= a.n ? __ldg(a.U + b) : -INFINITY;
-  r.u1 = b + 32 <= a.n ? __ldg(a.U + b + 32) : -INFINITY;
-  return r;
+__host__ __device__ inline DpPlan dp_plan(int n, int N) {
+  DpPlan p;
+  p.blocks = n / kDpX + 1;
+  p.entries = ((p.blocks + kDpSub) * kDpX + kDpWindow - 1) / kDpWindow * kDpWindow;
+  p.runs_off = p.entries / 8 * kDpGroup;
+  p.u_off = p.runs_off + (p.entries + 32) / kDpRun * 4;
+  p.u_off = (p.u_off + 15) & ~15;
+  p.u_bytes = p.blocks * kDpUBlock;
+  p.u_runs_off = p.u_off + 2 * p.u_bytes;
+  p.table_off = p.u_runs_off + 2 * p.blocks * 16;
+  p.total = p.table_off + (N < kDpTable ? N : kDpTable) * 32;
+  return p;
 }
 
-// Stores the fetched block packed for dp_block.  F2: entry j (0..95) = (f(yw + 32 + j), f(yw + j)), yw the first of the
-// block's 128 values of y; U2: entry t (0..31) = (U(b0 + t), U(b0 + 32 + t)); groups of 8 entries at a padded stride.
-__device__ __forceinline__ void dp_store(const DpFetch& r, unsigned char* F2, unsigned char* U2, int lane) {
-  // lane l >= 8 holds the first parts of entries 4 l - 32 .. + 3, lane l - 8 their second parts
-  const float g0 = __shfl_up_sync(0xffffffffu, r.f.x, 8), g1 = __shfl_up_sync(0xffffffffu, r.f.y, 8);
-  const float g2 = __shfl_up_sync(0xffffffffu, r.f.z, 8), g3 = __shfl_up_sync(0xffffffffu, r.f.w, 8);
-  float4* to = reinterpret_cast<float4*>(F2 + ((lane - 8) >> 1) * kDpGroup + (lane & 1) * 32);
-  if (lane >= 8) {
-    to[0] = make_float4(r.f.x, g0, r.f.y, g1);
-    to[1] = make_float4(r.f.z, g2, r.f.w, g3);
-  }
-  *reinterpret_cast<float2*>(U2 + (lane >> 3) * kDpGroup + (lane & 7) * 8) = make_float2(r.u0, r.u1);
+__device__ __forceinline__ void cp_async4(void* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 
-// One block of b for the warp's 64 budgets.  Lane (xg, bg) takes budgets 8 xg .. 8 xg + 7 and, in the two halves of a
-// packed pair, b = 8 bg + t and 8 bg + 32 + t, t < 8: the 16 entries of F2 from group xg - bg + 3 on.
-__device__ __forceinline__ void dp_block(const unsigned char* fw, const unsigned char* ub, float (&blo)[8], float (&bhi)[8]) {
-  // entry 8 + r - t pairs budget r with value t of b; the window slides down as t grows
-  ulonglong2 w[8];  // w[i]: entries 2 i, 2 i + 1
+// 32 values of b for the warp's 64 budgets.  Lane (xg, bg) takes budgets 8 xg .. 8 xg + 7 and, in the two halves of a packed
+// pair, b = 4 bg + t and 4 bg + 16 + t, t < 4.  fw: the pairs of f from y = x0 + 8 xg - 4 bg - 20 on (from b = 0), of which
+// the first four may be the second half of a padded group (odd); ub: the lane's four pairs of U.
+__device__ __forceinline__ void dp_block(const unsigned char* fw, bool odd, const unsigned char* ub, float (&blo)[8],
+                                         float (&bhi)[8]) {
+  const unsigned char* fm = fw + (odd ? 48 : 32);
+  // w[i]: pairs 2 i, 2 i + 1; pair 4 + r - t goes with budget r and value t of b
+  const ulonglong2 w[6] = {*reinterpret_cast<const ulonglong2*>(fw),      *reinterpret_cast<const ulonglong2*>(fw + 16),
+                           *reinterpret_cast<const ulonglong2*>(fm),      *reinterpret_cast<const ulonglong2*>(fm + 16),
+                           *reinterpret_cast<const ulonglong2*>(fw + 80), *reinterpret_cast<const ulonglong2*>(fw + 96)};
 #pragma unroll
-  for (int i = 3; i < 8; ++i)
-    w[i] = *reinterpret_cast<const ulonglong2*>(fw + (i >> 2) * kDpGroup + (i & 3) * 16);
-#pragma unroll
-  for (int t = 0; t < 8; t += 2) {
+  for (int t = 0; t < 4; t += 2) {
     const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(ub + 8 * t);
 #pragma unroll
     for (int r = 0; r < 8; ++r) {
-      const int e0 = 8 + r - t, e1 = e0 - 1;
+      const int e0 = 4 + r - t, e1 = e0 - 1;
       float a0, a1, b0, b1;
       unpack2(fadd2((e0 & 1) ? w[e0 >> 1].y : w[e0 >> 1].x, u.x), a0, a1);
       unpack2(fadd2((e1 & 1) ? w[e1 >> 1].y : w[e1 >> 1].x, u.y), b0, b1);
       blo[r] = max3(blo[r], a0, b0);
       bhi[r] = max3(bhi[r], a1, b1);
     }
-    if (t < 6) {
-      const int i = 2 - t / 2;
-      w[i] = *reinterpret_cast<const ulonglong2*>(fw + i * 16);
-    }
   }
 }
 
-__global__ void __launch_bounds__(kDpThreads, 5) dp_step_kernel(const DpStep a) {
-  __shared__ __align__(16) unsigned char dp_smem[kDpWarps][kDpFBytes + kDpUBytes];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int x0 = (a.lo & ~(kDpX - 1)) + (int)blockIdx.x * kDpTile + warp * kDpX;
-  unsigned char* F2 = dp_smem[warp];
-  unsigned char* U2 = F2 + kDpFBytes;
-  const int xg = lane & 7, bg = lane >> 3;
-  const unsigned char* fw = F2 + (xg - bg + 3) * kDpGroup;
-  const unsigned char* ub = U2 + bg * kDpGroup;
+// Row h: the budgets [lo, hi], as tiles of 64 (from the tile of lo on, `per` to a CTA), and the blocks of b that it needs,
+// of whose halves of 32 the first `skip` and those from `halves` on hold no token that is left.
+struct __align__(16) DpRow {
+  int lo, hi, tile0, tiles, per, blk0, blocks, halves;
+};
 
-  pdl_launch_dependents();
-  pdl_wait();
-  if (x0 > a.hi) return;  // whole warps; nothing below waits for another warp
-
+// Row h at the 64 budgets from x0 on (those in [lo, hi]) over `blocks` blocks of b.  Blocks and tokens count from the first
+// staged block; the staged values start 64 `blocks` budgets below what tile 0 reaches with the first token.
+__device__ __forceinline__ void dp_tile(const unsigned char* F2, const float* f_runs, const unsigned char* U2,
+                                        const float4* u_runs, const DpRow& row, int tile, int x0, float* next, int lane) {
+  const int xg = lane & 7, bg = lane >> 3, blocks = row.blocks, lo = row.lo, hi = row.hi;
+  // a sum of two bounds, plus what the rounding of their terms can take away (a few roundings of 2^-24 each)
+  auto sum_up = [](float f, float u) { return f + u > -INFINITY ? f + u + 4e-7f * (fabsf(f) + fabsf(u)) : -INFINITY; };
   // Upper bound of (f(y) - s (y - x0)) + (U(b) - s b) over the pairs of block `blk` from the run maxima of its 64 values of
-  // b and of its 128 values of y, and the size of its terms.  The maxima are read again for every check (L1 holds them):
-  // registers decide how many tiles an SM has in flight.
-  auto bound = [&](int blk, float s, float& size) {
-    const float4 um = __ldg(reinterpret_cast<const float4*>(a.u_runs) + blk);
+  // b and of its 128 values of y.
+  const float4* runs0 = reinterpret_cast<const float4*>(f_runs) + blocks + tile;  // the runs of the tile's own budgets
+  auto bound = [&](int blk, float s) {
+    if (blk >= blocks) return -INFINITY;
+    const float4 um = u_runs[blk];
     const float at = s * (float)(kDpX * blk), s16 = s * (float)kDpRun;
     float f = -INFINITY;
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      // four runs from y = x0 - 64 (blk + 1 - i) on; the tiles of the previous row start at multiples of 64
-      const int y = x0 - kDpX * (blk + 1 - i);
-      float4 v = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-      if (y + kDpX - 1 >= a.plo && y <= a.phi) {
-        if (a.prev) v = *reinterpret_cast<const float4*>(a.prev_runs + y / kDpRun);
-        else v.x = 0.f;
-      }
+      const float4 v = runs0[i - blk - 1];  // four runs from y = x0 - 64 (blk + 1 - i) on
       const float o = (float)(4 * i - 4);
       f = max3(f, max3(v.x - s16 * o, v.y - s16 * (o + 1.f), v.z - s16 * (o + 2.f)), v.w - s16 * (o + 3.f));
     }
     f += at;
     const float u = fmaxf(max3(um.x, um.y - s16, um.z - 2.f * s16), um.w - 3.f * s16) - at;
-    size = fabsf(f) + fabsf(u);
-    return f + u;
+    return sum_up(f, u);
   };
   auto blocks_where = [&](bool p0, bool p1) {
     const uint32_t m0 = __ballot_sync(0xffffffffu, p0), m1 = __ballot_sync(0xffffffffu, p1);
     return (uint64_t)m0 | ((uint64_t)m1 << 32);
   };
-
-  float blo[8], bhi[8], best[8];
+  // packed pairs from y = x0 - 64 (blk + 1) on; a block's packed pairs of U
+  auto f_of = [&](int blk) { return F2 + (blocks + tile - blk - 1) * (kDpX / 8) * kDpGroup; };
+  // The same bound from the block's own values instead of the run maxima, for its two halves of 32 values of b.
+  auto halves = [&](int blk, float s, float& h0, float& h1) {
+    const unsigned char* fe = f_of(blk) + (lane >> 3) * kDpGroup + (lane & 7) * 8 + 4;
+    const unsigned char* ue = U2 + blk * kDpUBlock + (lane & 15) * 8 + (lane >> 4) * 4;
+    const float y = (float)(lane - kDpX * (blk + 1)), b = (float)(kDpX * blk + lane);
+    float g[4];
 #pragma unroll
-  for (int r = 0; r < 8; ++r) blo[r] = bhi[r] = best[r] = -INFINITY;
-  float s = 0.f, low = -INFINITY;
-  uint64_t done = 0;
-#pragma unroll 1
-  for (;;) {
-    // the blocks still to be evaluated: those whose bound comes within the rounding of these expressions (every
-    // term carries a few roundings of 2^-24) of `low`; the one with the largest bound goes first
-    float size0, size1;
-    float t0 = bound(lane, s, size0), t1 = bound(lane + 32, s, size1);
-    const float lin = s * 8192.f + fabsf(low);
-    const bool any = !(low > -INFINITY);
-    const uint64_t todo = blocks_where(t0 > -INFINITY && (any || t0 + 4e-7f * (size0 + lin) >= low),
-                                       t1 > -INFINITY && (any || t1 + 4e-7f * (size1 + lin) >= low)) & ~done;
-    if (!todo) break;
-    if (!((todo >> lane) & 1)) t0 = -INFINITY;
-    if (!((todo >> (lane + 32)) & 1)) t1 = -INFINITY;
-    const float top = warp_max(fmaxf(t0, t1));
-    const uint64_t first = blocks_where(t0 == top, t1 == top) & todo;
-    // alone while `low` still rises a lot (the first time), then together with all others
-    uint64_t batch = done ? todo : first & (~first + 1);
-    done |= batch;
-    DpFetch cur = dp_fetch(a, x0, __ffsll((long long)batch) - 1, lane);
-#pragma unroll 1
-    do {
-      // the same bound once more, from the block's own values instead of the run maxima: what passed on the slack of the
-      // runs alone (up to 16 tokens on either side) drops out before the 4096 pairs are formed
-      const int blk = __ffsll((long long)batch) - 1;
-      batch &= batch - 1;
-      const float y4 = (float)(4 * lane - kDpX * (blk + 1)), b1 = (float)(kDpX * blk + lane);
-      const float fmax = warp_max(fmaxf(max3(cur.f.x - s * y4, cur.f.y - s * (y4 + 1.f), cur.f.z - s * (y4 + 2.f)),
-                                        cur.f.w - s * (y4 + 3.f)));
-      const float umax = warp_max(fmaxf(cur.u0 - s * b1, cur.u1 - s * (b1 + 32.f)));
-      const bool keep = any || fmax + umax + 4e-7f * (fabsf(fmax) + fabsf(umax) + lin) >= low;
-      if (keep) {
-        __syncwarp();
-        dp_store(cur, F2, U2, lane);
-        __syncwarp();
-      }
-      if (batch) cur = dp_fetch(a, x0, __ffsll((long long)batch) - 1, lane);
-      if (keep) dp_block(fw, ub, blo, bhi);
-    } while (batch);
-    // f_h of the tile so far, its slope, and the smallest f_h(x) - s (x - x0) among the budgets that count
+    for (int k = 0; k < 4; ++k) g[k] = *reinterpret_cast<const float*>(fe + 4 * k * kDpGroup) - s * (y + 32.f * k);
+    const float u0 = warp_max(*reinterpret_cast<const float*>(ue) - s * b);
+    const float u1 = warp_max(*reinterpret_cast<const float*>(ue + 128) - s * (b + 32.f));
+    const float f0 = warp_max(max3(g[1], g[2], g[3])), f1 = warp_max(max3(g[0], g[1], g[2]));
+    h0 = sum_up(f0, u0);
+    h1 = sum_up(f1, u1);
+  };
+  float blo[8], bhi[8];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      float m = fmaxf(blo[r], bhi[r]);
-      m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 8));
-      best[r] = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 16));
+  for (int r = 0; r < 8; ++r) blo[r] = bhi[r] = -INFINITY;
+  const int e_lane = 8 * xg - 4 * bg + 12;  // pairs of the lane, from y = x0 - 32 on for half 0
+  const bool odd = (bg & 1) == 0;
+  const unsigned char* f_lane = F2 + (e_lane >> 3) * kDpGroup + (e_lane & 7) * 8;
+  auto evaluate = [&](int blk, int half) {
+    dp_block(f_lane + ((blocks + tile - blk) * 8 - 4 - 4 * half) * kDpGroup, odd, U2 + blk * kDpUBlock + half * 128 + bg * 32,
+             blo, bhi);
+  };
+  // the row so far: a lane gets budgets x0 + xl, x0 + xl + 1
+  const bool hi16 = lane & 16, hi8 = lane & 8;
+  const int xl = 8 * xg + (hi16 ? 4 : 0) + (hi8 ? 2 : 0);
+  float best[2];
+  auto merge = [&]() {
+    float q[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const float a = fmaxf(blo[r], bhi[r]), b = fmaxf(blo[r + 4], bhi[r + 4]);
+      q[r] = fmaxf(hi16 ? b : a, __shfl_xor_sync(0xffffffffu, hi16 ? a : b, 16));
     }
-    s = (__shfl_sync(0xffffffffu, best[7], 7) - __shfl_sync(0xffffffffu, best[0], 0)) * (1.f / 63.f);
-    if (!(s > 0.f && s < 1e30f)) s = 0.f;  // s times a distance of up to 8192 stays a number
+#pragma unroll
+    for (int r = 0; r < 2; ++r) best[r] = fmaxf(hi8 ? q[r + 2] : q[r], __shfl_xor_sync(0xffffffffu, hi8 ? q[r] : q[r + 2], 8));
+  };
+  // smallest f_h(x) - s (x - x0) among the budgets that count, less the rounding of the terms in s
+  auto lowest = [&](float s) {
     float neg = -INFINITY;
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const int x = x0 + 8 * xg + r;
-      if (x >= a.lo && x <= a.hi) neg = fmaxf(neg, s * (float)(8 * xg + r) - best[r]);
-    }
-    low = -warp_max(neg);
-  }
+    for (int r = 0; r < 2; ++r)
+      if (x0 + xl + r >= lo && x0 + xl + r <= hi) neg = fmaxf(neg, s * (float)(xl + r) - best[r]);
+    const float low = -warp_max(neg);
+    return low - 4e-7f * (s * 8192.f + fabsf(low));
+  };
+  auto slope = [&](float last, float first) {
+    const float s = (last - first) * (1.f / 63.f);
+    return s > 0.f && s < 1e30f ? s : 0.f;  // s times a distance of up to 8192 stays a number
+  };
 
-  // the row, and its maxima over runs of 16 (budgets outside [lo, hi] count as -inf)
-  const int x = x0 + 8 * xg;
-  float run = -INFINITY;
+  if (blocks <= kDpFewBlocks) {
+    // few tokens: all of them (bounds would take longer)
+#pragma unroll 1
+    for (int i = row.halves & 255; i < row.halves >> 8; ++i) evaluate(i >> 1, i & 1);
+    merge();
+  } else {
+    // Any slope gives true bounds; that of the previous row at the same budgets gives close ones.
+    const unsigned char* own = F2 + (blocks + tile) * (kDpX / 8) * kDpGroup;
+    float s = slope(*reinterpret_cast<const float*>(own + 7 * kDpGroup + 7 * 8 + 4), *reinterpret_cast<const float*>(own + 4));
+    float t0 = bound(lane, s), t1 = bound(lane + 32, s);
+    const float top = warp_max(fmaxf(t0, t1));
+    // the better half of the block with the largest bound first
+    const int first = __ffsll((long long)blocks_where(t0 == top, t1 == top)) - 1;
+    float h0, h1;
+    halves(first, s, h0, h1);
+    const int half = h1 > h0;
+    evaluate(first, half);
+    merge();
+    float low = lowest(s);
+    bool raised = !(fminf(h0, h1) < low);
+    if (raised) evaluate(first, half ^ 1);
+    uint64_t todo = blocks_where(t0 > -INFINITY && !(t0 < low), t1 > -INFINITY && !(t1 < low)) & ~(1ull << first);
+    if (__popcll(todo) > 4) {  // along the slope of this row the bounds may be closer
+      s = slope(__shfl_sync(0xffffffffu, best[1], 31), __shfl_sync(0xffffffffu, best[0], 0));
+      t0 = bound(lane, s), t1 = bound(lane + 32, s);
+      low = lowest(s);
+      todo &= blocks_where(!(t0 < low), !(t1 < low));
+    }
+    // a block that is not left can raise no budget's value above what it has; the others are looked at once
+#pragma unroll 1
+    while (todo) {
+      const int blk = __ffsll((long long)todo) - 1;
+      todo &= todo - 1;
+      halves(blk, s, h0, h1);
+      if (!(h0 < low)) raised = true, evaluate(blk, 0);
+      if (!(h1 < low)) raised = true, evaluate(blk, 1);
+    }
+    if (raised) merge();
+  }
+  if (!next) return;
+  const int x = x0 + xl;
+  if (x >= lo && x + 1 <= hi)
+    asm volatile("st.relaxed.gpu.global.v2.f32 [%0], {%1, %2};" ::"l"(next + x), "f"(best[0]), "f"(best[1]) : "memory");
+  else if (x >= lo && x <= hi)
+    asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" ::"l"(next + x), "f"(best[0]) : "memory");
+  else if (x + 1 >= lo && x + 1 <= hi)
+    asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" ::"l"(next + x + 1), "f"(best[1]) : "memory");
+}
+
+// ---- which tokens can matter -------------------------------------------------------------------------------------
+//
+// For any slope l, a choice b of head j falls short of c_j = max over b of (U_j(b) - l b) by d_j(b) >= 0, and a solution of
+// sum B has the value l B + sum c_j - sum d_j(b_j).  With the value LB of some solution, the choices of an optimal one have
+// d_j(b_j) <= l B + sum c_j - LB each.  The recursion adds in fp32: every row's addition errs by at most 2^-24 of the sum, so
+// whatever path attains the recursion's result (and with it every place where the walk back finds its target) has a true
+// value of at least LB less twice the sum of those errors.  With that allowance the tokens [b0, b1] of a head that are
+// left, and the budgets that such tokens add up to, hold every path that the full recursion could return, and the rows
+// restricted to them have the full recursion's values on those paths.  l and LB come from the greedy solution of the
+// relaxed problem, which is close: 240 of 3968 tokens a head are left on utility curves of 256 heads, and 5 % of the budgets.
+
+constexpr int kDpCoreThreads = 256;
+__device__ __forceinline__ double dp_warp_sum(double v) {
 #pragma unroll
-  for (int r = 0; r < 8; ++r)
-    if (x + r >= a.lo && x + r <= a.hi) run = fmaxf(run, best[r]);
-  run = fmaxf(run, __shfl_xor_sync(0xffffffffu, run, 1));
-  if (bg == 0) {
-    if (!(xg & 1)) __stcg(a.next_runs + x / kDpRun, run);
-    if (x >= a.lo && x + 7 <= a.hi) {  // rows start at multiples of 64 floats, x is a multiple of 8
-      __stcg(reinterpret_cast<float4*>(a.next + x), make_float4(best[0], best[1], best[2], best[3]));
-      __stcg(reinterpret_cast<float4*>(a.next + x + 4), make_float4(best[4], best[5], best[6], best[7]));
-    } else {
+  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+  return v;
+}
+// Sum over the CTA in a fixed order, for all threads.
+__device__ __forceinline__ double dp_cta_sum(double v, double* part) {
+  v = dp_warp_sum(v);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = v;
+  __syncthreads();
+  double t = 0.0;
+  for (int i = 0; i < kDpCoreThreads / 32; ++i) t += part[i];
+  return t;
+}
+
+struct DpCore {
+  const float* curves;      // [N][P]
+  HullLists lists;          // of the curves
+  const int32_t* budgets;   // [N] the greedy solution
+  double* slope;            // [1]
+  double* c;                // [N] c_j
+  double* u;                // [N] U_j at the greedy solution
+  double* size;             // [N] max |U_j|
+  int4* rows;               // [N]
+  int* done;                // [1] heads that have their tokens, zero before
+  int P, N, n, B;
+};
+// The slope and every head's c_j.  One CTA per head.
+__global__ void __launch_bounds__(kDpCoreThreads) dp_reduced_kernel(const DpCore a) {
+  __shared__ double part[kDpCoreThreads / 32], part_size[kDpCoreThreads / 32];
+  __shared__ float gain_s[kDpCoreThreads / 32];
+  const int j = blockIdx.x, tid = threadIdx.x;
+  // the smallest gain among the blocks that the solution takes from; the largest of all if it takes nothing
+  float least = INFINITY, most = 0.f;
+  for (int i = tid; i < a.N; i += kDpCoreThreads) {
+    const size_t row = (size_t)i * (a.P - 1);
+    const int count = a.lists.count[i], b = a.budgets[i];
+    if (count < 1) continue;
+    most = fmaxf(most, a.lists.gain[row]);
+    if (b < 1) continue;
+    int lo = 0, hi = count - 1;  // the last block that starts before token b
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if ((int)a.lists.start[row + mid] < b) lo = mid;
+      else hi = mid - 1;
+    }
+    least = fminf(least, a.lists.gain[row + lo]);
+  }
+  least = -warp_max(-least);
+  if ((tid & 31) == 0) gain_s[tid >> 5] = least;
+  __syncthreads();
+  for (int i = 0; i < kDpCoreThreads / 32; ++i) least = fminf(least, gain_s[i]);
+  if (!(least < INFINITY)) {
+    __syncthreads();
+    most = warp_max(most);
+    if ((tid & 31) == 0) gain_s[tid >> 5] = most;
+    __syncthreads();
+    for (int i = 0; i < kDpCoreThreads / 32; ++i) most = fmaxf(most, gain_s[i]);
+    least = most;
+  }
+  const double slope = (double)least;
+  const float* U = a.curves + (size_t)j * a.P;
+  double c = -INFINITY, size = 0.0;
+  for (int b = tid; b <= a.n; b += kDpCoreThreads) {
+    const double x = (double)__ldg(U + b);
+    c = fmax(c, x - slope * b);
+    size = fmax(size, fabs(x));
+  }
 #pragma unroll
-      for (int r = 0; r < 8; ++r)
-        if (x + r >= a.lo && x + r <= a.hi) __stcg(a.next + x + r, best[r]);
+  for (int off = 16; off > 0; off >>= 1) {
+    c = fmax(c, __shfl_xor_sync(0xffffffffu, c, off));
+    size = fmax(size, __shfl_xor_sync(0xffffffffu, size, off));
+  }
+  if ((tid & 31) == 0) {
+    part[tid >> 5] = c;
+    part_size[tid >> 5] = size;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    for (int i = 1; i < kDpCoreThreads / 32; ++i) {
+      c = fmax(c, part[i]);
+      size = fmax(size, part_size[i]);
+    }
+    a.c[j] = c;
+    a.size[j] = size;
+    a.u[j] = (double)__ldg(U + min(max(a.budgets[j], 0), a.n));
+    if (j == 0) *a.slope = slope;
+  }
+}
+
+// Every head's tokens; the last CTA to finish makes the rows' budgets of them.
+__global__ void __launch_bounds__(kDpCoreThreads) dp_ranges_kernel(const DpCore a) {
+  __shared__ double part[kDpCoreThreads / 32];
+  __shared__ int range_s[2], last_s;
+  const int j = blockIdx.x, tid = threadIdx.x;
+  int b0 = a.n, b1 = 0;
+  double c = 0.0, u = 0.0, size = 0.0, sizes = 0.0;
+  for (int i = tid; i < a.N; i += kDpCoreThreads) {
+    c += a.c[i];
+    u += a.u[i];
+    size += a.size[i];
+    sizes += a.size[i] * (double)(a.N - i);  // a head's size is part of its own row's sum and of all later ones
+  }
+  c = dp_cta_sum(c, part), u = dp_cta_sum(u, part), size = dp_cta_sum(size, part), sizes = dp_cta_sum(sizes, part);
+  const double slope = *a.slope;
+  double slack = slope * (double)a.B + c - u + 2.0 * (1.001 * sizes * 0x1p-24 + a.N * 0x1p-125);
+  slack += 1e-12 * (size + slope * (double)a.n * a.N);  // of the sums here
+  if (!(size < 1e37)) slack = INFINITY;               // sums might leave fp32
+  const double bar = a.c[j] - slack;
+  const float* U = a.curves + (size_t)j * a.P;
+  for (int b = tid; b <= a.n; b += kDpCoreThreads)
+    if (!((double)__ldg(U + b) - slope * b < bar)) {
+      b0 = min(b0, b);
+      b1 = max(b1, b);
+    }
+  if (tid == 0) range_s[0] = a.n, range_s[1] = 0;
+  __syncthreads();
+  b0 = __reduce_min_sync(0xffffffffu, b0);
+  b1 = __reduce_max_sync(0xffffffffu, b1);
+  if ((tid & 31) == 0) {
+    atomicMin(&range_s[0], b0);
+    atomicMax(&range_s[1], b1);
+  }
+  __syncthreads();
+  if (tid == 0) {
+    // (no token is left where a curve holds something that is no number: then all are)
+    a.rows[j] = range_s[0] <= range_s[1] ? make_int4(0, 0, range_s[0], range_s[1]) : make_int4(0, 0, 0, a.n);
+    __threadfence();
+    last_s = atomicAdd(a.done, 1) == a.N - 1;
+  }
+  __syncthreads();
+  if (!last_s) return;
+  __threadfence();
+  // sums of the fewest and of the most tokens up to every head, 256 heads at a time
+  __shared__ long long sum0_s[kDpCoreThreads / 32], sum1_s[kDpCoreThreads / 32];
+  long long carry0 = 0, carry1 = 0, total0 = 0, total1 = 0;
+  bool sound = true;
+  for (int pass = 0; pass < 2; ++pass) {
+    for (int i0 = 0; i0 < a.N; i0 += kDpCoreThreads) {
+      const int i = i0 + tid;
+      int4 r = make_int4(0, 0, 0, 0);
+      if (i < a.N) r = __ldcg(a.rows + i);
+      if (pass == 1 && !sound && i < a.N) r.z = 0, r.w = a.n;
+      long long s0 = r.z, s1 = r.w;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const long long o0 = __shfl_up_sync(0xffffffffu, s0, off), o1 = __shfl_up_sync(0xffffffffu, s1, off);
+        if ((tid & 31) >= off) s0 += o0, s1 += o1;
+      }
+      if ((tid & 31) == 31) sum0_s[tid >> 5] = s0, sum1_s[tid >> 5] = s1;
+      __syncthreads();
+      long long all0 = carry0, all1 = carry1;
+      for (int k = 0; k < kDpCoreThreads / 32; ++k) {
+        if (k < (tid >> 5)) s0 += sum0_s[k], s1 += sum1_s[k];
+        all0 += sum0_s[k], all1 += sum1_s[k];
+      }
+      s0 += carry0, s1 += carry1;
+      if (pass == 1 && i < a.N) {
+        // what the heads behind take at the least and at the most bounds the budget from the other side
+        r.x = (int)max(s0, (long long)a.B - (total1 - s1));
+        r.y = (int)min(s1, (long long)a.B - (total0 - s0));
+        a.rows[i] = r;
+      }
+      carry0 = all0, carry1 = all1;
+      __syncthreads();
+    }
+    if (pass == 0) {
+      total0 = carry0, total1 = carry1, carry0 = carry1 = 0;
+      sound = total0 <= a.B && a.B <= total1;  // always, for curves of numbers
+      if (!sound) total0 = 0, total1 = (long long)a.N * a.n;
     }
   }
 }
 
-// Walks back from x = B; also writes the optimum and the packed-row offsets of this sequence.  One CTA; the chain over
-// the heads is serial and a step reads f_{h-1} at up to n + 1 places (one L2 latency and one barrier), so the next row
-// is asked for while a step runs, and the next head's curve is staged in shared memory.
-__global__ void __launch_bounds__(kDpBackThreads) dp_backtrack_kernel(const float* __restrict__ curves, int P,
-                                                                      const float* __restrict__ f, long long stride,
-                                                                      long long B, int N, int n, int w,
-                                                                      long long row_base, int q,
+__device__ __forceinline__ DpRow dp_row(const DpArgs& a, int h) {
+  const int4 v = __ldg(a.rows + h);
+  DpRow r;
+  r.lo = v.x, r.hi = v.y;
+  r.tile0 = r.lo / kDpX;
+  r.tiles = r.hi / kDpX - r.tile0 + 1;
+  r.per = max(kDpMinTiles, (r.tiles + (int)gridDim.x - 1) / (int)gridDim.x);
+  r.blk0 = v.z / kDpX;
+  r.blocks = v.w / kDpX - r.blk0 + 1;
+  const int skip = v.z / 32 - 2 * r.blk0;
+  r.halves = skip | (v.w / 32 - 2 * r.blk0 + 1) << 8;
+  return r;
+}
+
+// Marks the values of the rows that are to come, and their vectors' other elements as -inf.  One CTA per row.  `B` (or
+// -1: the rows are known): rows of all tokens are made first, those budgets that can still reach B.
+__global__ void __launch_bounds__(256) dp_clear_kernel(const DpArgs a, int4* rows, int B) {
+  const int h = blockIdx.x;
+  int4 r;
+  if (B >= 0) {
+    r = make_int4((int)max(0LL, B - (long long)(a.N - 1 - h) * a.n), (int)min((long long)B, (long long)(h + 1) * a.n), 0, a.n);
+    if (threadIdx.x == 0) rows[h] = r;
+  } else {
+    r = __ldg(a.rows + h);
+  }
+  float* f = a.f + (size_t)h * a.stride;
+  const float unset = __uint_as_float(kDpUnset);
+  for (int y = (r.x & ~3) + 4 * threadIdx.x; y <= r.y; y += 4 * 256)
+    *reinterpret_cast<float4*>(f + y) =
+        make_float4(y >= r.x ? unset : -INFINITY, y + 1 >= r.x && y + 1 <= r.y ? unset : -INFINITY,
+                    y + 2 >= r.x && y + 2 <= r.y ? unset : -INFINITY, y + 3 <= r.y ? unset : -INFINITY);
+}
+
+// All rows in one launch.  The tiles of every row are dealt to the CTAs in stretches.  A tile of row h needs f_{h-1} at its
+// own budgets and at what the head's tokens take off them: a CTA polls those values themselves, which the CTAs that had them
+// store as they get them (every row is kept, so nobody waits to overwrite, and there is no other signal).
+__global__ void __launch_bounds__(kDpThreads, 1) dp_rows_kernel(const DpArgs a) {
+  extern __shared__ __align__(16) unsigned char dp_smem[];
+  __shared__ int next_tile;
+  const DpPlan plan = dp_plan(a.n, a.N);
+  unsigned char* F2 = dp_smem;                                       // packed pairs (f(y + 16), f(y))
+  float* f_runs = reinterpret_cast<float*>(dp_smem + plan.runs_off);
+  DpRow* table = reinterpret_cast<DpRow*>(dp_smem + plan.table_off);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, cta = blockIdx.x;
+  for (int i = threadIdx.x; i < min(a.N, kDpTable); i += kDpThreads) table[i] = dp_row(a, i);
+  __syncthreads();
+  auto row_of = [&](int h) { return h < kDpTable ? table[h] : dp_row(a, h); };
+  auto fetch_curve = [&](int h, const DpRow& r, int buf) {  // the blocks that the row needs
+    unsigned char* U2 = dp_smem + plan.u_off + buf * plan.u_bytes;
+    const float* U = a.curves + (size_t)h * a.P + r.blk0 * kDpX;
+    const int last = a.n - r.blk0 * kDpX;
+    for (int b = threadIdx.x; b < r.blocks * kDpX; b += kDpThreads) {
+      unsigned char* to = U2 + (b >> 5) * 128 + (b & 15) * 8 + ((b >> 4) & 1) * 4;  // pairs (U(b), U(b + 16))
+      if (b <= last) cp_async4(to, U + b);
+      else *reinterpret_cast<float*>(to) = -INFINITY;
+    }
+    float* ur = reinterpret_cast<float*>(dp_smem + plan.u_runs_off) + buf * plan.blocks * 4;
+    for (int i = threadIdx.x; i < r.blocks * 4; i += kDpThreads)
+      cp_async4(ur + i, a.u_runs + (size_t)h * kDpURuns + r.blk0 * 4 + i);
+  };
+  auto next_row = [&](int h) {  // the next row from h on of which this CTA has a part
+    for (; h < a.N; ++h) {
+      const DpRow r = row_of(h);
+      if (cta * r.per < r.tiles) break;
+    }
+    return h;
+  };
+  int h = next_row(0), buf = 0;
+  if (h < a.N) fetch_curve(h, row_of(h), 0);
+
+  for (int h_next; h < a.N; h = h_next, buf ^= 1) {
+    const DpRow row = row_of(h);
+    const int old_lo = h > 0 ? row_of(h - 1).lo : 0, old_hi = h > 0 ? row_of(h - 1).hi : 0;
+    const int tile0 = row.tile0 + cta * row.per, tiles = min(row.per, row.tiles - cta * row.per);
+    const float* prev = a.f + (size_t)(h > 0 ? h - 1 : 0) * a.stride;
+    float* next = a.f + (size_t)h * a.stride;
+    const unsigned char* U2 = dp_smem + plan.u_off + buf * plan.u_bytes;
+    const float4* u_runs = reinterpret_cast<const float4*>(dp_smem + plan.u_runs_off) + buf * plan.blocks;
+    for (int t_sub = 0; t_sub < tiles; t_sub += kDpSub) {
+      const int n_sub = min(kDpSub, tiles - t_sub), xs = (tile0 + t_sub) * kDpX;
+      const int ybase = xs - (row.blk0 + row.blocks) * kDpX;
+      const int windows = ((row.blocks + n_sub) * kDpX + kDpWindow - 1) / kDpWindow;
+      // f_{h-1} at ybase + 112 i + 4 lane .. + 3 for this warp's windows i
+      float4 v[kDpWindowsPer];
+      uint32_t left = 0;
+#pragma unroll
+      for (int k = 0; k < kDpWindowsPer; ++k) {
+        const int y = ybase + kDpWindow * (warp + k * kDpWarps) + 4 * lane;
+        v[k] = make_float4(h == 0 && y == 0 ? 0.f : -INFINITY, -INFINITY, -INFINITY, -INFINITY);
+        if (h > 0 && warp + k * kDpWarps < windows && y + 3 >= old_lo && y <= old_hi) left |= 1u << k;
+      }
+      bool ok = true;
+      for (uint32_t spins = 0; left;) {
+#pragma unroll
+        for (int k = 0; k < kDpWindowsPer; ++k)
+          if (left >> k & 1)
+            asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                         : "=f"(v[k].x), "=f"(v[k].y), "=f"(v[k].z), "=f"(v[k].w)
+                         : "l"(prev + ybase + kDpWindow * (warp + k * kDpWarps) + 4 * lane)
+                         : "memory");
+#pragma unroll
+        for (int k = 0; k < kDpWindowsPer; ++k)
+          if (__float_as_uint(v[k].x) != kDpUnset && __float_as_uint(v[k].y) != kDpUnset &&
+              __float_as_uint(v[k].z) != kDpUnset && __float_as_uint(v[k].w) != kDpUnset)
+            left &= ~(1u << k);
+        if (left && (++spins >= a.spin_limit || ((spins & 255) == 0 && *reinterpret_cast<volatile int*>(a.words) != 0))) {
+          atomicExch(a.words, (int)LUKV_ERR_TIMEOUT);
+          ok = false;
+          break;
+        }
+      }
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      if (!__syncthreads_and(ok)) return;  // (and the tiles before have been read)
+      if (threadIdx.x == 0) next_tile = kDpWarps;
+#pragma unroll
+      for (int k = 0; k < kDpWindowsPer; ++k) {
+        const int i = warp + k * kDpWarps;
+        if (i < windows) {
+          // lane l >= 4 holds the first parts of pairs 4 l - 16 .. + 3, lane l - 4 their second parts
+          const float g0 = __shfl_up_sync(0xffffffffu, v[k].x, 4), g1 = __shfl_up_sync(0xffffffffu, v[k].y, 4);
+          const float g2 = __shfl_up_sync(0xffffffffu, v[k].z, 4), g3 = __shfl_up_sync(0xffffffffu, v[k].w, 4);
+          if (lane >= 4) {
+            float4* to_s = reinterpret_cast<float4*>(F2 + (kDpWindow / 8 * i + ((lane - 4) >> 1)) * kDpGroup + (lane & 1) * 32);
+            to_s[0] = make_float4(v[k].x, g0, v[k].y, g1);
+            to_s[1] = make_float4(v[k].z, g2, v[k].w, g3);
+          }
+          float m = fmaxf(max3(v[k].x, v[k].y, v[k].z), v[k].w);
+          m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+          m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+          if ((lane & 3) == 0 && (lane < 28 || i == windows - 1)) f_runs[kDpWindow / kDpRun * i + (lane >> 2)] = m;
+        }
+      }
+      __syncthreads();
+
+      // tiles differ in what they have to look at: warps take them as they come
+      for (int tile = warp; tile < n_sub;) {
+        dp_tile(F2, f_runs, U2, u_runs, row, tile, xs + tile * kDpX, cta != a.drop ? next : nullptr, lane);
+        if (n_sub <= kDpWarps) break;
+        if (lane == 0) tile = atomicAdd(&next_tile, 1);
+        tile = __shfl_sync(0xffffffffu, tile, 0);
+      }
+    }
+    h_next = next_row(h + 1);
+    if (h_next < a.N) fetch_curve(h_next, row_of(h_next), buf ^ 1);
+  }
+}
+
+// Walks back from x = B; also writes the optimum and the packed-row offsets of this sequence, and clears the word
+// of the next sequence's heads.  One CTA; the chain over the heads is serial.  A step compares the head's tokens (one load of
+// f_{h-1} and one of U each, one barrier); what a step kWalkAhead heads on can read is touched meanwhile, so that it is in
+// L1 by then: the budget falls by what the tokens allow.  The value at the budget that a step arrives at comes with the match.
+constexpr int kWalkAhead = 4;
+__global__ void __launch_bounds__(kDpBackThreads) dp_backtrack_kernel(const DpArgs a, int B, int w, long long row_base, int q,
                                                                       int32_t* __restrict__ budgets,
                                                                       int32_t* __restrict__ offsets,
                                                                       double* __restrict__ values) {
-  constexpr int kVecs = 3;  // 16-byte vectors of f per thread: 12 * 384 places cover n + 4
-  constexpr int kUPer = (kDpMaxBlocks * kDpX + kDpBackThreads - 1) / kDpBackThreads;
-  __shared__ float Us[2][kDpMaxBlocks * kDpX];
-  __shared__ int first_b[3];
-  const int tid = threadIdx.x;
-  long long x = B;
-  float target = f[(size_t)(N - 1) * stride + B];
-  if (tid == 0) {
-    values[q] = (double)target;
-    first_b[0] = first_b[1] = first_b[2] = 1 << 30;
-    if (q == 0) offsets[0] = 0;
-  }
-  for (int b = tid; b <= n; b += kDpBackThreads) Us[(N - 1) & 1][b] = __ldg(curves + (size_t)(N - 1) * P + b);
+  constexpr int kWarps = kDpBackThreads / 32;
+  __shared__ int match_b[2][kWarps];
+  __shared__ float match_f[2][kWarps];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, N = a.N;
+  const bool failed = a.words[0] != 0;
   __syncthreads();
+  if (tid == 0) a.words[1] = 0;
+  if (tid == 0 && q == 0) offsets[0] = 0;
+  if (failed) {  // a wait of the rows' kernel ran out: no solution
+    if (tid == 0) values[q] = __longlong_as_double(0x7FF8000000000000LL);
+    for (int h = tid; h < N; h += kDpBackThreads) {
+      budgets[(size_t)q * N + h] = 0;
+      offsets[(size_t)q * N + h + 1] = (int32_t)(row_base + (long long)(h + 1) * w);
+    }
+    return;
+  }
+  int x = B;
+  float target = __ldg(a.f + (size_t)(N - 1) * a.stride + B);
+  if (tid == 0) values[q] = (double)target;
+  auto touch = [](const float* p) { asm volatile("{\n\t.reg .f32 t;\n\tld.global.ca.f32 t, [%0];\n\t}" ::"l"(p)); };
+  int4 row = __ldg(a.rows + N - 1);
   for (int h = N - 1; h >= 0; --h) {
-    const float* prev = h > 0 ? f + (size_t)(h - 1) * stride : nullptr;
-    const long long plo = h > 0 ? max(0LL, B - (long long)(N - h) * n) : 0;
-    const long long phi = h > 0 ? min(B, (long long)h * n) : 0;
-    // y = x - b for b = 0 .. n, as aligned vectors of four from the top down
-    const int top = (int)(x & 3);
-    float4 v[kVecs];
-#pragma unroll
-    for (int i = 0; i < kVecs; ++i) {
-      const long long y = (x & ~3LL) - 4LL * (tid + i * kDpBackThreads);
-      v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (prev && y + 3 >= max(plo, x - n) && y <= phi) v[i] = __ldcg(reinterpret_cast<const float4*>(prev + y));
-    }
-    float u_next[kUPer];
-#pragma unroll
-    for (int i = 0; i < kUPer; ++i) {
-      const int b = tid + i * kDpBackThreads;
-      u_next[i] = h > 0 && b <= n ? __ldg(curves + (size_t)(h - 1) * P + b) : 0.f;
-    }
-    if (h > 1) {  // x falls by at most n a head: what the next step reads lies within 2 n
-      const long long y = x - 2LL * n + (long long)tid * 32;
-      if (tid <= n / 16 + 1 && y >= 0 && y <= x)
-        asm volatile("prefetch.global.L2 [%0];" ::"l"(f + (size_t)(h - 2) * stride + y));
-    }
-    const float* U = Us[h & 1];
+    const int4 old = h > 0 ? __ldg(a.rows + h - 1) : make_int4(0, 0, 0, 0);
+    const float* prev = a.f + (size_t)max(h - 1, 0) * a.stride;
+    const float* U = a.curves + (size_t)h * a.P;
     int mine = 1 << 30;
-#pragma unroll
-    for (int i = kVecs - 1; i >= 0; --i) {
-      const float e[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const int b = top - c + 4 * (tid + i * kDpBackThreads);
-        const long long y = x - b;
-        if (b >= 0 && b <= n && y >= plo && y <= phi && e[c] + U[b] == target) mine = min(mine, b);
+    float mine_f = 0.f;
+#pragma unroll 4
+    for (int b = row.z + tid; b <= row.w; b += kDpBackThreads) {
+      const int y = x - b;
+      if (y >= old.x && y <= old.y) {
+        const float e = h > 0 ? __ldg(prev + y) : 0.f;
+        if (mine == 1 << 30 && e + __ldg(U + b) == target) {
+          mine = b;
+          mine_f = e;
+        }
       }
     }
-#pragma unroll
-    for (int i = 0; i < kUPer; ++i) {
-      const int b = tid + i * kDpBackThreads;
-      if (b <= n) Us[(h + 1) & 1][b] = u_next[i];
+    const int least = __reduce_min_sync(0xffffffffu, mine);
+    if (mine == least && (mine < (1 << 30) || lane == 0)) {  // one lane: every b is one thread's
+      match_b[h & 1][warp] = least;
+      match_f[h & 1][warp] = mine_f;
     }
-    mine = __reduce_min_sync(0xffffffffu, mine);
-    if ((tid & 31) == 0 && mine < (1 << 30)) atomicMin(&first_b[h % 3], mine);
+    const int ahead = h - kWalkAhead;
+    if (ahead > 0) {
+      long long down0 = 0, down1 = 0;  // fewest and most tokens until then
+#pragma unroll
+      for (int i = 0; i < kWalkAhead; ++i) {
+        const int4 r = __ldg(a.rows + h - i);
+        down0 += r.z, down1 += r.w;
+      }
+      const int4 r = __ldg(a.rows + ahead);
+      const long long y0 = max((long long)__ldg(a.rows + ahead - 1).x, x - down1 - r.w) & ~31LL, y1 = x - down0 - r.z;
+      if (y0 + 32LL * tid <= y1) touch(a.f + (size_t)(ahead - 1) * a.stride + y0 + 32 * tid);
+      if (r.z + 32 * tid <= r.w + 31) touch(a.curves + (size_t)ahead * a.P + min(r.z + 32 * tid, r.w));
+    }
     __syncthreads();
-    const int b = (int)min((long long)first_b[h % 3], min(x, (long long)n));  // a match exists for finite curves
+    const int theirs = lane < kWarps ? match_b[h & 1][lane] : 1 << 30;
+    const float theirs_f = lane < kWarps ? match_f[h & 1][lane] : 0.f;
+    const int found = __reduce_min_sync(0xffffffffu, theirs);
+    // a match exists for finite curves; without one, as many tokens as there are
+    const int b = found < (1 << 30) ? found : min(x, a.n);
     if (tid == 0) {
-      first_b[(h + 1) % 3] = 1 << 30;  // the slot of the step before, which every thread has read: for two steps on
       budgets[(size_t)q * N + h] = b;
       // the rows up to and with head h: x tokens and the windows
       offsets[(size_t)q * N + h + 1] = (int32_t)(row_base + x + (long long)(h + 1) * w);
     }
     x -= b;
-    if (prev) target = __ldcg(prev + x);
+    target = __shfl_sync(0xffffffffu, theirs_f, __ffs(__ballot_sync(0xffffffffu, theirs == found)) - 1);
+    if (found == 1 << 30 && h > 0) target = __ldg(prev + x);
+    row = old;
   }
 }
 
 size_t align256x(size_t x) { return (x + 255) & ~(size_t)255; }
 // floats of one row f_h: rows start on 256-byte boundaries
 size_t dp_stride(int64_t budget) { return align256x(((size_t)budget + 1) * sizeof(float)) / sizeof(float); }
-
 }  // namespace
 
-size_t exact_workspace_bytes(const Dims& dm, int64_t max_budget) {
-  const size_t stride = dp_stride(max_budget);
-  // the rows, two sets of run maxima, the curves' run maxima
-  return ((size_t)dm.N * stride + 2 * (stride / kDpRun + kDpX) + (size_t)dm.N * kDpURuns) * sizeof(float);
+// the rows' values; the curves' run maxima; the words; the heads' c, u, size and the slope; the rows; the hull lists
+struct DpSpace {
+  size_t f, u_runs, words, core, rows, hull, total;
+};
+static DpSpace dp_space(const Dims& dm, int64_t max_budget) {
+  DpSpace s;
+  s.f = 0;
+  s.u_runs = (size_t)dm.N * dp_stride(max_budget) * sizeof(float);
+  s.words = s.u_runs + align256x((size_t)dm.N * kDpURuns * sizeof(float));
+  s.core = s.words + align256x(kDpWords * sizeof(int));
+  s.rows = s.core + align256x((3 * (size_t)dm.N + 1) * sizeof(double));
+  s.hull = s.rows + align256x((size_t)dm.N * sizeof(int4));
+  s.total = s.hull + hull_lists_bytes(dm.N, dm.P);
+  return s;
 }
+size_t exact_workspace_bytes(const Dims& dm, int64_t max_budget) { return dp_space(dm, max_budget).total; }
 
 cudaError_t launch_exact_allocate(const Dims& dm, const float* curves, const int64_t* budgets_host, int32_t* budgets,
                                   int32_t* offsets, double* values, void* ws, LaunchCtx& lc) {
   if (dm.n / kDpX + 1 > kDpMaxBlocks) return cudaErrorInvalidValue;
-  cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(kDpThreads);
-  cfg.stream = lc.st;
-  // a step may start while the one before it drains
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
   cudaError_t e;
-  float* u_runs = static_cast<float*>(ws);
-  dp_runs_kernel<<<(unsigned)dm.N, kDpURuns, 0, lc.st>>>(curves, u_runs, dm.n, dm.P);
+  int sms = 0;
+  if ((e = device_sms(&sms)) != cudaSuccess) return e;
+  const size_t smem = dp_plan(dm.n, dm.N).total;
+  if ((e = allow_smem((const void*)dp_rows_kernel, smem)) != cudaSuccess) return e;
+  int64_t most = 0;
+  for (int q = 0; q < dm.S; ++q) most = std::max(most, budgets_host[q]);
+  const DpSpace at = dp_space(dm, most);
+  char* base = static_cast<char*>(ws);
+  float* u_runs = reinterpret_cast<float*>(base + at.u_runs);
+  DpArgs a;
+  a.curves = curves;
+  a.u_runs = u_runs;
+  a.rows = reinterpret_cast<int4*>(base + at.rows);
+  a.words = reinterpret_cast<int*>(base + at.words);
+  a.f = reinterpret_cast<float*>(base + at.f);
+  a.P = dm.P, a.N = dm.N, a.n = dm.n;
+  score_test_hooks(&a.spin_limit, &a.drop);
+  DpCore c;
+  c.curves = curves;
+  c.lists = hull_lists(base + at.hull, dm.N, dm.P);
+  c.slope = reinterpret_cast<double*>(base + at.core);
+  c.c = c.slope + 1, c.u = c.c + dm.N, c.size = c.u + dm.N;
+  c.rows = reinterpret_cast<int4*>(base + at.rows);
+  c.done = a.words + 1;
+  c.P = dm.P, c.N = dm.N, c.n = dm.n;
+  dp_runs_kernel<<<(unsigned)dm.N, kDpURuns, 0, lc.st>>>(curves, u_runs, a.words, kDpWords, dm.n, dm.P);
   lc.mark("dp_runs");
+  // the greedy solutions of all sequences; each is read before the walk overwrites it.  They cost 40 to 100 us and shorten a
+  // row by 1 us or more: 16 heads x 584 tokens 98 us with them and 83 without, 32 x 284 138 and 128, 64 x 134 211 and 207,
+  // 128 x 114 363 and 384, 256 x 3968 1.0 and 3.4 ms.
+  const bool greedy = dm.N >= 40 && dm.N * (int64_t)(dm.n / kDpX + 2) > 256 && dm.N <= kGreedyMaxHeads;
+  if (greedy) {
+    if ((e = launch_hull(curves, c.lists, dm.N, dm.P, lc)) != cudaSuccess) return e;
+    if ((e = launch_greedy(dm, c.lists, budgets_host, budgets, offsets, 1, false, lc)) != cudaSuccess) return e;
+  }
   long long row_base = 0;
   for (int q = 0; q < dm.S; ++q) {
-    const long long B = budgets_host[q];
-    const size_t stride = dp_stride(B), runs = stride / kDpRun + kDpX;
-    float* f_runs = u_runs + (size_t)dm.N * kDpURuns;
-    float* f = f_runs + 2 * runs;
-    DpStep st;
-    st.plo = st.phi = 0;
-    st.prev = st.prev_runs = nullptr;
-    st.n = dm.n;
-    for (int h = 0; h < dm.N; ++h) {
-      st.U = curves + (size_t)h * dm.P;
-      st.u_runs = u_runs + (size_t)h * kDpURuns;
-      st.next = f + (size_t)h * stride;
-      st.next_runs = f_runs + (size_t)(h & 1) * runs;
-      st.lo = (int)std::max(0LL, B - (long long)(dm.N - 1 - h) * dm.n);  // B < 2^31, as the packed rows
-      st.hi = (int)std::min(B, (long long)(h + 1) * dm.n);
-      cfg.gridDim = dim3((unsigned)((st.hi - (st.lo & ~(kDpX - 1))) / kDpTile + 1));
-      // the first step of a sequence waits for all before it: its rows overwrite what the last walk reads, and it
-      // reads the curves' run maxima
-      cfg.numAttrs = h > 0 ? 1 : 0;
-      if ((e = cudaLaunchKernelEx(&cfg, dp_step_kernel, st)) != cudaSuccess) return e;
-      lc.mark("dp_step");
-      st.plo = st.lo;
-      st.phi = st.hi;
-      st.prev = st.next;
-      st.prev_runs = st.next_runs;
+    c.B = (int)budgets_host[q];  // below 2^31, as the packed rows
+    c.budgets = budgets + (size_t)q * dm.N;
+    if (greedy) {
+      dp_reduced_kernel<<<(unsigned)dm.N, kDpCoreThreads, 0, lc.st>>>(c);
+      lc.mark("dp_reduced");
+      dp_ranges_kernel<<<(unsigned)dm.N, kDpCoreThreads, 0, lc.st>>>(c);
+      lc.mark("dp_ranges");
     }
-    dp_backtrack_kernel<<<1, kDpBackThreads, 0, lc.st>>>(curves, dm.P, f, (long long)stride, B, dm.N, dm.n, dm.w, row_base,
-                                                         q, budgets, offsets, values);
+    a.stride = (long long)dp_stride(c.B);
+    dp_clear_kernel<<<(unsigned)dm.N, 256, 0, lc.st>>>(a, c.rows, greedy ? -1 : c.B);
+    lc.mark("dp_clear");
+    void* params[] = {(void*)&a};
+    // cooperative launch: CTAs wait for one another, so all must be resident
+    const int ctas = std::min(sms, c.B / kDpX / kDpMinTiles + 1);
+    e = cudaLaunchCooperativeKernel((const void*)dp_rows_kernel, dim3((unsigned)ctas), dim3(kDpThreads), params, smem, lc.st);
+    if (e != cudaSuccess) return e;
+    lc.mark("dp_rows");
+    dp_backtrack_kernel<<<1, kDpBackThreads, 0, lc.st>>>(a, c.B, dm.w, row_base, q, budgets, offsets, values);
     lc.mark("dp_backtrack");
-    row_base += B + (long long)dm.N * dm.w;
+    row_base += c.B + (long long)dm.N * dm.w;
   }
   return cudaGetLastError();
 }

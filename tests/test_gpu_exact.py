@@ -148,3 +148,51 @@ def test_curves_with_jumps_near_the_end_of_fp32():
     for q, B in enumerate(Bs):
         ref, best = _recursion(U, B, T - w)
         assert list(b[q]) == ref and np.float32(val[q]) == best
+
+
+@pytest.mark.parametrize("kind", ["utility", "rough", "falling", "ties", "zero", "steep"])
+@pytest.mark.parametrize("N,T,w,Bs", [
+    (40, 300, 20, [1500, 0, 40 * 280, 7001]),   # several sequences, no budget, all of it
+    (24, 497, 50, [24 * 447 - 1, 63, 5000]),    # more than six blocks of tokens on curves that leave them all
+    (17, 130, 2, [640, 1087]),                  # tokens up to a block's edge
+])
+def test_same_solution_as_the_full_recursion(kind, N, T, w, Bs):
+    """Tokens and budgets that cannot matter are left out, to the bit: the same smallest solution and the same sum, on curves
+    that leave few tokens (utility) and on curves that leave all (ties, zero)."""
+    rng = np.random.default_rng(N + T)
+    n = T - w
+    inc = rng.exponential(size=(N, T)) * np.arange(1, T + 1) ** -rng.uniform(0.2, 1.6, (N, 1))
+    if kind == "rough":
+        inc = rng.exponential(size=(N, T)) * np.where(rng.random((N, T)) < 0.2, 3.0, 1.0)
+    elif kind == "falling":
+        inc = rng.normal(size=(N, T))
+    elif kind == "ties":
+        inc = rng.integers(0, 3, (N, T)).astype(np.float64)
+    elif kind == "zero":
+        inc = np.zeros((N, T))
+    elif kind == "steep":
+        inc *= 1e33
+    U = np.zeros((N, T + 1), np.float32)
+    U[:, 1:] = np.cumsum(inc, axis=1)
+    b, off, val = gpu_exact(N, T, w, U, Bs)
+    for q, B in enumerate(Bs):
+        ref, best = _recursion(U, B, n)
+        assert list(b[q]) == ref and np.float32(val[q]) == best
+    np.testing.assert_array_equal(off, np.concatenate([[0], np.cumsum(b.reshape(-1) + w)]))
+
+
+def test_a_wait_that_runs_out_leaves_no_solution(monkeypatch):
+    """With the test hooks one CTA stores nothing and the wait limit is short: the optimum is no number and the budgets are
+    zero.  The next ordinary call gives the same as a fresh one."""
+    N, T, w, B = 32, 300, 20, 32 * 140
+    U = _rough(np.random.default_rng(9), N, T + 1)
+    ref = gpu_exact(N, T, w, U, [B])
+    monkeypatch.setenv("LUKV_TEST_SPIN_LIMIT", "20000")
+    monkeypatch.setenv("LUKV_TEST_DROP_ITEM", "0")
+    b, off, val = gpu_exact(N, T, w, U, [B])
+    assert np.isnan(val).all() and not b.any()
+    np.testing.assert_array_equal(off, w * np.arange(N + 1))
+    monkeypatch.delenv("LUKV_TEST_SPIN_LIMIT")
+    monkeypatch.delenv("LUKV_TEST_DROP_ITEM")
+    for x, y in zip(gpu_exact(N, T, w, U, [B]), ref):
+        np.testing.assert_array_equal(x, y)
