@@ -234,7 +234,15 @@ __global__ void __launch_bounds__(1024) imp_normalize_kernel(float* __restrict__
   __shared__ double total_s;
   float* base = importance + (size_t)blockIdx.x * count;
   double acc = 0.0;
-  for (long long i = threadIdx.x; i < count; i += blockDim.x) acc += (double)base[i];
+  // four loads at a time: the layer's few warps have nothing else to wait behind
+  constexpr int kAhead = 4;
+  for (long long i0 = threadIdx.x; i0 < count; i0 += kAhead * blockDim.x) {
+    float x[kAhead];
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) x[k] = i0 + k * blockDim.x < count ? base[i0 + k * blockDim.x] : 0.f;
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) acc += (double)x[k];
+  }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
   if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
@@ -247,7 +255,14 @@ __global__ void __launch_bounds__(1024) imp_normalize_kernel(float* __restrict__
   __syncthreads();
   const double total = total_s;
   if (total <= 0.0) return;  // (not a number: the whole layer is none)
-  for (long long i = threadIdx.x; i < count; i += blockDim.x) base[i] = (float)((double)base[i] / total);
+  for (long long i0 = threadIdx.x; i0 < count; i0 += kAhead * blockDim.x) {
+    float x[kAhead];
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) x[k] = i0 + k * blockDim.x < count ? base[i0 + k * blockDim.x] : 0.f;
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k)
+      if (i0 + k * blockDim.x < count) base[i0 + k * blockDim.x] = (float)((double)x[k] / total);
+  }
 }
 
 // LUKV_FORCE_SIMT=1 keeps the value norms on the FP32 pipes (for A/B checks; read at every call).

@@ -11,7 +11,7 @@
 // four accumulator buffers, warp 8 TMA producer, warp 9 tensor memory and MMA issue.  Every wait is bounded and between the
 // warps of one CTA only; should one run out, here or in the value norms, what depends on it becomes NaN.
 // Bound by the exp2 of the epilogue (2 x 2.6e8 for 256 heads x 256 rows x 4000 keys).  Measured there: 1.90 + 1.82 ms
-// on the FP32 pipes, 0.11 + 0.14 ms here.
+// on the FP32 pipes, 0.11 + 0.15 ms here.
 #define LUKV_POLY_SEL1(i) false  // every exp2 on the special-function unit: the values keep their precision
 #include <algorithm>
 
@@ -257,13 +257,21 @@ __global__ void __launch_bounds__(kItThreads, 1)
         }
         bar_sync(1, kItEpiThreads);
         const uint64_t sc2 = pack2(a.scale_log2, a.scale_log2);
+        // value norms of this thread's key: those of the quad's next tile are on their way during a tile
+        float vg[8], vg_next[8];
+        auto fetch_norms = [&](int t) {
+          const int j = (it.t0 + t) * 128 + qtid;
+#pragma unroll
+          for (int g = 0; g < 8; ++g)
+            vg_next[g] = g < a.G && t < it.nt && j < a.n ? __ldg(a.vnorm + ((size_t)it.u * a.G + g) * a.n + j) : 0.f;
+        };
+        fetch_norms((int)(tt & 1) == quad ? 0 : 1);
         for (int t = 0; t < it.nt; ++t, ++tt) {
           if ((int)(tt & 1) != quad) continue;
           const int j = (it.t0 + t) * 128 + qtid;
-          float vg[8];
 #pragma unroll
-          for (int g = 0; g < 8; ++g)
-            vg[g] = g < a.G && j < a.n ? __ldg(a.vnorm + ((size_t)it.u * a.G + g) * a.n + j) : 0.f;
+          for (int g = 0; g < 8; ++g) vg[g] = vg_next[g];
+          fetch_norms(t + 2);
           float best = a.accumulate && j < a.n ? a.importance[(size_t)it.u * a.n + j] : 0.f;  // importance is not negative
           for (int c = 0; c < it.nq; ++c) {
             const uint32_t buf = 2 * quad + (n_use & 1);
