@@ -261,7 +261,7 @@ __device__ __forceinline__ int hull_walk_regs(const float* __restrict__ U, int P
 // ---- long curves: drop the points that lie on or below the chord of their neighbours, until none does ----------------
 
 // Survivors of the first pass that the shared memory of a curve holds; a fifth of the points of a noisy curve survive.
-inline int hull_prune_cap(int P) { return (P * 2 / 5 + 63) & ~63; }
+inline int hull_prune_cap(int P) { return (P * 3 / 10 + 63) & ~63; }
 constexpr int kHullPasses = 48;
 
 // One warp per curve.  A point on or below the chord of two other points is no vertex of the majorant, whichever points
@@ -269,11 +269,13 @@ constexpr int kHullPasses = 48;
 // majorant.  The first pass reads the curve once, into registers, and drops what lies clearly below the chord of the points
 // 1, 2, 4, 8 or 16 places to either side (4001 points: about 800 stay); the survivors (value and index) are compacted in
 // shared memory and tested against their neighbours, exactly, until none is dropped (9 passes over 1900 points in all, 53
-// stay).  A curve of which more than two fifths survive the first pass, or that needs more than kHullPasses, is left to
+// stay).  A curve of which more than three tenths survive the first pass, or that needs more than kHullPasses, is left to
 // hull_dense_kernel (count -1).  Blocks beyond the last positive slope are one block of gain 0.
-// Bound by the latency of a warp's own instructions at 21 warps per SM (9600 bytes of shared memory each): 57 % of the issue
-// slots are used.  7680 curves of 4001 points: 3.07 ms as one serial stack walk per curve, 0.31 ms as a walk from
-// vertex to vertex over chunk maxima, 0.22 ms with neighbours alone in the first pass, 0.15 ms now.
+// Bound by the latency of a warp's own instructions at 27 warps per SM (7300 bytes of shared memory each; the 52 curves of an SM
+// are two rounds).  7680 curves of 4001 points: 3.07 ms as one serial stack walk per curve, 0.31 ms as a walk from
+// vertex to vertex over chunk maxima, 0.22 ms with neighbours alone in the first pass, 0.157 ms with room
+// for two fifths of the points (21 warps per SM, three rounds); the profile build 243 us with that and a dense-hull CTA per
+// curve, 227 now.
 __global__ void __launch_bounds__(32) hull_prune_kernel(const float* __restrict__ curves, HullLists lists, int P, int cap) {
   extern __shared__ float hull_smem[];
   const int hid = blockIdx.x, lane = threadIdx.x;
@@ -345,12 +347,8 @@ inline size_t hull_dense_smem_bytes(int P) { return (size_t)P * 4 + (size_t)hull
 // hulls are joined pairwise, five times: the block across the joint absorbs blocks from the left while their mean does
 // not exceed its own and from the right while its own does not exceed theirs, which is where the serial algorithm ends
 // up as well (the projection is unique).
-__global__ void hull_dense_kernel(const float* __restrict__ curves, HullLists lists, int P) {
-  extern __shared__ float hull_smem[];
-  const int hid = blockIdx.x, lane = threadIdx.x;
-  pdl_launch_dependents();
-  pdl_wait();
-  if (lists.count[hid] >= 0) return;  // the kernel before took this curve
+__device__ __noinline__ void hull_dense_curve(const float* __restrict__ curves, const HullLists& lists, int P, int hid,
+                                              float* hull_smem, int lane) {
   const float* U = curves + (size_t)hid * P;
   const int run = hull_run(P);
   float* Us = hull_smem;
@@ -483,6 +481,21 @@ __global__ void hull_dense_kernel(const float* __restrict__ curves, HullLists li
     s_out[i] = (unsigned short)l;
   }
   if (lane == 0) lists.count[hid] = total;
+}
+// One warp looks at up to 32 curves at a time, `gridDim` apart, for those that the kernel before left.
+__global__ void __launch_bounds__(32) hull_dense_kernel(const float* __restrict__ curves, HullLists lists, int P, int n_curves) {
+  extern __shared__ float hull_smem[];
+  const int lane = threadIdx.x, step = gridDim.x;
+  pdl_launch_dependents();
+  pdl_wait();
+  for (long long base = blockIdx.x; base < n_curves; base += 32LL * step) {
+    const long long mine = base + (long long)lane * step;
+    uint32_t todo = __ballot_sync(0xffffffffu, mine < n_curves && lists.count[mine] < 0);
+    for (; todo; todo &= todo - 1) {
+      __syncwarp();
+      hull_dense_curve(curves, lists, P, (int)(base + (long long)(__ffs(todo) - 1) * step), hull_smem, lane);
+    }
+  }
 }
 
 constexpr int kHullRegsMaxP = 32 * 17;
@@ -1099,8 +1112,10 @@ cudaError_t launch_hull(const float* curves, const HullLists& out, int64_t n_cur
   const int cap = hull_prune_cap(P);
   hull_prune_kernel<<<grid, 32, (size_t)cap * 6, lc.st>>>(curves, out, P, cap);
   lc.mark("hull_prune");
-  const cudaError_t e = launch_pdl(hull_dense_kernel, dim3(grid), dim3(32), hull_dense_smem_bytes(P), lc.st, true, curves,
-                                   out, P);  // at most 25 KB
+  // as many warps as the chip holds at 25 KB each: all curves may be left to it, most often none is
+  const unsigned dense = std::min(grid, 9u * 148u);
+  const cudaError_t e = launch_pdl(hull_dense_kernel, dim3(dense), dim3(32), hull_dense_smem_bytes(P), lc.st, true, curves,
+                                   out, P, (int)n_curves);
   if (e != cudaSuccess) return e;
   lc.mark("hull_dense");
   return cudaGetLastError();
