@@ -214,7 +214,9 @@ static SideStream* side_stream() {
 
 // The whole path.  Allocation depends only on the curves, scoring only on Q/K; selection needs both, the gather follows.
 // With `overlap` allocation runs beside the scorer.  Up to 32 heads: one CTA per sequence, on the caller's stream, behind a
-// persistent scorer (tensor-core, KeyDiff), which leaves it an SM, or ahead of the general-shape scorer's first sweep;
+// persistent scorer (tensor-core, KeyDiff), which leaves it an SM, behind the general-shape scorer where that has a CTA per
+// SM at most and so room for its sweeps and the allocation at once (4 heads x 1024 keys: 18.2 us a call, 20.5 with the
+// allocation ahead, whose time is longer than the first sweep's), or else ahead of its first sweep;
 // neighbours in the stream are programmatic dependents, and whichever of scorer and allocation comes second ends after the
 // first, so that the selection, which waits for the second, sees both.  More heads: hulls and greedy on an auxiliary
 // stream, whose hulls take the SMs before the scorer does (256 heads x 513 points with 1536 keys: 87 us a call; hulls by
@@ -229,9 +231,10 @@ static int run_compress(const Dims& dm, const void* q_win, const void* k, const 
     auto allocate = [&](bool beside) {
       return launch_allocate_small(dm, curves, budgets_in, budgets, offsets, beside, lc);
     };
-    if (!persistent && allocate(false) != cudaSuccess) return LUKV_ERR_CUDA;
-    if (run_score(dm, q_win, k, w, 1, true, lc) != cudaSuccess) return LUKV_ERR_CUDA;
-    if (persistent && allocate(true) != cudaSuccess) return LUKV_ERR_CUDA;
+    const bool behind = persistent || dm.heads() * score_chunks(dm) <= 148;
+    if (!behind && allocate(false) != cudaSuccess) return LUKV_ERR_CUDA;
+    if (run_score(dm, q_win, k, w, 1, !behind, lc) != cudaSuccess) return LUKV_ERR_CUDA;
+    if (behind && allocate(true) != cudaSuccess) return LUKV_ERR_CUDA;
     chained = true;
   } else if (SideStream* side = overlap ? side_stream() : nullptr) {
     std::lock_guard<std::mutex> in_use(side->use);
