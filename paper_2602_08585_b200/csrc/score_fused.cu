@@ -92,7 +92,7 @@ struct FusedArgs {
   int lse_rows;        // M rounded up to a multiple of 4
   int nheads;
   int item_tiles, items_per_head, tiles_T, tiles_n;
-  int adapt_items;     // host only: let the launcher pick a multiple of item_tiles
+  int adapt_items;     // host only: let the launcher pick a number of tiles from item_tiles on
   int npad;            // pass 2: query rows rounded up to a multiple of 32 (MMA N and columns read)
   int lag;             // 2..kMaxLag: pass 1 of item k+lag-1 precedes pass 2 of item k
   int l2_hints;        // 1: pass-1 key loads ask L2 to keep the lines, pass-2 loads to drop them first
@@ -641,9 +641,12 @@ cudaError_t launch_fused(const CUtensorMap& qm, const CUtensorMap& km, FusedArgs
     // per-item overhead); measured on 256 heads x 256 tiles and 148 CTAs: 0.89 ms with 8 tiles per item,
     // 0.84 with 16, 0.82 with 32, 0.81 with 64.  The price of large items is that pass 2 no longer finds all its key
     // tiles in L2; the kernel is bound by the exp2 unit, not by HBM, so re-reading part of K costs nothing.
+    // Any number of tiles is tried where all sequences have one length (a head's items are then as long as one another but for
+    // the last): 8 heads x 64 tiles 41.3 us a call with 8 and 35.3 with 4, 24 x 64 62.5 with 16 and 55 with 6, 48 x 32 (two row
+    // blocks) 89 with 16 and 77 with 6, 128 x 157 357 with 16 and 343 with 20.
     int best = args.item_tiles;
     double best_cost = 1e30;
-    for (int it = args.item_tiles; it <= 8 * args.item_tiles; it *= 2) {
+    for (int it = args.item_tiles; it <= 64; it = RAGGED ? 2 * it : it + 1) {
       const long long per_head = (args.tiles_T + it - 1) / it;
       const long long items = (long long)args.nheads * per_head;
       const long long ctas = items < sms ? items : sms;
@@ -695,17 +698,17 @@ void score_test_hooks(uint32_t* spin_limit, int* drop_item) {
   *drop_item = (drop && d >= 0 && d <= (1L << 30)) ? (int)d : -1;
 }
 
-// Key tiles per work item (the smallest the scorer uses; it grows for very long contexts).  Items of two tiles where eight
-// leave SMs without one are faster (8 heads x 8192 keys: 17.3 us instead of 23.4), but a row's sum is then added up in
-// another order, which changes the last bits of the scores and so, where two scores nearly tie, the kept positions.
-// LUKV_ITEM_TILES (1..64) overrides the default for tuning runs.
-int score_item_tiles() {
-  static const int v = env_int("LUKV_ITEM_TILES", 1, 64, 8);
-  return v;
+// Fewest key tiles per work item the launcher tries (it grows for very long contexts): eight, or two where items of eight
+// are fewer than two per SM.  The 148 is the chip this library is built for: the workspace depends on it.
+// LUKV_ITEM_TILES (1..64) overrides it for tuning runs.
+int score_item_tiles(const Dims& dm) {
+  static const int v = env_int("LUKV_ITEM_TILES", 1, 64, 0);
+  if (v) return v;
+  return dm.heads() * (((dm.T + kTileKeys - 1) / kTileKeys + 7) / 8) < 2 * 148 ? 2 : 8;
 }
 // Bytes of pass-1 partials the tensor-core scorer may write for these sizes.
 size_t score_tc_stats_bytes(const Dims& dm) {
-  const size_t tiles = ((size_t)dm.T + kTileKeys - 1) / kTileKeys, least = score_item_tiles();
+  const size_t tiles = ((size_t)dm.T + kTileKeys - 1) / kTileKeys, least = score_item_tiles(dm);
   return (size_t)dm.heads() * ((tiles + least - 1) / least) * 256 * sizeof(float);
 }
 // Bytes of the block that must be zero at launch: [heads] counters, the status word, then [heads][lse_rows][2] floats.
@@ -747,7 +750,7 @@ cudaError_t launch_score_tc(const Dims& dm, const void* q, const void* k, const 
   args.lse_rows = (dm.M + 3) & ~3;
   args.nheads = (int)dm.heads();
   args.tiles_T = (dm.T + kTileKeys - 1) / kTileKeys;
-  args.item_tiles = score_item_tiles();
+  args.item_tiles = score_item_tiles(dm);
   args.adapt_items = getenv("LUKV_ITEM_TILES") ? 0 : 1;
   args.tiles_n = (dm.n + kTileKeys - 1) / kTileKeys;
   args.items_per_head = 0;  // set by the launcher

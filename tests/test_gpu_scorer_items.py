@@ -49,3 +49,16 @@ def test_items_of_one_tile(S, L, H, G, d, w, kp, lens):
             ref = _reference(q[s].reshape(L * H, G * w, d)[u], k[s].reshape(L * H, T, d)[u], n + w, w, kp)
             err = (first[s, u, :n].double() - ref).abs()
             assert bool((err <= SCORE_RTOL * ref + SCORE_ATOL).all()), (s, u, float((err / ref).max()))
+
+
+@pytest.mark.parametrize("S,L,H,G,d,w,kp,lens", [
+    (1, 1, 2, 4, 128, 32, 7, [300]),          # three tiles in items of two: a job of one tile
+    (1, 1, 8, 4, 128, 32, 7, [8192]),         # 64 tiles in items of four
+    (1, 3, 8, 4, 64, 32, 7, [8320]),          # 65 tiles in eleven items of five or six
+    (1, 2, 4, 8, 128, 32, 5, [1999]),         # two row blocks, 16 tiles
+    (1, 1, 2, 4, 128, 16, 5, [40000]),        # 313 tiles of two heads, items of different sizes
+    (3, 1, 4, 4, 128, 32, 7, [3000, 640, 1000]), (5, 3, 8, 2, 64, 16, 7, [9000, 4125, 250, 7000, 875]),
+])
+def test_items_of_a_small_call(S, L, H, G, d, w, kp, lens):
+    """Calls with few heads share a head out over more and smaller items, of sizes that differ by one tile."""
+    test_items_of_one_tile(S, L, H, G, d, w, kp, lens)
