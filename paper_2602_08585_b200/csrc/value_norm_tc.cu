@@ -143,8 +143,10 @@ __global__ void __launch_bounds__(kVnThreads, 1)
   if (a.flags) {  // most often nothing is left to do
     int any = 0;
     for (long long k = threadIdx.x; blockIdx.x + (k >> 3) * gridDim.x < a.items; k += kVnThreads) {
-      const uint4 f = reinterpret_cast<const uint4*>(a.flags)[(blockIdx.x + (k >> 3) * gridDim.x) * 8 + (k & 7)];
-      any |= (f.x | f.y | f.z | f.w) != 0;  // entries past a head's last tile hold anything: the items look again
+      const long long idx = blockIdx.x + (k >> 3) * gridDim.x;
+      const int left = (a.n - (int)(idx % a.chunks) * kVnChunkRows + kVnRowTile - 1) / kVnRowTile - 4 * (int)(k & 7);
+      const uint4 f = reinterpret_cast<const uint4*>(a.flags)[idx * 8 + (k & 7)];  // a word per tile; those past the last hold anything
+      any |= (left > 0 && f.x) | (left > 1 && f.y) | (left > 2 && f.z) | (left > 3 && f.w);
     }
     if (!__syncthreads_or(any)) return;
   }
