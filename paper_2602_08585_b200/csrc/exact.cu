@@ -136,9 +136,11 @@ struct __align__(16) DpRow {
 };
 
 // Row h at the 64 budgets from x0 on (those in [lo, hi]) over `blocks` blocks of b.  Blocks and tokens count from the first
-// staged block; the staged values start 64 `blocks` budgets below what tile 0 reaches with the first token.
+// staged block; the staged values start 64 `blocks` budgets below what tile 0 reaches with the first token.  Of a row of few
+// blocks, `parts` warps can share a tile (part_s: room for 64 values each).
 __device__ __forceinline__ void dp_tile(const unsigned char* F2, const float* f_runs, const unsigned char* U2,
-                                        const float4* u_runs, const DpRow& row, int tile, int x0, float* next, int lane) {
+                                        const float4* u_runs, const DpRow& row, int tile, int x0, float* next, int lane,
+                                        int part, int parts, float* part_s) {
   const int xg = lane & 7, bg = lane >> 3, blocks = row.blocks, lo = row.lo, hi = row.hi;
   // a sum of two bounds, plus what the rounding of their terms can take away (a few roundings of 2^-24 each)
   auto sum_up = [](float f, float u) { return f + u > -INFINITY ? f + u + 4e-7f * (fabsf(f) + fabsf(u)) : -INFINITY; };
@@ -221,8 +223,20 @@ __device__ __forceinline__ void dp_tile(const unsigned char* F2, const float* f_
   if (blocks <= kDpFewBlocks) {
     // few tokens: all of them (bounds would take longer)
 #pragma unroll 1
-    for (int i = row.halves & 255; i < row.halves >> 8; ++i) evaluate(i >> 1, i & 1);
+    for (int i = (row.halves & 255) + part; i < row.halves >> 8; i += parts) evaluate(i >> 1, i & 1);
     merge();
+    if (parts > 1) {
+      float2* mine = reinterpret_cast<float2*>(part_s + part * kDpX + xl);
+      *mine = make_float2(best[0], best[1]);
+      bar_sync(1 + tile, 32 * parts);
+      if (part > 0) return;
+#pragma unroll 1
+      for (int i = 1; i < parts; ++i) {
+        const float2 o = mine[i * (kDpX / 2)];
+        best[0] = fmaxf(best[0], o.x);
+        best[1] = fmaxf(best[1], o.y);
+      }
+    }
   } else {
     // Any slope gives true bounds; that of the previous row at the same budgets gives close ones.
     const unsigned char* own = F2 + (blocks + tile) * (kDpX / 8) * kDpGroup;
@@ -493,6 +507,7 @@ __global__ void __launch_bounds__(256) dp_clear_kernel(const DpArgs a, int4* row
 __global__ void __launch_bounds__(kDpThreads, 1) dp_rows_kernel(const DpArgs a) {
   extern __shared__ __align__(16) unsigned char dp_smem[];
   __shared__ int next_tile;
+  __shared__ __align__(16) float part_s[kDpWarps * kDpX];
   const DpPlan plan = dp_plan(a.n, a.N);
   unsigned char* F2 = dp_smem;                                       // packed pairs (f(y + 16), f(y))
   float* f_runs = reinterpret_cast<float*>(dp_smem + plan.runs_off);
@@ -501,17 +516,18 @@ __global__ void __launch_bounds__(kDpThreads, 1) dp_rows_kernel(const DpArgs a) 
   for (int i = threadIdx.x; i < min(a.N, kDpTable); i += kDpThreads) table[i] = dp_row(a, i);
   __syncthreads();
   auto row_of = [&](int h) { return h < kDpTable ? table[h] : dp_row(a, h); };
-  auto fetch_curve = [&](int h, const DpRow& r, int buf) {  // the blocks that the row needs
+  auto fetch_curve = [&](int h, const DpRow& r, int buf, int warp0) {  // the blocks that the row needs, by warps from warp0 on
+    const int tid0 = threadIdx.x - 32 * warp0, threads = kDpThreads - 32 * warp0;
     unsigned char* U2 = dp_smem + plan.u_off + buf * plan.u_bytes;
     const float* U = a.curves + (size_t)h * a.P + r.blk0 * kDpX;
     const int last = a.n - r.blk0 * kDpX;
-    for (int b = threadIdx.x; b < r.blocks * kDpX; b += kDpThreads) {
+    for (int b = tid0; b < r.blocks * kDpX; b += threads) {
       unsigned char* to = U2 + (b >> 5) * 128 + (b & 15) * 8 + ((b >> 4) & 1) * 4;  // pairs (U(b), U(b + 16))
       if (b <= last) cp_async4(to, U + b);
       else *reinterpret_cast<float*>(to) = -INFINITY;
     }
     float* ur = reinterpret_cast<float*>(dp_smem + plan.u_runs_off) + buf * plan.blocks * 4;
-    for (int i = threadIdx.x; i < r.blocks * 4; i += kDpThreads)
+    for (int i = tid0; i < r.blocks * 4; i += threads)
       cp_async4(ur + i, a.u_runs + (size_t)h * kDpURuns + r.blk0 * 4 + i);
   };
   auto next_row = [&](int h) {  // the next row from h on of which this CTA has a part
@@ -522,9 +538,9 @@ __global__ void __launch_bounds__(kDpThreads, 1) dp_rows_kernel(const DpArgs a) 
     return h;
   };
   int h = next_row(0), buf = 0;
-  if (h < a.N) fetch_curve(h, row_of(h), 0);
+  if (h < a.N) fetch_curve(h, row_of(h), 0, 0);
 
-  for (int h_next; h < a.N; h = h_next, buf ^= 1) {
+  for (int h_next = a.N; h < a.N; h = h_next, buf ^= 1) {
     const DpRow row = row_of(h);
     const int old_lo = h > 0 ? row_of(h - 1).lo : 0, old_hi = h > 0 ? row_of(h - 1).hi : 0;
     const int tile0 = row.tile0 + cta * row.per, tiles = min(row.per, row.tiles - cta * row.per);
@@ -588,16 +604,34 @@ __global__ void __launch_bounds__(kDpThreads, 1) dp_rows_kernel(const DpArgs a) 
       }
       __syncthreads();
 
-      // tiles differ in what they have to look at: warps take them as they come
-      for (int tile = warp; tile < n_sub;) {
-        dp_tile(F2, f_runs, U2, u_runs, row, tile, xs + tile * kDpX, cta != a.drop ? next : nullptr, lane);
-        if (n_sub <= kDpWarps) break;
-        if (lane == 0) tile = atomicAdd(&next_tile, 1);
-        tile = __shfl_sync(0xffffffffu, tile, 0);
+      // several warps to a tile where there are few, one warp to several tiles (as they come: they differ in what there is to
+      // look at) where there are many; warps without one fetch the next curve at once
+      const int halves = (row.halves >> 8) - (row.halves & 255);
+      const int parts = row.blocks <= kDpFewBlocks ? max(1, min(kDpWarps / n_sub, halves)) : 1, busy = n_sub * parts;
+      if (busy <= kDpWarps) {
+        const bool last = t_sub + n_sub == tiles;
+        if (warp < busy) {
+          const int tile = warp / parts;
+          dp_tile(F2, f_runs, U2, u_runs, row, tile, xs + tile * kDpX, cta != a.drop ? next : nullptr, lane,
+                  warp - tile * parts, parts, part_s + tile * parts * kDpX);
+        }
+        if (last) {
+          h_next = next_row(h + 1);
+          const int from = busy < kDpWarps ? busy : 0;
+          if (h_next < a.N && warp >= from) fetch_curve(h_next, row_of(h_next), buf ^ 1, from);
+        }
+      } else {
+        for (int tile = warp; tile < n_sub;) {
+          dp_tile(F2, f_runs, U2, u_runs, row, tile, xs + tile * kDpX, cta != a.drop ? next : nullptr, lane, 0, 1, part_s);
+          if (lane == 0) tile = atomicAdd(&next_tile, 1);
+          tile = __shfl_sync(0xffffffffu, tile, 0);
+        }
+        if (t_sub + n_sub == tiles) {
+          h_next = next_row(h + 1);
+          if (h_next < a.N) fetch_curve(h_next, row_of(h_next), buf ^ 1, 0);
+        }
       }
     }
-    h_next = next_row(h + 1);
-    if (h_next < a.N) fetch_curve(h_next, row_of(h_next), buf ^ 1);
   }
 }
 
@@ -629,7 +663,7 @@ __global__ void __launch_bounds__(kDpBackThreads) dp_backtrack_kernel(const DpAr
   int x = B;
   float target = __ldg(a.f + (size_t)(N - 1) * a.stride + B);
   if (tid == 0) values[q] = (double)target;
-  auto touch = [](const float* p) { asm volatile("{\n\t.reg .f32 t;\n\tld.global.ca.f32 t, [%0];\n\t}" ::"l"(p)); };
+  auto touch = [](const float* p) { asm volatile("{\n\t.reg .f32 t;\n\tld.global.nc.f32 t, [%0];\n\t}" ::"l"(p)); };
   int4 row = __ldg(a.rows + N - 1);
   for (int h = N - 1; h >= 0; --h) {
     const int4 old = h > 0 ? __ldg(a.rows + h - 1) : make_int4(0, 0, 0, 0);
