@@ -12,7 +12,7 @@
 //           exp2(x - lse_row) over all rows in registers -> the un-pooled score of the key
 // Both operand tiles are K-major, so the same shared-memory tiles serve as A or B.
 //
-// Work item = (head, run of item_tiles key tiles).  Items are dealt round-robin to a grid of
+// Work item = (head, run of at most item_tiles key tiles).  Items are dealt round-robin to a grid of
 // at most one CTA per SM, launched cooperatively (all CTAs resident).  A CTA runs pass 1
 // lag-1 items ahead of pass 2, so that the log-sum-exp of a head is normally complete before
 // pass 2 needs it.  With small items the key tiles pass 2 re-reads are still in L2 (K crosses
@@ -92,6 +92,7 @@ struct FusedArgs {
   int lse_rows;        // M rounded up to a multiple of 4
   int nheads;
   int item_tiles, items_per_head, tiles_T, tiles_n;
+  uint32_t iph_magic;  // div_magic(items_per_head)
   int adapt_items;     // host only: let the launcher pick a number of tiles from item_tiles on
   int npad;            // pass 2: query rows rounded up to a multiple of 32 (MMA N and columns read)
   int lag;             // 2..kMaxLag: pass 1 of item k+lag-1 precedes pass 2 of item k
@@ -100,7 +101,8 @@ struct FusedArgs {
   // sequences of different lengths in one launch (RAGGED kernels): seq_T[q] = context length of sequence q,
   // seq_item0[q] = number of its first work item; heads_per_seq heads each.  The uniform fields above then hold
   // the maxima (strides and capacities).  The tables travel by value in the launch arguments.
-  int seq_T[kMaxRaggedSeqs], seq_item0[kMaxRaggedSeqs];
+  int seq_T[kMaxRaggedSeqs], seq_item0[kMaxRaggedSeqs], seq_iph[kMaxRaggedSeqs];
+  uint32_t seq_magic[kMaxRaggedSeqs];  // div_magic(seq_iph)
   int n_seq, heads_per_seq, total_items;
   int T_stride, n_stride;  // rows between consecutive heads in K and in the raw scores
   uint32_t spin_limit; // iterations a wait may take
@@ -117,36 +119,51 @@ struct Job {
   bool p2;
 };
 
+// Quotients by a number of items without a division: that would go through the special-function unit, where it would queue
+// behind the exponentials of the epilogue, and every role works its job out when it changes jobs (128 heads x 157 tiles, 14 jobs a
+// CTA: 367 us a call with three divisions a job, 347 with none).  Exact while dividend times divisor stays below 2^32.
+__host__ __device__ inline uint32_t div_magic(int d) { return d > 1 ? (uint32_t)((1ull << 32) / (uint32_t)d) + 1u : 0u; }
+__device__ __forceinline__ int div_by(int x, uint32_t magic) { return magic ? (int)__umulhi((uint32_t)x, magic) : x; }
+
 template <bool RAGGED>
 __device__ __forceinline__ Job make_job(int k, bool p2, const FusedArgs& a) {
   Job j;
   j.p2 = p2;
   const int item = (int)blockIdx.x + k * (int)gridDim.x;
-  int tiles_T = a.tiles_T, tiles_n = a.tiles_n;
-  if (!RAGGED) {
-    j.n = a.n;
-    j.iph = a.items_per_head;
-    const int hu = item / a.items_per_head;
-    j.c = item - hu * a.items_per_head;
-    j.u = hu;
-  } else {
+  int tiles_T = a.tiles_T, tiles_n = a.tiles_n, local = item, head0 = 0;
+  uint32_t magic = a.iph_magic;
+  j.n = a.n;
+  j.iph = a.items_per_head;
+  if (RAGGED) {
     int lo = 0, hi = a.n_seq;  // the sequence whose items contain `item`
     while (hi - lo > 1) {
       const int mid = (lo + hi) >> 1;
       if (a.seq_item0[mid] <= item) lo = mid; else hi = mid;
     }
-    const int2 sq = make_int2(a.seq_T[lo], a.seq_item0[lo]);
-    j.n = sq.x - a.w;
-    tiles_T = (sq.x + kTileKeys - 1) / kTileKeys;
+    j.n = a.seq_T[lo] - a.w;
+    tiles_T = (a.seq_T[lo] + kTileKeys - 1) / kTileKeys;
     tiles_n = (j.n + kTileKeys - 1) / kTileKeys;
-    j.iph = (tiles_T + a.item_tiles - 1) / a.item_tiles;
-    const int local = item - sq.y, hu = local / j.iph;
-    j.c = local - hu * j.iph;
-    j.u = lo * a.heads_per_seq + hu;
+    j.iph = a.seq_iph[lo];
+    magic = a.seq_magic[lo];
+    local = item - a.seq_item0[lo];
+    head0 = lo * a.heads_per_seq;
   }
-  j.tile0 = j.c * a.item_tiles;
-  const int lim = p2 ? tiles_n : tiles_T;
-  j.ntiles = max(0, min(a.item_tiles, lim - j.tile0));
+  const int hu = div_by(local, magic);
+  j.c = local - hu * j.iph;
+  j.u = head0 + hu;
+  int end;
+  if (RAGGED) {
+    // a head's items differ by one tile at most: with full items and a short last one a CTA could be dealt the long ones every
+    // time (eight sequences of 1750 to 16000 keys: 1493 us a call with full items, 1438 so)
+    const int base = div_by(tiles_T, magic), rest = tiles_T - base * j.iph;
+    j.tile0 = j.c * base + min(j.c, rest);
+    end = j.tile0 + base + (j.c < rest ? 1 : 0);
+  } else {
+    // where all heads are alike the short items fall to all CTAs (128 x 157 tiles: 343 us a call, 347 with equal items)
+    j.tile0 = j.c * a.item_tiles;
+    end = min(j.tile0 + a.item_tiles, tiles_T);
+  }
+  j.ntiles = max(0, (p2 ? min(end, tiles_n) : end) - j.tile0);
   return j;
 }
 
@@ -623,6 +640,39 @@ __global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
 
 // ---- host side --------------------------------------------------------------------------------
 
+// Tiles, and one more per item, of the CTA with the most of them, when the items of `groups` groups of heads (heads each, T[g]
+// keys long, at most `it` tiles an item) are dealt to `ctas` CTAs in turn.
+double deal_cost(const int32_t* T, int groups, int heads, int it, int ctas) {
+  constexpr int kMaxCtas = 256;
+  constexpr double kItem = 1.05;
+  double step[kMaxCtas + 1] = {};  // what a group's last, incomplete round adds: differences from CTA to CTA
+  if (ctas > kMaxCtas) ctas = kMaxCtas;
+  double base = 0.0;
+  int first = 0;  // the CTA that gets the group's first item
+  for (int g = 0; g < groups; ++g) {
+    const long long tiles = (T[g] + kTileKeys - 1) / kTileKeys, per_head = (tiles + it - 1) / it, items = heads * per_head;
+    const double time = (double)tiles / (double)per_head + kItem;
+    const int rest = (int)(items % ctas);
+    base += time * (double)(items / ctas);
+    if (rest) {
+      step[first] += time;
+      if (first + rest <= ctas) {
+        step[first + rest] -= time;
+      } else {
+        step[0] += time;
+        step[first + rest - ctas] -= time;
+      }
+      first = (first + rest) % ctas;
+    }
+  }
+  double run = 0.0, most = 0.0;
+  for (int c = 0; c < (groups > 1 ? ctas : 1); ++c) {
+    run += step[c];
+    if (run > most) most = run;
+  }
+  return base + most;
+}
+
 template <int MT, int NQ, int NH, bool RAGGED = false>
 cudaError_t launch_fused(const CUtensorMap& qm, const CUtensorMap& km, FusedArgs args, int spare_sms, LaunchCtx& lc,
                          const int32_t* seq_T_host = nullptr) {
@@ -636,21 +686,17 @@ cudaError_t launch_fused(const CUtensorMap& qm, const CUtensorMap& km, FusedArgs
   // A CTA runs pass 1 of later items before pass 2 of the current one, so a head's items must
   // not outnumber the CTAs (else a CTA would wait for partials that it is due to produce itself).
   if (args.adapt_items) {
-    // Larger work items mean fewer job changes and fewer partials to fold per head, but coarser dealing.
-    // A CTA's critical path is its number of items times (tiles per item + about one tile's time of
-    // per-item overhead); measured on 256 heads x 256 tiles and 148 CTAs: 0.89 ms with 8 tiles per item,
-    // 0.84 with 16, 0.82 with 32, 0.81 with 64.  The price of large items is that pass 2 no longer finds all its key
-    // tiles in L2; the kernel is bound by the exp2 unit, not by HBM, so re-reading part of K costs nothing.
-    // Any number of tiles is tried where all sequences have one length (a head's items are then as long as one another but for
-    // the last): 8 heads x 64 tiles 41.3 us a call with 8 and 35.3 with 4, 24 x 64 62.5 with 16 and 55 with 6, 48 x 32 (two row
-    // blocks) 89 with 16 and 77 with 6, 128 x 157 357 with 16 and 343 with 20.
+    // Larger work items mean fewer job changes and fewer partials to fold per head, but coarser dealing.  The time is that of
+    // the CTA with the most to do: its tiles and about one tile's time per item (256 heads x 256 tiles on 148 CTAs: 0.89 ms with
+    // 8 tiles per item, 0.84 with 16, 0.82 with 32, 0.81 with 64).  The price of large items is that pass 2 no longer finds all
+    // its key tiles in L2; the kernel is bound by the exp2 unit, not by HBM, so re-reading part of K costs nothing.
+    // Any number of tiles up to 64 is tried: 8 heads x 64 tiles 41.3 us a call with 8 and 35.7 with 4, 24 x 64 61.6 with 16 and
+    // 55 with 6, 48 x 32 (two row blocks) 89 with 16 and 76 with 6.
     int best = args.item_tiles;
     double best_cost = 1e30;
-    for (int it = args.item_tiles; it <= 64; it = RAGGED ? 2 * it : it + 1) {
-      const long long per_head = (args.tiles_T + it - 1) / it;
-      const long long items = (long long)args.nheads * per_head;
-      const long long ctas = items < sms ? items : sms;
-      const double cost = (double)((items + ctas - 1) / ctas) * (it + 1.05);
+    for (int it = args.item_tiles; it <= 64; ++it) {
+      const double cost = RAGGED ? deal_cost(seq_T_host, args.n_seq, args.heads_per_seq, it, sms)
+                                 : deal_cost(&args.T, 1, args.nheads, it, sms);
       if (cost < best_cost * 0.995) {
         best_cost = cost;
         best = it;
@@ -660,6 +706,7 @@ cudaError_t launch_fused(const CUtensorMap& qm, const CUtensorMap& km, FusedArgs
   }
   while ((args.tiles_T + args.item_tiles - 1) / args.item_tiles > sms) ++args.item_tiles;
   args.items_per_head = (args.tiles_T + args.item_tiles - 1) / args.item_tiles;
+  args.iph_magic = div_magic(args.items_per_head);
   int total_items = args.nheads * args.items_per_head;
   if (RAGGED) {
     int base = 0;
@@ -667,7 +714,9 @@ cudaError_t launch_fused(const CUtensorMap& qm, const CUtensorMap& km, FusedArgs
       args.seq_T[q] = seq_T_host[q];
       args.seq_item0[q] = base;
       const int tiles = (seq_T_host[q] + kTileKeys - 1) / kTileKeys;
-      base += args.heads_per_seq * ((tiles + args.item_tiles - 1) / args.item_tiles);
+      args.seq_iph[q] = (tiles + args.item_tiles - 1) / args.item_tiles;
+      args.seq_magic[q] = div_magic(args.seq_iph[q]);
+      base += args.heads_per_seq * args.seq_iph[q];
     }
     total_items = base;
   }
