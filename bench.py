@@ -204,15 +204,6 @@ def measured_peak():
         return FALLBACK_HBM_GBS, "fallback"
 
 
-def bf16_peak_tflops():
-    """Measured dense bf16 rate of a kernel timed alone (burst), else the earlier measurement on this machine."""
-    try:
-        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as f:
-            return float(json.load(f)["bf16_tflops"])
-    except Exception:
-        return 1590.0
-
-
 def kernel_bytes(name, wl, rows):
     """Algorithmic bytes one launch of a kernel must move (inputs read once + outputs written once)."""
     es = 2 if wl.dtype == "bf16" else 4

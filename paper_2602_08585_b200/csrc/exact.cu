@@ -19,11 +19,12 @@
 //   - all rows in one launch: a CTA keeps its part of the row before and the curve in shared memory and polls the values that
 //     others compute themselves, so that a row costs one trip through L2.
 // The values are those of the full recursion wherever its solutions pass, bit for bit.
-// What bounds it now: the latency of a row (2.9 us: store, poll, two barriers and a tile's 2000 to 4000 dependent clocks) and
+// What bounds it now: the latency of a row (2.7 us: store, poll, two barriers and a tile's dependent clocks) and
 // of the walk back (0.6 us a head).  256 heads x 3968 tokens, B = 304742: 57.2 ms with every pair evaluated one by one and the
 // argmax kept; 3.95 ms with bounds and a launch per row; 2.7 + 0.4 ms in one launch over all budgets, its parts signalled by
-// flags; 1.0 ms now, of which the greedy solution takes 0.09, the rows 0.74 and the walk 0.17.  CTAs of at least ten tiles
-// instead of two 1171 us, five 1070; the curve's tokens read from L2 in the walk 1.7 us a head.
+// flags; 0.99 ms over what can matter (greedy solution 0.09, rows 0.74, walk 0.17); 0.95 ms now, with several warps to a tile of
+// a narrow row.  CTAs of at least ten tiles instead of two 1171 us, five 1070 (before that); the curve's tokens read from L2 in
+// the walk 1.7 us a head.
 #include <math.h>
 
 #include <algorithm>
