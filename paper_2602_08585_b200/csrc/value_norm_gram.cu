@@ -222,18 +222,23 @@ __global__ void __launch_bounds__(kGmThreads, 1)
     // two quads of warps take alternate tiles: a quad alone is slower than the MMAs
     const int quad = warp & 3, parity = (warp - 4) >> 2, row = 32 * quad + lane;
     const uint32_t lane_addr = (uint32_t)(32 * quad) << 16;
-    uint32_t tt = 0, it = 0, vs = 0;
+    uint32_t tt = 0, it = 0, vs = 0, vph = 0;
     bool ok = true;
     for (int idx = blockIdx.x; idx < a.items && ok; idx += gridDim.x, ++it) {
       const int slice = idx / a.items_per_slice, t0 = (idx % a.items_per_slice) * a.per_item;
       const int t1 = min(t0 + a.per_item, all_tiles);
       const int uh = slice / a.G, g = slice - uh * a.G;
       for (int t = t0; t < t1; ++t, ++tt) {
-        const uint32_t stage = vs;
-        if (++vs == P::kVStages) vs = 0;
+        const uint32_t stage = vs, stage_ph = vph;
+        if (++vs == P::kVStages) vs = 0, vph ^= 1;
         if ((int)(tt & 1) != parity) continue;
         const uint32_t s = tt & 1, ph = (tt >> 1) & 1;
-        if (!(ok = wait(bar(kGmDFull, s), ph))) break;  // behind the MMAs, which waited for the tile of values
+        // The accumulator, and what ordinary loads below read beside it: the maxima (published by the Gram warps) and the
+        // tile of values (by its copy).  The MMAs waited for both, but their completion orders only the accumulator for
+        // this thread.  None of the three barriers can be a phase ahead: this tile's buffers are still to be given back.
+        if (!(ok = wait(bar(kGmDFull, s), ph) && wait(bar(kGmBFull, it & 3), (it >> 2) & 1) &&
+                   wait(bar(kGmVFull, stage), stage_ph)))
+          break;
         tc_fence_after();
         // a slot is written again four items on, when this tile's buffer has long been given back
         float gmax = 0.f;
