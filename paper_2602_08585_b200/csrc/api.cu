@@ -25,13 +25,17 @@ Workspace carve_workspace(const Dims& dm, void* base) {
   };
   const size_t heads = (size_t)dm.heads();
   ws.raw = static_cast<float*>(take(heads * dm.raw_stride() * sizeof(float)));
-  ws.pooled = static_cast<float*>(take(heads * dm.raw_stride() * sizeof(float)));
+  const size_t pooled_bytes = align256(heads * dm.raw_stride() * sizeof(float));
+  ws.pooled = static_cast<float*>(take(pooled_bytes));
   const size_t stats_simt = heads * score_chunks(dm) * dm.M * 2 * sizeof(float);
   size_t stats_bytes = score_tc_stats_bytes(dm);
   if (stats_simt > stats_bytes) stats_bytes = stats_simt;
   if (score_onepass_stats_bytes(dm) > stats_bytes) stats_bytes = score_onepass_stats_bytes(dm);
   if (keydiff_scratch_bytes(dm) > stats_bytes) stats_bytes = keydiff_scratch_bytes(dm);
+  // a small call's partials start at `pooled` and may run on into `stats`
+  if (score_tc_small_stats_bytes(dm) > pooled_bytes + stats_bytes) stats_bytes = score_tc_small_stats_bytes(dm) - pooled_bytes;
   ws.stats = static_cast<float*>(take(stats_bytes));
+  ws.tc_stats = score_tc_small(dm) ? ws.pooled : ws.stats;
   ws.hull = hull_lists(take(hull_lists_bytes(dm.N, dm.P)), dm.N, dm.P);
   ws.head_flags = static_cast<int*>(take(score_tc_flag_bytes(dm)));
   ws.bytes = off;

@@ -48,6 +48,8 @@ struct Workspace {
   float* pooled;     // [S*N][raw_stride]  pooled scores (whole path, where the selection does not pool)
   float* stats;      // partials per row: (reference, sum-exp) [S*N][chunks][M][2] (FP32-pipe scorer) or the
                      // log-sum-exp [S*N][items][128 or 256] (tensor-core scorer); pieces and anchors (KeyDiff)
+  float* tc_stats;   // those of the two-sweep tensor-core scorer: `stats`, or for small calls, whose work items are more and
+                     // smaller, from `pooled` on, which is not written before they have been read
   HullLists hull;    // blocks of equal gain of every head's curve
   int* head_flags;   // tensor-core scorer: [S*N] items delivered per head and the status word, then the (lse, tag) rows
   size_t bytes;
@@ -55,6 +57,8 @@ struct Workspace {
 
 int score_chunks(const Dims& dm);                       // key chunks per head of the SIMT scorer
 size_t score_tc_stats_bytes(const Dims& dm);            // pass-1 partials of the two-sweep tensor-core scorer
+bool score_tc_small(const Dims& dm);                    // a call in items of two tiles; its partials:
+size_t score_tc_small_stats_bytes(const Dims& dm);
 size_t score_tc_flag_bytes(const Dims& dm);             // zero-initialised block: [heads] counters, status, then the (lse, tag) rows
 inline int* score_tc_status(const Dims& dm, const Workspace& ws) { return ws.head_flags + dm.heads(); }
 size_t score_tc_lse_offset(const Dims& dm);             // offset of the (lse, tag) rows inside that block

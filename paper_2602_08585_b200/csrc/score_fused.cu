@@ -750,15 +750,25 @@ void score_test_hooks(uint32_t* spin_limit, int* drop_item) {
 // Fewest key tiles per work item the launcher tries (it grows for very long contexts): eight, or two where items of eight
 // are fewer than two per SM.  The 148 is the chip this library is built for: the workspace depends on it.
 // LUKV_ITEM_TILES (1..64) overrides it for tuning runs.
-int score_item_tiles(const Dims& dm) {
+static int forced_item_tiles() {
   static const int v = env_int("LUKV_ITEM_TILES", 1, 64, 0);
-  if (v) return v;
-  return dm.heads() * (((dm.T + kTileKeys - 1) / kTileKeys + 7) / 8) < 2 * 148 ? 2 : 8;
+  return v;
 }
-// Bytes of pass-1 partials the tensor-core scorer may write for these sizes.
+static size_t tiles_of(const Dims& dm) { return ((size_t)dm.T + kTileKeys - 1) / kTileKeys; }
+bool score_tc_small(const Dims& dm) {
+  return !forced_item_tiles() && (size_t)dm.heads() * ((tiles_of(dm) + 7) / 8) < 2 * 148;
+}
+int score_item_tiles(const Dims& dm) { return forced_item_tiles() ? forced_item_tiles() : score_tc_small(dm) ? 2 : 8; }
+// Bytes of pass-1 partials the tensor-core scorer may write for these sizes, in items of eight tiles and in a small call's of
+// two.  The latter stay at the largest small call's where small calls end: a call must not need less than a smaller one.
 size_t score_tc_stats_bytes(const Dims& dm) {
-  const size_t tiles = ((size_t)dm.T + kTileKeys - 1) / kTileKeys, least = score_item_tiles(dm);
-  return (size_t)dm.heads() * ((tiles + least - 1) / least) * 256 * sizeof(float);
+  const size_t least = forced_item_tiles() ? forced_item_tiles() : 8;
+  return (size_t)dm.heads() * ((tiles_of(dm) + least - 1) / least) * 256 * sizeof(float);
+}
+size_t score_tc_small_stats_bytes(const Dims& dm) {
+  if (forced_item_tiles()) return 0;
+  const size_t items = (size_t)dm.heads() * ((tiles_of(dm) + 1) / 2), most = 4 * (2 * 148 - 1);  // a small call's items of two
+  return (items < most ? items : most) * 256 * sizeof(float);
 }
 // Bytes of the block that must be zero at launch: [heads] counters, the status word, then [heads][lse_rows][2] floats.
 size_t score_tc_flag_bytes(const Dims& dm) {
@@ -783,7 +793,7 @@ cudaError_t launch_score_tc(const Dims& dm, const void* q, const void* k, const 
   if (!make_map(&qm, q, (uint64_t)dm.heads() * dm.M, dm.d) || !make_map(&km, k, (uint64_t)dm.heads() * dm.T, dm.d))
     return cudaErrorInvalidValue;
   FusedArgs args;
-  args.stats = ws.stats;
+  args.stats = ws.tc_stats;
   args.lse = reinterpret_cast<float*>(reinterpret_cast<char*>(ws.head_flags) + score_tc_lse_offset(dm));
   args.raw = ws.raw;
   args.head_cnt = ws.head_flags;

@@ -52,6 +52,17 @@ def test_workspace_bytes_grows_with_the_problem():
     assert 0 < a < b and a < c and a % 256 == 0
 
 
+@pytest.mark.parametrize("small,large", [
+    # 288 and 320, 256 and 320, 288 and 324 work items of eight key tiles: below 296 the scorer makes smaller and more ones
+    (dict(S=9, L=1, H=8, T=4096), dict(S=10, L=1, H=8, T=4096)), (dict(S=4, L=1, H=8, T=8192), dict(S=5, L=1, H=8, T=8192)),
+    (dict(L=1, H=36, T=8192), dict(L=1, H=36, T=8320)),
+])
+@pytest.mark.parametrize("kw", [dict(G=1, w=16, d=128), dict(G=8, w=16, d=64), dict(G=1, w=256, d=64)])
+def test_scratch_for_a_call_is_enough_for_a_smaller_one(small, large, kw):
+    kw = dict(kw, P=2, kp=7)
+    assert lukv.lukv_workspace_bytes(_p(**small, **kw)) <= lukv.lukv_workspace_bytes(_p(**large, **kw))
+
+
 @pytest.mark.parametrize("kw,code", [
     (dict(d=96), lukv.ERR_UNSUPPORTED), (dict(dtype=7), lukv.ERR_UNSUPPORTED), (dict(kp=4), lukv.ERR_UNSUPPORTED),
     (dict(P=18), lukv.ERR_UNSUPPORTED), (dict(G=64), lukv.ERR_UNSUPPORTED), (dict(P=8193, T=8192), lukv.ERR_UNSUPPORTED),
