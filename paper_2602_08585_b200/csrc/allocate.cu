@@ -65,45 +65,49 @@ __device__ __forceinline__ bool mean_le(float u_l1, float u_r1, int len1, float 
 }
 
 // The vertices among cnt points (values us, places is, ascending; the first and the last are ends) in the warp's shared
-// memory: a point on or below the chord of its neighbours is dropped, all of them tested at once, until a pass drops none.
-// In place; returns how many are left, or -1 if that took more than max_passes.
-__device__ __forceinline__ int hull_passes(float* us, unsigned short* is, int cnt, int max_passes, int lane) {
+// memory: a point on or below the chord of its neighbours is dropped, all of them tested at once.  One pass, in place; returns
+// how many are left.
+__device__ __forceinline__ int hull_pass(float* us, unsigned short* is, int cnt, int lane) {
   const uint32_t lt_mask = (1u << lane) - 1u;
+  __syncwarp();
+  int out = 0;
+#pragma unroll 1
+  for (int base = 0; base < cnt; base += 32) {
+    // in place: the writes of a turn end before the points that the next one reads, but for the last, unless nothing
+    // was dropped yet, when they write what is there
+    const int i = base + lane, ii = min(i, cnt - 1), il = max(ii - 1, 0), ir = min(ii + 1, cnt - 1);
+    const float um = us[ii], ul = us[il], ur = us[ir];
+    const int km = is[ii], kl = is[il], kr = is[ir];
+    // 2^23 + k as a float: differences of two are the lengths
+    auto place = [](int k) { return __int_as_float(0x4B000000 | k); };
+    const float d1 = um - ul, d2 = ur - um;
+    bool keep;
+    if (__all_sync(0xffffffffu, exact_range(um) & exact_diff(um, ul, d1) & exact_diff(ur, um, d2)))
+      keep = !exact_le(d1, place(km) - place(kl), d2, place(kr) - place(km));
+    else
+      keep = !mean_le(ul, um, km - kl, um, ur, kr - km);
+    keep = (i < cnt) & ((i == 0) | (i == cnt - 1) | keep);
+    const uint32_t kept = __ballot_sync(0xffffffffu, keep);
+    if (keep) {
+      const int at = out + __popc(kept & lt_mask);
+      us[at] = um;
+      is[at] = (unsigned short)km;
+    }
+    out += __popc(kept);
+    __syncwarp();
+  }
+  return out;
+}
+// Passes until one drops none; returns how many points are left, or -1 if that took more than max_passes.
+__device__ __forceinline__ int hull_passes(float* us, unsigned short* is, int cnt, int max_passes, int lane) {
 #pragma unroll 1
   for (int pass = 0; pass < max_passes; ++pass) {
-    __syncwarp();
-    int out = 0;
-#pragma unroll 1
-    for (int base = 0; base < cnt; base += 32) {
-      // in place: the writes of a turn end before the points that the next one reads, but for the last, unless nothing
-      // was dropped yet, when they write what is there
-      const int i = base + lane, ii = min(i, cnt - 1), il = max(ii - 1, 0), ir = min(ii + 1, cnt - 1);
-      const float um = us[ii], ul = us[il], ur = us[ir];
-      const int km = is[ii], kl = is[il], kr = is[ir];
-      // 2^23 + k as a float: differences of two are the lengths
-      auto place = [](int k) { return __int_as_float(0x4B000000 | k); };
-      const float d1 = um - ul, d2 = ur - um;
-      bool keep;
-      if (__all_sync(0xffffffffu, exact_range(um) & exact_diff(um, ul, d1) & exact_diff(ur, um, d2)))
-        keep = !exact_le(d1, place(km) - place(kl), d2, place(kr) - place(km));
-      else
-        keep = !mean_le(ul, um, km - kl, um, ur, kr - km);
-      keep = (i < cnt) & ((i == 0) | (i == cnt - 1) | keep);
-      const uint32_t kept = __ballot_sync(0xffffffffu, keep);
-      if (keep) {
-        const int at = out + __popc(kept & lt_mask);
-        us[at] = um;
-        is[at] = (unsigned short)km;
-      }
-      out += __popc(kept);
-      __syncwarp();
-    }
+    const int out = hull_pass(us, is, cnt, lane);
     if (out == cnt) return cnt;
     cnt = out;
   }
   return -1;
 }
-
 // The blocks between cnt vertices; the part without a positive slope is one block of gain 0.  The output may be the place
 // of the vertices.  Returns the number of blocks.
 __device__ __forceinline__ int hull_emit(const float* us, const unsigned short* is, int cnt, float* gain, unsigned short* start,
@@ -264,19 +268,47 @@ __device__ __forceinline__ int hull_walk_regs(const float* __restrict__ U, int P
 inline int hull_prune_cap(int P) { return (P * 3 / 10 + 63) & ~63; }
 constexpr int kHullPasses = 48;
 
+// The survivors of points base .. base + count - 1 behind the cnt (at most cap) there are, when they are too many to be added
+// as they are: passes over what is there make room.  Returns how many there are then, or cap + 1 if a pass does not make enough.
+__device__ __noinline__ int hull_squeeze(const float* __restrict__ U, int P, int base, int count, float* us, unsigned short* is,
+                                         int cnt, int cap, int lane) {
+#pragma unroll 1
+  for (int v = 0; v < count; v += 32) {
+    const int j = base + v + lane, jj = min(j, P - 1);
+    const float u = __ldg(U + jj), lim = fmaf(5e-7f, fabsf(u), 2.f * u);
+    bool below = false;  // clearly below a chord, as in the first pass
+#pragma unroll
+    for (int k = 4; k <= 16; k <<= 1)
+      if (j >= k && j + k < P) below |= __ldg(U + j - k) + __ldg(U + j + k) > lim;
+    const uint32_t kept = __ballot_sync(0xffffffffu, j < P && !below);
+    if (cnt + __popc(kept) > cap) cnt = hull_pass(us, is, cnt, lane);
+    if (cnt + __popc(kept) > cap) return cap + 1;
+    if ((kept >> lane) & 1) {
+      const int at = cnt + __popc(kept & ((1u << lane) - 1u));
+      us[at] = u;
+      is[at] = (unsigned short)j;
+    }
+    cnt += __popc(kept);
+  }
+  __syncwarp();
+  return cnt;
+}
+
 // One warp per curve.  A point on or below the chord of two other points is no vertex of the majorant, whichever points
 // they are, so a pass may test all points against their current neighbours at once; a polygon without such a point is the
 // majorant.  The first pass reads the curve once, into registers, and drops what lies clearly below the chord of the points
 // 1, 2, 4, 8 or 16 places to either side (4001 points: about 800 stay); the survivors (value and index) are compacted in
 // shared memory and tested against their neighbours, exactly, until none is dropped (9 passes over 1900 points in all, 53
-// stay).  A curve of which more than three tenths survive the first pass, or that needs more than kHullPasses, is left to
-// hull_dense_kernel (count -1).  Blocks beyond the last positive slope are one block of gain 0.
+// stay).  Where there is no room for 256 points' survivors, those before them go through a pass of their own (hull_squeeze); a
+// curve for which that is not enough, or that needs more than kHullPasses, is left to hull_dense_kernel (count -1).  Blocks
+// beyond the last positive slope are one block of gain 0.
 // Bound by the latency of a warp's own instructions at 27 warps per SM (7300 bytes of shared memory each; the 52 curves of an SM
 // are two rounds).  7680 curves of 4001 points: 3.07 ms as one serial stack walk per curve, 0.31 ms as a walk from
 // vertex to vertex over chunk maxima, 0.22 ms with neighbours alone in the first pass, 0.157 ms with room
 // for two fifths of the points (21 warps per SM, three rounds); the profile build 243 us with that and a dense-hull CTA per
-// curve, 227 now.
-__global__ void __launch_bounds__(32) hull_prune_kernel(const float* __restrict__ curves, HullLists lists, int P, int cap) {
+// curve, 227 now.  Smooth curves with 2 % noise in the increments (0.29 of the points survive) 484 us, 502 with room for two
+// fifths, 966 if hull_dense_kernel takes them; without noise (0.65 survive) 1874, 1886 and 2123.
+__global__ void __launch_bounds__(32, 27) hull_prune_kernel(const float* __restrict__ curves, HullLists lists, int P, int cap) {
   extern __shared__ float hull_smem[];
   const int hid = blockIdx.x, lane = threadIdx.x;
   const float* U = curves + (size_t)hid * P;
@@ -291,6 +323,7 @@ __global__ void __launch_bounds__(32) hull_prune_kernel(const float* __restrict_
   for (int t = 0; t < kAhead; ++t) nxt[t] = __ldg(U + min(32 * t + lane, P - 1));
 #pragma unroll 1
   for (int base = 0; base < P; base += 32 * kAhead) {
+    const int before = cnt;
 #pragma unroll
     for (int t = 0; t < kAhead; ++t) cur[t] = nxt[t];
 #pragma unroll
@@ -329,6 +362,7 @@ __global__ void __launch_bounds__(32) hull_prune_kernel(const float* __restrict_
       cnt += __popc(kept);
     }
     prev = cur[kAhead - 1];
+    if (cnt > cap && before <= cap) cnt = hull_squeeze(U, P, base, 32 * kAhead, us, is, before, cap, lane);
   }
   int total = -1;
   if (cnt <= cap && (cnt = hull_passes(us, is, cnt, kHullPasses, lane)) > 0)
@@ -347,7 +381,7 @@ inline size_t hull_dense_smem_bytes(int P) { return (size_t)P * 4 + (size_t)hull
 // hulls are joined pairwise, five times: the block across the joint absorbs blocks from the left while their mean does
 // not exceed its own and from the right while its own does not exceed theirs, which is where the serial algorithm ends
 // up as well (the projection is unique).
-__device__ __noinline__ void hull_dense_curve(const float* __restrict__ curves, const HullLists& lists, int P, int hid,
+__device__ __forceinline__ void hull_dense_curve(const float* __restrict__ curves, const HullLists& lists, int P, int hid,
                                               float* hull_smem, int lane) {
   const float* U = curves + (size_t)hid * P;
   const int run = hull_run(P);

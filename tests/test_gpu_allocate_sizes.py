@@ -115,6 +115,30 @@ def test_curves_of_many_vertices(oracle, N, P, kind):
     np.testing.assert_array_equal(o, o_ref)
 
 
+@pytest.mark.parametrize("noise", [0.0, 0.003, 0.01, 0.02, 0.03, "half", "late"])
+@pytest.mark.parametrize("N,P", [(40, 545), (40, 1030), (36, 4001), (33, 4097)])
+def test_long_curves_whose_first_pass_leaves_many_points(oracle, N, P, noise):
+    """Long curves that are smooth but for a little noise: between all points and a fifth of them are left by the first pass
+    (at 4001 points 0.65, 0.45, 0.35, 0.29 and 0.27 of them), more than the shared memory of a curve holds at once.  "half":
+    smooth up to the middle, rough behind it; "late": the other way round."""
+    rng = np.random.default_rng(P)
+    t = np.arange(1, P)[None, :]
+    sigma = np.full((1, P - 1), 0.8 if isinstance(noise, str) else noise)
+    if isinstance(noise, str):
+        sigma[:, slice(0, P // 2) if noise == "half" else slice(P // 2, P)] = 0.0
+    inc = t ** -rng.uniform(0.5, 0.9, (N, 1)) * (1 + sigma * rng.standard_normal((N, P - 1)))
+    U = np.zeros((N, P), np.float32)
+    U[:, 1:] = np.cumsum(inc, axis=1)
+    T, w = 2 * (P - 1), 4
+    most = N * (T - w)
+    Bs = [most // 7, most // 3 + 1, most * 4 // 5]
+    p = lukv.make_params(len(Bs), 1, N, 1, 64, T, w, 1, "bf16", P)
+    b, o = gpu_allocate(p, U, Bs)
+    b_ref, o_ref = oracle.allocate(U, T, w, Bs)
+    np.testing.assert_array_equal(b, b_ref)
+    np.testing.assert_array_equal(o, o_ref)
+
+
 @pytest.mark.parametrize("exponent", [-105, -90, 90, 112, 117])
 @pytest.mark.parametrize("kind", ["rough", "concave", "mixed"])
 @pytest.mark.parametrize("N,P", [(6, 513), (40, 257), (6, 1025), (3, 4001)])
