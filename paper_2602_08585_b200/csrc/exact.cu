@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(kDpCoreThreads) dp_reduced_kernel(const DpCore
   for (int b = tid; b <= a.n; b += kDpCoreThreads) {
     const double x = (double)__ldg(U + b);
     c = fmax(c, x - slope * b);
-    size = fmax(size, fabs(x));
+    size = fmax(size, fabs(x) < INFINITY ? fabs(x) : INFINITY);  // no number: the greedy solution may be none
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {

@@ -181,6 +181,25 @@ def test_same_solution_as_the_full_recursion(kind, N, T, w, Bs):
     np.testing.assert_array_equal(off, np.concatenate([[0], np.cumsum(b.reshape(-1) + w)]))
 
 
+@pytest.mark.parametrize("seed", [3, 10, 17])
+def test_values_that_are_no_numbers_bound_nothing(seed):
+    """Where some values are no numbers the greedy solution need not have the sum of the budget (seed 10: 12189 instead of
+    12117), and its value is no bound for leaving tokens out."""
+    rng = np.random.default_rng(seed)
+    N, T, w = 40, 404, 20
+    inc = rng.exponential(size=(N, T)) * np.arange(1, T + 1) ** -rng.uniform(0.2, 1.6, (N, 1))
+    U = np.zeros((N, T + 1), np.float32)
+    U[:, 1:] = np.cumsum(inc, axis=1)
+    none = rng.random(U[:, 1:].shape) < 10 ** rng.uniform(-4, -0.2)
+    none[rng.random(N) < rng.uniform(0, 0.8)] = False
+    U[:, 1:][none] = np.nan
+    B = int(rng.integers(1, N * (T - w)))
+    b, _, val = gpu_exact(N, T, w, U, [B])
+    with np.errstate(invalid="ignore"):
+        ref, best = _recursion(U, B, T - w)
+    assert list(b[0]) == ref and np.float32(val[0]) == best
+
+
 def test_a_wait_that_runs_out_leaves_no_solution(monkeypatch):
     """With the test hooks one CTA stores nothing and the wait limit is short: the optimum is no number and the budgets are
     zero.  The next ordinary call gives the same as a fresh one."""
