@@ -150,17 +150,8 @@ def test_curves_with_jumps_near_the_end_of_fp32():
         assert list(b[q]) == ref and np.float32(val[q]) == best
 
 
-@pytest.mark.parametrize("kind", ["utility", "rough", "falling", "ties", "zero", "steep"])
-@pytest.mark.parametrize("N,T,w,Bs", [
-    (40, 300, 20, [1500, 0, 40 * 280, 7001]),   # several sequences, no budget, all of it
-    (24, 497, 50, [24 * 447 - 1, 63, 5000]),    # more than six blocks of tokens on curves that leave them all
-    (17, 130, 2, [640, 1087]),                  # tokens up to a block's edge
-])
-def test_same_solution_as_the_full_recursion(kind, N, T, w, Bs):
-    """Tokens and budgets that cannot matter are left out, to the bit: the same smallest solution and the same sum, on curves
-    that leave few tokens (utility) and on curves that leave all (ties, zero)."""
+def _curves(kind, N, T):
     rng = np.random.default_rng(N + T)
-    n = T - w
     inc = rng.exponential(size=(N, T)) * np.arange(1, T + 1) ** -rng.uniform(0.2, 1.6, (N, 1))
     if kind == "rough":
         inc = rng.exponential(size=(N, T)) * np.where(rng.random((N, T)) < 0.2, 3.0, 1.0)
@@ -174,11 +165,37 @@ def test_same_solution_as_the_full_recursion(kind, N, T, w, Bs):
         inc *= 1e33
     U = np.zeros((N, T + 1), np.float32)
     U[:, 1:] = np.cumsum(inc, axis=1)
+    if kind in ("nan", "-inf", "inf"):  # no number at some tokens of every other head, its last ones among them
+        U[::2, 1:][rng.random(U[::2, 1:].shape) < (0.3 if kind != "inf" else 0.01)] = float(kind)
+        U[::4, -T // 2:] = float(kind)
+    return U
+
+
+@pytest.mark.parametrize("kind", ["utility", "rough", "falling", "ties", "zero", "steep", "nan", "-inf", "inf"])
+@pytest.mark.parametrize("N,T,w,Bs,reduced", [
+    (40, 300, 20, [1500, 0, 40 * 280, 7001], False),   # several sequences, no budget, all of it
+    (24, 497, 50, [24 * 447 - 1, 63, 5000], False),    # more than six blocks of tokens on curves that leave them all
+    (17, 130, 2, [640, 1087], False),                  # tokens up to a block's edge
+    # from here on tokens and budgets are left out
+    (40, 404, 20, [2300, 0, 40 * 384, 64, 40 * 384 - 1, 9001], True),
+    (300, 100, 12, [300 * 88 // 3, 2000], True),      # more heads than the threads that add up their tokens
+    (48, 700, 28, [48 * 672 // 4], True),              # eleven blocks on curves that leave all tokens; long curves' hulls
+])
+def test_same_solution_as_the_full_recursion(kind, N, T, w, Bs, reduced):
+    """To the bit: the same smallest solution and the same sum, on curves that leave few tokens (utility), on curves that
+    leave all (ties, zero), and where some values are no numbers, which no solution takes, or infinite."""
+    n, U = T - w, _curves(kind, N, T)
     b, off, val = gpu_exact(N, T, w, U, Bs)
+    # one kernel and three a sequence, or the hulls, the greedy solution and two more a sequence before the rows
+    assert (lukv.lukv_last_launch_count() > 1 + 3 * len(Bs)) == reduced
     for q, B in enumerate(Bs):
-        ref, best = _recursion(U, B, n)
-        assert list(b[q]) == ref and np.float32(val[q]) == best
-    np.testing.assert_array_equal(off, np.concatenate([[0], np.cumsum(b.reshape(-1) + w)]))
+        with np.errstate(invalid="ignore"):
+            ref, best = _recursion(U, B, n)
+        assert np.float32(val[q]) == best
+        if best > -np.inf:  # else no solution: every one is as good
+            assert list(b[q]) == ref
+    if kind not in ("-inf", "nan"):
+        np.testing.assert_array_equal(off, np.concatenate([[0], np.cumsum(b.reshape(-1) + w)]))
 
 
 @pytest.mark.parametrize("seed", [3, 10, 17])
@@ -200,10 +217,11 @@ def test_values_that_are_no_numbers_bound_nothing(seed):
     assert list(b[0]) == ref and np.float32(val[0]) == best
 
 
-def test_a_wait_that_runs_out_leaves_no_solution(monkeypatch):
+@pytest.mark.parametrize("N,T,w", [(32, 300, 20), (40, 404, 20)])  # all tokens; those that can matter
+def test_a_wait_that_runs_out_leaves_no_solution(monkeypatch, N, T, w):
     """With the test hooks one CTA stores nothing and the wait limit is short: the optimum is no number and the budgets are
     zero.  The next ordinary call gives the same as a fresh one."""
-    N, T, w, B = 32, 300, 20, 32 * 140
+    B = N * (T - w) // 2
     U = _rough(np.random.default_rng(9), N, T + 1)
     ref = gpu_exact(N, T, w, U, [B])
     monkeypatch.setenv("LUKV_TEST_SPIN_LIMIT", "20000")
