@@ -186,15 +186,15 @@ cudaError_t launch_keydiff(const Dims& dm, const void* k, float* scores, int str
                            int spare_sms, LaunchCtx& lc);
 // Value norms || v_j W_O^(g) ||_2 of the oracle importance on the tensor cores (bf16): vnorm [heads][G][n].  Here and in
 // the attention part a bounded wait that runs out stores LUKV_ERR_TIMEOUT to status.
-// flags (or null: every position): the 128-byte entries, one per (head, query head, 4096 positions), of the chunks to compute.
+// left (or null: all): [heads][G][128-position tiles][4] a bit per position to compute.
 bool value_norm_tc_supported(const Dims& dm);
 cudaError_t launch_value_norm_tc(const Dims& dm, int d_model, const void* v, const void* w_o, float* vnorm,
-                                 const unsigned char* flags, int32_t* status, LaunchCtx& lc);
-// The same through the Gram matrix of the projection; positions for which it is not sound are flagged for the kernel above.
+                                 const uint32_t* left, int32_t* status, LaunchCtx& lc);
+// The same through the Gram matrix of the projection; positions for which it is not sound are left to the kernel above.
 bool value_norm_gram_pays(const Dims& dm, int d_model, const void* w_o);
-size_t value_norm_gram_flag_bytes(const Dims& dm);
+size_t value_norm_gram_left_bytes(const Dims& dm);
 cudaError_t launch_value_norm_gram(const Dims& dm, int d_model, const void* v, const void* w_o, float* vnorm,
-                                   unsigned char* flags, int32_t* status, LaunchCtx& lc);
+                                   uint32_t* left, int32_t* status, LaunchCtx& lc);
 // Attention part of the oracle importance on the tensor cores (bf16, up to 8 query heads per KV head): needs the value
 // norms, leaves the un-normalised importance; part: importance_tc_part_bytes() of scratch.
 bool importance_tc_supported(const Dims& dm, int k_max);

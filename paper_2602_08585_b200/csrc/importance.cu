@@ -287,12 +287,12 @@ cudaError_t launch_importance_t(const Dims& dm, ImpDims id, const void* q_dec, c
   const unsigned pos_tiles = (unsigned)((dm.n + kTile - 1) / kTile);
   const bool norms_tc = value_norm_tc_supported(dm) && !value_norm_force_simt();
   if (norms_tc) {
-    unsigned char* flags = nullptr;
+    uint32_t* left = nullptr;
     if (value_norm_gram_pays(dm, id.Dm, w_o)) {
-      flags = reinterpret_cast<unsigned char*>(lse);  // the log-sum-exps come later
-      if ((e = launch_value_norm_gram(dm, id.Dm, v, w_o, vnorm, flags, status, lc)) != cudaSuccess) return e;
+      left = reinterpret_cast<uint32_t*>(lse);  // the log-sum-exps come later
+      if ((e = launch_value_norm_gram(dm, id.Dm, v, w_o, vnorm, left, status, lc)) != cudaSuccess) return e;
     }
-    if ((e = launch_value_norm_tc(dm, id.Dm, v, w_o, vnorm, flags, status, lc)) != cudaSuccess) return e;
+    if ((e = launch_value_norm_tc(dm, id.Dm, v, w_o, vnorm, left, status, lc)) != cudaSuccess) return e;
   } else {
     kn<<<dim3(heads * id.G, pos_tiles), kSimtThreads, smem, lc.st>>>((const TIn*)v, (const TIn*)w_o, vnorm, id);
     lc.mark("value_norm");
@@ -316,11 +316,11 @@ cudaError_t launch_importance_t(const Dims& dm, ImpDims id, const void* q_dec, c
 
 }  // namespace
 
-// value norms, row log-sum-exps (or their partials; before them the value norms' flags), the status word
+// value norms, row log-sum-exps (or their partials; before them the bits of the positions that the Gram form leaves), the status word
 static size_t importance_status_offset(const Dims& dm, int k_max) {
   const size_t a = ((size_t)dm.heads() * dm.G * dm.n * sizeof(float) + 255) & ~(size_t)255;
   const size_t rows = (size_t)dm.heads() * dm.G * k_max * sizeof(float);  // row log-sum-exps; room for their partials
-  const size_t b = std::max(rows + (dm.G <= 8 ? importance_tc_part_bytes(dm, k_max) : 0), value_norm_gram_flag_bytes(dm));
+  const size_t b = std::max(rows + (dm.G <= 8 ? importance_tc_part_bytes(dm, k_max) : 0), value_norm_gram_left_bytes(dm));
   return a + ((b + 255) & ~(size_t)255);
 }
 size_t importance_workspace_bytes(const Dims& dm, int k_max) { return importance_status_offset(dm, k_max) + 256; }

@@ -13,20 +13,30 @@
 //   warps 12-19 Gram sums: every 64 (d = 64: 32) projection columns the accumulator is added to fp32 sums in registers; at
 //               the end B
 // Precision.  Products of bf16 are exact; the tensor core, whose sums err towards zero, adds four (two) instructions' worth
-// before they continue in round-to-nearest fp32 registers.  The matrix enters the second contraction as three bf16 pieces (24 bits).  It is
-// symmetric, so only blocks of 16 channels on and above the diagonal are multiplied, those above it doubled.
-// q loses digits when it is small beside max |G| |v|^2 (a value close to the null space of an ill-conditioned projection)
-// and the squares of extreme inputs leave fp32: a tile that holds such a position is flagged, and the direct kernel
-// recomputes its chunk of positions.  With q >= max |G| |v|^2 / 32 the entries of G, wrong by about 2^-24 each, move the norm
-// by at most 16 * 2^-24.
-// Against 64 bits (normal values, projections of 520 to 4096 columns) the norms' error is 0.87e-7 rms here and 1.16e-7
-// multiplied out (d = 64: 0.66e-7 and 0.74e-7); with twice the columns between the fp32 additions it would be 1.28e-7.
+// before they continue in round-to-nearest fp32 registers.  The matrix enters the second contraction as three bf16 pieces
+// (24 bits).  It is symmetric, so only blocks of 16 channels on and above the diagonal are multiplied, those above it doubled.
+// Cancellation.  With y_b the projection of a position's first b blocks of 16 channels, q = |y_last|^2, and the terms D[c] v[c]
+// of block b add up to |y_b|^2 - |y_b-1|^2.  q is taken where t, the sum of the blocks' sums without their signs, and s, the sum of
+// G[c][c] v[c]^2, are both at most 1.5 q.  t >= 2 max |y_b|^2 - q, so that |y_b|^2 <= 1.25 q and no partial sum of D[c] is beyond
+// 2.3 |w_c| sqrt(q).  With e a few 2^-24: an entry of G is wrong by e |w_c| |w_k|, which moves q by at most e d s, and by about e s
+// as the errors have either sign; a step of D is wrong by e |w_c| sqrt(q), which moves q by at most e sqrt(d s q).  Other
+// positions, and those whose squares leave fp32 or its normal range, are left to the direct kernel, a bit each.  Without the
+// rule a projection with a common component in its rows, and values that cancel it, loses 1e-7 to 3e-5 of the norm, and
+// t and s are 1.5 to 1100 q there (multiplied out: 0.5e-7 to 1.2e-7).
+// Against 64 bits (normal values, projections of 520 to 4096 columns) the norms' error is 0.75e-7 to 0.87e-7 rms here and
+// 1.15e-7 multiplied out (d = 64: 0.66e-7 to 0.73e-7 and 0.76e-7); with twice the columns between the fp32 additions it would
+// be 1.28e-7.  Where rows share components, single rows are a hundred times the others or singular values fall as k^-1/4 to k^-2,
+// what is taken is as good as multiplied out (0.75e-7 to 1.1e-7).  With a limit of 3 instead of 1.5 the first of these would lose
+// half as much again.
 // What bounds it: shared-memory bandwidth (an MMA reads both operands there: 24 steps per tile, 256 per projection slice)
-// beside the 1.07 GB of projections at 256 heads x 4 query heads x 4096 columns.  There, with 3968 positions a head: 0.37 ms
-// against 2.81 ms multiplied out; 0.26 ms with one tile per slice, 0.28 ms with 512 columns.  A single epilogue quad 0.39 ms;
-// blocks below the diagonal multiplied too 0.43 ms.
+// beside the 1.07 GB of projections at 256 heads x 4 query heads x 4096 columns.  There, with 3968 positions a head: 0.38 ms
+// against 2.81 ms multiplied out, 0.37 without t and s, and 0.44 where rows differ in length (s added up for every
+// position: 0.43 if it were so for all); 0.26 ms with one tile per slice, 0.28 ms with 512 columns.  A single epilogue quad
+// 0.39 ms and blocks below the diagonal multiplied too 0.43 ms (both without t and s).
 // Every wait is bounded; the waits are between the warps of one CTA only.
 #include <algorithm>
+#include <cstdlib>
+#include <type_traits>
 
 #include "tc_ptx.cuh"
 
@@ -35,7 +45,7 @@ namespace {
 
 constexpr int kGmThreads = 640;
 constexpr int kGmGramWarps = 8;
-constexpr float kGmMinShare = 1.f / 32.f;  // least q / (max |G| |v|^2) that is taken
+constexpr float kGmMost = 1.5f;  // most (sum of a position's terms without their signs) / q that is taken
 
 template <int NH>  // halves of 64 channels: d = 64 NH
 struct GmPlan {
@@ -62,14 +72,14 @@ enum {
 
 struct GmArgs {
   float* vnorm;          // [heads][G][n]
-  unsigned char* flags;  // [heads][G][chunks4k][32 tiles][4]: 1 where a warp's positions are left to the direct kernel
+  uint32_t* left;        // [heads][G][tiles][4] a bit per position that is left to the direct kernel
   int S, LH, G, T, n, Dm;
   int tiles;             // 128-position tiles per head
-  int chunks4k;          // chunks of the direct kernel per head
   int per_item;          // tiles per item (of the S * tiles that a slice has)
   int items_per_slice;
   int items;
   uint32_t spin_limit;
+  int drop_item;         // test hook: the value tiles of this item are never loaded (-1: none)
   int32_t* status;
 };
 
@@ -83,7 +93,8 @@ __global__ void __launch_bounds__(kGmThreads, 1)
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   unsigned char* v_tiles = smem + P::kVOff;
   __shared__ __align__(8) uint64_t bars[kGmBars];
-  __shared__ float gmax_s[4][kGmGramWarps];  // largest |G| of an item, per warp, for the last items
+  __shared__ __align__(16) float diag_s[4][128];  // the diagonal of G, for the last items
+  __shared__ float gmax_s[4][kGmGramWarps];       // its largest entry, per warp
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_s;
   volatile int* abort_flag = &abort_s;
@@ -132,6 +143,7 @@ __global__ void __launch_bounds__(kGmThreads, 1)
       for (int idx = blockIdx.x; idx < a.items && ok; idx += gridDim.x) {
         const int slice = idx / a.items_per_slice, t0 = (idx % a.items_per_slice) * a.per_item;
         const int t1 = min(t0 + a.per_item, all_tiles);
+        if (idx == a.drop_item) break;
         for (int t = t0; t < t1; ++t) {
           if (!(ok = wait(bar(kGmVEmpty, s), ph))) break;
           mbar_expect_tx(bar(kGmVFull, s), P::kVTile);
@@ -222,71 +234,113 @@ __global__ void __launch_bounds__(kGmThreads, 1)
     // two quads of warps take alternate tiles: a quad alone is slower than the MMAs
     const int quad = warp & 3, parity = (warp - 4) >> 2, row = 32 * quad + lane;
     const uint32_t lane_addr = (uint32_t)(32 * quad) << 16;
-    uint32_t tt = 0, it = 0, vs = 0, vph = 0;
+    uint32_t tt = 0, it = 0, vs = 0, vph = 0, seen = ~0u;  // seen: the last item whose diagonal was waited for
     bool ok = true;
     for (int idx = blockIdx.x; idx < a.items && ok; idx += gridDim.x, ++it) {
       const int slice = idx / a.items_per_slice, t0 = (idx % a.items_per_slice) * a.per_item;
       const int t1 = min(t0 + a.per_item, all_tiles);
       const int uh = slice / a.G, g = slice - uh * a.G;
+      bool uneven = false;  // the projection's rows differ in length (as far as this warp has seen)
       for (int t = t0; t < t1; ++t, ++tt) {
         const uint32_t stage = vs, stage_ph = vph;
         if (++vs == P::kVStages) vs = 0, vph ^= 1;
         if ((int)(tt & 1) != parity) continue;
         const uint32_t s = tt & 1, ph = (tt >> 1) & 1;
-        // The accumulator, and what ordinary loads below read beside it: the maxima (published by the Gram warps) and the
-        // tile of values (by its copy).  The MMAs waited for both, but their completion orders only the accumulator for
+        // The accumulator, and what ordinary loads below read beside it: the tile of values (by its copy) and the diagonal
+        // (published by the Gram warps).  The MMAs waited for both, but their completion orders only the accumulator for
         // this thread.  None of the three barriers can be a phase ahead: this tile's buffers are still to be given back.
-        if (!(ok = wait(bar(kGmDFull, s), ph) && wait(bar(kGmBFull, it & 3), (it >> 2) & 1) &&
-                   wait(bar(kGmVFull, stage), stage_ph)))
-          break;
+        if (!(ok = (seen == it || wait(bar(kGmBFull, it & 3), (it >> 2) & 1)) && wait(bar(kGmDFull, s), ph))) break;
+        seen = it;
         tc_fence_after();
         // a slot is written again four items on, when this tile's buffer has long been given back
         float gmax = 0.f;
 #pragma unroll
         for (int i = 0; i < kGmGramWarps; ++i) gmax = fmaxf(gmax, gmax_s[it & 3][i]);
         const unsigned char* vrow = v_tiles + stage * P::kVTile + row * 128;
-        uint64_t q2[2] = {0, 0}, vv2[2] = {0, 0};
+        auto value8 = [&](int c8) {  // channels 8 c8 .. + 7
+          return *reinterpret_cast<const uint4*>(vrow + (c8 >> 3) * kHalfBytes + (((c8 & 7) ^ (row & 7)) << 4));
+        };
+        auto pair_of = [](uint32_t w) { return pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); };
+        const float* diag = diag_s[it & 3];
+        float q = 0.f, terms = 0.f;
+        uint64_t vv2[2] = {0, 0}, own2[2] = {0, 0};
         uint32_t any = 0;
-#pragma unroll
-        for (int c0 = 0; c0 < 2 * NH; ++c0) {
-          float d[32];
-          tmem_ld32(tmem_base + lane_addr + s * 128 + 32 * c0, d);
-          uint4 v[4];
-#pragma unroll
-          for (int c = 0; c < 4; ++c)
-            v[c] = *reinterpret_cast<const uint4*>(vrow + (c0 >> 1) * kHalfBytes + (((4 * (c0 & 1) + c) ^ (row & 7)) << 4));
+        float d[32];
+        tmem_ld32(tmem_base + lane_addr + s * 128, d);
+        ok = wait(bar(kGmVFull, stage), stage_ph);  // (behind the load: the test is a round trip to shared memory)
+        if (!ok) {
           tmem_ld_wait(d);
+          break;
+        }
+        auto add_up = [&](auto with_own) {
 #pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            const uint32_t w4[4] = {v[c].x, v[c].y, v[c].z, v[c].w};
+          for (int c0 = 0; c0 < 2 * NH; ++c0) {
+            if (c0 > 0) tmem_ld32(tmem_base + lane_addr + s * 128 + 32 * c0, d);
+            uint4 v[4];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const uint64_t x = pack2(__uint_as_float(w4[i] << 16), __uint_as_float(w4[i] & 0xFFFF0000u));
-              q2[i & 1] = ffma2(pack2(d[8 * c + 2 * i], d[8 * c + 2 * i + 1]), x, q2[i & 1]);
-              vv2[i & 1] = ffma2(x, x, vv2[i & 1]);
-              any |= w4[i];
+            for (int c = 0; c < 4; ++c) v[c] = value8(4 * c0 + c);
+            tmem_ld_wait(d);
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {  // a block of 16 channels
+              uint64_t sum = 0;
+#pragma unroll
+              for (int c = 2 * b; c < 2 * b + 2; ++c) {
+                const uint32_t w4[4] = {v[c].x, v[c].y, v[c].z, v[c].w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                  const uint64_t x = pair_of(w4[i]);
+                  sum = ffma2(pack2(d[8 * c + 2 * i], d[8 * c + 2 * i + 1]), x, sum);
+                  vv2[b] = ffma2(x, x, vv2[b]);
+                  if constexpr (decltype(with_own)::value) {
+                    const uint64_t g = *reinterpret_cast<const uint64_t*>(diag + 32 * c0 + 8 * c + 2 * i);
+                    own2[b] = ffma2(fmul2(g, x), x, own2[b]);
+                  }
+                  any |= w4[i];
+                }
+              }
+              float even, odd;
+              unpack2(sum, even, odd);
+              q += even + odd, terms += fabsf(even + odd);
             }
           }
-        }
+        };
+        const bool with_own = uneven;
+        if (with_own) add_up(std::true_type{});
+        else add_up(std::false_type{});
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) {
-          mbar_arrive(bar(kGmDEmpty, s), 1);
-          mbar_arrive(bar(kGmVEmpty, stage), 1);
+        if (lane == 0) mbar_arrive(bar(kGmDEmpty, s), 1);
+        const float vv = sum4(vv2[0], vv2[1]), most = kGmMost * q;
+        bool sound = terms <= most && q >= 1e-30f && q <= 1e37f && vv >= 1e-30f && vv <= 1e30f && q >= 1e-25f * vv;
+        // rows of alike length: the longest bounds the sum of G[c][c] v[c]^2; else it is added up, from the next tile on above
+        if (!with_own && __any_sync(0xffffffffu, sound && !(gmax * vv <= most))) {
+          uneven = true;
+#pragma unroll 2
+          for (int c = 0; c < 8 * NH; ++c) {
+            const uint4 v = value8(c);
+            const ulonglong2 g0 = *reinterpret_cast<const ulonglong2*>(diag + 8 * c);
+            const ulonglong2 g1 = *reinterpret_cast<const ulonglong2*>(diag + 8 * c + 4);
+            const uint64_t x0 = pair_of(v.x), x1 = pair_of(v.y), x2 = pair_of(v.z), x3 = pair_of(v.w);
+            own2[0] = ffma2(fmul2(g0.x, x0), x0, own2[0]);
+            own2[1] = ffma2(fmul2(g0.y, x1), x1, own2[1]);
+            own2[0] = ffma2(fmul2(g1.x, x2), x2, own2[0]);
+            own2[1] = ffma2(fmul2(g1.y, x3), x3, own2[1]);
+          }
+          __syncwarp();
         }
-        const float q = sum4(q2[0], q2[1]), vv = sum4(vv2[0], vv2[1]);
-        const bool sound = (q >= kGmMinShare * gmax * vv && q <= 1e37f && vv >= 1e-30f && vv <= 1e30f && gmax >= 1e-25f &&
-                            gmax <= 1e30f) || ((any & 0x7FFF7FFFu) == 0 && q == 0.f);
+        if (uneven) sound = sound && sum4(own2[0], own2[1]) <= most;
+        if (lane == 0) mbar_arrive(bar(kGmVEmpty, stage), 1);
+        sound = sound || ((any & 0x7FFF7FFFu) == 0 && q == 0.f);
         const int seq = t / a.tiles, tile = t - seq * a.tiles, j = tile * 128 + row;
         const size_t ug = (size_t)(seq * a.LH + uh) * a.G + g;
         if (j < a.n) a.vnorm[ug * a.n + j] = sqrtf(q);
-        const bool bad = __any_sync(0xffffffffu, j < a.n && !sound);
-        if (lane == 0) a.flags[((ug * a.chunks4k + tile / 32) * 32 + tile % 32) * 4 + quad] = bad;
+        const uint32_t left = __ballot_sync(0xffffffffu, j < a.n && !sound);
+        if (lane == 0) a.left[(ug * a.tiles + tile) * 4 + quad] = left;
       }
     }
   } else {
     // ---------------- Gram sums and pieces ----------------
-    const int quad = warp & 3, half = (warp - 12) >> 2, gw = warp - 12;
+    const int quad = warp & 3, half = (warp - 12) >> 2;
     const int row = 32 * quad + lane;               // row of G = column of D
     constexpr int kCols = 32 * NH;                  // this warp's columns of G, from kCols * half on
     const uint32_t lane_addr = (uint32_t)(32 * quad) << 16;
@@ -320,15 +374,9 @@ __global__ void __launch_bounds__(kGmThreads, 1)
         if (lane == 0) mbar_arrive(bar(kGmGEmpty, b), 1);
       }
       if (!ok) break;
-      float mx = 0.f;
-      if (live) {
-#pragma unroll
-        for (int i = 0; i < kCols; ++i) mx = fmaxf(mx, fabsf(acc[i]));
-      }
-      mx = warp_max(mx);
+      float own = 0.f;  // G[row][row], where it is one of this thread's columns
       // the tiles of the item before have been multiplied
       if (!(ok = wait(bar(kGmBEmpty, 0), (it & 1) ^ 1))) break;
-      if (lane == 0) gmax_s[it & 3][gw] = mx;
       if (live) {
 #pragma unroll
         for (int c = 0; c < kCols / 8; ++c) {
@@ -338,6 +386,8 @@ __global__ void __launch_bounds__(kGmThreads, 1)
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             float x = acc[8 * c + 2 * i] * f, y = acc[8 * c + 2 * i + 1] * f;
+            if (k0 + 2 * i == row) own = x;  // f is 1 there
+            if (k0 + 2 * i + 1 == row) own = y;
 #pragma unroll
             for (int piece = 0; piece < 3; ++piece) {
               const __nv_bfloat162 p = __floats2bfloat162_rn(x, y);
@@ -354,6 +404,9 @@ __global__ void __launch_bounds__(kGmThreads, 1)
                 make_uint4(w[piece][0], w[piece][1], w[piece][2], w[piece][3]);
         }
       }
+      if (live && row / kCols == half) diag_s[it & 3][row] = own;
+      own = warp_max(own);
+      if (lane == 0) gmax_s[it & 3][warp - 12] = own;
       // the MMA reads shared memory through the asynchronous proxy: order these writes before it
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       __syncwarp();
@@ -388,7 +441,6 @@ bool make_panel_map(CUtensorMap* map, const void* base, uint64_t rows, int cols,
 }
 
 int gm_tiles(const Dims& dm) { return (dm.n + 127) / 128; }
-int gm_chunks4k(const Dims& dm) { return (dm.n + 4095) / 4096; }
 
 // Tiles per item and the time that the call would take, by this kernel and by the direct one.
 struct GmChoice {
@@ -397,7 +449,8 @@ struct GmChoice {
 };
 GmChoice gm_choose(const Dims& dm, int d_model, int sms) {
   const bool wide = dm.d == 128;
-  // measured with every SM busy (48 query heads x 3 to 1024 x 31 tiles, 512 to 4096 columns), us: 64 projection columns into the Gram matrix, a tile through it, a tile times 256 columns
+  // measured with every SM busy (48 query heads x 3 to 1024 x 31 tiles, 512 to 4096 columns), us: 64 projection columns into
+  // the Gram matrix, a tile through it, a tile times 256 columns
   const double panel = wide ? 0.55 : 0.4, tile = wide ? 1.1 : 0.7, direct = wide ? 0.72 : 0.4;
   const long long slices = (long long)dm.N * dm.G, all = (long long)dm.S * gm_tiles(dm);
   const double gram = panel * ((d_model + 63) / 64);
@@ -408,13 +461,13 @@ GmChoice gm_choose(const Dims& dm, int d_model, int sms) {
     if (us < 0.99 * best.gram_us) best.gram_us = us, best.per_item = (int)per;
   }
   best.gram_us += 5.0;  // the direct kernel's look at the flags
-  const long long chunks = gm_chunks4k(dm), items = dm.heads() * dm.G * chunks;
+  const long long items = dm.heads() * dm.G * ((dm.n + 4095) / 4096);  // of the direct kernel
   best.direct_us = direct * (double)((items + sms - 1) / sms) * std::min(32, gm_tiles(dm)) * ((d_model + 255) / 256);
   return best;
 }
 }  // namespace
 
-size_t value_norm_gram_flag_bytes(const Dims& dm) { return (size_t)dm.heads() * dm.G * gm_chunks4k(dm) * 128; }
+size_t value_norm_gram_left_bytes(const Dims& dm) { return (size_t)dm.heads() * dm.G * gm_tiles(dm) * 16; }
 
 bool value_norm_gram_pays(const Dims& dm, int d_model, const void* w_o) {
   if (!value_norm_tc_supported(dm) || (d_model & 7) || (reinterpret_cast<uintptr_t>(w_o) & 15)) return false;
@@ -422,25 +475,26 @@ bool value_norm_gram_pays(const Dims& dm, int d_model, const void* w_o) {
     return false;
   int sms = 0;
   if (device_sms(&sms) != cudaSuccess) return false;
+  // LUKV_VALUE_NORM=gram or direct: that form wherever the shape allows it (for A/B checks; read at every call)
+  const char* form = getenv("LUKV_VALUE_NORM");
+  if (form && (form[0] == 'g' || form[0] == 'd')) return form[0] == 'g';
   const GmChoice c = gm_choose(dm, d_model, sms);
   return c.gram_us < c.direct_us;
 }
 
 cudaError_t launch_value_norm_gram(const Dims& dm, int d_model, const void* v, const void* w_o, float* vnorm,
-                                   unsigned char* flags, int32_t* status, LaunchCtx& lc) {
+                                   uint32_t* left, int32_t* status, LaunchCtx& lc) {
   CUtensorMap vm, wm;
   if (!make_map(&vm, v, (uint64_t)dm.heads() * dm.T, dm.d) ||
       !make_panel_map(&wm, w_o, (uint64_t)dm.L * dm.H * dm.G * dm.d, d_model, dm.d))
     return cudaErrorNotSupported;
   GmArgs a;
   a.vnorm = vnorm;
-  a.flags = flags;
+  a.left = left;
   a.S = dm.S, a.LH = dm.N, a.G = dm.G, a.T = dm.T, a.n = dm.n, a.Dm = d_model;
   a.tiles = gm_tiles(dm);
-  a.chunks4k = gm_chunks4k(dm);
   a.status = status;
-  int drop = 0;
-  score_test_hooks(&a.spin_limit, &drop);
+  score_test_hooks(&a.spin_limit, &a.drop_item);
   int sms = 0;
   cudaError_t e;
   if ((e = device_sms(&sms)) != cudaSuccess) return e;

@@ -104,6 +104,102 @@ def test_value_norms_through_the_gram_matrix(monkeypatch, kind, S, L, H, G, d, T
     np.testing.assert_allclose(gram, simt, rtol=2e-5, atol=1e-30)
 
 
+FORMS = {"gram": 1, "direct": 0}  # launches beyond the direct form's
+
+
+@pytest.mark.parametrize("S,L,H,G,d,T,w,Dm", [
+    (1, 1, 1, 1, 128, 130, 2, 2048),      # one tile, filled to the last position
+    (1, 3, 8, 7, 128, 161, 32, 1032),     # a tile with one position; 168 slices on 148 SMs; a last panel of 8 columns
+    (1, 5, 8, 7, 128, 761, 32, 2056),     # 280 slices: several items a CTA, the next Gram matrix beside the present tiles
+    (1, 5, 8, 7, 64, 761, 32, 2056),
+    (2, 1, 3, 5, 128, 4096 + 700, 16, 264),  # two chunks of positions; five panels
+    (3, 2, 2, 2, 64, 300, 5, 24),         # one panel, not full
+])
+@pytest.mark.parametrize("kind", ["normal", "null", "zero", "large"])
+@pytest.mark.parametrize("form", FORMS)
+def test_both_forms_of_the_value_norms(monkeypatch, form, kind, S, L, H, G, d, T, w, Dm):
+    """The Gram matrix and the projection multiplied out, each at every size, against the FP32 pipes.  Every kind but "normal"
+    has projections or positions that the Gram form leaves beside ones that it takes."""
+    q, k, v, kd, wo = _inputs(S, L, H, G, d, T, 2, Dm, torch.bfloat16, seed=T + Dm)
+    if kind == "null":
+        wo[:, 0, -1] *= 1e-4
+        v[:, :, :, 5::131, :-1] = 0
+    elif kind == "zero":
+        v[:, :, :, ::3] = 0
+        wo[:, -1] = 0
+    elif kind == "large":
+        wo[:, 0] *= 2.0 ** 70
+        v[:, :, 0, ::64] *= 2.0 ** -60
+    p = lukv.make_params(S, L, H, G, d, T, w, 1, torch.bfloat16, 2)
+    monkeypatch.setenv("LUKV_VALUE_NORM", form)
+    got = gpu_importance(p, 2, Dm, q, k, v, kd, wo, False)
+    launches = lukv.lukv_last_launch_count()
+    monkeypatch.setenv("LUKV_VALUE_NORM", "direct")
+    gpu_importance(p, 2, Dm, q, k, v, kd, wo, False)
+    assert launches - lukv.lukv_last_launch_count() == FORMS[form]
+    monkeypatch.setenv("LUKV_FORCE_SIMT", "1")
+    simt = gpu_importance(p, 2, Dm, q, k, v, kd, wo, False)
+    np.testing.assert_allclose(got, simt, rtol=2e-5, atol=1e-30)
+
+
+@pytest.mark.parametrize("d,Dm", [(128, 4096), (128, 1032), (64, 4096)])
+@pytest.mark.parametrize("kind", ["normal", "common0.5", "common1", "common2", "common5", "halves", "row10", "row100", "decay1",
+                                  "decay2"])
+def test_value_norms_keep_their_digits(monkeypatch, kind, d, Dm):
+    """Against 64 bits, where the terms of the quadratic form cancel: projections whose rows share a component that the values
+    take out again, single large rows, singular values that fall.  The Gram form has to be as good as the projection
+    multiplied out, whose error is that of sums rounded to 24 bits in 64 to 128 steps (1e-7 rms, 4e-7 at most for these inputs);
+    half as much again leaves room for the sums' other order."""
+    T, w = 4096, 8
+    n = T - w
+    g = torch.Generator(device="cuda").manual_seed(17)
+    r = lambda *s: torch.randn(s, generator=g, device="cuda", dtype=torch.float64)
+    W, V, common = r(d, Dm), r(T, d), r(Dm)
+    if kind.startswith("common"):
+        W += float(kind[6:]) * common
+        V -= V.mean(1, keepdim=True)
+    elif kind == "halves":
+        W += 5.2 * common
+        V = V.abs()
+        V[:, d // 2:] *= -1
+        V -= V.mean(1, keepdim=True)
+    elif kind.startswith("row"):
+        W[3] *= float(kind[3:])
+    elif kind.startswith("decay"):
+        u, _ = torch.linalg.qr(r(d, d))
+        c, _ = torch.linalg.qr(r(Dm, d))
+        W = (u * torch.arange(1, d + 1, device="cuda", dtype=torch.float64) ** -float(kind[5:])) @ c.T * 30
+    v, wo = V.bfloat16()[None, None, None], W.bfloat16()[None, None]
+    ref = (v[0, 0, 0].double() @ wo[0, 0].double()).square().sum(1).sqrt()[:n].cpu().numpy() / T
+    q = torch.zeros((1, 1, 1, 1, d), dtype=torch.bfloat16)          # equal weights 1/T: the importance is the norm over T
+    k = torch.zeros((1, 1, 1, T, d), dtype=torch.bfloat16)
+    p = lukv.make_params(1, 1, 1, 1, d, T, w, 1, torch.bfloat16, 2)
+    err = {}
+    for form in FORMS:
+        monkeypatch.setenv("LUKV_VALUE_NORM", form)
+        err[form] = gpu_importance(p, 1, Dm, q, k, v, None, wo, False)[0, 0].astype(np.float64) / ref - 1
+    rms = {form: np.sqrt((e ** 2).mean()) for form, e in err.items()}
+    print(kind, d, Dm, rms, {form: np.abs(e).max() for form, e in err.items()})
+    assert rms["gram"] <= 1.5 * rms["direct"] and np.abs(err["gram"]).max() <= 1e-6
+
+
+def test_a_wait_of_the_gram_form_that_runs_out_leaves_nan(monkeypatch):
+    """With the test hooks the value tiles of item 31, which only the Gram kernel has, are never loaded (32 slices, of at most
+    three items; the other kernels have up to 12 items).  The next ordinary call gives the bits of a fresh one."""
+    S, L, H, G, d, T, w, Kmax, Dm = 1, 1, 4, 8, 64, 300, 32, 2, 128
+    q, k, v, kd, wo = _inputs(S, L, H, G, d, T, Kmax, Dm, torch.bfloat16, seed=6)
+    p = lukv.make_params(S, L, H, G, d, T, w, 1, torch.bfloat16, 2)
+    monkeypatch.setenv("LUKV_VALUE_NORM", "gram")
+    ref = gpu_importance(p, Kmax, Dm, q, k, v, kd, wo, False)
+    assert not np.isnan(ref).any()
+    monkeypatch.setenv("LUKV_TEST_SPIN_LIMIT", "20000")
+    monkeypatch.setenv("LUKV_TEST_DROP_ITEM", "31")
+    assert np.isnan(gpu_importance(p, Kmax, Dm, q, k, v, kd, wo, False)).all()
+    monkeypatch.delenv("LUKV_TEST_DROP_ITEM")
+    monkeypatch.delenv("LUKV_TEST_SPIN_LIMIT")
+    np.testing.assert_array_equal(gpu_importance(p, Kmax, Dm, q, k, v, kd, wo, False), ref)
+
+
 @pytest.mark.parametrize("S,L,H,G,d,T,w,Kmax,Dm,with_kd", [
     (1, 1, 2, 1, 64, 130, 1, 1, 64, True),        # one step, one query head; a key tile with two keys
     (1, 1, 2, 2, 128, 129, 32, 65, 40, True),     # steps just past one query tile; odd panel width
