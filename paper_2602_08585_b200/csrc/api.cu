@@ -219,8 +219,10 @@ static SideStream* side_stream() {
 // The whole path.  Allocation depends only on the curves, scoring only on Q/K; selection needs both, the gather follows.
 // With `overlap` allocation runs beside the scorer.  Up to 32 heads: one CTA per sequence, on the caller's stream, behind a
 // persistent scorer (tensor-core, KeyDiff), which leaves it an SM, behind the general-shape scorer where that has a CTA per
-// SM at most and so room for its sweeps and the allocation at once (4 heads x 1024 keys: 18.2 us a call, 20.5 with the
-// allocation ahead, whose time is longer than the first sweep's), or else ahead of its first sweep;
+// SM at most and so room for its sweeps and the allocation at once (4 heads x 1024 keys: 17.0 us a call where calls are queued
+// ahead, 20.5 with the allocation in front, whose time is longer than the first sweep's; 16 x 512 24.6 and 30.8, 4 heads x 4
+// query heads x 1024, d = 128, 40.0 and 40.3; where the host's launches are in the way 20.2 and 20.5), or else ahead of its
+// first sweep;
 // neighbours in the stream are programmatic dependents, and whichever of scorer and allocation comes second ends after the
 // first, so that the selection, which waits for the second, sees both.  More heads: hulls and greedy on an auxiliary
 // stream, whose hulls take the SMs before the scorer does (256 heads x 513 points with 1536 keys: 87 us a call; hulls by

@@ -20,8 +20,8 @@
 // little else to hide their loads behind.  Chunks of which more than three quarters are left are computed whole, as in the other
 // form (a gathered tile takes 0.95 us a panel, a whole chunk's 0.75).  The chunk's positions are listed by all threads, so its
 // roles meet at its ends.  256 heads x 4 query heads x 3968 positions x 4096 columns, a call of one step: nothing left 0.53 ms,
-// 1 % of the positions 0.89, 9 % 1.03, 27 % 1.9, 70 % 2.9, all 3.9; every position in this form at once 3.0 to 3.5.  One
-// gathering warp took 1.05, 6.8 and 11.7 ms where 1, 9 and 70 % are left.
+// 1 % of the positions 0.89, 9 % 1.03, 27 % 1.9, 70 % 2.9, all 3.9 (11.7 with a single gathering warp); every position in the
+// other form at once 3.0 to 3.5.
 // Every wait is bounded; the waits are between the warps of one CTA only.
 #include "tc_ptx.cuh"
 

@@ -65,8 +65,8 @@ def test_importance_matches_oracle(oracle, shape):
 
 
 def test_value_norms_tensor_core_against_fp32_pipes(monkeypatch):
-    """The two value-norm kernels (tensor cores; FP32 pipes, kept for other shapes) agree far inside the tolerance:
-    bf16 products are exact in fp32 and both accumulate in fp32."""
+    """The value norms on the tensor cores (in the form that the cost model takes) and on the FP32 pipes, kept for other shapes,
+    agree far inside the tolerance: bf16 products are exact in fp32 and both accumulate in fp32."""
     S, L, H, G, d, T, w, Kmax, Dm = 1, 2, 2, 4, 128, 2000, 32, 4, 1024
     q, k, v, kd, wo = _inputs(S, L, H, G, d, T, Kmax, Dm, torch.bfloat16, seed=21)
     p = lukv.make_params(S, L, H, G, d, T, w, 1, torch.bfloat16, 2)
@@ -84,9 +84,10 @@ def test_value_norms_tensor_core_against_fp32_pipes(monkeypatch):
 ])
 @pytest.mark.parametrize("kind", ["normal", "null", "zero", "large"])
 def test_value_norms_through_the_gram_matrix(monkeypatch, kind, S, L, H, G, d, T, w, Dm):
-    """Sizes that take the Gram matrix of the projection against the FP32 pipes, which multiply it out.  Both round sums of
-    exact products to 24 bits.  "null": some values lie where the projection is 1e-4 of its size, their chunks are left to the
-    direct kernel; "zero": zero values and a zero projection; "large": squares beyond fp32's range are left to it as well."""
+    """The form that the cost model takes (the Gram matrix of the projection for the last two sizes, the projection multiplied out
+    for the first two) against the FP32 pipes.  All round sums of exact products to 24 bits.  "null": some values lie where the
+    projection is 1e-4 of its size and are left to the direct kernel; "zero": zero values and a zero projection; "large": squares
+    beyond fp32's range are left to it as well."""
     q, k, v, kd, wo = _inputs(S, L, H, G, d, T, 2, Dm, torch.bfloat16, seed=T + Dm)
     if kind == "null":
         wo[:, 0, -1] *= 1e-4

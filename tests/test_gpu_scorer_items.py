@@ -60,5 +60,5 @@ def test_items_of_one_tile(S, L, H, G, d, w, kp, lens):
     (3, 1, 4, 4, 128, 32, 7, [3000, 640, 1000]), (5, 3, 8, 2, 64, 16, 7, [9000, 4125, 250, 7000, 875]),
 ])
 def test_items_of_a_small_call(S, L, H, G, d, w, kp, lens):
-    """Calls with few heads share a head out over more and smaller items, of sizes that differ by one tile."""
+    """Calls with few heads share a head out over more and smaller items; with several lengths their sizes differ by one tile."""
     test_items_of_one_tile(S, L, H, G, d, w, kp, lens)
