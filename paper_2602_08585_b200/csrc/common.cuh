@@ -190,9 +190,9 @@ cudaError_t launch_keydiff(const Dims& dm, const void* k, float* scores, int str
 bool value_norm_tc_supported(const Dims& dm);
 cudaError_t launch_value_norm_tc(const Dims& dm, int d_model, const void* v, const void* w_o, float* vnorm,
                                  const uint32_t* left, int32_t* status, LaunchCtx& lc);
-// The same through the Gram matrix of the projection; positions for which it is not sound are left to the kernel above.
+// The same through the Gram matrix of the projection; positions for which it is not sound are left to the kernel above (left:
+// as many bytes as the importance has at most, where the form pays).
 bool value_norm_gram_pays(const Dims& dm, int d_model, const void* w_o);
-size_t value_norm_gram_left_bytes(const Dims& dm);
 cudaError_t launch_value_norm_gram(const Dims& dm, int d_model, const void* v, const void* w_o, float* vnorm,
                                    uint32_t* left, int32_t* status, LaunchCtx& lc);
 // Attention part of the oracle importance on the tensor cores (bf16, up to 8 query heads per KV head): needs the value

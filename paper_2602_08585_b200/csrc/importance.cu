@@ -9,7 +9,6 @@
 //   imp_lse_kernel      row log-sum-exp of every (head, g, step), exp2 domain
 //   imp_kernel          probabilities x value norms, summed over g inside a thread, maximum over the steps
 //   imp_normalize_kernel  one CTA per (sequence, layer): fp64 total in a fixed order, then the division
-#include <algorithm>
 #include <cstdlib>
 
 #include "simt_tile.cuh"
@@ -289,7 +288,7 @@ cudaError_t launch_importance_t(const Dims& dm, ImpDims id, const void* q_dec, c
   if (norms_tc) {
     uint32_t* left = nullptr;
     if (value_norm_gram_pays(dm, id.Dm, w_o)) {
-      left = reinterpret_cast<uint32_t*>(lse);  // the log-sum-exps come later
+      left = reinterpret_cast<uint32_t*>(importance);  // which is written by the kernels behind
       if ((e = launch_value_norm_gram(dm, id.Dm, v, w_o, vnorm, left, status, lc)) != cudaSuccess) return e;
     }
     if ((e = launch_value_norm_tc(dm, id.Dm, v, w_o, vnorm, left, status, lc)) != cudaSuccess) return e;
@@ -316,12 +315,12 @@ cudaError_t launch_importance_t(const Dims& dm, ImpDims id, const void* q_dec, c
 
 }  // namespace
 
-// value norms, row log-sum-exps (or their partials; before them the bits of the positions that the Gram form leaves), the status word
+// value norms, row log-sum-exps (or their partials), the status word
 static size_t importance_status_offset(const Dims& dm, int k_max) {
   const size_t a = ((size_t)dm.heads() * dm.G * dm.n * sizeof(float) + 255) & ~(size_t)255;
   const size_t rows = (size_t)dm.heads() * dm.G * k_max * sizeof(float);  // row log-sum-exps; room for their partials
-  const size_t b = std::max(rows + (dm.G <= 8 ? importance_tc_part_bytes(dm, k_max) : 0), value_norm_gram_left_bytes(dm));
-  return a + ((b + 255) & ~(size_t)255);
+  const size_t b = (rows + (dm.G <= 8 ? importance_tc_part_bytes(dm, k_max) : 0) + 255) & ~(size_t)255;
+  return a + b;
 }
 size_t importance_workspace_bytes(const Dims& dm, int k_max) { return importance_status_offset(dm, k_max) + 256; }
 

@@ -467,12 +467,12 @@ GmChoice gm_choose(const Dims& dm, int d_model, int sms) {
 }
 }  // namespace
 
-size_t value_norm_gram_left_bytes(const Dims& dm) { return (size_t)dm.heads() * dm.G * gm_tiles(dm) * 16; }
-
 bool value_norm_gram_pays(const Dims& dm, int d_model, const void* w_o) {
   if (!value_norm_tc_supported(dm) || (d_model & 7) || (reinterpret_cast<uintptr_t>(w_o) & 15)) return false;
   if ((int64_t)dm.N * dm.G * dm.d >= ((int64_t)1 << 31) || dm.heads() * dm.G * (int64_t)gm_tiles(dm) >= ((int64_t)1 << 31))
     return false;
+  // the bits of the positions that are left lie where the importance will (groups beyond 32, or a few positions: no room)
+  if ((int64_t)dm.G * gm_tiles(dm) * 16 > (int64_t)dm.n * 4) return false;
   int sms = 0;
   if (device_sms(&sms) != cudaSuccess) return false;
   // LUKV_VALUE_NORM=gram or direct: that form wherever the shape allows it (for A/B checks; read at every call)

@@ -141,6 +141,18 @@ def test_profile_argument_errors_come_back_before_any_launch():
     assert lukv.lukv_profile_budgets(p, None, grid, [0.5, 0.5], f, f, check=False) == lukv.ERR_INVALID_ARG
 
 
+@pytest.mark.parametrize("S,L,H,G,d,T,w,steps", [(1, 1, 8, 1, 128, 130, 32, 1), (1, 32, 8, 4, 128, 130, 32, 1), (1, 2, 4, 7, 64, 130, 16, 1),
+                                                  (2, 4, 8, 8, 128, 500, 32, 2), (1, 32, 8, 4, 128, 8192, 32, 1)])
+def test_importance_scratch_holds_norms_and_row_sums_only(S, L, H, G, d, T, w, steps):
+    """A value norm per (query head, position), a log-sum-exp per (query head, step), and as many partial ones as the keys are
+    split: at most one split for every four key tiles, 128 rows each."""
+    p = lukv.make_params(S, L, H, G, d, T, w, 1, "bf16", 2)
+    heads, n, rows = S * L * H, T - w, steps * (1 << (G - 1).bit_length())
+    partials = heads * -(-rows // 128) * max(1, -(-T // 128) // 4) * 128 * 4
+    need = 4 * heads * G * n + 4 * heads * G * steps + partials
+    assert lukv.lukv_importance_workspace_bytes(p, steps) <= need + 3 * 256
+
+
 def test_importance_argument_errors_come_back_before_any_launch():
     p = _p()
     f = _Fake()
