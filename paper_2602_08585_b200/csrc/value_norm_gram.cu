@@ -264,7 +264,6 @@ __global__ void __launch_bounds__(kGmThreads, 1)
         const float* diag = diag_s[it & 3];
         float q = 0.f, terms = 0.f;
         uint64_t vv2[2] = {0, 0}, own2[2] = {0, 0};
-        uint32_t any = 0;
         float d[32];
         tmem_ld32(tmem_base + lane_addr + s * 128, d);
         ok = wait(bar(kGmVFull, stage), stage_ph);  // (behind the load: the test is a round trip to shared memory)
@@ -295,7 +294,6 @@ __global__ void __launch_bounds__(kGmThreads, 1)
                     const uint64_t g = *reinterpret_cast<const uint64_t*>(diag + 32 * c0 + 8 * c + 2 * i);
                     own2[b] = ffma2(fmul2(g, x), x, own2[b]);
                   }
-                  any |= w4[i];
                 }
               }
               float even, odd;
@@ -329,8 +327,18 @@ __global__ void __launch_bounds__(kGmThreads, 1)
           __syncwarp();
         }
         if (uneven) sound = sound && sum4(own2[0], own2[1]) <= most;
+        // a value of zeros has the norm zero (if the projection holds numbers); squares below fp32's range look the same
+        if (__any_sync(0xffffffffu, vv == 0.f)) {
+          uint32_t any = 0;
+#pragma unroll 2
+          for (int c = 0; c < 8 * NH; ++c) {
+            const uint4 v = value8(c);
+            any |= v.x | v.y | v.z | v.w;
+          }
+          sound = sound || ((any & 0x7FFF7FFFu) == 0 && q == 0.f);
+          __syncwarp();
+        }
         if (lane == 0) mbar_arrive(bar(kGmVEmpty, stage), 1);
-        sound = sound || ((any & 0x7FFF7FFFu) == 0 && q == 0.f);
         const int seq = t / a.tiles, tile = t - seq * a.tiles, j = tile * 128 + row;
         const size_t ug = (size_t)(seq * a.LH + uh) * a.G + g;
         if (j < a.n) a.vnorm[ug * a.n + j] = sqrtf(q);
