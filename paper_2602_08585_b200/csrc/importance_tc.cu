@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kItThreads, 1)
           const float2 o = merge_s[qtid];
           const float mn = fmaxf(m, o.x);
           float v = -INFINITY;
-          if (row_ok && mn > -INFINITY) v = mn + log2f((l > 0.f ? l * ex2(m - mn) : 0.f) + (o.y > 0.f ? o.y * ex2(o.x - mn) : 0.f));
+          if (row_ok && mn > -INFINITY) v = p1_log(mn, (l > 0.f ? l * ex2(m - mn) : 0.f) + (o.y > 0.f ? o.y * ex2(o.x - mn) : 0.f));
           a.part[(((size_t)it.u * a.chunks + it.c0) * a.splits + it.split) * 128 + qtid] = v;
         }
         bar_sync(1, kItEpiThreads);

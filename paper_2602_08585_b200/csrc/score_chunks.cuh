@@ -6,6 +6,18 @@
 namespace lukv {
 namespace {
 
+// Largest sum of a chunk or tile relative to the running reference before pass 1 takes a new one.  fp32 keeps its relative
+// precision all the way, so the limit only guards the exponent: 2^80 times the tiles of an item stays far below 2^127, and a sum
+// that is merged with one at a reference 126 or more binary orders higher still counts for less than 2^-30 of it.
+constexpr float kP1Limit = 1.2e24f;
+// m + log2(l) of such a sum, the binary exponent apart so that the logarithm's own error stays that of [1, 2).
+__device__ __forceinline__ float p1_log(float m, float l) {
+  if (!(l > 0.f)) return -INFINITY;
+  const uint32_t b = __float_as_uint(l);
+  if (b >= 0x7F800000u) return m + l;
+  return (m + (float)((int)(b >> 23) - 127)) + log2f(__uint_as_float((b & 0x007FFFFFu) | 0x3F800000u));
+}
+
 // Pass 1, 32 columns (keys jbase..jbase+31) of one query row: fold into the running (m, l).
 // (m, l) means sum over the keys seen so far of exp2(x - m); m is a reference point, not
 // necessarily the maximum: the common path adds the new terms relative to the current m and
@@ -33,10 +45,53 @@ __device__ __forceinline__ void p1_chunk(const float (&v)[32], int jbase, int li
     }
   }
   const float cs = sum4(acc0, acc1);
-  if (cs <= 1e12f && fmaf(pmax, scale_log2, -m) <= 100.f) {  // false for inf and NaN
+  if (cs <= kP1Limit && fmaf(pmax, scale_log2, -m) <= 100.f) {  // false for inf and NaN
     l += cs;
     return;
   }
+  float cmax = x[0];
+#pragma unroll
+  for (int i = 1; i < 32; ++i) cmax = fmaxf(cmax, x[i]);
+  if (cmax == -INFINITY) return;  // every key of the chunk is masked
+  const float mn = fmaxf(m, cmax * scale_log2);  // scale > 0
+  float a0 = l * ex2(m - mn), a1 = 0.f;
+#pragma unroll
+  for (int i = 0; i < 32; i += 2) {
+    a0 += ex2(fmaf(x[i], scale_log2, -mn));
+    a1 += ex2(fmaf(x[i + 1], scale_log2, -mn));
+  }
+  l = a0 + a1;
+  m = mn;
+}
+
+// The same in parts, for a whole tile whose keys are all visible: reference point, terms without a branch, test, and the exact
+// form, chunk by chunk, for tiles that fail it or have hidden keys.
+__device__ __forceinline__ float p1_reference(const float (&v)[32], float scale_log2) {
+  float c = v[0];
+#pragma unroll
+  for (int i = 1; i < 32; ++i) c = fmaxf(c, v[i]);
+  return c * scale_log2;
+}
+__device__ __forceinline__ void p1_terms(const float (&x)[32], uint64_t sc2, uint64_t nm2, uint64_t& acc0, uint64_t& acc1,
+                                         float& pmax) {
+#pragma unroll
+  for (int i = 0; i < 32; i += 4) {
+    acc0 = fadd2(acc0, ex2_pair(ffma2(pack2(x[i], x[i + 1]), sc2, nm2)));
+    if (LUKV_POLY_SEL1(i)) {
+      pmax = fmaxf(pmax, fmaxf(x[i + 2], x[i + 3]));
+      acc1 = fadd2(acc1, ex2_poly_pair<false>(ffma2(pack2(x[i + 2], x[i + 3]), sc2, nm2)));
+    } else {
+      acc1 = fadd2(acc1, ex2_pair(ffma2(pack2(x[i + 2], x[i + 3]), sc2, nm2)));
+    }
+  }
+}
+__device__ __forceinline__ bool p1_in_range(float sum, float pmax, float scale_log2, float m) {
+  return sum <= kP1Limit && fmaf(pmax, scale_log2, -m) <= 100.f;  // false for inf and NaN
+}
+__device__ __forceinline__ void p1_exact(const float (&v)[32], int jbase, int lim, float scale_log2, float& m, float& l) {
+  float x[32];
+#pragma unroll
+  for (int i = 0; i < 32; ++i) x[i] = jbase + i <= lim ? v[i] : -INFINITY;
   float cmax = x[0];
 #pragma unroll
   for (int i = 1; i < 32; ++i) cmax = fmaxf(cmax, x[i]);

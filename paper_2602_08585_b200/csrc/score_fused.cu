@@ -16,8 +16,7 @@
 // at most one CTA per SM, launched cooperatively (all CTAs resident).  A CTA runs pass 1
 // lag-1 items ahead of pass 2, so that the log-sum-exp of a head is normally complete before
 // pass 2 needs it.  With small items the key tiles pass 2 re-reads are still in L2 (K crosses
-// HBM once); the launcher prefers large items where there are enough of them, which re-read K
-// from HBM but change jobs less often (the kernel is bound by the exp2 evaluation, not by HBM).
+// HBM once); large ones re-read K from HBM but change jobs less often (the launcher weighs it).
 //
 // Warp roles per CTA: 4*NQ epilogue warps in NQ quads (a warp may only read the TMEM lanes
 // 32*(warp%4)..+31), then one warp each: TMA producer, MMA issuer 0 and TMEM owner, MMA issuer 1,
@@ -38,12 +37,9 @@ namespace {
 template <int MT, int NQ, int NH>
 struct Plan {
   static_assert(MT == 1 || NQ == 2, "two query-row blocks are split over exactly two quads");
-  // An mbarrier wait only knows the parity of the phase it waits for, so the successive phases of a
-  // barrier must be waited for by the same threads in order.  Accumulator buffer b = tile % kNumBufs is
-  // read by quad tile % NQ and written by issuer tile % 2: both must be functions of b.
-  // With three quads the buffers rotate over the quads, so "accumulator complete" has two barriers per
-  // buffer, used alternately: a quad that runs ahead then still waits on a barrier whose previous
-  // phase (eight tiles back) is long complete.
+  // An mbarrier wait only knows the parity of the phase it waits for, so a thread must not wait for a phase whose predecessor may
+  // be incomplete.  An accumulator buffer takes one row block of one key tile, buffer (tile * MT + block) % kNumBufs, and is
+  // written by issuer tile % 2; see kFullSets for its readers.
   static_assert(NQ == 2 || (MT == 1 && NQ == 3), "two quads, or three that take the tiles in turn");
   static constexpr int kEpiWarps = 4 * NQ;
   // + TMA producer, two MMA issuers, helper.  The count stays a multiple of 4 warps: the register
@@ -54,10 +50,13 @@ struct Plan {
   // odd count the two issuers would take turns on a stage, and the one that runs ahead could wait
   // for a phase two ahead of the barrier -- which a parity wait reports as complete while the
   // previous load of that stage is still in flight.
-  static constexpr int kStages = (MT == 1 ? 4 : 2) * (3 - NH);
+  static constexpr int kStages = 4 * (3 - NH);
   static constexpr int kStageBytes = NH * kHalfBytes;
   static_assert(kStages % 2 == 0, "a key stage must always be consumed by the same MMA issuer");
-  static constexpr int kQSlots = 2;                    // query tiles of the job in the tensor pipe and the next one
+  // Query tiles of the job in the tensor pipe and of the next one.  One slot where two of 256 rows x 128 channels would leave room
+  // for two key stages only, which do not cover the latency of their loads (eight 16k sequences of 256 rows: 7690 us a call with
+  // two slots and two stages, 7615 so).
+  static constexpr int kQSlots = MT == 2 && NH == 2 ? 1 : 2;
   static constexpr int kQBytes = MT * kStageBytes;     // [half][MT*128 rows][128 B]
   static constexpr int kFinBufs = 1;                   // blocks of partials in flight while a head is folded
   static constexpr int kFinBytes = 16384;              // one block
@@ -65,12 +64,17 @@ struct Plan {
   static constexpr int kKOff = kQSlots * kQBytes;
   static constexpr int kFinOff = kKOff + kStages * kStageBytes;
   static constexpr int kBarOff = kFinOff + kFinBufs * kFinBytes;
-  static constexpr int kNumBufs = 4 / MT;              // accumulator buffers in TMEM
-  static constexpr int kBufCols = 128 * MT;
-  // barriers: full[kStages], empty[kStages], qfull[kQSlots], qempty[kQSlots], tfull[2][kNumBufs],
+  static constexpr int kNumBufs = 4;                   // accumulator buffers in TMEM, one row block of a key tile each
+  static constexpr int kBufCols = 128;
+  // "Accumulator complete" barriers per buffer, used in turn, so that a quad that runs ahead waits on a barrier whose previous phase
+  // is long complete.  With one row block a quad only ever reads what one issuer wrote (or, with three quads, is held back by the
+  // key ring), two sets do.  With two it reads one block of every tile in pass 1 and both of every other one in pass 2: a set per
+  // key stage, since a tile 2 kFullSets back that is not issued keeps the key ring from loading the tile before this one.
+  static constexpr int kFullSets = MT == 2 ? kStages : 2;
+  // barriers: full[kStages], empty[kStages], qfull[kQSlots], qempty[kQSlots], tfull[kFullSets][kNumBufs],
   // tempty[kNumBufs], pub_full[NQ], pub_empty[NQ], lse_full[kMaxLag], lse_empty[kMaxLag], fin[kFinBufs]
   static constexpr int kBarFull = 0, kBarEmpty = kStages, kBarQFull = 2 * kStages, kBarQEmpty = kBarQFull + kQSlots,
-                       kBarTFull = kBarQEmpty + kQSlots, kBarTEmpty = kBarTFull + 2 * kNumBufs,
+                       kBarTFull = kBarQEmpty + kQSlots, kBarTEmpty = kBarTFull + kFullSets * kNumBufs,
                        kBarPubFull = kBarTEmpty + kNumBufs, kBarPubEmpty = kBarPubFull + NQ,
                        kBarLseFull = kBarPubEmpty + NQ, kBarLseEmpty = kBarLseFull + kMaxLag,
                        kBarFin = kBarLseEmpty + kMaxLag, kNumBars = kBarFin + kFinBufs;
@@ -215,9 +219,8 @@ __global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
       mbar_init(bar(P::kBarQEmpty, s), 2);  // both MMA issuers
     }
     for (int b = 0; b < kNumBufs; ++b) {
-      mbar_init(bar(P::kBarTFull, b), 1);
-      mbar_init(bar(P::kBarTFull, kNumBufs + b), 1);
-      mbar_init(bar(P::kBarTEmpty, b), MT == 2 ? 8 : 4);
+      for (int f = 0; f < P::kFullSets; ++f) mbar_init(bar(P::kBarTFull, f * kNumBufs + b), 1);
+      mbar_init(bar(P::kBarTEmpty, b), 4);
     }
     for (int q = 0; q < NQ; ++q) {
       mbar_init(bar(P::kBarPubFull, q), 4);
@@ -245,18 +248,24 @@ __global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
       for (int idx = 0; idx < njobs; ++idx) {
         const Job j = decode_job<RAGGED>(idx, K, a);
         if (j.ntiles == 0) continue;
-        const uint32_t slot = jq % P::kQSlots;
-        if (!mbar_wait(bar(P::kBarQEmpty, slot), ((jq / P::kQSlots) & 1) ^ 1, abort_flag, a.dev_status, a.spin_limit)) break;
-        mbar_expect_tx(bar(P::kBarQFull, slot), P::kQBytes);
-        const uint32_t qd = q_s + slot * P::kQBytes;
-        for (int h = 0; h < NH; ++h)
-          for (int mt = 0; mt < MT; ++mt) {
-            const uint32_t dst = qd + h * (MT * kHalfBytes) + mt * kHalfBytes;
-            if (a.l2_hints) tma_load_2d_hint(dst, &q_map, bar(P::kBarQFull, slot), h * 64, j.u * a.M + mt * 128, keep);
-            else tma_load_2d(dst, &q_map, bar(P::kBarQFull, slot), h * 64, j.u * a.M + mt * 128);
-          }
-        ++jq;
+        // With one slot the query tiles follow the first key tiles, which need not wait for the job before to end.
+        const int q_after = P::kQSlots == 1 ? min(kStages, j.ntiles) : 0;
         bool ok = true;
+        auto load_q = [&]() -> bool {
+          const uint32_t slot = jq % P::kQSlots;
+          if (!mbar_wait(bar(P::kBarQEmpty, slot), ((jq / P::kQSlots) & 1) ^ 1, abort_flag, a.dev_status, a.spin_limit)) return false;
+          mbar_expect_tx(bar(P::kBarQFull, slot), P::kQBytes);
+          const uint32_t qd = q_s + slot * P::kQBytes;
+          for (int h = 0; h < NH; ++h)
+            for (int mt = 0; mt < MT; ++mt) {
+              const uint32_t dst = qd + h * (MT * kHalfBytes) + mt * kHalfBytes;
+              if (a.l2_hints) tma_load_2d_hint(dst, &q_map, bar(P::kBarQFull, slot), h * 64, j.u * a.M + mt * 128, keep);
+              else tma_load_2d(dst, &q_map, bar(P::kBarQFull, slot), h * 64, j.u * a.M + mt * 128);
+            }
+          ++jq;
+          return true;
+        };
+        if (q_after == 0 && !load_q()) break;
         for (int t = 0; t < j.ntiles; ++t, ++tt) {
           const uint32_t s = tt % kStages, ph = (tt / kStages) & 1;
           if (!(ok = mbar_wait(bar(P::kBarEmpty, s), ph ^ 1, abort_flag, a.dev_status, a.spin_limit))) break;
@@ -269,6 +278,7 @@ __global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
           } else {
             for (int h = 0; h < NH; ++h) tma_load_2d(dst + h * kHalfBytes, &k_map, bar(P::kBarFull, s), h * 64, row);
           }
+          if (t + 1 == q_after && !(ok = load_q())) break;
         }
         if (!ok) break;
       }
@@ -295,37 +305,28 @@ __global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
             have_q = true;
           }
           const uint32_t s = tt % kStages, ph = (tt / kStages) & 1;
-          const uint32_t buf = tt % kNumBufs, use = tt / kNumBufs;
-          if (!(ok = mbar_wait(bar(P::kBarTEmpty, buf), (use & 1) ^ 1, abort_flag, a.dev_status, a.spin_limit))) break;
           if (!(ok = mbar_wait(bar(P::kBarFull, s), ph, abort_flag, a.dev_status, a.spin_limit))) break;
-          tc_fence_after();
           const uint32_t kt = k_s + s * kStageBytes;
-          const uint32_t d_tmem = tmem_base + buf * P::kBufCols;
-          if (!j.p2) {
-            // D[q row][key]: A = Q (M-tile mt), B = K tile
-            constexpr uint32_t idesc = instr_desc_bf16(128, kTileKeys);
-#pragma unroll
-            for (int mt = 0; mt < MT; ++mt)
-#pragma unroll
-              for (int ks = 0; ks < 4 * NH; ++ks) {
-                const int h = ks >> 2, sub = ks & 3;
-                const uint64_t da = smem_desc_sw128(qd + h * (MT * kHalfBytes) + mt * kHalfBytes) + (uint64_t)(sub * 2);
-                const uint64_t db = smem_desc_sw128(kt + h * kHalfBytes) + (uint64_t)(sub * 2);
-                umma_bf16(d_tmem + mt * 128, da, db, idesc, ks > 0);
-              }
-          } else {
-            // D[key][q row]: A = K tile, B = Q (npad rows)
-            const uint32_t idesc = instr_desc_bf16(128, a.npad);
+          for (int mt = 0; mt < MT; ++mt) {
+            const uint32_t st = tt * MT + mt, buf = st % kNumBufs, use = st / kNumBufs;
+            if (!(ok = mbar_wait(bar(P::kBarTEmpty, buf), (use & 1) ^ 1, abort_flag, a.dev_status, a.spin_limit))) break;
+            tc_fence_after();
+            const uint32_t d_tmem = tmem_base + buf * P::kBufCols;
+            const uint32_t qb = qd + mt * kHalfBytes;
+            // pass 1: D[q row][key], A = 128 query rows, B = K tile; pass 2: D[key][q row], A = K tile, B = the query rows (up to
+            // 128, padded to a multiple of 32)
+            const uint32_t idesc = j.p2 ? instr_desc_bf16(128, min(128, a.npad - 128 * mt)) : instr_desc_bf16(128, kTileKeys);
 #pragma unroll
             for (int ks = 0; ks < 4 * NH; ++ks) {
               const int h = ks >> 2, sub = ks & 3;
-              const uint64_t da = smem_desc_sw128(kt + h * kHalfBytes) + (uint64_t)(sub * 2);
-              const uint64_t db = smem_desc_sw128(qd + h * (MT * kHalfBytes)) + (uint64_t)(sub * 2);
-              umma_bf16(d_tmem, da, db, idesc, ks > 0);
+              const uint64_t dq = smem_desc_sw128(qb + h * (MT * kHalfBytes)) + (uint64_t)(sub * 2);
+              const uint64_t dk = smem_desc_sw128(kt + h * kHalfBytes) + (uint64_t)(sub * 2);
+              umma_bf16(d_tmem, j.p2 ? dk : dq, j.p2 ? dq : dk, idesc, ks > 0);
             }
+            umma_commit(bar(P::kBarTFull, buf + kNumBufs * (use % P::kFullSets)));   // the accumulator is complete
           }
+          if (!ok) break;
           umma_commit(bar(P::kBarEmpty, s));     // the stage may be refilled once these MMAs have read it
-          umma_commit(bar(P::kBarTFull, buf + kNumBufs * (use & 1)));   // the accumulator is complete
         }
         // An issuer without a tile in this job (a job of one tile) waits all the same: else it could hand the slot back twice
         // while the other issuer still works on the job before in it, which would free that job's query tiles, and its
@@ -379,7 +380,7 @@ __global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
                   }
                 }
               }
-              dst[rr + lane] = v.y > 0.f ? v.x + log2f(v.y) : -INFINITY;
+              dst[rr + lane] = p1_log(v.x, v.y);
             }
           }
           __syncwarp();
@@ -531,52 +532,88 @@ __global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
     const uint32_t lane_addr = (uint32_t)(32 * (warp & 3)) << 16;
     const uint64_t sc2 = pack2(a.scale_log2, a.scale_log2);
     uint32_t tt = 0, p1c = 0, p2c = 0;
+    // Row block `st` (counted over all tiles of the CTA) lies in buffer st % 4.  The waits give one answer to the whole warp, which
+    // goes on to warp-wide loads.
+    auto full_wait = [&](uint32_t st) {
+      const uint32_t buf = st % kNumBufs, use = st / kNumBufs;
+      return __all_sync(0xffffffffu, mbar_wait(bar(P::kBarTFull, buf + kNumBufs * (use % P::kFullSets)), (use / P::kFullSets) & 1,
+                                               abort_flag, a.dev_status, a.spin_limit));
+    };
+    auto column = [&](uint32_t st) { return tmem_base + lane_addr + (st % kNumBufs) * P::kBufCols; };
+    auto release = [&](uint32_t st) {  // this warp has the last columns it needs in registers
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar(P::kBarTEmpty, st % kNumBufs), 1);
+    };
+    float va[32], vb[32];
     for (int idx = 0; idx < njobs; ++idx) {
       const Job j = decode_job<RAGGED>(idx, K, a);
       if (j.ntiles == 0) continue;
+      // The quads take the tiles in turn; with two row blocks pass 1 gives each quad one block of every tile.  Buffers of one block
+      // instead of whole tiles let the MMAs of a quad's next tile start when half of this one is read, not all of it.
+      const bool every = MT == 2 && !j.p2;
+      const int step = every ? 1 : NQ;
+      int t = every ? 0 : (int)((quad + NQ - tt % NQ) % NQ);
       if (!j.p2) {
-        // ---- pass 1: (reference, sum-exp) of this thread's query row over the job's keys
+        // ---- pass 1: (reference, sum-exp) of this thread's query row over the job's keys.  A tile is one stretch of code without a
+        // branch, relative to the reference so far (the maximum of the job's first 32 keys to begin with); a sum that leaves the
+        // safe range, or a tile with keys hidden from some row, is done again chunk by chunk, exactly.  The range is wide (2^80):
+        // with one of 2^40, tested per chunk, outlier channels at head size 64 (logits of 23 binary orders' standard deviation)
+        // sent every tenth chunk through the exact form (128 heads x 20011 keys: 345 us a call; 323 with the wide range, 305
+        // tested per tile; 256 heads x 32768 keys at head size 128 1217 and 1163).
         const int r = (MT == 2 ? 128 * quad : 0) + qtid;
         const int lim = r < a.M ? j.n + (r % a.w) : -1;           // last visible key; -1: padded row
+        const bool live = (r & ~31) < a.M;                        // a row of this warp is no padding
         float m = -INFINITY, l = 0.f;
-        for (int t = 0; t < j.ntiles; ++t, ++tt) {
-          if (MT == 1 && (int)(tt % NQ) != quad) continue;
-          const uint32_t buf = tt % kNumBufs, use = tt / kNumBufs;
-          const bool ok = mbar_wait(bar(P::kBarTFull, buf + kNumBufs * (use & 1)), (use >> 1) & 1, abort_flag, a.dev_status, a.spin_limit);
-          if (ok) {
-            tc_fence_after();
-            const int j0 = (j.tile0 + t) * kTileKeys;
-            const bool masked = j0 + kTileKeys > j.n;             // tile reaches into the window / past T
-            const uint32_t tcol = tmem_base + lane_addr + buf * P::kBufCols + (MT == 2 ? 128 * quad : 0);
-            // the accumulator is free as soon as its last columns are in registers
-            auto release = [&](uint32_t n) {
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(bar(P::kBarTEmpty, buf), n);
-            };
-            float va[32], vb[32];
-            tmem_ld32(tcol, va);
-#pragma unroll
-            for (int c = 0; c < 4; c += 2) {
-              tmem_ld_wait(va);
-              tmem_ld32(tcol + 32 * (c + 1), vb);
-              if (lim >= 0) {
-                if (masked) p1_chunk<true>(va, j0 + 32 * c, lim, a.scale_log2, m, l);
-                else p1_chunk<false>(va, j0 + 32 * c, lim, a.scale_log2, m, l);
-              }
-              tmem_ld_wait(vb);
-              if (c + 2 < 4) tmem_ld32(tcol + 32 * (c + 2), va);
-              else release(1);
-              if (lim >= 0) {
-                if (masked) p1_chunk<true>(vb, j0 + 32 * (c + 1), lim, a.scale_log2, m, l);
-                else p1_chunk<false>(vb, j0 + 32 * (c + 1), lim, a.scale_log2, m, l);
-              }
+        bool first = true;
+        for (; t < j.ntiles; t += step) {
+          const uint32_t st = MT == 2 ? 2 * (tt + t) + quad : tt + t;
+          if (!full_wait(st)) continue;
+          tc_fence_after();
+          if (!live) {
+            release(st);
+            continue;
+          }
+          const uint32_t tcol = column(st);
+          tmem_ld32(tcol, va);
+          const int j0 = (j.tile0 + t) * kTileKeys;
+          bool redo = true;
+          if (j0 + kTileKeys <= j.n) {  // all keys are visible to all rows
+            uint64_t acc0 = 0ull, acc1 = 0ull;
+            float pmax = -INFINITY;
+            tmem_ld_wait(va);
+            tmem_ld32(tcol + 32, vb);
+            if (first) m = p1_reference(va, a.scale_log2);
+            const uint64_t nm2 = pack2(-m, -m);
+            p1_terms(va, sc2, nm2, acc0, acc1, pmax);
+            tmem_ld_wait(vb);
+            tmem_ld32(tcol + 64, va);
+            p1_terms(vb, sc2, nm2, acc0, acc1, pmax);
+            tmem_ld_wait(va);
+            tmem_ld32(tcol + 96, vb);
+            p1_terms(va, sc2, nm2, acc0, acc1, pmax);
+            tmem_ld_wait(vb);
+            p1_terms(vb, sc2, nm2, acc0, acc1, pmax);
+            const float cs = sum4(acc0, acc1);
+            if (p1_in_range(cs, pmax, a.scale_log2, m)) {
+              l += cs;
+              redo = false;
             }
           }
+          first = false;
+          if (__any_sync(0xffffffffu, redo && lim >= 0)) {
+#pragma unroll 1
+            for (int c = 0; c < 4; ++c) {
+              tmem_ld32(tcol + 32 * c, vb);
+              tmem_ld_wait(vb);
+              if (redo) p1_exact(vb, j0 + 32 * c, lim, a.scale_log2, m, l);
+            }
+          }
+          release(st);
         }
         // hand the partial to the publisher warp
         const bool ok = mbar_wait(bar(P::kBarPubEmpty, quad), (p1c & 1) ^ 1, abort_flag, a.dev_status, a.spin_limit);
-        if (ok) pub_s[quad * 128 + qtid] = make_float2(m, l);
+        if (ok) pub_s[quad * 128 + qtid] = lim >= 0 ? make_float2(m, l) : make_float2(-INFINITY, 0.f);
         __syncwarp();
         if (lane == 0 && ok) mbar_arrive(bar(P::kBarPubFull, quad), 1);
         ++p1c;
@@ -584,44 +621,49 @@ __global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
         // ---- pass 2: this thread's key, summed over all query rows
         const uint32_t slot = p2c % a.lag;
         const bool have_lse = mbar_wait(bar(P::kBarLseFull, slot), (p2c / a.lag) & 1, abort_flag, a.dev_status, a.spin_limit);
-        const float* nlse = nlse_s + slot * 256;
-        for (int t = 0; t < j.ntiles; ++t, ++tt) {
-          if ((int)(tt % NQ) != quad) continue;
-          const uint32_t buf = tt % kNumBufs, use = tt / kNumBufs;
-          const bool ok = mbar_wait(bar(P::kBarTFull, buf + kNumBufs * (use & 1)), (use >> 1) & 1, abort_flag, a.dev_status, a.spin_limit);
-          if (ok) {
-            tc_fence_after();
-            const int key = (j.tile0 + t) * kTileKeys + qtid;
-            const uint32_t tcol = tmem_base + lane_addr + buf * P::kBufCols;
-            uint64_t acc0 = 0ull, acc1 = 0ull;
-            auto release = [&](uint32_t n) {
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(bar(P::kBarTEmpty, buf), n);
-            };
-            float va[32], vb[32];
-            tmem_ld32(tcol, va);
+        for (; t < j.ntiles; t += step) {
+          uint64_t acc0 = 0ull, acc1 = 0ull;
+          bool ok = true;
 #pragma unroll 1
-            for (int c0 = 0; c0 < a.npad; c0 += 64) {
+          for (int mt = 0; mt < MT; ++mt) {  // 128 rows unrolled: 7850 -> 7640 us for eight 16k sequences of 256 rows
+            const uint32_t st = (tt + t) * MT + mt;
+            const float* nlse = nlse_s + slot * 256 + 128 * mt;
+            const uint32_t tcol = column(st);
+            if (!(ok = full_wait(st))) break;
+            tc_fence_after();
+            tmem_ld32(tcol, va);
+            const int cols = a.npad - 128 * mt;
+            if (cols >= 128) {
               tmem_ld_wait(va);
-              const bool two = c0 + 32 < a.npad;
-              if (two) tmem_ld32(tcol + c0 + 32, vb);
-              else release(MT == 2 ? 2 : 1);
-              p2_chunk(va, nlse + c0, sc2, acc0, acc1);
-              if (two) {
-                tmem_ld_wait(vb);
-                if (c0 + 64 < a.npad) tmem_ld32(tcol + c0 + 64, va);
-                else release(MT == 2 ? 2 : 1);
-                p2_chunk(vb, nlse + c0 + 32, sc2, acc0, acc1);
+              tmem_ld32(tcol + 32, vb);
+              p2_chunk(va, nlse, sc2, acc0, acc1);
+              tmem_ld_wait(vb);
+              tmem_ld32(tcol + 64, va);
+              p2_chunk(vb, nlse + 32, sc2, acc0, acc1);
+              tmem_ld_wait(va);
+              tmem_ld32(tcol + 96, vb);
+              p2_chunk(va, nlse + 64, sc2, acc0, acc1);
+              tmem_ld_wait(vb);
+              release(st);
+              p2_chunk(vb, nlse + 96, sc2, acc0, acc1);
+            } else {
+#pragma unroll 1
+              for (int c = 0; c < cols; c += 32) {
+                tmem_ld_wait(va);
+                if (c + 32 >= cols) release(st);
+                p2_chunk(va, nlse + c, sc2, acc0, acc1);
+                if (c + 32 < cols) tmem_ld32(tcol + c + 32, va);
               }
             }
-            if (key < j.n) a.raw[(size_t)j.u * a.n_stride + key] = sum4(acc0, acc1);
           }
+          const int key = (j.tile0 + t) * kTileKeys + qtid;
+          if (ok && key < j.n) a.raw[(size_t)j.u * a.n_stride + key] = sum4(acc0, acc1);
         }
         __syncwarp();
         if (lane == 0 && have_lse) mbar_arrive(bar(P::kBarLseEmpty, slot), 1);
         ++p2c;
       }
+      tt += j.ntiles;
     }
   }
 
@@ -640,18 +682,17 @@ __global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
 
 // ---- host side --------------------------------------------------------------------------------
 
-// Tiles, and one more per item, of the CTA with the most of them, when the items of `groups` groups of heads (heads each, T[g]
+// Tiles, and `item` more per item, of the CTA with the most of them, when the items of `groups` groups of heads (heads each, T[g]
 // keys long, at most `it` tiles an item) are dealt to `ctas` CTAs in turn.
-double deal_cost(const int32_t* T, int groups, int heads, int it, int ctas) {
+double deal_cost(const int32_t* T, int groups, int heads, int it, int ctas, double item) {
   constexpr int kMaxCtas = 256;
-  constexpr double kItem = 1.05;
   double step[kMaxCtas + 1] = {};  // what a group's last, incomplete round adds: differences from CTA to CTA
   if (ctas > kMaxCtas) ctas = kMaxCtas;
   double base = 0.0;
   int first = 0;  // the CTA that gets the group's first item
   for (int g = 0; g < groups; ++g) {
     const long long tiles = (T[g] + kTileKeys - 1) / kTileKeys, per_head = (tiles + it - 1) / it, items = heads * per_head;
-    const double time = (double)tiles / (double)per_head + kItem;
+    const double time = (double)tiles / (double)per_head + item;
     const int rest = (int)(items % ctas);
     base += time * (double)(items / ctas);
     if (rest) {
@@ -687,16 +728,23 @@ cudaError_t launch_fused(const CUtensorMap& qm, const CUtensorMap& km, FusedArgs
   // not outnumber the CTAs (else a CTA would wait for partials that it is due to produce itself).
   if (args.adapt_items) {
     // Larger work items mean fewer job changes and fewer partials to fold per head, but coarser dealing.  The time is that of
-    // the CTA with the most to do: its tiles and about one tile's time per item (256 heads x 256 tiles on 148 CTAs: 0.89 ms with
-    // 8 tiles per item, 0.84 with 16, 0.82 with 32, 0.81 with 64).  The price of large items is that pass 2 no longer finds all
-    // its key tiles in L2; the kernel is bound by the exp2 unit, not by HBM, so re-reading part of K costs nothing.
-    // Any number of tiles up to 64 is tried: 8 heads x 64 tiles 41.3 us a call with 8 and 35.7 with 4, 24 x 64 61.6 with 16 and
-    // 55 with 6, 48 x 32 (two row blocks) 89 with 16 and 76 with 6.
+    // the CTA with the most to do: its tiles and about half a row block's time per item (128 heads x 157 tiles, head size 64: 223 us
+    // of scorer in items of 20 tiles, 231 in 16, 237 in 8; two row blocks 2048 x 128 tiles 5.84 ms in 64 and 5.94 in 8).
+    // Large items do not leave pass 2 its key tiles in L2.  With one row block of 128 channels reading them from HBM again is a
+    // bound of its own (7 TB/s at the speed of the arithmetic): items of up to nine tiles, whose two sweeps' keys fit L2, are
+    // a tenth faster per tile (256 heads x 256 tiles: 1163 us a call in 64 tiles, 1172 in 32, 1176 in 12, 1143 in 10, 1129 in 8
+    // and 9).  Any number of tiles up to 64 is tried: 8 heads x 64 tiles 33 us a call with 4, 37 with 6 or 8.
+    constexpr double kItem = 0.5 / MT, kReread = 1.1;
+    constexpr long long kL2Tiles = (90ll << 20) / (2 * kHalfBytes);
+    long long all_tiles = 0;
+    for (int q = 0; q < (RAGGED ? args.n_seq : 1); ++q)
+      all_tiles += (long long)(RAGGED ? args.heads_per_seq : args.nheads) * (((RAGGED ? seq_T_host[q] : args.T) + kTileKeys - 1) / kTileKeys);
     int best = args.item_tiles;
     double best_cost = 1e30;
     for (int it = args.item_tiles; it <= 64; ++it) {
-      const double cost = RAGGED ? deal_cost(seq_T_host, args.n_seq, args.heads_per_seq, it, sms)
-                                 : deal_cost(&args.T, 1, args.nheads, it, sms);
+      double cost = RAGGED ? deal_cost(seq_T_host, args.n_seq, args.heads_per_seq, it, sms, kItem)
+                           : deal_cost(&args.T, 1, args.nheads, it, sms, kItem);
+      if (MT == 1 && NH == 2 && all_tiles > kL2Tiles && 2ll * sms * it > kL2Tiles) cost *= kReread;
       if (cost < best_cost * 0.995) {
         best_cost = cost;
         best = it;

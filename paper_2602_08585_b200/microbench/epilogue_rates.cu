@@ -70,7 +70,7 @@ __global__ void __launch_bounds__(512, 1) epilogue_rate(float* out, long long* c
   const long long t0 = clock64();
   const uint64_t sc2 = pack2(0.1275f, 0.1275f), nm2 = pack2(-2.f, -2.f);
   uint64_t acc0 = 0ull, acc1 = 0ull;
-  float m_run = -INFINITY, l_run = 0.f;
+  float m_run = -2.f, l_run = 0.f, pmax = -INFINITY;
   const float4 mine4 = *reinterpret_cast<const float4*>(nlse + 4 * lane);
   const int quad = warp >> 2;
   if (quad < q1 + q2) {
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(512, 1) epilogue_rate(float* out, long long* c
         tmem_ld_wait(va);
         tmem_ld32(tcol + 32 * (c + 1), vb);
         if (first) {
-          if (ROLE == kRoleKernel || ROLE == kRoleShfl) p1_chunk<false>(va, 0, 1 << 30, 0.1275f, m_run, l_run);
+          if (ROLE == kRoleKernel || ROLE == kRoleShfl) p1_terms(va, sc2, pack2(-m_run, -m_run), acc0, acc1, pmax);
           else if (ROLE == kRoleSfu || ROLE == kRoleMixed) sfu_chunk(va, sc2, nm2, acc0, acc1);
           else poly_chunk(va, nlse + 32 * c, sc2, acc0, acc1);
         } else {
@@ -97,7 +97,15 @@ __global__ void __launch_bounds__(512, 1) epilogue_rate(float* out, long long* c
         tmem_ld_wait(vb);
         if (c + 2 < 4) tmem_ld32(tcol + 32 * (c + 2), va);
         if (first) {
-          if (ROLE == kRoleKernel || ROLE == kRoleShfl) p1_chunk<false>(vb, 0, 1 << 30, 0.1275f, m_run, l_run);
+          if (ROLE == kRoleKernel || ROLE == kRoleShfl) {
+            p1_terms(vb, sc2, pack2(-m_run, -m_run), acc0, acc1, pmax);
+            if (c == 2) {  // the end of the tile
+              const float cs = sum4(acc0, acc1);
+              if (p1_in_range(cs, pmax, 0.1275f, m_run)) l_run += cs;
+              acc0 = acc1 = 0ull;
+              pmax = -INFINITY;
+            }
+          }
           else if (ROLE == kRoleSfu || ROLE == kRoleMixed) sfu_chunk(vb, sc2, nm2, acc0, acc1);
           else poly_chunk(vb, nlse + 32 * (c + 1), sc2, acc0, acc1);
         } else {

@@ -146,3 +146,25 @@ def test_bounded_wait_expiry_is_reported_and_leaves_the_library_usable(monkeypat
     assert torch.equal(out.kept_idx, fresh.kept_idx)
     assert torch.equal(out.k_out.view(torch.int16), fresh.k_out.view(torch.int16))
     assert torch.equal(out.v_out.view(torch.int16), fresh.v_out.view(torch.int16))
+
+
+# Rows of logits that rise by so many binary orders above the reference (the first 32 keys' maximum): below, at and above the range
+# of the tile's sum (80) and of the polynomial's arguments (100), in a slot of either kind; one and two row blocks, the last of
+# them with all its 128 rows or fewer, both head sizes, a first tile with hidden keys.
+@pytest.mark.parametrize("rise", [40, 79, 82, 99, 102, 140])
+@pytest.mark.parametrize("shape", [(1, 16, 128, 700), (4, 32, 64, 2100), (5, 32, 128, 1500), (7, 32, 64, 1111), (4, 64, 128, 1300),
+                                   (4, 32, 128, 150)])
+def test_sums_that_rise_within_an_item(oracle, shape, rise):
+    Gq, w, d, T = shape
+    g = torch.Generator().manual_seed(1000 * rise + T)
+    base = torch.randn(d, generator=g)
+    base = base / base.norm()
+    q = (torch.randn((1, 1, 2 * Gq, w, d), generator=g) * 0.05 + 10.0 * base).to(torch.bfloat16)
+    k = (torch.randn((1, 1, 2, T, d), generator=g) * 0.05).to(torch.bfloat16)
+    height = rise / (10.0 * 1.4426950408889634) * d ** 0.5  # logit = height * 10 / sqrt(d)
+    last = T - w - 1
+    for h, j in ((0, min(last, 128 + 34)), (1, min(last, 128 + 37))):  # element 2 of a chunk goes through the polynomial, 5 does not
+        k[0, 0, h, j] = (height * base).to(torch.bfloat16)
+    p = lukv.make_params(1, 1, 2, Gq, d, T, w, 7, torch.bfloat16, 2)
+    got = gpu_score(p, q.cuda(), k.cuda()).cpu().numpy()
+    assert_scores_close(got, oracle.score(bits(q), bits(k), Gq, 7))
