@@ -7,11 +7,11 @@
 // the group and the maximum over the steps stay in the thread that owns a key.
 //   imp_tc_kernel<LSE>  D[row][key]: a thread owns a query row, as in pass 1 of the tensor-core scorer
 //   imp_tc_kernel       D[key][row] (operands swapped): a thread owns a key and runs over the rows
-// Both are persistent with static items and warp roles: warps 0-7 two epilogue quads that take alternate key tiles out of
+// Both are persistent with static items (equal shares of the key tiles for the second) and warp roles: warps 0-7 two epilogue quads that take alternate key tiles out of
 // four accumulator buffers, warp 8 TMA producer, warp 9 tensor memory and MMA issue.  Every wait is bounded and between the
 // warps of one CTA only; should one run out, here or in the value norms, what depends on it becomes NaN.
 // Bound by the exp2 of the epilogue (2 x 2.6e8 for 256 heads x 256 rows x 4000 keys).  Measured there: 1.90 + 1.82 ms
-// on the FP32 pipes, 0.11 + 0.15 ms here.
+// on the FP32 pipes, 0.106 + 0.112 ms here.
 #define LUKV_POLY_SEL1(i) false  // every exp2 on the special-function unit: the values keep their precision
 #include <algorithm>
 
@@ -26,9 +26,10 @@ constexpr int kItThreads = kItEpiThreads + 64;
 template <int NH, bool LSE>  // halves of 64 channels: d = 64 NH
 struct ItPlan {
   static constexpr int kTile = NH * kHalfBytes;  // one tile of 128 rows
-  static constexpr int kQPer = LSE ? 1 : 2;      // query tiles per item, for two items
-  static constexpr int kStages = LSE ? 4 : 2;    // key tiles in flight
-  static constexpr int kKOff = 2 * kQPer * kTile;
+  static constexpr int kQPer = LSE ? 1 : 2;      // query tiles per item
+  static constexpr int kQSlots = LSE ? 2 : 1;    // items whose query tiles are held
+  static constexpr int kStages = 4;              // key tiles in flight
+  static constexpr int kKOff = kQSlots * kQPer * kTile;
   static constexpr int kNlseOff = kKOff + kStages * kTile;     // [2][256] floats
   static constexpr int kMergeOff = kNlseOff + 2 * 256 * 4;       // [128] (reference, sum) of the second quad
   static constexpr int kTotal = kMergeOff + 128 * 8 + 1024;
@@ -44,8 +45,7 @@ struct ItArgs {
   int chunk0, nchunk; // imp: the query tiles of this launch (at most two)
   int accumulate;     // imp: the maximum goes on from what `importance` holds
   int splits, tiles_per_split, tiles_T, tiles_D;  // lse: tiles_D tiles of decode keys follow the cached ones
-  int run, runs;      // imp: key tiles per item, items per head
-  int items;
+  int items;          // lse: items; imp: key tiles of all heads
   float scale_log2;
   uint32_t spin_limit;
   int drop_item;      // test hook: the query tiles of this item are never loaded (-1: none)
@@ -53,7 +53,7 @@ struct ItArgs {
 };
 
 // Both kernels (LSE: the row log-sum-exps): one item is a head, its query tiles (one, or up to two) and a run of key tiles.
-template <int NH, bool LSE>
+template <int NH, bool LSE, int GPL>  // GPL: log2 of GP (the form without LSE)
 __global__ void __launch_bounds__(kItThreads, 1)
     imp_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map,
                   const __grid_constant__ CUtensorMap kd_map, const ItArgs a) {
@@ -100,47 +100,69 @@ __global__ void __launch_bounds__(kItThreads, 1)
   struct Item {
     int u, c0, nq, split, t0, nt;
   };
-  auto item_of = [&](int idx) {
-    Item it;
+  // The items of this CTA in order: for the log-sum-exps every gridDim-th of all; for the importance its share of the key tiles of
+  // all heads, cut where a head ends.  (Eight items per SM of a few tiles of one head each spent as long on the start of an item,
+  // its row log-sum-exps and value norms, as on its tiles: 256 heads x 31 tiles x 2 query tiles 154 us, 112 so.)
+  struct Walk {
+    int idx, pos, end;
+  };
+  auto walk = [&]() {
+    const long long all = a.items;
+    return Walk{(int)blockIdx.x, (int)(all * blockIdx.x / gridDim.x), (int)(all * (blockIdx.x + 1) / gridDim.x)};
+  };
+  auto next = [&](Walk& w, Item& it) -> bool {
     if (LSE) {
-      it.split = idx % a.splits;
-      const int uc = idx / a.splits;
+      if (w.idx >= a.items) return false;
+      it.split = w.idx % a.splits;
+      const int uc = w.idx / a.splits;
       it.c0 = uc % a.chunks;
       it.u = uc / a.chunks;
       it.nq = 1;
       it.t0 = it.split * a.tiles_per_split;
       it.nt = max(0, min(a.tiles_per_split, a.tiles_T + a.tiles_D - it.t0));
     } else {
-      it.u = idx / a.runs;
+      if (w.pos >= w.end) return false;
+      it.u = w.pos / a.tiles_T;
       it.split = 0;
       it.c0 = a.chunk0;
       it.nq = a.nchunk;
-      it.t0 = (idx % a.runs) * a.run;
-      it.nt = min(a.run, a.tiles_T - it.t0);
+      it.t0 = w.pos - it.u * a.tiles_T;
+      it.nt = min(a.tiles_T - it.t0, w.end - w.pos);
+      w.pos += it.nt;
     }
-    return it;
+    w.idx += gridDim.x;
+    return true;
   };
-  const int steps_log2 = 7 - a.gp_log2;  // a query tile holds 128 / GP steps
+  const int gp_log2 = LSE ? a.gp_log2 : GPL;
+  const int steps_log2 = 7 - gp_log2;  // a query tile holds 128 / GP steps
 
   if (warp == 8) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
       uint32_t tt = 0, jq = 0;
       bool ok = true;
-      for (int idx = blockIdx.x; idx < a.items && ok; idx += gridDim.x, ++jq) {
-        const Item it = item_of(idx);
-        const uint32_t slot = jq & 1;
-        if (!(ok = wait(bar(kItQEmpty, slot), ((jq >> 1) & 1) ^ 1))) break;
-        mbar_expect_tx(bar(kItQFull, slot), it.nq * P::kTile);
-        for (int c = 0; c < it.nq && idx != a.drop_item; ++c)
-          for (int h = 0; h < NH; ++h) {
-            const uint32_t dst = smem_u32(smem) + (P::kQPer * slot + c) * P::kTile + h * kHalfBytes;
-            asm volatile(
-                "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-                ::"r"(dst), "l"(&q_map), "r"(bar(kItQFull, slot)), "r"(h * 64), "r"(0), "r"((it.c0 + c) << steps_log2),
-                "r"(it.u)
-                : "memory");
-          }
+      Walk w = walk();
+      Item it;
+      while (ok && next(w, it)) {
+        const uint32_t slot = jq % P::kQSlots;
+        // with one slot the query tiles follow the first key tiles, which need not wait for the item before to end
+        const int q_after = P::kQSlots == 1 ? min(kItStages, it.nt) : 0;
+        auto load_q = [&]() -> bool {
+          if (!wait(bar(kItQEmpty, slot), ((jq / P::kQSlots) & 1) ^ 1)) return false;
+          mbar_expect_tx(bar(kItQFull, slot), it.nq * P::kTile);
+          for (int c = 0; c < it.nq && w.idx - (int)gridDim.x != a.drop_item; ++c)
+            for (int h = 0; h < NH; ++h) {
+              const uint32_t dst = smem_u32(smem) + (P::kQPer * slot + c) * P::kTile + h * kHalfBytes;
+              asm volatile(
+                  "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
+                  ::"r"(dst), "l"(&q_map), "r"(bar(kItQFull, slot)), "r"(h * 64), "r"(0), "r"((it.c0 + c) << steps_log2),
+                  "r"(it.u)
+                  : "memory");
+            }
+          ++jq;
+          return true;
+        };
+        if (q_after == 0 && !(ok = load_q())) break;
         for (int t = 0; t < it.nt; ++t, ++tt) {
           const uint32_t s = tt % kItStages, ph = (tt / kItStages) & 1;
           if (!(ok = wait(bar(kItKEmpty, s), ph ^ 1))) break;
@@ -151,6 +173,7 @@ __global__ void __launch_bounds__(kItThreads, 1)
             if (!LSE || tile < a.tiles_T) tma_load_2d(dst + h * kHalfBytes, &k_map, bar(kItKFull, s), h * 64, it.u * a.T + tile * 128);
             else tma_load_2d(dst + h * kHalfBytes, &kd_map, bar(kItKFull, s), h * 64, it.u * a.Kmax + (tile - a.tiles_T) * 128);
           }
+          if (t + 1 == q_after && !(ok = load_q())) break;
         }
       }
     }
@@ -160,10 +183,11 @@ __global__ void __launch_bounds__(kItThreads, 1)
       constexpr uint32_t idesc = instr_desc_bf16(128, 128);
       uint32_t tt = 0, jq = 0, used[2] = {0, 0};
       bool ok = true;
-      for (int idx = blockIdx.x; idx < a.items && ok; idx += gridDim.x, ++jq) {
-        const Item it = item_of(idx);
-        const uint32_t slot = jq & 1;
-        if (!(ok = wait(bar(kItQFull, slot), (jq >> 1) & 1))) break;
+      Walk w = walk();
+      Item it;
+      for (; ok && next(w, it); ++jq) {
+        const uint32_t slot = jq % P::kQSlots;
+        if (!(ok = wait(bar(kItQFull, slot), (jq / P::kQSlots) & 1))) break;
         for (int t = 0; t < it.nt && ok; ++t, ++tt) {
           const uint32_t s = tt % kItStages, quad = tt & 1;
           if (!(ok = wait(bar(kItKFull, s), (tt / kItStages) & 1))) break;
@@ -192,11 +216,13 @@ __global__ void __launch_bounds__(kItThreads, 1)
     const uint32_t lane_addr = (uint32_t)(32 * (warp & 3)) << 16;
     uint32_t tt = 0, n_use = 0, jq = 0;
     bool ok = true;
-    for (int idx = blockIdx.x; idx < a.items; idx += gridDim.x, ++jq) {
-      const Item it = item_of(idx);
+    Walk w = walk();
+    Item it;
+    for (; next(w, it); ++jq) {
       if (LSE) {
-        const int step = (it.c0 << steps_log2) + (qtid >> a.gp_log2);
-        const bool row_ok = step < a.Kmax && (qtid & ((1 << a.gp_log2) - 1)) < a.G;
+        const int step = (it.c0 << steps_log2) + (qtid >> gp_log2);
+        const bool row_ok = step < a.Kmax && (qtid & ((1 << gp_log2) - 1)) < a.G;
+        const uint64_t sc2 = pack2(a.scale_log2, a.scale_log2);
         float m = -INFINITY, l = 0.f;
         for (int t = 0; t < it.nt; ++t, ++tt) {
           if ((int)(tt & 1) != quad) continue;
@@ -211,18 +237,39 @@ __global__ void __launch_bounds__(kItThreads, 1)
           const int lim = !row_ok ? -1 : decode ? step : a.T - 1;  // last visible key
           const bool masked = decode || j0 + 128 > a.T;
           const uint32_t tcol = tmem_base + lane_addr + buf * 128;
+          // a tile in one stretch where all its keys are visible, chunk by chunk where not, as in the scorer's pass 1
           float va[32], vb[32];
-          tmem_ld32(tcol, va);
-#pragma unroll
-          for (int c = 0; c < 4; c += 2) {
+          bool redo = true;
+          if (!masked) {
+            uint64_t acc0 = 0ull, acc1 = 0ull;
+            float pmax = -INFINITY;  // (no argument goes through the polynomial here)
+            tmem_ld32(tcol, va);
             tmem_ld_wait(va);
-            tmem_ld32(tcol + 32 * (c + 1), vb);
-            if (masked) p1_chunk<true>(va, j0 + 32 * c, lim, a.scale_log2, m, l);
-            else p1_chunk<false>(va, j0 + 32 * c, lim, a.scale_log2, m, l);
+            tmem_ld32(tcol + 32, vb);
+            if (m == -INFINITY) m = p1_reference(va, a.scale_log2);
+            const uint64_t nm2 = pack2(-m, -m);
+            p1_terms(va, sc2, nm2, acc0, acc1, pmax);
             tmem_ld_wait(vb);
-            if (c + 2 < 4) tmem_ld32(tcol + 32 * (c + 2), va);
-            if (masked) p1_chunk<true>(vb, j0 + 32 * (c + 1), lim, a.scale_log2, m, l);
-            else p1_chunk<false>(vb, j0 + 32 * (c + 1), lim, a.scale_log2, m, l);
+            tmem_ld32(tcol + 64, va);
+            p1_terms(vb, sc2, nm2, acc0, acc1, pmax);
+            tmem_ld_wait(va);
+            tmem_ld32(tcol + 96, vb);
+            p1_terms(va, sc2, nm2, acc0, acc1, pmax);
+            tmem_ld_wait(vb);
+            p1_terms(vb, sc2, nm2, acc0, acc1, pmax);
+            const float cs = sum4(acc0, acc1);
+            if (cs <= kP1Limit) {
+              l += cs;
+              redo = false;
+            }
+          }
+          if (__any_sync(0xffffffffu, redo)) {
+#pragma unroll 1
+            for (int c = 0; c < 4; ++c) {
+              tmem_ld32(tcol + 32 * c, vb);
+              tmem_ld_wait(vb);
+              if (redo) p1_exact(vb, j0 + 32 * c, lim, a.scale_log2, m, l);
+            }
           }
           tc_fence_before();
           __syncwarp();
@@ -250,19 +297,20 @@ __global__ void __launch_bounds__(kItThreads, 1)
             float m = -INFINITY, l = 0.f;
             for (int s = 0; s < a.splits; ++s) m = fmaxf(m, __ldg(p + (size_t)s * 128));
             for (int s = 0; s < a.splits; ++s) l += ex2(__ldg(p + (size_t)s * 128) - m);
-            const int step = ((it.c0 + c) << steps_log2) + (qtid >> a.gp_log2);
-            if (step < a.Kmax && (qtid & ((1 << a.gp_log2) - 1)) < a.G) v = -(m + (a.splits > 1 ? log2f(l) : 0.f));
+            const int step = ((it.c0 + c) << steps_log2) + (qtid >> gp_log2);
+            if (step < a.Kmax && (qtid & ((1 << gp_log2) - 1)) < a.G) v = -(m + (a.splits > 1 ? log2f(l) : 0.f));
           }
           nlse[threadIdx.x] = v;
         }
         bar_sync(1, kItEpiThreads);
         const uint64_t sc2 = pack2(a.scale_log2, a.scale_log2);
         // value norms of this thread's key: those of the quad's next tile are on their way during a tile
-        float vg[8], vg_next[8];
+        constexpr int GP = 1 << GPL;
+        float vg[GP], vg_next[GP];
         auto fetch_norms = [&](int t) {
           const int j = (it.t0 + t) * 128 + qtid;
 #pragma unroll
-          for (int g = 0; g < 8; ++g)
+          for (int g = 0; g < GP; ++g)
             vg_next[g] = g < a.G && t < it.nt && j < a.n ? __ldg(a.vnorm + ((size_t)it.u * a.G + g) * a.n + j) : 0.f;
         };
         fetch_norms((int)(tt & 1) == quad ? 0 : 1);
@@ -270,7 +318,7 @@ __global__ void __launch_bounds__(kItThreads, 1)
           if ((int)(tt & 1) != quad) continue;
           const int j = (it.t0 + t) * 128 + qtid;
 #pragma unroll
-          for (int g = 0; g < 8; ++g) vg[g] = vg_next[g];
+          for (int g = 0; g < GP; ++g) vg[g] = vg_next[g];
           fetch_norms(t + 2);
           float best = a.accumulate && j < a.n ? a.importance[(size_t)it.u * a.n + j] : 0.f;  // importance is not negative
           for (int c = 0; c < it.nq; ++c) {
@@ -290,29 +338,17 @@ __global__ void __launch_bounds__(kItThreads, 1)
                 unpack2(ex2_pair(ffma2(pack2(v[i], v[i + 1]), sc2, ls.x)), e[i], e[i + 1]);
                 unpack2(ex2_pair(ffma2(pack2(v[i + 2], v[i + 3]), sc2, ls.y)), e[i + 2], e[i + 3]);
               }
-              if (a.gp_log2 == 2) {
 #pragma unroll
-                for (int i = 0; i < 32; i += 4)
-                  best = fmaxf(best, fmaf(e[i + 3], vg[3], fmaf(e[i + 2], vg[2], fmaf(e[i + 1], vg[1], e[i] * vg[0]))));
-              } else if (a.gp_log2 == 3) {
+              for (int i = 0; i < 32; i += 1 << GPL) {
+                float s = e[i] * vg[0];
 #pragma unroll
-                for (int i = 0; i < 32; i += 8) {
-                  float s = e[i] * vg[0];
-#pragma unroll
-                  for (int g = 1; g < 8; ++g) s = fmaf(e[i + g], vg[g], s);
-                  best = fmaxf(best, s);
-                }
-              } else if (a.gp_log2 == 1) {
-#pragma unroll
-                for (int i = 0; i < 32; i += 2) best = fmaxf(best, fmaf(e[i + 1], vg[1], e[i] * vg[0]));
-              } else {
-#pragma unroll
-                for (int i = 0; i < 32; ++i) best = fmaxf(best, e[i] * vg[0]);
+                for (int g = 1; g < 1 << GPL; ++g) s = fmaf(e[i + g], vg[g], s);
+                best = fmaxf(best, s);
               }
             };
             float va[32], vb[32];
             tmem_ld32(tcol, va);
-#pragma unroll 1
+#pragma unroll 1  // (unrolled: spills, 119 against 112 us)
             for (int i = 0; i < 4; i += 2) {
               tmem_ld_wait(va);
               tmem_ld32(tcol + 32 * (i + 1), vb);
@@ -396,8 +432,9 @@ cudaError_t launch_importance_tc_t(const Dims& dm, int k_max, const void* q_dec,
   int sms = 0;
   cudaError_t e;
   if ((e = device_sms(&sms)) != cudaSuccess) return e;
-  auto lse = imp_tc_kernel<NH, true>;
-  auto imp = imp_tc_kernel<NH, false>;
+  auto lse = imp_tc_kernel<NH, true, 0>;
+  auto imp = gp_log2 == 0 ? imp_tc_kernel<NH, false, 0> : gp_log2 == 1 ? imp_tc_kernel<NH, false, 1>
+             : gp_log2 == 2 ? imp_tc_kernel<NH, false, 2> : imp_tc_kernel<NH, false, 3>;
   constexpr int lse_smem = ItPlan<NH, true>::kTotal, imp_smem = ItPlan<NH, false>::kTotal;
   if ((e = allow_smem((const void*)lse, lse_smem)) != cudaSuccess) return e;
   if ((e = allow_smem((const void*)imp, imp_smem)) != cudaSuccess) return e;
@@ -408,10 +445,7 @@ cudaError_t launch_importance_tc_t(const Dims& dm, int k_max, const void* q_dec,
   lse<<<std::min(a.items, sms), kItThreads, lse_smem, lc.st>>>(qm, km, kdm, a);
   lc.mark("imp_lse_tc");
   a.tiles_T = (dm.n + 127) / 128;
-  // key tiles per item: about eight items per SM, so that the last round is short
-  a.run = std::max(1, std::min(a.tiles_T, (int)(dm.heads() * a.tiles_T / (8LL * sms))));
-  a.runs = (a.tiles_T + a.run - 1) / a.run;
-  a.items = (int)dm.heads() * a.runs;
+  a.items = (int)dm.heads() * a.tiles_T;
   for (a.chunk0 = 0; a.chunk0 < a.chunks; a.chunk0 += 2) {
     a.nchunk = std::min(2, a.chunks - a.chunk0);
     a.accumulate = a.chunk0 > 0;
