@@ -7,24 +7,23 @@
 // maximum.
 //
 // 2.2e11 pairs (x, b) for 256 heads x 3968 tokens at B = 0.3 N n if every one is evaluated.  What is done instead:
-//   - tokens that no optimal solution can contain, and budgets that such tokens cannot add up to, are left out before (see
-//     "which tokens can matter" below): 5 % of the budgets and 6 % of the tokens are left there;
-//   - of those, a warp owns 64 budgets and skips every block of 64 values of b that an upper bound rules out: for any slope s
-//     a pair (y, b) can only matter if (f(y) - s y) + (U(b) - s b) reaches the smallest f_h(x) - s x found so far, and maxima
-//     of f and U over runs of 16 bound the left side; half a block at a time is then bounded by its own values.  Where six
-//     blocks or fewer are left all are evaluated: the bounds would take longer (256 heads, B = 0.05 N n: 891 us with, 784
-//     without);
+//   - tokens that no optimal solution can contain, and budgets on which none can pass, are left out before (see "which tokens
+//     can matter" below): 1 % of the budgets and 6 % of the tokens are left there;
+//   - of those, a warp owns 64 budgets; where many blocks of 64 values of b are left it skips every one that an upper bound
+//     rules out: for any slope s a pair (y, b) can only matter if (f(y) - s y) + (U(b) - s b) reaches the smallest
+//     f_h(x) - s x found so far, and maxima of f and U over runs of 16 bound the left side; half a block at a time is then
+//     bounded by its own values.  Where a CTA has few blocks all are evaluated, by many warps: the bounds would take longer;
 //   - in a block, a pair of additions is one packed instruction and two comparisons are one three-input maximum, on a
 //     register tile of 8 budgets x 8 pairs of b per lane; the argmax is not carried along;
 //   - all rows in one launch: a CTA keeps its part of the row before and the curve in shared memory and polls the values that
-//     others compute themselves, so that a row costs one trip through L2.
+//     others compute themselves, so that a row costs one trip through L2; two narrow rows share one.
 // The values are those of the full recursion wherever its solutions pass, bit for bit.
-// What bounds it now: the latency of a row (2.7 us: store, poll, two barriers and a tile's dependent clocks) and
-// of the walk back (0.6 us a head).  256 heads x 3968 tokens, B = 304742: 57.2 ms with every pair evaluated one by one and the
-// argmax kept; 3.95 ms with bounds and a launch per row; 2.7 + 0.4 ms in one launch over all budgets, its parts signalled by
-// flags; 0.99 ms over what can matter (greedy solution 0.09, rows 0.74, walk 0.17); 0.95 ms now, with several warps to a tile of
-// a narrow row.  CTAs of at least ten tiles instead of two 1171 us, five 1070 (before that); the curve's tokens read from L2 in
-// the walk 1.7 us a head.
+// What bounds it now: the latency of a row's straight-line code (1.8 us: poll, staging, a barrier, an evaluation spread over 18
+// warps and its maxima) and of the walk back (0.5 us a head).  256 heads x 3968 tokens, B = 304742: 57.2 ms with every pair
+// evaluated one by one and the argmax kept; 3.95 ms with bounds and a launch per row; 2.7 + 0.4 ms in one launch over all
+// budgets; 0.99 ms over the tokens that can matter and all budgets that they add up to (rows 0.72, walk 0.20, greedy solution 0.09);
+// 0.73 ms with the budgets' bands (335 -> 55 tiles a row: rows 0.69 -> 0.57), steps of narrow rows (0.47) and a walk by one warp
+// (0.13).  Three rows a step 745 us, two where a CTA has up to 64, 100 or 160 blocks 733, 748, 753; two tiles to a CTA 776.
 #include <math.h>
 
 #include <algorithm>
@@ -46,10 +45,14 @@ constexpr int kDpGroup = 80;                  // bytes of 8 packed pairs of f, p
 constexpr int kDpWindow = 112;                // packed pairs of f that a warp makes of 128 values
 constexpr int kDpUBlock = 2 * 128;            // bytes of a block's 32 packed pairs of U
 constexpr int kDpWindowsPer = ((kDpMaxBlocks + kDpSub) * kDpX / kDpWindow + kDpWarps) / kDpWarps;  // per warp
-constexpr int kDpMinTiles = 2;                // least tiles of a CTA in a row
+constexpr int kDpMinTiles = 1;                // least tiles of a CTA in a row
 constexpr int kDpWords = 2;                   // status, heads that have their tokens
 constexpr int kDpTable = 1024;                // rows whose parts are worked out ahead
-constexpr int kDpFewBlocks = 6;               // blocks of b that are evaluated without bounds
+constexpr int kDpFewWork = 40;                // blocks of b times tiles that a CTA evaluates without bounds
+constexpr int kDpJoin = 2;                    // rows that are made together where they are narrow
+constexpr int kDpJoinTiles = 32;              // most tiles of the row before that a narrow step stages
+constexpr int kDpStepWarps = kDpWarps - 2;    // warps that evaluate tiles in a narrow step; the others fetch the next curves
+constexpr int kDpStepBytes = (kDpJoinTiles * kDpX + kDpWindow) / 8 * kDpGroup;  // one of a narrow step's two buffers of f
 constexpr uint32_t kDpUnset = 0xFFFFFFFFu;    // a value that is still to come (a NaN that no addition or maximum makes)
 constexpr int kDpBackThreads = 384;
 
@@ -85,7 +88,7 @@ struct DpArgs {
 // Shared memory: the staged part of the previous row as packed pairs and its run maxima; the curve of this head and the
 // next one as packed pairs and their run maxima; the rows' parts.
 struct DpPlan {
-  int blocks, entries, runs_off, u_off, u_bytes, u_runs_off, table_off, total;
+  int blocks, entries, runs_off, u_off, u_blocks, u_bytes, u_runs_off, table_off, total;
 };
 __host__ __device__ inline DpPlan dp_plan(int n, int N) {
   DpPlan p;
@@ -94,10 +97,11 @@ __host__ __device__ inline DpPlan dp_plan(int n, int N) {
   p.runs_off = p.entries / 8 * kDpGroup;
   p.u_off = p.runs_off + (p.entries + 32) / kDpRun * 4;
   p.u_off = (p.u_off + 15) & ~15;
-  p.u_bytes = p.blocks * kDpUBlock;
+  p.u_blocks = p.blocks > kDpJoinTiles ? p.blocks : kDpJoinTiles;
+  p.u_bytes = p.u_blocks * kDpUBlock;
   p.u_runs_off = p.u_off + 2 * p.u_bytes;
   p.table_off = p.u_runs_off + 2 * p.blocks * 16;
-  p.total = p.table_off + (N < kDpTable ? N : kDpTable) * 32;
+  p.total = p.table_off + (N < kDpTable ? N : kDpTable) * (32 + 16);
   return p;
 }
 
@@ -131,10 +135,37 @@ __device__ __forceinline__ void dp_block(const unsigned char* fw, bool odd, cons
 }
 
 // Row h: the budgets [lo, hi], as tiles of 64 (from the tile of lo on, `per` to a CTA), and the blocks of b that it needs,
-// of whose halves of 32 the first `skip` and those from `halves` on hold no token that is left.
+// of whose halves of 32 only those from byte 0 of `halves` to byte 1 (not included) hold tokens that are left; bit 17: all blocks
+// are evaluated, without bounds.
 struct __align__(16) DpRow {
+  __device__ int half0() const { return halves & 255; }
+  __device__ int half1() const { return halves >> 8 & 255; }
+  __device__ bool few() const { return halves >> 17 & 1; }
   int lo, hi, tile0, tiles, per, blk0, blocks, halves;
 };
+
+// A tile's maxima out of the lanes' parts: a lane gets budgets dp_budget(lane) and the one behind it.
+__device__ __forceinline__ int dp_budget(int lane) { return 8 * (lane & 7) + (lane & 16 ? 4 : 0) + (lane & 8 ? 2 : 0); }
+__device__ __forceinline__ void dp_merge(const float (&blo)[8], const float (&bhi)[8], int lane, float (&best)[2]) {
+  const bool hi16 = lane & 16, hi8 = lane & 8;
+  float q[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const float a = fmaxf(blo[r], bhi[r]), b = fmaxf(blo[r + 4], bhi[r + 4]);
+    q[r] = fmaxf(hi16 ? b : a, __shfl_xor_sync(0xffffffffu, hi16 ? a : b, 16));
+  }
+#pragma unroll
+  for (int r = 0; r < 2; ++r) best[r] = fmaxf(hi8 ? q[r + 2] : q[r], __shfl_xor_sync(0xffffffffu, hi8 ? q[r] : q[r + 2], 8));
+}
+// Stores those of budgets x, x + 1 that the row has.
+__device__ __forceinline__ void dp_store(float* next, int x, int lo, int hi, const float (&best)[2]) {
+  if (x >= lo && x + 1 <= hi)
+    asm volatile("st.relaxed.gpu.global.v2.f32 [%0], {%1, %2};" ::"l"(next + x), "f"(best[0]), "f"(best[1]) : "memory");
+  else if (x >= lo && x <= hi)
+    asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" ::"l"(next + x), "f"(best[0]) : "memory");
+  else if (x + 1 >= lo && x + 1 <= hi)
+    asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" ::"l"(next + x + 1), "f"(best[1]) : "memory");
+}
 
 // Row h at the 64 budgets from x0 on (those in [lo, hi]) over `blocks` blocks of b.  Blocks and tokens count from the first
 // staged block; the staged values start 64 `blocks` budgets below what tile 0 reaches with the first token.  Of a row of few
@@ -193,20 +224,9 @@ __device__ __forceinline__ void dp_tile(const unsigned char* F2, const float* f_
     dp_block(f_lane + ((blocks + tile - blk) * 8 - 4 - 4 * half) * kDpGroup, odd, U2 + blk * kDpUBlock + half * 128 + bg * 32,
              blo, bhi);
   };
-  // the row so far: a lane gets budgets x0 + xl, x0 + xl + 1
-  const bool hi16 = lane & 16, hi8 = lane & 8;
-  const int xl = 8 * xg + (hi16 ? 4 : 0) + (hi8 ? 2 : 0);
+  const int xl = dp_budget(lane);
   float best[2];
-  auto merge = [&]() {
-    float q[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const float a = fmaxf(blo[r], bhi[r]), b = fmaxf(blo[r + 4], bhi[r + 4]);
-      q[r] = fmaxf(hi16 ? b : a, __shfl_xor_sync(0xffffffffu, hi16 ? a : b, 16));
-    }
-#pragma unroll
-    for (int r = 0; r < 2; ++r) best[r] = fmaxf(hi8 ? q[r + 2] : q[r], __shfl_xor_sync(0xffffffffu, hi8 ? q[r] : q[r + 2], 8));
-  };
+  auto merge = [&]() { dp_merge(blo, bhi, lane, best); };
   // smallest f_h(x) - s (x - x0) among the budgets that count, less the rounding of the terms in s
   auto lowest = [&](float s) {
     float neg = -INFINITY;
@@ -221,10 +241,10 @@ __device__ __forceinline__ void dp_tile(const unsigned char* F2, const float* f_
     return s > 0.f && s < 1e30f ? s : 0.f;  // s times a distance of up to 8192 stays a number
   };
 
-  if (blocks <= kDpFewBlocks) {
+  if (row.few()) {
     // few tokens: all of them (bounds would take longer)
 #pragma unroll 1
-    for (int i = (row.halves & 255) + part; i < row.halves >> 8; i += parts) evaluate(i >> 1, i & 1);
+    for (int i = row.half0() + part; i < row.half1(); i += parts) evaluate(i >> 1, i & 1);
     merge();
     if (parts > 1) {
       float2* mine = reinterpret_cast<float2*>(part_s + part * kDpX + xl);
@@ -272,14 +292,55 @@ __device__ __forceinline__ void dp_tile(const unsigned char* F2, const float* f_
     }
     if (raised) merge();
   }
-  if (!next) return;
-  const int x = x0 + xl;
-  if (x >= lo && x + 1 <= hi)
-    asm volatile("st.relaxed.gpu.global.v2.f32 [%0], {%1, %2};" ::"l"(next + x), "f"(best[0]), "f"(best[1]) : "memory");
-  else if (x >= lo && x <= hi)
-    asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" ::"l"(next + x), "f"(best[0]) : "memory");
-  else if (x + 1 >= lo && x + 1 <= hi)
-    asm volatile("st.relaxed.gpu.global.f32 [%0], %1;" ::"l"(next + x + 1), "f"(best[1]) : "memory");
+  if (next) dp_store(next, x0 + xl, lo, hi, best);
+}
+
+// One row of a narrow step: `count` tiles from tile t0 on, their halves of blocks shared out over kDpStepWarps warps.  The values go to
+// `next` (global memory; the tiles from `own` on) and, as staged values of the row behind it, to `onward` (shared memory), where given.
+__device__ __forceinline__ void dp_narrow(const unsigned char* F2, const unsigned char* U2, const DpRow& row, int t0, int count,
+                                          int own, float* next, unsigned char* onward, const unsigned short* parts_of, int warp,
+                                          int lane, float* part_s) {
+  const int xg = lane & 7, bg = lane >> 3, e_lane = 8 * xg - 4 * bg + 12, xl = dp_budget(lane);
+  const bool odd = (bg & 1) == 0;
+  const unsigned char* f_lane = F2 + (e_lane >> 3) * kDpGroup + (e_lane & 7) * 8;
+  const int half0 = row.half0(), half1 = row.half1();
+  const int parts = min((int)parts_of[min(count, kDpStepWarps)], half1 - half0);
+  const int per = parts_of[32 + parts];  // 1024 / parts, rounded up: the quotients below are exact
+#pragma unroll 1
+  for (int v = warp; v < count * parts; v += kDpStepWarps) {
+    const int tile = v * per >> 10, part = v - tile * parts;
+    float blo[8], bhi[8], best[2];
+#pragma unroll
+    for (int r = 0; r < 8; ++r) blo[r] = bhi[r] = -INFINITY;
+    const unsigned char* f = f_lane + ((row.blocks + tile) * 8 - 4) * kDpGroup;
+#pragma unroll 1
+    for (int i = half0 + part; i < half1; i += parts) dp_block(f - 4 * kDpGroup * i, odd, U2 + 128 * i + bg * 32, blo, bhi);
+    dp_merge(blo, bhi, lane, best);
+    if (parts > 1) {
+      float2* mine = reinterpret_cast<float2*>(part_s + v * kDpX + xl);
+      *mine = make_float2(best[0], best[1]);
+      bar_sync(1 + tile, 32 * parts);
+      if (part > 0) break;
+#pragma unroll 4
+      for (int i = 1; i < parts; ++i) {
+        const float2 o = mine[i * (kDpX / 2)];
+        best[0] = fmaxf(best[0], o.x);
+        best[1] = fmaxf(best[1], o.y);
+      }
+    }
+    const int x = (t0 + tile) * kDpX + xl;
+    if (onward) {
+      const int e = kDpX * tile + xl;
+      const float g0 = x >= row.lo && x <= row.hi ? best[0] : -INFINITY, g1 = x + 1 >= row.lo && x + 1 <= row.hi ? best[1] : -INFINITY;
+      float* second = reinterpret_cast<float*>(onward + (e >> 3) * kDpGroup + (e & 7) * 8 + 4);
+      second[0] = g0, second[2] = g1;
+      if (e >= 16) {  // (the last 16 pairs of a row are never read)
+        float* first = reinterpret_cast<float*>(onward + ((e >> 3) - 2) * kDpGroup + (e & 7) * 8);
+        first[0] = g0, first[2] = g1;
+      }
+    }
+    if (next && tile >= own) dp_store(next, x, row.lo, row.hi, best);
+  }
 }
 
 // ---- which tokens can matter -------------------------------------------------------------------------------------
@@ -291,7 +352,8 @@ __device__ __forceinline__ void dp_tile(const unsigned char* F2, const float* f_
 // value of at least LB less twice the sum of those errors.  With that allowance the tokens [b0, b1] of a head that are
 // left, and the budgets that such tokens add up to, hold every path that the full recursion could return, and the rows
 // restricted to them have the full recursion's values on those paths.  l and LB come from the greedy solution of the
-// relaxed problem, which is close: 240 of 3968 tokens a head are left on utility curves of 256 heads, and 5 % of the budgets.
+// relaxed problem, which is close: 240 of 3968 tokens a head are left on utility curves of 256 heads, and 5 % of the budgets, of
+// which the bands (dp_band) leave a sixth.
 
 constexpr int kDpCoreThreads = 256;
 __device__ __forceinline__ double dp_warp_sum(double v) {
@@ -318,11 +380,20 @@ struct DpCore {
   double* c;                // [N] c_j
   double* u;                // [N] U_j at the greedy solution
   double* size;             // [N] max |U_j|
+  float* f;                 // [N][stride]: before the rows are made, kDpSlopes doubles at the start of each hold the bounds' sums
+  long long stride;
   int4* rows;               // [N]
   int* done;                // [1] heads that have their tokens, zero before
   int P, N, n, B;
 };
-// The slope and every head's c_j.  One CTA per head.
+// Slopes whose bounds are used: l and l (1 +- 2^-i), i = 1 .. 7 (15 is l again).  Steps by two lose at most 6 % of a quadratic's
+// width; i up to 15 leaves as many budgets.
+constexpr int kDpSlopes = 16;
+__device__ __forceinline__ double dp_slope(double l, int k) {
+  const int i = (k + 1) >> 1;
+  return k == 0 || k == kDpSlopes - 1 ? l : l + ((k & 1) ? l : -l) * __longlong_as_double((long long)(1023 - i) << 52);
+}
+// The slope, every head's c_j, and c_j for the slopes next to it.  One CTA per head.
 __global__ void __launch_bounds__(kDpCoreThreads) dp_reduced_kernel(const DpCore a) {
   __shared__ double part[kDpCoreThreads / 32], part_size[kDpCoreThreads / 32];
   __shared__ float gain_s[kDpCoreThreads / 32];
@@ -382,6 +453,23 @@ __global__ void __launch_bounds__(kDpCoreThreads) dp_reduced_kernel(const DpCore
     a.size[j] = size;
     a.u[j] = (double)__ldg(U + min(max(a.budgets[j], 0), a.n));
     if (j == 0) *a.slope = slope;
+  }
+  constexpr int kPer = kDpSlopes / (kDpCoreThreads / 32);  // slopes a warp
+  const int lane = tid & 31, k0 = kPer * (tid >> 5);
+  double s[kPer], most_at[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) s[k] = -dp_slope(slope, k0 + k), most_at[k] = -INFINITY;
+  double at = (double)lane;
+  for (int b = lane; b <= a.n; b += 32, at += 32.0) {
+    const double x = (double)__ldg(U + b);
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) most_at[k] = fmax(most_at[k], fma(s[k], at, x));
+  }
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) most_at[k] = fmax(most_at[k], __shfl_xor_sync(0xffffffffu, most_at[k], off));
+    if (lane == k) reinterpret_cast<double*>(a.f + (size_t)j * a.stride)[k0 + k] = most_at[k];
   }
 }
 
@@ -467,6 +555,60 @@ __global__ void __launch_bounds__(kDpCoreThreads) dp_ranges_kernel(const DpCore 
       if (!sound) total0 = 0, total1 = (long long)a.N * a.n;
     }
   }
+  // running sums over the heads of every slope's c_j, in place; all heads' sums take the place of `size`, and the least value that
+  // a solution must have that of `u` (both have been read)
+  __shared__ double seg_s[kDpCoreThreads / 32][32];
+  const int lane = tid & 31, warp = tid >> 5, per = (a.N + kDpCoreThreads / 32 - 1) / (kDpCoreThreads / 32);
+  const int first = warp * per, end = min(a.N, first + per);
+  auto sum_at = [&](int i) { return reinterpret_cast<double*>(a.f + (size_t)i * a.stride) + lane; };
+  double run = 0.0;
+  auto over_heads = [&](bool store) {
+    for (int i = first; i < end; i += 8) {
+      double v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = i + k < end && lane < kDpSlopes ? __ldcg(sum_at(i + k)) : 0.0;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        run += v[k];
+        if (store && i + k < end && lane < kDpSlopes) *sum_at(i + k) = run;
+      }
+    }
+  };
+  over_heads(false);
+  seg_s[warp][lane] = run;
+  __syncthreads();
+  run = 0.0;
+  double all = 0.0;
+  for (int i = 0; i < kDpCoreThreads / 32; ++i) {
+    if (i < warp) run += seg_s[i][lane];
+    all += seg_s[i][lane];
+  }
+  over_heads(true);
+  if (warp == 0 && lane < kDpSlopes) a.size[lane] = all;
+  if (tid == 0) a.u[0] = sound ? slope * (double)a.B + c - slack : -INFINITY;
+}
+
+// The budgets of row h on which a solution can pass.  With C(l) the sum of c_j(l) over the heads up to h and S(l) that over the
+// others, a solution that has x tokens up to h is worth at most C(l) + l x + S(l') + l' (B - x) for any two slopes; where that is
+// below the least value that it must have, x does not count.  The heads share the slack here, instead of each having all of it:
+// 2 000 budgets a row are left on average instead of 12 600 (256 heads x 3968 tokens).  Lane k takes slope k against all others.
+__device__ __forceinline__ int4 dp_band(const DpCore& a, int h, int4 r) {
+  const int lane = threadIdx.x & (kDpSlopes - 1);
+  const double l = dp_slope(*a.slope, lane), up_to = reinterpret_cast<const double*>(a.f + (size_t)h * a.stride)[lane];
+  const double others = a.size[lane] - up_to + l * (double)a.B, need = a.u[0] - up_to;
+  int lo = r.x, hi = r.y;
+  for (int k = 0; k < kDpSlopes - 1; ++k) {
+    const double lk = __shfl_sync(0xffffffffu, l, k), sk = __shfl_sync(0xffffffffu, others, k);
+    const double x = (need - sk) / (l - lk);
+    if (x > -1e9 && x < 1e9) {  // (a number; not for equal slopes)
+      if (l > lk) lo = max(lo, (int)floor(x));
+      if (l < lk) hi = min(hi, (int)ceil(x));
+    }
+  }
+  lo = __reduce_max_sync(0xffffffffu, lo);
+  hi = __reduce_min_sync(0xffffffffu, hi);
+  if (lo <= hi) r.x = lo, r.y = hi;
+  return r;
 }
 
 __device__ __forceinline__ DpRow dp_row(const DpArgs& a, int h) {
@@ -479,20 +621,27 @@ __device__ __forceinline__ DpRow dp_row(const DpArgs& a, int h) {
   r.blk0 = v.z / kDpX;
   r.blocks = v.w / kDpX - r.blk0 + 1;
   const int skip = v.z / 32 - 2 * r.blk0;
-  r.halves = skip | (v.w / 32 - 2 * r.blk0 + 1) << 8;
+  r.halves = skip | (v.w / 32 - 2 * r.blk0 + 1) << 8 | (r.blocks * min(r.per, r.tiles) <= kDpFewWork) << 17;
   return r;
 }
 
 // Marks the values of the rows that are to come, and their vectors' other elements as -inf.  One CTA per row.  `B` (or
-// -1: the rows are known): rows of all tokens are made first, those budgets that can still reach B.
-__global__ void __launch_bounds__(256) dp_clear_kernel(const DpArgs a, int4* rows, int B) {
+// -1: the rows are known, but for the bands): rows of all tokens are made first, those budgets that can still reach B.
+__global__ void __launch_bounds__(256) dp_clear_kernel(const DpArgs a, const DpCore core, int4* rows, int B) {
   const int h = blockIdx.x;
   int4 r;
   if (B >= 0) {
     r = make_int4((int)max(0LL, B - (long long)(a.N - 1 - h) * a.n), (int)min((long long)B, (long long)(h + 1) * a.n), 0, a.n);
     if (threadIdx.x == 0) rows[h] = r;
   } else {
-    r = __ldg(a.rows + h);
+    __shared__ int4 row_s;
+    if (threadIdx.x < 32) {
+      r = dp_band(core, h, rows[h]);
+      __syncwarp();
+      if (threadIdx.x == 0) row_s = rows[h] = r;
+    }
+    __syncthreads();  // (the sums at the start of the row are read)
+    r = row_s;
   }
   float* f = a.f + (size_t)h * a.stride;
   const float unset = __uint_as_float(kDpUnset);
@@ -508,6 +657,8 @@ __global__ void __launch_bounds__(256) dp_clear_kernel(const DpArgs a, int4* row
 __global__ void __launch_bounds__(kDpThreads, 1) dp_rows_kernel(const DpArgs a) {
   extern __shared__ __align__(16) unsigned char dp_smem[];
   __shared__ int next_tile;
+  __shared__ volatile int stop_s[2];  // a wait of a narrow step ran out (steps take them in turn)
+  __shared__ unsigned short parts_of[64];
   __shared__ __align__(16) float part_s[kDpWarps * kDpX];
   const DpPlan plan = dp_plan(a.n, a.N);
   unsigned char* F2 = dp_smem;                                       // packed pairs (f(y + 16), f(y))
@@ -516,10 +667,40 @@ __global__ void __launch_bounds__(kDpThreads, 1) dp_rows_kernel(const DpArgs a) 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, cta = blockIdx.x;
   for (int i = threadIdx.x; i < min(a.N, kDpTable); i += kDpThreads) table[i] = dp_row(a, i);
   __syncthreads();
+  // Narrow steps: kDpJoin rows of few blocks (those whose numbers follow a multiple of it), or one.  A CTA makes the values that it
+  // needs of all but the last row itself, from the row before all of them, so that one trip through L2 serves all of a step.
+  // steps[h]: first tile and number of tiles to be staged, tiles of this CTA in the last row, rows (0: not a narrow step).
+  const int listed = min(a.N, kDpTable);
+  int4* steps = reinterpret_cast<int4*>(table + listed);
+  for (int h = threadIdx.x; h < listed; h += kDpThreads) {
+    int4 st = make_int4(0, 0, 0, 0);
+    for (int rows = kDpJoin; rows > 0 && st.w == 0; rows = rows > 1 ? 1 : 0) {
+      if (h + rows > listed || (rows > 1 && h % rows != 0)) continue;
+      const DpRow last = table[h + rows - 1];
+      const int mine = min(last.per, last.tiles - cta * last.per);
+      int t = last.tile0 + cta * last.per, tiles = min(last.per, last.tiles);  // (the same answer in all CTAs)
+      bool narrow = true;
+      for (int i = rows - 1; i >= 0; --i) {
+        const DpRow r = table[h + i];
+        narrow = narrow && tiles * r.blocks <= kDpFewWork;
+        tiles += r.blocks;
+        t -= r.blk0 + r.blocks;
+      }
+      if (narrow && tiles <= kDpJoinTiles) st = make_int4(t, tiles - min(last.per, last.tiles) + mine, mine, rows);
+    }
+    steps[h] = st;
+  }
+  if (threadIdx.x < 64) {
+    const int i = threadIdx.x & 31;
+    parts_of[threadIdx.x] = i == 0 ? 1 : threadIdx.x < 32 ? max(1, kDpStepWarps / i) : (1024 + i - 1) / i;
+  }
+  if (threadIdx.x < 2) stop_s[threadIdx.x] = 0;
+  __syncthreads();
   auto row_of = [&](int h) { return h < kDpTable ? table[h] : dp_row(a, h); };
-  auto fetch_curve = [&](int h, const DpRow& r, int buf, int warp0) {  // the blocks that the row needs, by warps from warp0 on
+  auto step_of = [&](int h) { return h < listed ? steps[h] : make_int4(0, 0, 0, 0); };
+  auto fetch_curve = [&](int h, const DpRow& r, int buf, int at, int warp0) {  // the blocks that the row needs, by warps from warp0 on
     const int tid0 = threadIdx.x - 32 * warp0, threads = kDpThreads - 32 * warp0;
-    unsigned char* U2 = dp_smem + plan.u_off + buf * plan.u_bytes;
+    unsigned char* U2 = dp_smem + plan.u_off + buf * plan.u_bytes + at * kDpUBlock;
     const float* U = a.curves + (size_t)h * a.P + r.blk0 * kDpX;
     const int last = a.n - r.blk0 * kDpX;
     for (int b = tid0; b < r.blocks * kDpX; b += threads) {
@@ -527,88 +708,178 @@ __global__ void __launch_bounds__(kDpThreads, 1) dp_rows_kernel(const DpArgs a) 
       if (b <= last) cp_async4(to, U + b);
       else *reinterpret_cast<float*>(to) = -INFINITY;
     }
+    if (r.few()) return;
     float* ur = reinterpret_cast<float*>(dp_smem + plan.u_runs_off) + buf * plan.blocks * 4;
     for (int i = tid0; i < r.blocks * 4; i += threads)
       cp_async4(ur + i, a.u_runs + (size_t)h * kDpURuns + r.blk0 * 4 + i);
   };
-  auto next_row = [&](int h) {  // the next row from h on of which this CTA has a part
-    for (; h < a.N; ++h) {
-      const DpRow r = row_of(h);
-      if (cta * r.per < r.tiles) break;
+  auto next_row = [&](int h) {  // the next step from row h on in which this CTA has a part
+    while (h < a.N) {
+      const int4 st = step_of(h);
+      if (st.w > 0) {
+        if (st.z > 0) break;
+        h += st.w;
+      } else {
+        const DpRow r = row_of(h);
+        if (cta * r.per < r.tiles) break;
+        ++h;
+      }
     }
     return h;
   };
+  auto fetch_curves = [&](int h, int buf, int warp0) {
+    if (h >= a.N) return;
+    const int rows = max(1, step_of(h).w);
+    for (int i = 0, at = 0; i < rows; ++i) {
+      const DpRow r = row_of(h + i);
+      fetch_curve(h + i, r, buf, at, warp0);
+      at += r.blocks;
+    }
+  };
   int h = next_row(0), buf = 0;
-  if (h < a.N) fetch_curve(h, row_of(h), 0, 0);
+  fetch_curves(h, 0, 0);
 
-  for (int h_next = a.N; h < a.N; h = h_next, buf ^= 1) {
-    const DpRow row = row_of(h);
+  // Stages f_{h-1} from budget ybase on (at least 64 `tiles` values); false if a wait ran out.
+  auto stage = [&](int h, int ybase, int tiles) -> bool {
     const int old_lo = h > 0 ? row_of(h - 1).lo : 0, old_hi = h > 0 ? row_of(h - 1).hi : 0;
-    const int tile0 = row.tile0 + cta * row.per, tiles = min(row.per, row.tiles - cta * row.per);
     const float* prev = a.f + (size_t)(h > 0 ? h - 1 : 0) * a.stride;
+    const int windows = (tiles * kDpX + kDpWindow - 1) / kDpWindow;
+    // f_{h-1} at ybase + 112 i + 4 lane .. + 3 for this warp's windows i
+    float4 v[kDpWindowsPer];
+    uint32_t left = 0;
+#pragma unroll
+    for (int k = 0; k < kDpWindowsPer; ++k) {
+      const int y = ybase + kDpWindow * (warp + k * kDpWarps) + 4 * lane;
+      v[k] = make_float4(h == 0 && y == 0 ? 0.f : -INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      if (h > 0 && warp + k * kDpWarps < windows && y + 3 >= old_lo && y <= old_hi) left |= 1u << k;
+    }
+    bool ok = true;
+    for (uint32_t spins = 0; left;) {
+#pragma unroll
+      for (int k = 0; k < kDpWindowsPer; ++k)
+        if (left >> k & 1)
+          asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                       : "=f"(v[k].x), "=f"(v[k].y), "=f"(v[k].z), "=f"(v[k].w)
+                       : "l"(prev + ybase + kDpWindow * (warp + k * kDpWarps) + 4 * lane)
+                       : "memory");
+#pragma unroll
+      for (int k = 0; k < kDpWindowsPer; ++k)
+        if (__float_as_uint(v[k].x) != kDpUnset && __float_as_uint(v[k].y) != kDpUnset &&
+            __float_as_uint(v[k].z) != kDpUnset && __float_as_uint(v[k].w) != kDpUnset)
+          left &= ~(1u << k);
+      if (left && (++spins >= a.spin_limit || ((spins & 255) == 0 && *reinterpret_cast<volatile int*>(a.words) != 0))) {
+        atomicExch(a.words, (int)LUKV_ERR_TIMEOUT);
+        ok = false;
+        break;
+      }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    if (!__syncthreads_and(ok)) return false;  // (and the tiles before have been read)
+    if (threadIdx.x == 0) next_tile = kDpWarps;
+#pragma unroll
+    for (int k = 0; k < kDpWindowsPer; ++k) {
+      const int i = warp + k * kDpWarps;
+      if (i < windows) {
+        // lane l >= 4 holds the first parts of pairs 4 l - 16 .. + 3, lane l - 4 their second parts
+        const float g0 = __shfl_up_sync(0xffffffffu, v[k].x, 4), g1 = __shfl_up_sync(0xffffffffu, v[k].y, 4);
+        const float g2 = __shfl_up_sync(0xffffffffu, v[k].z, 4), g3 = __shfl_up_sync(0xffffffffu, v[k].w, 4);
+        if (lane >= 4) {
+          float4* to_s = reinterpret_cast<float4*>(F2 + (kDpWindow / 8 * i + ((lane - 4) >> 1)) * kDpGroup + (lane & 1) * 32);
+          to_s[0] = make_float4(v[k].x, g0, v[k].y, g1);
+          to_s[1] = make_float4(v[k].z, g2, v[k].w, g3);
+        }
+        float m = fmaxf(max3(v[k].x, v[k].y, v[k].z), v[k].w);
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+        if ((lane & 3) == 0 && (lane < 28 || i == windows - 1)) f_runs[kDpWindow / kDpRun * i + (lane >> 2)] = m;
+      }
+    }
+    __syncthreads();
+    return true;
+  };
+
+  bool settled = true;  // no warp may still read staged values of a step that is not narrow
+  int turn = 0;
+  int side = 0;         // buffer that the next narrow step is staged in: none of its warps may still read from it
+  for (int h_next = a.N; h < a.N; h = h_next, buf ^= 1) {
+    const int4 st = step_of(h);
+    if (st.w > 0) {
+      // f_{h-1} from the first tile on, a window of 112 values a warp; no barrier ahead of the stores: the step before ended in
+      // the other buffer
+      if (!settled) __syncthreads();
+      settled = true;
+      unsigned char* F = F2 + side * kDpStepBytes;
+      if (warp * kDpWindow < st.y * kDpX) {
+        const int y = st.x * kDpX + kDpWindow * warp + 4 * lane;
+        float4 v = make_float4(h == 0 && y == 0 ? 0.f : -INFINITY, -INFINITY, -INFINITY, -INFINITY);
+        if (h > 0) {
+          const DpRow* before = table + h - 1;
+          if (y + 3 >= before->lo && y <= before->hi) {
+            const float* from = a.f + (size_t)(h - 1) * a.stride + y;
+            for (uint32_t spins = 0;;) {
+              asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
+                           : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(from) : "memory");
+              if (__float_as_uint(v.x) != kDpUnset && __float_as_uint(v.y) != kDpUnset && __float_as_uint(v.z) != kDpUnset &&
+                  __float_as_uint(v.w) != kDpUnset)
+                break;
+              if (++spins >= a.spin_limit || ((spins & 255) == 0 && *reinterpret_cast<volatile int*>(a.words) != 0)) {
+                atomicExch(a.words, (int)LUKV_ERR_TIMEOUT);
+                stop_s[turn] = 1;
+                break;
+              }
+            }
+          }
+        }
+        __syncwarp();
+        const float g0 = __shfl_up_sync(0xffffffffu, v.x, 4), g1 = __shfl_up_sync(0xffffffffu, v.y, 4);
+        const float g2 = __shfl_up_sync(0xffffffffu, v.z, 4), g3 = __shfl_up_sync(0xffffffffu, v.w, 4);
+        if (lane >= 4) {
+          float4* to_s = reinterpret_cast<float4*>(F + (kDpWindow / 8 * warp + ((lane - 4) >> 1)) * kDpGroup + (lane & 1) * 32);
+          to_s[0] = make_float4(v.x, g0, v.y, g1);
+          to_s[1] = make_float4(v.z, g2, v.w, g3);
+        }
+      }
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncthreads();
+      if (stop_s[turn]) return;
+      turn ^= 1;
+      h_next = next_row(h + st.w);
+      const bool next_narrow = step_of(h_next).w > 0;
+      if (warp >= kDpStepWarps && next_narrow) fetch_curves(h_next, buf ^ 1, kDpStepWarps);
+      const unsigned char* U2 = dp_smem + plan.u_off + buf * plan.u_bytes;
+      int t0 = st.x, count = st.y;
+#pragma unroll 1
+      for (int i = 0; i < st.w; ++i) {
+        const DpRow row = table[h + i];
+        t0 += row.blk0 + row.blocks;
+        count -= row.blocks;
+        if (i > 0) __syncthreads();
+        // The row's top st.z tiles are this CTA's to store (the walk back reads every row), and all of them the first one's.
+        if (warp < kDpStepWarps)
+          dp_narrow(F2 + (side ^ (i & 1)) * kDpStepBytes, U2, row, t0, count, cta == 0 ? 0 : count - st.z,
+                    cta != a.drop ? a.f + (size_t)(h + i) * a.stride : nullptr,
+                    i + 1 < st.w ? F2 + (side ^ (~i & 1)) * kDpStepBytes : nullptr, parts_of, warp, lane, part_s);
+        U2 += row.blocks * kDpUBlock;
+      }
+      side = (side + st.w) & 1;
+      if (!next_narrow) fetch_curves(h_next, buf ^ 1, 0);
+      continue;
+    }
+    settled = false;
+    const DpRow row = row_of(h);
+    const int tile0 = row.tile0 + cta * row.per, tiles = min(row.per, row.tiles - cta * row.per);
     float* next = a.f + (size_t)h * a.stride;
     const unsigned char* U2 = dp_smem + plan.u_off + buf * plan.u_bytes;
     const float4* u_runs = reinterpret_cast<const float4*>(dp_smem + plan.u_runs_off) + buf * plan.blocks;
     for (int t_sub = 0; t_sub < tiles; t_sub += kDpSub) {
       const int n_sub = min(kDpSub, tiles - t_sub), xs = (tile0 + t_sub) * kDpX;
       const int ybase = xs - (row.blk0 + row.blocks) * kDpX;
-      const int windows = ((row.blocks + n_sub) * kDpX + kDpWindow - 1) / kDpWindow;
-      // f_{h-1} at ybase + 112 i + 4 lane .. + 3 for this warp's windows i
-      float4 v[kDpWindowsPer];
-      uint32_t left = 0;
-#pragma unroll
-      for (int k = 0; k < kDpWindowsPer; ++k) {
-        const int y = ybase + kDpWindow * (warp + k * kDpWarps) + 4 * lane;
-        v[k] = make_float4(h == 0 && y == 0 ? 0.f : -INFINITY, -INFINITY, -INFINITY, -INFINITY);
-        if (h > 0 && warp + k * kDpWarps < windows && y + 3 >= old_lo && y <= old_hi) left |= 1u << k;
-      }
-      bool ok = true;
-      for (uint32_t spins = 0; left;) {
-#pragma unroll
-        for (int k = 0; k < kDpWindowsPer; ++k)
-          if (left >> k & 1)
-            asm volatile("ld.relaxed.gpu.global.v4.f32 {%0, %1, %2, %3}, [%4];"
-                         : "=f"(v[k].x), "=f"(v[k].y), "=f"(v[k].z), "=f"(v[k].w)
-                         : "l"(prev + ybase + kDpWindow * (warp + k * kDpWarps) + 4 * lane)
-                         : "memory");
-#pragma unroll
-        for (int k = 0; k < kDpWindowsPer; ++k)
-          if (__float_as_uint(v[k].x) != kDpUnset && __float_as_uint(v[k].y) != kDpUnset &&
-              __float_as_uint(v[k].z) != kDpUnset && __float_as_uint(v[k].w) != kDpUnset)
-            left &= ~(1u << k);
-        if (left && (++spins >= a.spin_limit || ((spins & 255) == 0 && *reinterpret_cast<volatile int*>(a.words) != 0))) {
-          atomicExch(a.words, (int)LUKV_ERR_TIMEOUT);
-          ok = false;
-          break;
-        }
-      }
-      asm volatile("cp.async.wait_all;" ::: "memory");
-      if (!__syncthreads_and(ok)) return;  // (and the tiles before have been read)
-      if (threadIdx.x == 0) next_tile = kDpWarps;
-#pragma unroll
-      for (int k = 0; k < kDpWindowsPer; ++k) {
-        const int i = warp + k * kDpWarps;
-        if (i < windows) {
-          // lane l >= 4 holds the first parts of pairs 4 l - 16 .. + 3, lane l - 4 their second parts
-          const float g0 = __shfl_up_sync(0xffffffffu, v[k].x, 4), g1 = __shfl_up_sync(0xffffffffu, v[k].y, 4);
-          const float g2 = __shfl_up_sync(0xffffffffu, v[k].z, 4), g3 = __shfl_up_sync(0xffffffffu, v[k].w, 4);
-          if (lane >= 4) {
-            float4* to_s = reinterpret_cast<float4*>(F2 + (kDpWindow / 8 * i + ((lane - 4) >> 1)) * kDpGroup + (lane & 1) * 32);
-            to_s[0] = make_float4(v[k].x, g0, v[k].y, g1);
-            to_s[1] = make_float4(v[k].z, g2, v[k].w, g3);
-          }
-          float m = fmaxf(max3(v[k].x, v[k].y, v[k].z), v[k].w);
-          m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
-          m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
-          if ((lane & 3) == 0 && (lane < 28 || i == windows - 1)) f_runs[kDpWindow / kDpRun * i + (lane >> 2)] = m;
-        }
-      }
-      __syncthreads();
+      if (!stage(h, ybase, row.blocks + n_sub)) return;
 
       // several warps to a tile where there are few, one warp to several tiles (as they come: they differ in what there is to
       // look at) where there are many; warps without one fetch the next curve at once
-      const int halves = (row.halves >> 8) - (row.halves & 255);
-      const int parts = row.blocks <= kDpFewBlocks ? max(1, min(kDpWarps / n_sub, halves)) : 1, busy = n_sub * parts;
+      const int halves = row.half1() - row.half0();
+      const int parts = row.few() ? max(1, min(kDpWarps / n_sub, halves)) : 1, busy = n_sub * parts;
       if (busy <= kDpWarps) {
         const bool last = t_sub + n_sub == tiles;
         if (warp < busy) {
@@ -619,7 +890,7 @@ __global__ void __launch_bounds__(kDpThreads, 1) dp_rows_kernel(const DpArgs a) 
         if (last) {
           h_next = next_row(h + 1);
           const int from = busy < kDpWarps ? busy : 0;
-          if (h_next < a.N && warp >= from) fetch_curve(h_next, row_of(h_next), buf ^ 1, from);
+          if (warp >= from) fetch_curves(h_next, buf ^ 1, from);
         }
       } else {
         for (int tile = warp; tile < n_sub;) {
@@ -629,7 +900,7 @@ __global__ void __launch_bounds__(kDpThreads, 1) dp_rows_kernel(const DpArgs a) 
         }
         if (t_sub + n_sub == tiles) {
           h_next = next_row(h + 1);
-          if (h_next < a.N) fetch_curve(h_next, row_of(h_next), buf ^ 1, 0);
+          fetch_curves(h_next, buf ^ 1, 0);
         }
       }
     }
@@ -719,6 +990,105 @@ __global__ void __launch_bounds__(kDpBackThreads) dp_backtrack_kernel(const DpAr
   }
 }
 
+// The same where few tokens of a head are left: one warp walks, its step a load out of L1 (a lane has eight values of b), a comparison
+// and a reduction, no barrier; the curve's values and the next rows' ranges are asked for a step ahead.  The other warps bring
+// what the steps up to kWalkReach heads on can read into L1, following the walk through shared memory.
+constexpr int kWalkWarps = 8, kWalkReach = 8, kWalkPer = 8;
+__global__ void __launch_bounds__(32 * kWalkWarps) dp_walk_kernel(const DpArgs a, int B, int w, long long row_base, int q,
+                                                                  int32_t* __restrict__ budgets, int32_t* __restrict__ offsets,
+                                                                  double* __restrict__ values) {
+  __shared__ volatile unsigned long long at_s;  // the step the walk is at: head << 32 | budget
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, N = a.N;
+  const bool failed = a.words[0] != 0;
+  if (threadIdx.x == 0) at_s = (unsigned long long)(N - 1) << 32 | (uint32_t)B;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    a.words[1] = 0;
+    if (q == 0) offsets[0] = 0;
+  }
+  if (failed) {  // a wait of the rows' kernel ran out: no solution
+    if (threadIdx.x == 0) values[q] = __longlong_as_double(0x7FF8000000000000LL);
+    for (int h = threadIdx.x; h < N; h += 32 * kWalkWarps) {
+      budgets[(size_t)q * N + h] = 0;
+      offsets[(size_t)q * N + h + 1] = (int32_t)(row_base + (long long)(h + 1) * w);
+    }
+    return;
+  }
+  if (warp > 0) {
+    auto touch = [](const float* p) { asm volatile("{\n\t.reg .f32 t;\n\tld.global.nc.f32 t, [%0];\n\t}" ::"l"(p)); };
+    for (int t = N - warp; t > 0; t -= kWalkWarps - 1) {
+      int h = 0, x = 0;
+      for (int spin = 0; spin < 1 << 20; ++spin) {
+        const unsigned long long at = at_s;
+        h = (int)(at >> 32), x = (int)(uint32_t)at;
+        if (h - t <= kWalkReach) break;
+      }
+      if (h < t) continue;
+      // what the heads from t + 1 to h take at the least and at the most, then this one's tokens
+      int4 r = make_int4(0, 0, 0, 0);
+      if (lane <= h - t && lane <= kWalkReach) r = __ldg(a.rows + t + lane);
+      const long long y1 = x - (long long)__reduce_add_sync(0xffffffffu, r.z);
+      const long long y0 = max((long long)__ldg(a.rows + t - 1).x, x - (long long)__reduce_add_sync(0xffffffffu, r.w)) & ~31LL;
+      for (long long y = y0 + 32 * lane; y <= y1; y += 32 * 32) touch(a.f + (size_t)(t - 1) * a.stride + y);
+      const int z = __shfl_sync(0xffffffffu, r.z, 0), most = __shfl_sync(0xffffffffu, r.w, 0);
+      for (int b = z + 32 * lane; b <= most + 31; b += 32 * 32) touch(a.curves + (size_t)t * a.P + min(b, most));
+    }
+    return;
+  }
+  int x = B;
+  float target = __ldg(a.f + (size_t)(N - 1) * a.stride + B);
+  if (lane == 0) values[q] = (double)target;
+  const int4 nothing = make_int4(0, 0, 0, 0);
+  int4 row = __ldg(a.rows + N - 1), old = N > 1 ? __ldg(a.rows + N - 2) : nothing;
+  const float* prev = a.f + (size_t)max(N - 2, 0) * a.stride;
+  const float* U = a.curves + (size_t)(N - 1) * a.P;
+  int32_t* out_b = budgets + (size_t)q * N + N - 1;
+  int32_t* out_o = offsets + (size_t)q * N + N;
+  int rows = (int)(row_base + (long long)N * w);  // the windows' rows up to and with head h
+  const float none = __uint_as_float(kDpUnset);   // equals nothing
+  for (int h = N - 1; h > 0; --h) {
+    const int4 older = __ldg(a.rows + max(h - 2, 0));
+    // the tokens of the head with which the row before has a value
+    const int b0 = max(row.z, x - old.y), last = min(row.w, x - old.x);
+    int found = 1 << 30;
+    for (int b1 = b0 + lane; b1 - lane <= last; b1 += 32 * kWalkPer) {
+      const float* ep = prev + (x - b1);
+      const float* up = U + b1;
+      float e[kWalkPer], u[kWalkPer];
+#pragma unroll
+      for (int k = 0; k < kWalkPer; ++k) {
+        const bool in = b1 + 32 * k <= last;
+        e[k] = in ? __ldg(ep - 32 * k) : none;
+        u[k] = in ? __ldg(up + 32 * k) : 0.f;
+      }
+      int mine = 1 << 30;
+#pragma unroll
+      for (int k = kWalkPer - 1; k >= 0; --k)
+        if (e[k] + u[k] == target) mine = b1 + 32 * k;
+      found = __reduce_min_sync(0xffffffffu, mine);
+      if (found < 1 << 30) break;
+    }
+    // a match exists for finite curves; without one, as many tokens as there are
+    const int b = found < (1 << 30) ? found : min(x, a.n);
+    if (lane == 0) {
+      *out_b = b;
+      *out_o = rows + x;  // the rows up to and with head h: x tokens and the windows
+      at_s = (unsigned long long)(h - 1) << 32 | (uint32_t)(x - b);
+    }
+    x -= b;
+    target = __ldg(prev + x);
+    --out_b, --out_o, rows -= w;
+    prev -= h > 1 ? a.stride : 0, U -= a.P;
+    row = old, old = older;
+  }
+  // the first head: what is left
+  if (lane == 0) {
+    const float u = row.z <= x && x <= row.w ? __ldg(U + x) : none;
+    *out_b = u == target ? x : min(x, a.n);
+    *out_o = rows + x;
+  }
+}
+
 size_t align256x(size_t x) { return (x + 255) & ~(size_t)255; }
 // floats of one row f_h: rows start on 256-byte boundaries
 size_t dp_stride(int64_t budget) { return align256x(((size_t)budget + 1) * sizeof(float)) / sizeof(float); }
@@ -772,10 +1142,11 @@ cudaError_t launch_exact_allocate(const Dims& dm, const float* curves, const int
   c.P = dm.P, c.N = dm.N, c.n = dm.n;
   dp_runs_kernel<<<(unsigned)dm.N, kDpURuns, 0, lc.st>>>(curves, u_runs, a.words, kDpWords, dm.n, dm.P);
   lc.mark("dp_runs");
-  // the greedy solutions of all sequences; each is read before the walk overwrites it.  They cost 40 to 100 us and shorten a
-  // row by 1 us or more: 16 heads x 584 tokens 98 us with them and 83 without, 32 x 284 138 and 128, 64 x 134 211 and 207,
-  // 128 x 114 363 and 384, 256 x 3968 1.0 and 3.4 ms.
-  const bool greedy = dm.N >= 40 && dm.N * (int64_t)(dm.n / kDpX + 2) > 256 && dm.N <= kGreedyMaxHeads;
+  // the greedy solutions of all sequences; each is read before the walk overwrites it.  They and what is made of them cost 30 to
+  // 90 us and shorten a row by up to 5 us: 16 heads x 968 tokens 92 us with them and 67 without, x 1968 100 and 90, x 3968 121
+  // and 170; 32 x 568 117 and 110, x 968 127 both, x 3968 166 and 295; 48 x 268 133 and 130, x 468 137 and 155; 128 x 68 237 and
+  // 247.  (From 16 heads on also because kDpSlopes sums find room in what N heads have.)
+  const bool greedy = dm.N >= kDpSlopes && (int64_t)dm.N * dm.N * dm.n >= 600000 && dm.N <= kGreedyMaxHeads;
   if (greedy) {
     if ((e = launch_hull(curves, c.lists, dm.N, dm.P, lc)) != cudaSuccess) return e;
     if ((e = launch_greedy(dm, c.lists, budgets_host, budgets, offsets, 1, false, lc)) != cudaSuccess) return e;
@@ -784,14 +1155,15 @@ cudaError_t launch_exact_allocate(const Dims& dm, const float* curves, const int
   for (int q = 0; q < dm.S; ++q) {
     c.B = (int)budgets_host[q];  // below 2^31, as the packed rows
     c.budgets = budgets + (size_t)q * dm.N;
+    a.stride = (long long)dp_stride(c.B);
+    c.f = a.f, c.stride = a.stride;
     if (greedy) {
       dp_reduced_kernel<<<(unsigned)dm.N, kDpCoreThreads, 0, lc.st>>>(c);
       lc.mark("dp_reduced");
       dp_ranges_kernel<<<(unsigned)dm.N, kDpCoreThreads, 0, lc.st>>>(c);
       lc.mark("dp_ranges");
     }
-    a.stride = (long long)dp_stride(c.B);
-    dp_clear_kernel<<<(unsigned)dm.N, 256, 0, lc.st>>>(a, c.rows, greedy ? -1 : c.B);
+    dp_clear_kernel<<<(unsigned)dm.N, 256, 0, lc.st>>>(a, c, c.rows, greedy ? -1 : c.B);
     lc.mark("dp_clear");
     void* params[] = {(void*)&a};
     // cooperative launch: CTAs wait for one another, so all must be resident
@@ -799,7 +1171,9 @@ cudaError_t launch_exact_allocate(const Dims& dm, const float* curves, const int
     e = cudaLaunchCooperativeKernel((const void*)dp_rows_kernel, dim3((unsigned)ctas), dim3(kDpThreads), params, smem, lc.st);
     if (e != cudaSuccess) return e;
     lc.mark("dp_rows");
-    dp_backtrack_kernel<<<1, kDpBackThreads, 0, lc.st>>>(a, c.B, dm.w, row_base, q, budgets, offsets, values);
+    // (tokens left out: mostly a few hundred a head are left)
+    if (greedy) dp_walk_kernel<<<1, 32 * kWalkWarps, 0, lc.st>>>(a, c.B, dm.w, row_base, q, budgets, offsets, values);
+    else dp_backtrack_kernel<<<1, kDpBackThreads, 0, lc.st>>>(a, c.B, dm.w, row_base, q, budgets, offsets, values);
     lc.mark("dp_backtrack");
     row_base += c.B + (long long)dm.N * dm.w;
   }

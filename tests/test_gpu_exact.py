@@ -198,6 +198,25 @@ def test_same_solution_as_the_full_recursion(kind, N, T, w, Bs, reduced):
         np.testing.assert_array_equal(off, np.concatenate([[0], np.cumsum(b.reshape(-1) + w)]))
 
 
+@pytest.mark.parametrize("kind", ["utility", "rough", "ties", "nan"])
+@pytest.mark.parametrize("N,T,w,Bs", [
+    (16, 2400, 32, [16 * 2368 // 5]),                  # fewest heads; rows of more blocks than a narrow step has, between narrow ones
+    (33, 600, 24, [33 * 576 // 3, 33 * 576 - 5, 70]),  # an odd number of heads: the last one has a step of its own
+    (150, 100, 36, [150 * 64 // 2, 1]),                # bands of few budgets, tokens up to a block's edge
+])
+def test_bands_and_narrow_steps(kind, N, T, w, Bs):
+    """To the bit, where budgets are left out by the bounds at neighbouring slopes and narrow rows are made two at a time."""
+    n, U = T - w, _curves(kind, N, T)
+    b, off, val = gpu_exact(N, T, w, U, Bs)
+    assert lukv.lukv_last_launch_count() > 1 + 3 * len(Bs)  # the greedy solution came first
+    for q, B in enumerate(Bs):
+        with np.errstate(invalid="ignore"):
+            ref, best = _recursion(U, B, n)
+        assert np.float32(val[q]) == best
+        if best > -np.inf:
+            assert list(b[q]) == ref
+
+
 @pytest.mark.parametrize("seed", [3, 10, 17])
 def test_values_that_are_no_numbers_bound_nothing(seed):
     """Where some values are no numbers the greedy solution need not have the sum of the budget (seed 10: 12189 instead of
