@@ -100,22 +100,26 @@ __global__ void __launch_bounds__(kCurveThreads) build_curves_kernel(const float
 constexpr int kSortMaxN = 16384;   // positions (rounded up to a power of two) the bucket kernel takes
 constexpr int kBucketLimit = 64;   // entries of one bucket up to which ranking inside it beats sorting
 
+// Where a bucket's word lies: threads that read 2 EPT consecutive ones, 16 bytes at a time, hit all banks.
+__device__ __forceinline__ uint32_t bucket_place(uint32_t b) { return b ^ ((b >> 5 & 7) << 2); }
+
 // npow2 / EPT threads; a thread owns EPT positions (tid + t * threads) while ranking and EPT consecutive ranks while
-// summing.  A bucket is a stretch of 2^sh keys, at most 4 npow2 buckets cover the range of the head's keys; float keys are
+// summing.  A bucket is a stretch of 2^sh keys, at most 2 npow2 buckets cover the range of the head's keys; float keys are
 // logarithmic, which spreads scores over orders of magnitude evenly: the fullest buckets of a log-normal distribution hold
 // some five positions.  Inside a bucket the lower sh bits of the key and the inverted position, together at most 32 bits,
 // decide the order in one comparison.  Should a bucket hold more than kBucketLimit entries (long runs of equal scores), the
 // CTA sorts 64-bit keys instead (bitonic).
-// Bound by shared-memory round trips (63 % of the issue slots are used).  30 queries x 256 heads x 3968 positions: 1.94 ms for the bitonic
-// sort of every head with sums by one warp, 0.29 ms now.
+// Bound by shared-memory wavefronts (the random accesses to buckets and ranks) and issue slots.  30 queries x 256 heads x 3968
+// positions: 1.94 ms for the bitonic sort of every head with sums by one warp; 285 us with four 16-bit buckets a position, whose
+// reading by threads hit four times the same bank and took half the instructions, and all of a thread's positions compared as
+// far as the fullest bucket of all; 221 so.  2560 heads of 2084 positions 84 and 57 us, 512 of 8968 119 and 62.
 template <int EPT>
 __global__ void __launch_bounds__(EPT == 8 ? 512 : 1024, EPT == 8 ? 3 : 1)
     build_curves_bucket_kernel(const float* __restrict__ scores, const float* __restrict__ importance,
                                float* __restrict__ curves, int n, int npow2, int P, int seg, int n_sink) {
   extern __shared__ __align__(16) unsigned char curve_smem[];
   uint32_t* local_key = reinterpret_cast<uint32_t*>(curve_smem);                  // [npow2], bucket by bucket
-  unsigned short* bins = reinterpret_cast<unsigned short*>(local_key + npow2);   // [4 npow2 + 1], two to a word
-  uint32_t* words = reinterpret_cast<uint32_t*>(bins);
+  uint32_t* words = local_key + npow2;                                           // [2 npow2], a bucket each, see bucket_place
   unsigned long long* comp = reinterpret_cast<unsigned long long*>(curve_smem);  // [npow2], when sorting
   float* sorted = reinterpret_cast<float*>(curve_smem);                           // [npow2], once the ranks are known
   __shared__ uint32_t red[2][32];
@@ -137,7 +141,8 @@ __global__ void __launch_bounds__(EPT == 8 ? 512 : 1024, EPT == 8 ? 3 : 1)
 #pragma unroll
     for (int t = 0; t < EPT; ++t) key[t] = curve_key(x[t], tid + t * nthr, n_sink);
   }
-  for (int i = tid; i < 2 * npow2; i += nthr) words[i] = 0u;
+#pragma unroll
+  for (int i = 0; i < EPT / 2; ++i) reinterpret_cast<uint4*>(words)[tid + i * nthr] = make_uint4(0u, 0u, 0u, 0u);
   uint32_t lo = 0xFFFFFFFFu, hi = 0u;  // range of the scored positions' keys
 #pragma unroll
   for (int t = 0; t < EPT; ++t) {
@@ -157,10 +162,10 @@ __global__ void __launch_bounds__(EPT == 8 ? 512 : 1024, EPT == 8 ? 3 : 1)
   lo = __reduce_min_sync(0xffffffffu, lane < warps ? red[0][lane] : 0xFFFFFFFFu);
   hi = __reduce_max_sync(0xffffffffu, lane < warps ? red[1][lane] : 0u);
   const int pos_bits = 31 - __clz(npow2);
-  const int sh = max(0, 32 - __clz(hi > lo ? hi - lo : 0u) - pos_bits - 2);  // (hi - lo) >> sh is below 4 npow2
+  const int sh = max(0, 32 - __clz(hi > lo ? hi - lo : 0u) - pos_bits - 1);  // (hi - lo) >> sh is below 2 npow2
   const uint32_t top = hi > lo ? (hi - lo) >> sh : 0u, low_mask = (1u << sh) - 1u;
   uint32_t mine[EPT];
-  uint32_t where[EPT];  // bucket << 16 | slot in it; bucket 0 holds the largest keys
+  uint32_t where[EPT];  // place of the bucket << 16 | slot in it; bucket 0 holds the largest keys
 #pragma unroll
   for (int t = 0; t < EPT; ++t) {
     const int j = tid + t * nthr;
@@ -168,25 +173,20 @@ __global__ void __launch_bounds__(EPT == 8 ? 512 : 1024, EPT == 8 ? 3 : 1)
     if (j < n) {
       const bool sink = j < n_sink;  // before everything else: they have the lowest positions
       const uint32_t off = key[t] - lo;
-      const uint32_t b = sink ? 0u : top - (off >> sh), half = 16 * (b & 1);
+      const uint32_t place = bucket_place(sink ? 0u : top - (off >> sh));
       mine[t] = ((sink ? low_mask : off & low_mask) << pos_bits) | (uint32_t)(npow2 - 1 - j);
-      where[t] = (b << 16) | ((atomicAdd(words + (b >> 1), 1u << half) >> half) & 0xFFFFu);
+      where[t] = (place << 16) | atomicAdd(words + place, 1u);
     }
   }
   __syncthreads();
   // exclusive offsets of the buckets; the fullest one
-  uint4* own = reinterpret_cast<uint4*>(words + tid * 2 * EPT);  // 4 EPT bins per thread
-  int local = 0, most = 0;
+  auto own = [&](int i) { return reinterpret_cast<uint4*>(words + bucket_place((uint32_t)(tid * 2 * EPT + 4 * i))); };
+  int local = 0, most = 0;  // a thread has 2 EPT buckets
 #pragma unroll
   for (int i = 0; i < EPT / 2; ++i) {
-    const uint4 c = own[i];
-    const uint32_t w4[4] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int lo16 = (int)(w4[k] & 0xFFFFu), hi16 = (int)(w4[k] >> 16);
-      local += lo16 + hi16;
-      most = max(most, max(lo16, hi16));
-    }
+    const uint4 c = *own(i);
+    local += (int)((c.x + c.y) + (c.z + c.w));
+    most = max(most, (int)max(max(c.x, c.y), max(c.z, c.w)));
   }
   int incl = local;
 #pragma unroll
@@ -200,49 +200,47 @@ __global__ void __launch_bounds__(EPT == 8 ? 512 : 1024, EPT == 8 ? 3 : 1)
   __syncthreads();
   int run = __reduce_add_sync(0xffffffffu, lane < wv ? scan[lane] : 0) + incl - local;
   most = __reduce_max_sync(0xffffffffu, lane < warps ? most_s[lane] : 0);
+  // a bucket's word: where its entries start << 16 | their number
+  uint32_t at = (uint32_t)run;
 #pragma unroll
   for (int i = 0; i < EPT / 2; ++i) {
-    const uint4 c = own[i];
-    uint32_t w4[4] = {c.x, c.y, c.z, c.w};
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int lo16 = (int)(w4[k] & 0xFFFFu), hi16 = (int)(w4[k] >> 16);
-      w4[k] = (uint32_t)run | ((uint32_t)(run + lo16) << 16);
-      run += lo16 + hi16;
-    }
-    own[i] = make_uint4(w4[0], w4[1], w4[2], w4[3]);
+    const uint4 c = *own(i);
+    const uint32_t a1 = at + c.x, a2 = a1 + c.y, a3 = a2 + c.z;
+    *own(i) = make_uint4(at << 16 | c.x, a1 << 16 | c.y, a2 << 16 | c.z, a3 << 16 | c.w);
+    at = a3 + c.w;
   }
-  if (tid == nthr - 1) bins[4 * npow2] = (unsigned short)n;
   __syncthreads();
 
   int rank[EPT];
   if (most <= kBucketLimit) {
-    int left[EPT], longest = 0;
+#pragma unroll
+    for (int t = 0; t < EPT; ++t)
+      if (tid + t * nthr < n) {
+        const uint32_t word = words[where[t] >> 16];
+        local_key[(word >> 16) + (where[t] & 0xFFFFu)] = mine[t];
+        where[t] = word;
+      }
+    __syncthreads();
+    // Most buckets hold one entry: position by position, as far as the fullest of the warp's 32 buckets.
 #pragma unroll
     for (int t = 0; t < EPT; ++t) {
-      rank[t] = left[t] = 0;
-      if (tid + t * nthr < n) {
-        const uint32_t b = where[t] >> 16;
-        rank[t] = bins[b];
-        left[t] = bins[b + 1] - rank[t];
-        local_key[rank[t] + (where[t] & 0xFFFF)] = mine[t];
-        longest = max(longest, left[t]);
-      }
-      where[t] = rank[t];  // where the bucket's entries start
-    }
-    __syncthreads();
-    longest = __reduce_max_sync(0xffffffffu, longest);
+      const int left = (int)(where[t] & 0xFFFFu), longest = __reduce_max_sync(0xffffffffu, left);
+      const uint32_t* entries = local_key + (where[t] >> 16);
+      rank[t] = (int)(where[t] >> 16);
+      if (longest > 1) {
 #pragma unroll 1
-    for (int x = 0; x < longest; ++x) {
-#pragma unroll
-      for (int t = 0; t < EPT; ++t)
-        if (x < left[t]) rank[t] += local_key[where[t] + x] > mine[t];
+        for (int x = 0; x < longest; x += 2) {
+          if (x < left) rank[t] += entries[x] > mine[t];
+          if (x + 1 < left) rank[t] += entries[x + 1] > mine[t];
+        }
+      }
     }
   } else {
 #pragma unroll
     for (int t = 0; t < EPT; ++t) {
       const int j = tid + t * nthr;
-      comp[j] = j < n ? ((unsigned long long)key[t] << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)j) : 0ull;
+      comp[j] = j < n ? ((unsigned long long)curve_key(__ldg(sc + j), j, n_sink) << 32) | (unsigned long long)(0xFFFFFFFFu - (uint32_t)j)
+                      : 0ull;
     }
     __syncthreads();
     const int pairs = npow2 >> 1;
@@ -311,10 +309,7 @@ __global__ void __launch_bounds__(EPT == 8 ? 512 : 1024, EPT == 8 ? 3 : 1)
                           __double2float_rn(__dadd_rn(before, acc[4 * q + 2])),
                           __double2float_rn(__dadd_rn(before, acc[4 * q + 3])));
   __syncthreads();
-  for (int k = tid; k < P; k += nthr) {
-    const long long upto = (long long)k * seg;
-    out[k] = k == 0 ? 0.f : sorted[(int)(upto < n ? upto : n) - 1];
-  }
+  for (int k = tid; k < P; k += nthr) out[k] = k == 0 ? 0.f : sorted[min(k * seg, n) - 1];
 }
 
 int curve_pow2(int n) {
