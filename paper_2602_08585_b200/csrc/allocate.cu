@@ -296,18 +296,18 @@ __device__ __noinline__ int hull_squeeze(const float* __restrict__ U, int P, int
 
 // One warp per curve.  A point on or below the chord of two other points is no vertex of the majorant, whichever points
 // they are, so a pass may test all points against their current neighbours at once; a polygon without such a point is the
-// majorant.  The first pass reads the curve once, into registers, and drops what lies clearly below the chord of the points
-// 1, 2, 4, 8 or 16 places to either side (4001 points: about 800 stay); the survivors (value and index) are compacted in
+// majorant.  The first pass reads the curve once and drops what lies clearly below the chord of the points
+// 1, 2, 4, 8 or 32 places to either side (4001 points: about 700 stay); the survivors (value and index) are compacted in
 // shared memory and tested against their neighbours, exactly, until none is dropped (9 passes over 1900 points in all, 53
-// stay).  Where there is no room for 256 points' survivors, those before them go through a pass of their own (hull_squeeze); a
+// stay).  Where there is no room for 128 points' survivors, those before them go through a pass of their own (hull_squeeze); a
 // curve for which that is not enough, or that needs more than kHullPasses, is left to hull_dense_kernel (count -1).  Blocks
 // beyond the last positive slope are one block of gain 0.
 // Bound by the latency of a warp's own instructions at 27 warps per SM (7300 bytes of shared memory each; the 52 curves of an SM
 // are two rounds).  7680 curves of 4001 points: 3.07 ms as one serial stack walk per curve, 0.31 ms as a walk from
 // vertex to vertex over chunk maxima, 0.22 ms with neighbours alone in the first pass, 0.157 ms with room
-// for two fifths of the points (21 warps per SM, three rounds); the profile build 243 us with that and a dense-hull CTA per
-// curve, 227 now.  Smooth curves with 2 % noise in the increments (0.29 of the points survive) 484 us, 502 with room for two
-// fifths, 966 if hull_dense_kernel takes them; without noise (0.65 survive) 1874, 1886 and 2123.
+// for two fifths of the points (21 warps per SM, three rounds), 0.140 ms with a point a lane and five exchanges of 32 (chords of 16
+// places instead of 32), 0.119 ms now; the profile build 223 and 196 us.  Smooth curves with 2 % noise in the increments (0.29 of
+// the points survive) 485 and 475 us a build; without noise (0.65 survive, hull_dense_kernel takes them) 1880 and 1505.
 __global__ void __launch_bounds__(32, 27) hull_prune_kernel(const float* __restrict__ curves, HullLists lists, int P, int cap) {
   extern __shared__ float hull_smem[];
   const int hid = blockIdx.x, lane = threadIdx.x;
@@ -316,53 +316,82 @@ __global__ void __launch_bounds__(32, 27) hull_prune_kernel(const float* __restr
   unsigned short* is = reinterpret_cast<unsigned short*>(hull_smem + cap);  // [cap]
   const uint32_t lt_mask = (1u << lane) - 1u;
   pdl_launch_dependents();
-  constexpr int kAhead = 8;  // vectors of 32 points at a time; the next ones are on their way
+  // Four consecutive points a lane, in aligned 16-byte units (the curve starts `phase` floats into the first one): the points 4, 8
+  // and 32 places to either side are whole lanes away, those 1 and 2 places away mostly in the lane itself.  (Loading them instead
+  // of exchanging them: 167 us, the shared memory leaves L1 too little room; tests of the ends in every turn: 181, all of them ALU
+  // instructions.)
+  const int phase = (int)(reinterpret_cast<uintptr_t>(U) >> 2 & 3), last = (P + phase - 1) >> 2;
+  const float4* units = reinterpret_cast<const float4*>(U - phase);
+  auto load = [&](int q, float (&x)[4]) {
+    const float4 v = __ldg(units + min(max(q, 0), last));
+    x[0] = v.x, x[1] = v.y, x[2] = v.z, x[3] = v.w;
+  };
   int cnt = 0;
-  float cur[kAhead], nxt[kAhead], prev = 0.f;
-#pragma unroll
-  for (int t = 0; t < kAhead; ++t) nxt[t] = __ldg(U + min(32 * t + lane, P - 1));
+  float prev[4] = {}, u[4], nxt[4], ahead[4];
+  load(lane, u), load(lane + 32, nxt);
 #pragma unroll 1
-  for (int base = 0; base < P; base += 32 * kAhead) {
-    const int before = cnt;
+  for (int base = 0; base <= last; base += 32) {  // 32 units
+    const int before = cnt, q = base + lane, j0 = 4 * q - phase;
+    load(q + 64, ahead);
+    float l1[4], r1[4], l2[4], r2[4], l8[4], r8[4];
+    auto exchange = [&](int lanes, float (&l)[4], float (&r)[4]) {  // lanes whose value wraps around stand for the units before, or behind
 #pragma unroll
-    for (int t = 0; t < kAhead; ++t) cur[t] = nxt[t];
-#pragma unroll
-    for (int t = 0; t < kAhead; ++t) nxt[t] = __ldg(U + min(base + 32 * (kAhead + t) + lane, P - 1));
-#pragma unroll
-    for (int t = 0; t < kAhead; ++t) {
-      const int j = base + 32 * t + lane;
-      const float u = cur[t], up = t > 0 ? cur[t > 0 ? t - 1 : 0] : prev, un = t + 1 < kAhead ? cur[t + 1 < kAhead ? t + 1 : 0] : nxt[0];
-      // below the chord by more than the roundings of the two sides (2.4e-7 |u| where they are close)
-      const float lim = fmaf(5e-7f, fabsf(u), 2.f * u), small = 0.25f * fabsf(u);
-      bool below = false;
-      const bool edge = base + 32 * t < 32 || base + 32 * t + 48 > P;
-#pragma unroll
-      for (int k = 1; k <= 16; k <<= 1) {
-        // lanes whose value wraps around stand for the vector before, or behind
-        const float l = __shfl_sync(0xffffffffu, lane >= 32 - k ? up : u, (lane + 32 - k) & 31);
-        const float r = __shfl_sync(0xffffffffu, lane < k ? un : u, (lane + k) & 31);
-        bool b;
-        if (k <= 2) {
-          // rises of at most a quarter of u are exact in fp32 (late on a curve they are a few units in the last place)
-          const float d1 = u - l, d2 = r - u;
-          b = (d1 <= d2) & (fmaxf(fabsf(d1), fabsf(d2)) <= small);
-        } else {
-          b = l + r > lim;
-        }
-        if (edge) b = b & (j >= k) & (j + k < P);
-        below |= b;
+      for (int c = 0; c < 4; ++c) {
+        l[c] = __shfl_sync(0xffffffffu, lane >= 32 - lanes ? prev[c] : u[c], (lane + 32 - lanes) & 31);
+        r[c] = __shfl_sync(0xffffffffu, lane < lanes ? nxt[c] : u[c], (lane + lanes) & 31);
       }
-      const bool keep = (j < P) & !below;
-      const uint32_t kept = __ballot_sync(0xffffffffu, keep);
-      const int at = cnt + __popc(kept & lt_mask);
-      if (keep && at < cap) {
-        us[at] = u;
-        is[at] = (unsigned short)j;
+    };
+    exchange(1, l1, r1), exchange(2, l2, r2), exchange(8, l8, r8);
+    const float x[8] = {l1[2], l1[3], u[0], u[1], u[2], u[3], r1[0], r1[1]};
+    // rises of at most a quarter of u are exact in fp32 (late on a curve they are a few units in the last place); the other chords
+    // must pass by more than the roundings of the two sides (2.4e-7 |u| where they are close)
+    bool keep[4];
+    float d1[5], d2[6];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) d1[c] = x[c + 2] - x[c + 1];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) d2[c] = x[c + 2] - x[c];
+    if (base > 0 && base + 40 < last) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float lim = fmaf(5e-7f, fabsf(u[c]), 2.f * u[c]), small = 0.25f * fabsf(u[c]);
+        const float far = fmaxf(fmaxf(l1[c] + r1[c], l2[c] + r2[c]), l8[c] + r8[c]);
+        bool below = far > lim;
+        if (d1[c] <= d1[c + 1] && fmaxf(fabsf(d1[c]), fabsf(d1[c + 1])) <= small) below = true;
+        if (d2[c] <= d2[c + 2] && fmaxf(fabsf(d2[c]), fabsf(d2[c + 2])) <= small) below = true;
+        keep[c] = !below;
       }
+    } else {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float lim = fmaf(5e-7f, fabsf(u[c]), 2.f * u[c]), small = 0.25f * fabsf(u[c]);
+        const int j = j0 + c, room = min(j, P - 1 - j);  // points to the nearer end
+        bool below = room >= 4 && l1[c] + r1[c] > lim;
+        below = below || (room >= 8 && l2[c] + r2[c] > lim) || (room >= 32 && l8[c] + r8[c] > lim);
+        below = below || (room >= 1 && d1[c] <= d1[c + 1] && fmaxf(fabsf(d1[c]), fabsf(d1[c + 1])) <= small);
+        below = below || (room >= 2 && d2[c] <= d2[c + 2] && fmaxf(fabsf(d2[c]), fabsf(d2[c + 2])) <= small);
+        keep[c] = room >= 0 && !below;
+      }
+    }
+    int at = cnt;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const uint32_t kept = __ballot_sync(0xffffffffu, keep[c]);
+      at += __popc(kept & lt_mask);
       cnt += __popc(kept);
     }
-    prev = cur[kAhead - 1];
-    if (cnt > cap && before <= cap) cnt = hull_squeeze(U, P, base, 32 * kAhead, us, is, before, cap, lane);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      if (keep[c] && at < cap) {
+        us[at] = u[c];
+        is[at] = (unsigned short)(j0 + c);
+      }
+      at += keep[c];
+    }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) prev[c] = u[c], u[c] = nxt[c], nxt[c] = ahead[c];
+    // (not in the first turn: there is room for all of its points)
+    if (cnt > cap && before <= cap) cnt = hull_squeeze(U, P, 4 * base - phase, 128, us, is, before, cap, lane);
   }
   int total = -1;
   if (cnt <= cap && (cnt = hull_passes(us, is, cnt, kHullPasses, lane)) > 0)
@@ -520,7 +549,7 @@ __device__ __forceinline__ void hull_dense_curve(const float* __restrict__ curve
 __global__ void __launch_bounds__(32) hull_dense_kernel(const float* __restrict__ curves, HullLists lists, int P, int n_curves) {
   extern __shared__ float hull_smem[];
   const int lane = threadIdx.x, step = gridDim.x;
-  pdl_launch_dependents();
+  // (the next launch comes when this one ends: the greedy kernel's CTAs would wait in the shared memory that the CTAs here need)
   pdl_wait();
   for (long long base = blockIdx.x; base < n_curves; base += 32LL * step) {
     const long long mine = base + (long long)lane * step;
@@ -1146,8 +1175,9 @@ cudaError_t launch_hull(const float* curves, const HullLists& out, int64_t n_cur
   const int cap = hull_prune_cap(P);
   hull_prune_kernel<<<grid, 32, (size_t)cap * 6, lc.st>>>(curves, out, P, cap);
   lc.mark("hull_prune");
-  // as many warps as the chip holds at 25 KB each: all curves may be left to it, most often none is
-  const unsigned dense = std::min(grid, 9u * 148u);
+  // as many warps as the chip holds at 25 KB each: all curves may be left to it, most often none is.  (7680 smooth curves: 2180 us a
+  // profile build with nine to an SM, which do not fit, and the next launch beside them, 1960 with eight, 1505 with eight alone.)
+  const unsigned dense = std::min(grid, 8u * 148u);
   const cudaError_t e = launch_pdl(hull_dense_kernel, dim3(dense), dim3(32), hull_dense_smem_bytes(P), lc.st, true, curves,
                                    out, P, (int)n_curves);
   if (e != cudaSuccess) return e;

@@ -157,3 +157,25 @@ def test_curves_far_from_one(oracle, N, P, kind, exponent):
     b_ref, o_ref = oracle.allocate(U, T, w, Bs)
     np.testing.assert_array_equal(b, b_ref)
     np.testing.assert_array_equal(o, o_ref)
+
+
+@pytest.mark.parametrize("kind", ["rough", "concave", "mixed"])
+@pytest.mark.parametrize("P,shift", [(545, 1), (607, 2), (640, 3), (641, 0), (673, 1), (801, 3), (1281, 2), (3997, 1)])
+def test_long_curves_at_any_alignment(oracle, kind, P, shift):
+    """The first pass over a long curve reads aligned groups of four points, 128 a turn: curves that start anywhere in a group
+    and end anywhere in a turn, of which some leave all their points."""
+    rng = np.random.default_rng(P)
+    N, w = 6, 2
+    T = P - 1
+    U = _curves(rng, N, P, kind)
+    Bs = [0, N * (T - w) // 3, N * (T - w) - 1]
+    p = lukv.make_params(len(Bs), 1, N, 1, 64, T, w, 1, "bf16", P)
+    store = torch.full((N * P + 8,), float("nan"), device="cuda")
+    curves = store[shift:shift + N * P].view(N, P)
+    curves.copy_(torch.from_numpy(U))
+    b = torch.empty((len(Bs), N), dtype=torch.int32, device="cuda")
+    o = torch.empty(len(Bs) * N + 1, dtype=torch.int32, device="cuda")
+    lukv.lukv_allocate(p, curves, Bs, b, o, lukv.alloc_workspace(p))
+    b_ref, o_ref = oracle.allocate(U, T, w, Bs)
+    np.testing.assert_array_equal(b.cpu().numpy(), b_ref)
+    np.testing.assert_array_equal(o.cpu().numpy(), o_ref)
