@@ -25,6 +25,8 @@
 // Every wait is bounded; a wait that runs out raises the CTA's abort flag and stores
 // LUKV_ERR_TIMEOUT to the status word; the CTA then skips the remaining work and tears down
 // normally.
+#include <algorithm>
+
 #include "score_chunks.cuh"
 
 namespace lukv {
@@ -682,9 +684,12 @@ __global__ void __launch_bounds__(Plan<MT, NQ, NH>::kThreads, 1)
 
 // ---- host side --------------------------------------------------------------------------------
 
-// Tiles, and `item` more per item, of the CTA with the most of them, when the items of `groups` groups of heads (heads each, T[g]
-// keys long, at most `it` tiles an item) are dealt to `ctas` CTAs in turn.
-double deal_cost(const int32_t* T, int groups, int heads, int it, int ctas, double item) {
+// Clocks of the CTA with the most to do when the items of `groups` groups of heads (heads each, T[g] keys long, at most `it` tiles an
+// item) are dealt to `ctas` CTAs in turn: `tile` a tile and kItem an item, and what pass 2 waits for the row log-sum-exps of its head.
+// Those come kFold clocks after the head's last partial, and kFoldItem for each of the partials that they are put together from; pass 1
+// of the next item (`sweep` clocks a tile) runs meanwhile.
+double deal_cost(const int32_t* T, int groups, int heads, int it, int ctas, double tile, double sweep) {
+  constexpr double kItem = 1300.0, kFold = 8000.0, kFoldItem = 130.0;
   constexpr int kMaxCtas = 256;
   double step[kMaxCtas + 1] = {};  // what a group's last, incomplete round adds: differences from CTA to CTA
   if (ctas > kMaxCtas) ctas = kMaxCtas;
@@ -692,7 +697,8 @@ double deal_cost(const int32_t* T, int groups, int heads, int it, int ctas, doub
   int first = 0;  // the CTA that gets the group's first item
   for (int g = 0; g < groups; ++g) {
     const long long tiles = (T[g] + kTileKeys - 1) / kTileKeys, per_head = (tiles + it - 1) / it, items = heads * per_head;
-    const double time = (double)tiles / (double)per_head + item;
+    const double own = (double)tiles / (double)per_head, fold = kFold + kFoldItem * (double)per_head;
+    const double time = own * tile + kItem + std::max(0.0, fold - own * sweep);
     const int rest = (int)(items % ctas);
     base += time * (double)(items / ctas);
     if (rest) {
@@ -727,24 +733,27 @@ cudaError_t launch_fused(const CUtensorMap& qm, const CUtensorMap& km, FusedArgs
   // A CTA runs pass 1 of later items before pass 2 of the current one, so a head's items must
   // not outnumber the CTAs (else a CTA would wait for partials that it is due to produce itself).
   if (args.adapt_items) {
-    // Larger work items mean fewer job changes and fewer partials to fold per head, but coarser dealing.  The time is that of
-    // the CTA with the most to do: its tiles and about half a row block's time per item (128 heads x 157 tiles, head size 64: 223 us
-    // of scorer in items of 20 tiles, 231 in 16, 237 in 8; two row blocks 2048 x 128 tiles 5.84 ms in 64 and 5.94 in 8).
-    // Large items do not leave pass 2 its key tiles in L2.  With one row block of 128 channels reading them from HBM again is a
-    // bound of its own (7 TB/s at the speed of the arithmetic): items of up to nine tiles, whose two sweeps' keys fit L2, are
-    // a tenth faster per tile (256 heads x 256 tiles: 1163 us a call in 64 tiles, 1172 in 32, 1176 in 12, 1143 in 10, 1129 in 8
-    // and 9).  Any number of tiles up to 64 is tried: 8 heads x 64 tiles 33 us a call with 4, 37 with 6 or 8.
-    constexpr double kItem = 0.5 / MT, kReread = 1.1;
-    constexpr long long kL2Tiles = (90ll << 20) / (2 * kHalfBytes);
+    // Larger work items mean fewer job changes and fewer partials to fold per head, but coarser dealing.  A tile takes the time of
+    // its arithmetic in both sweeps, or of its way out of HBM where that is longer (128 heads x 157 tiles, head size 64: 223 us of
+    // scorer in items of 20 tiles, 231 in 16, 237 in 8; 2048 x 128 tiles of two row blocks 5.84 ms in 64 and 5.94 in 8).  Pass 1
+    // takes a row block's time however few of its rows there are, pass 2 what its columns take.  Large items do not leave pass 2 its
+    // key tiles in L2: items of up to eight tiles do, whose two sweeps' keys fit (256 heads x 256 tiles of 128 rows: 1163 us a call
+    // in 64 tiles, 1172 in 32, 1176 in 12, 1143 in 10, 1129 in 8 and 9; of 64 rows 982 in 64, 980 in 32, 977 in 16, 941 in 9, 926 in 8).  But a head of many items
+    // has its row log-sum-exps late (8 heads x 938 tiles: 187 us a call in 53 tiles, 218 in 9).  Any number of tiles up to 64 is
+    // tried: 8 heads x 64 tiles 33 us a call with 4, 37 with 6 or 8.
+    constexpr double kBlock = 1290.0, kRead = 710.0 * NH;
+    constexpr long long kL2Tiles = (80ll << 20) / (NH * kHalfBytes);
+    const double clocks = kBlock * (MT + args.npad / 128.0);
     long long all_tiles = 0;
     for (int q = 0; q < (RAGGED ? args.n_seq : 1); ++q)
       all_tiles += (long long)(RAGGED ? args.heads_per_seq : args.nheads) * (((RAGGED ? seq_T_host[q] : args.T) + kTileKeys - 1) / kTileKeys);
     int best = args.item_tiles;
     double best_cost = 1e30;
     for (int it = args.item_tiles; it <= 64; ++it) {
-      double cost = RAGGED ? deal_cost(seq_T_host, args.n_seq, args.heads_per_seq, it, sms, kItem)
-                           : deal_cost(&args.T, 1, args.nheads, it, sms, kItem);
-      if (MT == 1 && NH == 2 && all_tiles > kL2Tiles && 2ll * sms * it > kL2Tiles) cost *= kReread;
+      const bool twice = all_tiles > kL2Tiles && 2ll * sms * it > kL2Tiles;  // K comes out of HBM twice
+      const double tile = std::max(clocks, (twice ? 2.0 : 1.0) * kRead);
+      const double cost = RAGGED ? deal_cost(seq_T_host, args.n_seq, args.heads_per_seq, it, sms, tile, kBlock * MT)
+                                 : deal_cost(&args.T, 1, args.nheads, it, sms, tile, kBlock * MT);
       if (cost < best_cost * 0.995) {
         best_cost = cost;
         best = it;
