@@ -790,28 +790,53 @@ __device__ __forceinline__ void greedy_problem(const ListView<STAGED> lists, con
           }
           grp.sync();
           uint2* list = reinterpret_cast<uint2*>(bins);
-          each_block(lists, N, seg, n, floor_tok, from, to, grp, [&](unsigned g, unsigned tokens) {
+          auto add = [&](unsigned g, unsigned tokens) {
             const unsigned x = atomicAdd(&sh.listed, 1u);
             if (x < kGreedyList) list[x] = make_uint2(g, tokens);
-          });
+          };
+          if (lists.at_[N] > 8 * nthr) {
+            // many blocks: a search in every head's list, which is sorted, instead of a look at all of them (256 heads of 53
+            // blocks, 256 threads: 7500 clocks and 900)
+            for (int h = h_begin; h < h_end; ++h) {
+              const int c = lists.blocks(h);
+              int x = 0, r = c;  // first block that is not steeper than the range
+              while (x < r) {
+                const int m = (x + r) >> 1;
+                if (__float_as_uint(lists.gain(h, m)) > to) x = m + 1; else r = m;
+              }
+              for (; x < c; ++x) {
+                const unsigned g = __float_as_uint(lists.gain(h, x));
+                if (g < from) break;
+                add(g, (unsigned)max(0, capsum(lists.start(h, x + 1), seg, n, floor_tok) - capsum(lists.start(h, x), seg, n, floor_tok)));
+              }
+            }
+          } else {
+            each_block(lists, N, seg, n, floor_tok, from, to, grp, add);
+          }
           grp.sync();
           const int m = (int)sh.listed;
           if (m <= kGreedyList) {
             unsigned all = 0;
-            for (int e = tid; e < m; e += nthr) {
-              const unsigned g = list[e].x;
+            for (int e0 = 0; e0 < m; e0 += nthr >> 2) {  // four lanes a block
+              const int e = e0 + (tid >> 2);
+              const uint2 own = e < m ? list[e] : make_uint2(0u, 0u);
               unsigned steeper = 0, same = 0;
 #pragma unroll 4
-              for (int x = 0; x < m; ++x) {
+              for (int x = tid & 3; x < m; x += 4) {
                 const uint2 o = list[x];
-                steeper += o.x > g ? o.y : 0u;
-                same += o.x == g ? o.y : 0u;
+                steeper += o.x > own.x ? o.y : 0u;
+                same += o.x == own.x ? o.y : 0u;
               }
-              if (steeper <= R && R < steeper + same) {  // one gain; every thread that holds it writes the same
-                sh.cut[0] = g;
+#pragma unroll
+              for (int off = 1; off < 4; off <<= 1) {
+                steeper += __shfl_xor_sync(0xffffffffu, steeper, off);
+                same += __shfl_xor_sync(0xffffffffu, same, off);
+              }
+              if (e < m && steeper <= R && R < steeper + same) {  // one gain; every thread that holds it writes the same
+                sh.cut[0] = own.x;
                 sh.cut[1] = R - steeper;
               }
-              all += list[e].y;
+              if ((tid & 3) == 0) all += own.y;
             }
             all = group_sum2(all, 0u, sh.sum[round++ & 1], grp).x;
             grp.sync();
@@ -988,7 +1013,8 @@ inline size_t greedy_smem_bytes(int N, int cap, int groups, bool one) {
 // Bound by latency (a pass over the blocks, a scan, a ranking), hence several groups per CTA where there are that many
 // problems.  65536 segments in 256 heads: 91 us beside the scorer with a search per head for each of the 64 bits of (gain,
 // k, hid) over expanded segments, 34 us with the bits of the gain over block lists, 16 us now; 2970 problems of
-// 256 x 4000 segments 0.6 ms, 0.12 ms, 0.07 ms now that the first split is shared.
+// 256 x 4000 segments 0.6 ms, 0.12 ms, 0.07 ms with the first split shared, 0.056 ms with the cut's blocks searched for and ranked by
+// four lanes each.
 // blockIdx.y selects one of several independent curve sets (the calibration queries of the offline profile, which
 // share the budgets): set i reads the lists of curves i*N .., writes budgets + i*set.budgets and offsets +
 // i*set.offsets.  The hot path launches one set.
