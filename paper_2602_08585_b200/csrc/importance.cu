@@ -8,7 +8,9 @@
 //   value_norm_kernel   || v_j W_O^(g) ||_2 for every (head, g, rankable position)
 //   imp_lse_kernel      row log-sum-exp of every (head, g, step), exp2 domain
 //   imp_kernel          probabilities x value norms, summed over g inside a thread, maximum over the steps
-//   imp_normalize_kernel  one CTA per (sequence, layer): fp64 total in a fixed order, then the division
+//   imp_normalize_kernel  a cluster per (sequence, layer): fp64 total in a fixed order, then the quotients
+#include <cooperative_groups.h>
+
 #include <cstdlib>
 
 #include "simt_tile.cuh"
@@ -227,41 +229,51 @@ __global__ void __launch_bounds__(kSimtThreads) imp_kernel(const TIn* __restrict
   }
 }
 
-// One CTA per (sequence, layer): the layer's H*n values are contiguous.  fp64 sum in a fixed order, then x / total.
-__global__ void __launch_bounds__(1024) imp_normalize_kernel(float* __restrict__ importance, long long count) {
-  __shared__ double part[32];
-  __shared__ double total_s;
-  float* base = importance + (size_t)blockIdx.x * count;
+// One cluster of kNormCtas CTAs per (sequence, layer): the layer's H*n values are contiguous, a CTA has a stretch of them.  fp64 sum
+// in a fixed order, then x / total (times the fp64 reciprocal, rounded once).  Bound by latency: a trip to L2 each for the sum
+// and the products, and the cluster's barrier.  32 layers of 31744 values: 14 us with one CTA each and fp64 divisions, 5 so.
+constexpr int kNormCtas = 8, kNormThreads = 512;
+__global__ void __cluster_dims__(kNormCtas) __launch_bounds__(kNormThreads) imp_normalize_kernel(float* __restrict__ importance,
+                                                                                                   long long count) {
+  __shared__ double part[kNormThreads / 32];
+  __shared__ double sum_s;
+  cooperative_groups::cluster_group cluster = cooperative_groups::this_cluster();
+  const int rank = (int)cluster.block_rank(), tid = threadIdx.x;
+  const long long own = (count + kNormCtas - 1) / kNormCtas, first = own * rank, end = first + own < count ? first + own : count;
+  float* base = importance + (size_t)(blockIdx.x / kNormCtas) * count;
+  constexpr int kKeep = 8;  // values of a thread that stay in registers
+  float keep[kKeep];
   double acc = 0.0;
-  // four loads at a time: the layer's few warps have nothing else to wait behind
-  constexpr int kAhead = 4;
-  for (long long i0 = threadIdx.x; i0 < count; i0 += kAhead * blockDim.x) {
-    float x[kAhead];
 #pragma unroll
-    for (int k = 0; k < kAhead; ++k) x[k] = i0 + k * blockDim.x < count ? base[i0 + k * blockDim.x] : 0.f;
+  for (int k = 0; k < kKeep; ++k) keep[k] = first + tid + k * kNormThreads < end ? base[first + tid + k * kNormThreads] : 0.f;
 #pragma unroll
-    for (int k = 0; k < kAhead; ++k) acc += (double)x[k];
+  for (int k = 0; k < kKeep; ++k) acc += (double)keep[k];
+  for (long long i0 = first + tid + kKeep * kNormThreads; i0 < end; i0 += 4 * kNormThreads) {
+    float x[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) x[k] = i0 + k * kNormThreads < end ? base[i0 + k * kNormThreads] : 0.f;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc += (double)x[k];
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+  if ((tid & 31) == 0) part[tid >> 5] = acc;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     double t = 0.0;
-    for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += part[i];
-    total_s = t;
+    for (int i = 0; i < kNormThreads / 32; ++i) t += part[i];
+    sum_s = t;
   }
-  __syncthreads();
-  const double total = total_s;
+  cluster.sync();
+  double total = 0.0;
+  for (int c = 0; c < kNormCtas; ++c) total += *cluster.map_shared_rank(&sum_s, c);
+  cluster.sync();  // (no CTA exits while another may still read its sum)
   if (total <= 0.0) return;  // (not a number: the whole layer is none)
-  for (long long i0 = threadIdx.x; i0 < count; i0 += kAhead * blockDim.x) {
-    float x[kAhead];
+  const double scale = 1.0 / total;
 #pragma unroll
-    for (int k = 0; k < kAhead; ++k) x[k] = i0 + k * blockDim.x < count ? base[i0 + k * blockDim.x] : 0.f;
-#pragma unroll
-    for (int k = 0; k < kAhead; ++k)
-      if (i0 + k * blockDim.x < count) base[i0 + k * blockDim.x] = (float)((double)x[k] / total);
-  }
+  for (int k = 0; k < kKeep; ++k)
+    if (first + tid + k * kNormThreads < end) base[first + tid + k * kNormThreads] = (float)((double)keep[k] * scale);
+  for (long long i = first + tid + kKeep * kNormThreads; i < end; i += kNormThreads) base[i] = (float)((double)base[i] * scale);
 }
 
 // LUKV_FORCE_SIMT=1 keeps the value norms on the FP32 pipes (for A/B checks; read at every call).
@@ -307,7 +319,7 @@ cudaError_t launch_importance_t(const Dims& dm, ImpDims id, const void* q_dec, c
     lc.mark("importance");
   }
   if (normalize) {
-    imp_normalize_kernel<<<(unsigned)(dm.S * dm.L), 1024, 0, lc.st>>>(importance, (long long)dm.H * dm.n);
+    imp_normalize_kernel<<<(unsigned)(dm.S * dm.L * kNormCtas), kNormThreads, 0, lc.st>>>(importance, (long long)dm.H * dm.n);
     lc.mark("imp_normalize");
   }
   return cudaGetLastError();
