@@ -8,7 +8,7 @@
 //
 // 2.2e11 pairs (x, b) for 256 heads x 3968 tokens at B = 0.3 N n if every one is evaluated.  What is done instead:
 //   - tokens that no optimal solution can contain, and budgets on which none can pass, are left out before (see "which tokens
-//     can matter" below): 1 % of the budgets and 6 % of the tokens are left there;
+//     can matter" below): 1 % of the budgets and 8 % of the tokens are left there;
 //   - of those, a warp owns 64 budgets; where many blocks of 64 values of b are left it skips every one that an upper bound
 //     rules out: for any slope s a pair (y, b) can only matter if (f(y) - s y) + (U(b) - s b) reaches the smallest
 //     f_h(x) - s x found so far, and maxima of f and U over runs of 16 bound the left side; half a block at a time is then
@@ -352,7 +352,7 @@ __device__ __forceinline__ void dp_narrow(const unsigned char* F2, const unsigne
 // value of at least LB less twice the sum of those errors.  With that allowance the tokens [b0, b1] of a head that are
 // left, and the budgets that such tokens add up to, hold every path that the full recursion could return, and the rows
 // restricted to them have the full recursion's values on those paths.  l and LB come from the greedy solution of the
-// relaxed problem, which is close: 240 of 3968 tokens a head are left on utility curves of 256 heads, and 5 % of the budgets, of
+// relaxed problem, which is close: 325 of 3968 tokens a head are left on utility curves of 256 heads, and 7 % of the budgets, of
 // which the bands (dp_band) leave a sixth.
 
 constexpr int kDpCoreThreads = 256;
@@ -591,7 +591,7 @@ __global__ void __launch_bounds__(kDpCoreThreads) dp_ranges_kernel(const DpCore 
 // The budgets of row h on which a solution can pass.  With C(l) the sum of c_j(l) over the heads up to h and S(l) that over the
 // others, a solution that has x tokens up to h is worth at most C(l) + l x + S(l') + l' (B - x) for any two slopes; where that is
 // below the least value that it must have, x does not count.  The heads share the slack here, instead of each having all of it:
-// 2 000 budgets a row are left on average instead of 12 600 (256 heads x 3968 tokens).  Lane k takes slope k against all others.
+// 55 tiles of budgets a row are left on average instead of 333 (256 heads x 3968 tokens).  Lane k takes slope k against all others.
 __device__ __forceinline__ int4 dp_band(const DpCore& a, int h, int4 r) {
   const int lane = threadIdx.x & (kDpSlopes - 1);
   const double l = dp_slope(*a.slope, lane), up_to = reinterpret_cast<const double*>(a.f + (size_t)h * a.stride)[lane];

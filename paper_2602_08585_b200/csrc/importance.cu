@@ -24,27 +24,33 @@ constexpr int kTile = 64;  // rows and keys (or projection columns) per shared-m
 template <int D>
 __device__ __forceinline__ void tile_dots(const float* As, const float* Bs, int rg, int kg, float (&acc)[4][4]) {
   constexpr int kPitch = D + 4;
+  // even and odd channels apart, two products an instruction (8 heads x 2000 keys x 256 rows, fp32: 736 -> 719 us a call; the
+  // scorer's larger register tiles lose by it)
+  uint64_t pair[4][4];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
-    for (int kk = 0; kk < 4; ++kk) acc[a][kk] = 0.f;
+    for (int kk = 0; kk < 4; ++kk) pair[a][kk] = 0ull;
 #pragma unroll 4
   for (int c = 0; c < D; c += 4) {
-    float4 bv[4];
+    ulonglong2 bv[4];
 #pragma unroll
-    for (int kk = 0; kk < 4; ++kk) bv[kk] = *reinterpret_cast<const float4*>(Bs + (kg + 16 * kk) * kPitch + c);
+    for (int kk = 0; kk < 4; ++kk) bv[kk] = *reinterpret_cast<const ulonglong2*>(Bs + (kg + 16 * kk) * kPitch + c);
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
-      const float4 av = *reinterpret_cast<const float4*>(As + (rg + 16 * a) * kPitch + c);
+      const ulonglong2 av = *reinterpret_cast<const ulonglong2*>(As + (rg + 16 * a) * kPitch + c);
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        acc[a][kk] = fmaf(av.x, bv[kk].x, acc[a][kk]);
-        acc[a][kk] = fmaf(av.y, bv[kk].y, acc[a][kk]);
-        acc[a][kk] = fmaf(av.z, bv[kk].z, acc[a][kk]);
-        acc[a][kk] = fmaf(av.w, bv[kk].w, acc[a][kk]);
-      }
+      for (int kk = 0; kk < 4; ++kk) pair[a][kk] = ffma2(av.y, bv[kk].y, ffma2(av.x, bv[kk].x, pair[a][kk]));
     }
   }
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int kk = 0; kk < 4; ++kk) {
+      float even, odd;
+      unpack2(pair[a][kk], even, odd);
+      acc[a][kk] = even + odd;
+    }
 }
 
 struct ImpDims {

@@ -1,6 +1,6 @@
 // Shared-memory tile loader of the FP32-pipe kernels (general-shape scorer, oracle importance).
 #pragma once
-#include "common.cuh"
+#include "tc_ptx.cuh"
 
 namespace lukv {
 namespace {
