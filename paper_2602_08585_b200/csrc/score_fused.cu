@@ -741,10 +741,11 @@ cudaError_t launch_fused(const CUtensorMap& qm, const CUtensorMap& km, FusedArgs
     // scorer in items of 20 tiles, 231 in 16, 237 in 8; 2048 x 128 tiles of two row blocks 5.84 ms in 64 and 5.94 in 8).  Pass 1
     // takes a row block's time however few of its rows there are, pass 2 what its columns take.  Large items do not leave pass 2 its
     // key tiles in L2: items of up to eight tiles do, whose two sweeps' keys fit (256 heads x 256 tiles of 128 rows: 1163 us a call
-    // in 64 tiles, 1172 in 32, 1176 in 12, 1143 in 10, 1129 in 8 and 9; of 64 rows 982 in 64, 980 in 32, 977 in 16, 941 in 9, 926 in 8).  But a head of many items
-    // has its row log-sum-exps late (8 heads x 938 tiles: 187 us a call in 53 tiles, 218 in 9).  Any number of tiles up to 64 is
-    // tried: 8 heads x 64 tiles 33 us a call with 4, 37 with 6 or 8.
-    constexpr double kBlock = 1290.0, kRead = 710.0 * NH;
+    // in 64 tiles, 1172 in 32, 1176 in 12, 1143 in 10, 1129 in 8 and 9; of 64 rows 982 in 64, 980 in 32, 977 in 16, 941 in 9, 926
+    // in 8); some of a cache not much larger than L2 is there in any case (32 heads x 256 tiles 181 us in 8, 174 in 29).  But a head
+    // of many items has its row log-sum-exps late (8 heads x 938 tiles: 187 us a call in 53 tiles, 218 in 9).  Any number of tiles up
+    // to 64 is tried: 8 heads x 64 tiles 33 us a call with 4, 37 with 6 or 8.
+    constexpr double kBlock = 1290.0, kRead = 760.0 * NH;
     constexpr long long kL2Tiles = (80ll << 20) / (NH * kHalfBytes);
     const double clocks = kBlock * (MT + args.npad / 128.0);
     long long all_tiles = 0;
@@ -754,7 +755,7 @@ cudaError_t launch_fused(const CUtensorMap& qm, const CUtensorMap& km, FusedArgs
     double best_cost = 1e30;
     for (int it = args.item_tiles; it <= 64; ++it) {
       const bool twice = all_tiles > kL2Tiles && 2ll * sms * it > kL2Tiles;  // K comes out of HBM twice
-      const double tile = std::max(clocks, (twice ? 2.0 : 1.0) * kRead);
+      const double tile = std::max(clocks, (twice ? 2.0 - (double)kL2Tiles / (double)all_tiles : 1.0) * kRead);
       const double cost = RAGGED ? deal_cost(seq_T_host, args.n_seq, args.heads_per_seq, it, sms, tile, kBlock * MT)
                                  : deal_cost(&args.T, 1, args.nheads, it, sms, tile, kBlock * MT);
       if (cost < best_cost * 0.995) {
