@@ -323,8 +323,13 @@ __global__ void __launch_bounds__(32, 27) hull_prune_kernel(const float* __restr
   const int phase = (int)(reinterpret_cast<uintptr_t>(U) >> 2 & 3), last = (P + phase - 1) >> 2;
   const float4* units = reinterpret_cast<const float4*>(U - phase);
   auto load = [&](int q, float (&x)[4]) {
-    const float4 v = __ldg(units + min(max(q, 0), last));
-    x[0] = v.x, x[1] = v.y, x[2] = v.z, x[3] = v.w;
+    if (q > 0 && q < last) {
+      const float4 v = __ldg(units + q);
+      x[0] = v.x, x[1] = v.y, x[2] = v.z, x[3] = v.w;
+    } else {  // the ends, which may lie inside a unit
+#pragma unroll
+      for (int c = 0; c < 4; ++c) x[c] = __ldg(U + min(max(4 * q - phase + c, 0), P - 1));
+    }
   };
   int cnt = 0;
   float prev[4] = {}, u[4], nxt[4], ahead[4];
